@@ -4,18 +4,22 @@
 // acc = fma(a_d - b_d, a_d - b_d, acc).  That exact operation sequence is kept whatever the
 // tiling, so the order of neighbours does not depend on how the work is split.
 //
-// Small D (<= 32): one CTA per code computes its V keys straight into shared memory.
-// Large D: a tiled SIMT kernel writes the keys of a block of rows to global scratch (each
-// (i, j) accumulator still runs over d in order), and the per-row CTA reads its row of keys.
-// Per row (the code itself excluded; it goes to slot 0): the keys' range, one 2048-bin histogram of
-// the top 11 bits of key - min, the bin that holds the (k-1)-th smallest key and every bin's offset
-// by one block scan, then a counting sort -- the index of every key up to that bin is scattered to
-// its bin's place, ranked inside its bin by (key, index), and stored at its final position, so that
-// ties at the threshold are taken by smaller index.  A row in which one of those bins holds more
-// than 256 keys (massive ties, an outlier that stretches the range) takes the general path:
-// further histogram passes down to the exact threshold key, compaction of the selected
-// (key, index) pairs, bitonic sort of the 64-bit composites.
+// Small D (<= 32): a CTA takes R codes (rows of the table) at once and computes their keys against the
+// whole codebook, two rows to a packed fp32 instruction.  Large D: a tiled SIMT kernel writes the keys
+// of all pairs to global scratch first (each (i, j) accumulator still runs over d in order), and the same row
+// kernel reads them from there.
+//
+// Selection per row.  Only about k of the V keys matter, so no pass but the first looks at the others:
+//   1. a sample of 1024 keys gives a bound t below which, with room to spare, the k smallest lie;
+//   2. one pass over all keys keeps those <= t (composites key << 32 | index + 1; the code itself, 0);
+//   3. the keep list -- some 1.5 k entries -- is counting-sorted into 1024 bins of equal width, every entry
+//      ranked inside its bin by (key, index) and stored at its final position, so that ties are taken
+//      by smaller index.
+// A row whose sample misled (fewer than k kept, or more than fit) or whose keys crowd a bin (massive ties)
+// takes the general path: radix select down to the exact threshold key over all V keys, compaction, bitonic
+// sort of the composites.
 #include <cuda_runtime.h>
+#include <math.h>
 #include <stdint.h>
 
 #include "lantern.h"
@@ -23,21 +27,26 @@
 
 namespace lantern {
 
-constexpr int BT = 512;          // threads of the per-row kernel
-constexpr int BW = BT / 32;
+constexpr int KT = 1024;         // threads of the row kernel: one CTA per SM
+constexpr int KW = KT / 32;
 constexpr int SMALL_D = 32;
 constexpr int TM = 128;          // distance tile edge (rows and columns of one CTA)
 constexpr int DK = 16;           // dimensions staged per step
-constexpr int HB = 11;           // radix-select digit: 2048 bins, kept in the (still unused) list area
+constexpr int HB = 11;           // general path: radix-select digit, 2048 bins, kept in the (still unused) list area
 constexpr int HBINS = 1 << HB;
-constexpr int FAST_POP = 256;    // largest bin the counting-sort path ranks by pairwise comparison
+constexpr int SAMPLE = 1024;     // keys sampled per row
+constexpr int NBINS = 1024;      // bins of the counting sort
+constexpr int CROWD = 256;       // largest bin that is ranked by pairwise comparison
+static_assert(SAMPLE <= NBINS, "the sample is kept where the bins will be");
 
 struct BuildParams {
   const float* codebook;
-  const uint32_t* scratch;       // [rows, V] key bits of rows row0.. (large-D path), else null
+  const uint32_t* scratch;       // [V, V] key bits of all pairs (large-D path), else null
   int32_t* idx;
   float* dist;
-  int V, D, k, row0;
+  int V, D, k;
+  int cap;                       // entries of a row's keep list
+  int want;                      // rank in the sample that bounds the k smallest keys; 0 = keep everything (cap = V)
 };
 
 // Two fp32 lanes in one 64-bit register; each lane of the packed operations rounds exactly like the
@@ -59,10 +68,14 @@ __device__ __forceinline__ unsigned long long fma2(unsigned long long a, unsigne
 }
 
 // ---------------------------------------------------------------------------------------
-// keys of a block of rows, large D: a 128 x 128 tile per CTA, 8 x 8 accumulators per thread
+// keys of all pairs, large D: a 128 x 128 tile per CTA, 8 x 8 accumulators per thread
 // (rows ty*4.. and 64+ty*4.., columns tx*4.. and 64+tx*4.., so that every shared-memory read is
 // one conflict-free 16-byte load), the next 16 dimensions fetched into registers while the
 // current ones are used.  Every (i, j) accumulator still runs over d in order.
+//
+// (a - b)^2 and (b - a)^2 round alike, so key(j, i) = key(i, j) to the bit: only the tiles on and above the
+// diagonal are computed, and every tile is stored a second time transposed.  The kernel is bound by the fp32
+// pipes (two operations per pair and dimension).
 // ---------------------------------------------------------------------------------------
 __device__ __forceinline__ float4 fetch_quad(const float* __restrict__ cb, int row, int row_end, int D, int d, bool vec) {
   float4 v = make_float4(0.0f, 0.0f, 0.0f, 0.0f);   // zero padding adds fma(0, 0, acc) = acc exactly
@@ -81,12 +94,16 @@ __device__ __forceinline__ float4 fetch_quad(const float* __restrict__ cb, int r
 }
 
 __global__ void __launch_bounds__(256, 2) lantern_distance_tile_kernel(const float* __restrict__ cb, uint32_t* out, int V,
-                                                                       int D, int row0, int rows) {
+                                                                       int D) {
   __shared__ __align__(16) float As[DK][TM];
   __shared__ __align__(16) float Bs[DK][TM];
   const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
-  const int rbase = row0 + blockIdx.y * TM, cbase = blockIdx.x * TM;
-  const int row_end = (row0 + rows < V) ? row0 + rows : V;
+  // tile (tr, tc) with tr <= tc, numbered column by column: tc (tc + 1) / 2 + tr
+  int tc = static_cast<int>((sqrtf(8.0f * static_cast<float>(blockIdx.x) + 1.0f) - 1.0f) * 0.5f);
+  while (tc * (tc + 1) / 2 > static_cast<int>(blockIdx.x)) --tc;
+  while ((tc + 1) * (tc + 2) / 2 <= static_cast<int>(blockIdx.x)) ++tc;
+  const int tr = blockIdx.x - tc * (tc + 1) / 2;
+  const int rbase = tr * TM, cbase = tc * TM;
   const bool vec = (D & 3) == 0;
   unsigned long long acc[8][4];
 #pragma unroll
@@ -98,7 +115,7 @@ __global__ void __launch_bounds__(256, 2) lantern_distance_tile_kernel(const flo
   float4 ra[2], rb[2];
 #pragma unroll
   for (int l = 0; l < 2; ++l) {
-    ra[l] = fetch_quad(cb, rbase + srow, row_end, D, 4 * (squad + 2 * l), vec);
+    ra[l] = fetch_quad(cb, rbase + srow, V, D, 4 * (squad + 2 * l), vec);
     rb[l] = fetch_quad(cb, cbase + srow, V, D, 4 * (squad + 2 * l), vec);
   }
   for (int d0 = 0; d0 < D; d0 += DK) {
@@ -118,7 +135,7 @@ __global__ void __launch_bounds__(256, 2) lantern_distance_tile_kernel(const flo
     if (d0 + DK < D) {
 #pragma unroll
       for (int l = 0; l < 2; ++l) {
-        ra[l] = fetch_quad(cb, rbase + srow, row_end, D, d0 + DK + 4 * (squad + 2 * l), vec);
+        ra[l] = fetch_quad(cb, rbase + srow, V, D, d0 + DK + 4 * (squad + 2 * l), vec);
         rb[l] = fetch_quad(cb, cbase + srow, V, D, d0 + DK + 4 * (squad + 2 * l), vec);
       }
     }
@@ -143,25 +160,36 @@ __global__ void __launch_bounds__(256, 2) lantern_distance_tile_kernel(const flo
     __syncthreads();
   }
   const bool vec_out = (V & 3) == 0;
+  auto store4 = [&](int row, int col, uint32_t w0, uint32_t w1, uint32_t w2, uint32_t w3) {
+    if (row >= V) return;
+    uint32_t* o = out + static_cast<size_t>(row) * V + col;
+    if (vec_out && col + 3 < V) {
+      *reinterpret_cast<uint4*>(o) = make_uint4(w0, w1, w2, w3);
+    } else {
+      if (col < V) o[0] = w0;
+      if (col + 1 < V) o[1] = w1;
+      if (col + 2 < V) o[2] = w2;
+      if (col + 3 < V) o[3] = w3;
+    }
+  };
+  auto lo = [](unsigned long long v) { return static_cast<uint32_t>(v); };
+  auto hi = [](unsigned long long v) { return static_cast<uint32_t>(v >> 32); };
 #pragma unroll
   for (int r = 0; r < 8; ++r) {
-    const int gr = rbase + (r < 4 ? ty * 4 + r : 64 + ty * 4 + (r - 4));
-    if (gr >= row_end) continue;
-    uint32_t* orow = out + static_cast<size_t>(gr - row0) * V;
+    const int row = rbase + (r < 4 ? ty * 4 + r : 64 + ty * 4 + (r - 4));
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      const int gc = cbase + 64 * h + tx * 4;
-      const unsigned long long p0 = acc[r][2 * h], p1 = acc[r][2 * h + 1];
-      const uint32_t w[4] = {static_cast<uint32_t>(p0), static_cast<uint32_t>(p0 >> 32), static_cast<uint32_t>(p1),
-                             static_cast<uint32_t>(p1 >> 32)};
-      if (vec_out && gc + 3 < V) {
-        *reinterpret_cast<uint4*>(orow + gc) = make_uint4(w[0], w[1], w[2], w[3]);
-      } else {
+    for (int h = 0; h < 2; ++h)
+      store4(row, cbase + 64 * h + tx * 4, lo(acc[r][2 * h]), hi(acc[r][2 * h]), lo(acc[r][2 * h + 1]), hi(acc[r][2 * h + 1]));
+  }
+  if (tr != tc) {   // the mirror image: the two rows of threads of a warp fill one 32-byte sector per column
 #pragma unroll
-        for (int c = 0; c < 4; ++c)
-          if (gc + c < V) orow[gc + c] = w[c];
+    for (int c = 0; c < 4; ++c)
+#pragma unroll
+      for (int g = 0; g < 2; ++g) {
+        const int col = rbase + 64 * g + ty * 4, row = cbase + (c < 2 ? tx * 4 + 2 * c : 64 + tx * 4 + 2 * (c - 2));
+        store4(row, col, lo(acc[4 * g][c]), lo(acc[4 * g + 1][c]), lo(acc[4 * g + 2][c]), lo(acc[4 * g + 3][c]));
+        store4(row + 1, col, hi(acc[4 * g][c]), hi(acc[4 * g + 1][c]), hi(acc[4 * g + 2][c]), hi(acc[4 * g + 3][c]));
       }
-    }
   }
 }
 
@@ -200,96 +228,71 @@ __device__ __forceinline__ void bitonic_block64(unsigned long long* list, int bl
   list[e1] = x1;
 }
 
-__global__ void __launch_bounds__(BT) lantern_knn_row_kernel(BuildParams P, int P2 /* pow2 >= max(k-1, 64) */) {
-  extern __shared__ __align__(16) unsigned char dsm[];
+// squared distance of codes i (already in `ai`) and j, in the canonical operation sequence
+__device__ __forceinline__ float key_of(const float* ai, const float* __restrict__ b, int D, bool vec) {
+  float acc = 0.0f;
+  if (vec) {
+    for (int d = 0; d < D; d += 4) {
+      const float4 v = __ldg(reinterpret_cast<const float4*>(b + d));
+      float t = __fsub_rn(ai[d], v.x);
+      acc = __fmaf_rn(t, t, acc);
+      t = __fsub_rn(ai[d + 1], v.y);
+      acc = __fmaf_rn(t, t, acc);
+      t = __fsub_rn(ai[d + 2], v.z);
+      acc = __fmaf_rn(t, t, acc);
+      t = __fsub_rn(ai[d + 3], v.w);
+      acc = __fmaf_rn(t, t, acc);
+    }
+  } else {
+    for (int d = 0; d < D; ++d) {
+      const float t = __fsub_rn(ai[d], __ldg(b + d));
+      acc = __fmaf_rn(t, t, acc);
+    }
+  }
+  return acc;
+}
+
+struct GeneralShared {
+  int wcnt[KW];
+  uint32_t wmin[KW], wmax[KW];
+  float ai[SMALL_D];
+  int s_digit, s_below, s_ties, s_cnt;
+};
+
+// The general path for row i, by the whole CTA: dsm = V keys, then the list of P2 composites.
+__device__ __noinline__ void knn_row_general(const BuildParams& P, int i, int P2, unsigned char* dsm, GeneralShared& S) {
   uint32_t* keys = reinterpret_cast<uint32_t*>(dsm);                                  // [V]
   unsigned long long* list =
       reinterpret_cast<unsigned long long*>(dsm + ((static_cast<size_t>(P.V) * 4 + 15) & ~size_t(15)));  // [P2]
-  // [HBINS] 16-bit counters, two to a word (a row has fewer than 65536 keys); used before the list is filled
-  unsigned* hist = reinterpret_cast<unsigned*>(list);
-  unsigned short* list16 = reinterpret_cast<unsigned short*>(hist + HBINS / 2);   // [k - 1 + FAST_POP] indices, fast path
+  unsigned* hist = reinterpret_cast<unsigned*>(list);   // [HBINS] 16-bit counters, two to a word; used before the list is filled
   auto bin_count = [hist](int b) { return static_cast<int>((hist[b >> 1] >> ((b & 1) << 4)) & 0xffffu); };
-  __shared__ int wcnt[BW];
-  __shared__ uint32_t wmin[BW], wmax[BW];
-  __shared__ float ai[SMALL_D];
-  __shared__ int s_digit, s_below, s_ties, s_cnt;
-
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int V = P.V, D = P.D, K = P.k - 1;
-  const int i = P.row0 + blockIdx.x;
 
   // ---- keys (and their range over j != i) ----
   uint32_t kmin = 0xffffffffu, kmax = 0u;
-  if (P.scratch) {
-    const uint32_t* src = P.scratch + static_cast<size_t>(blockIdx.x) * V;
-    for (int j = tid; j < V; j += BT) {
-      const uint32_t key = src[j];
-      keys[j] = key;
-      if (j != i) {
-        kmin = key < kmin ? key : kmin;
-        kmax = key > kmax ? key : kmax;
-      }
-    }
-  } else {
-    if (tid < D) ai[tid] = P.codebook[static_cast<size_t>(i) * D + tid];
-    __syncthreads();
-    if ((D & 3) == 0) {
-      for (int j = tid; j < V; j += BT) {
-        const float4* b = reinterpret_cast<const float4*>(P.codebook + static_cast<size_t>(j) * D);
-        float acc = 0.0f;
-        for (int d = 0; d < D; d += 4) {
-          const float4 v = __ldg(b + (d >> 2));
-          float t = __fsub_rn(ai[d], v.x);
-          acc = __fmaf_rn(t, t, acc);
-          t = __fsub_rn(ai[d + 1], v.y);
-          acc = __fmaf_rn(t, t, acc);
-          t = __fsub_rn(ai[d + 2], v.z);
-          acc = __fmaf_rn(t, t, acc);
-          t = __fsub_rn(ai[d + 3], v.w);
-          acc = __fmaf_rn(t, t, acc);
-        }
-        const uint32_t key = __float_as_uint(acc);
-        keys[j] = key;
-        if (j != i) {
-          kmin = key < kmin ? key : kmin;
-          kmax = key > kmax ? key : kmax;
-        }
-      }
-    } else {
-      for (int j = tid; j < V; j += BT) {
-        const float* b = P.codebook + static_cast<size_t>(j) * D;
-        float acc = 0.0f;
-        for (int d = 0; d < D; ++d) {
-          const float t = __fsub_rn(ai[d], __ldg(b + d));
-          acc = __fmaf_rn(t, t, acc);
-        }
-        const uint32_t key = __float_as_uint(acc);
-        keys[j] = key;
-        if (j != i) {
-          kmin = key < kmin ? key : kmin;
-          kmax = key > kmax ? key : kmax;
-        }
-      }
+  if (!P.scratch && tid < D) S.ai[tid] = P.codebook[static_cast<size_t>(i) * D + tid];
+  __syncthreads();
+  for (int j = tid; j < V; j += KT) {
+    const uint32_t key = P.scratch ? P.scratch[static_cast<size_t>(i) * V + j]
+                                   : __float_as_uint(key_of(S.ai, P.codebook + static_cast<size_t>(j) * D, D, (D & 3) == 0));
+    keys[j] = key;
+    if (j != i) {
+      kmin = key < kmin ? key : kmin;
+      kmax = key > kmax ? key : kmax;
     }
   }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    const uint32_t a = __shfl_xor_sync(kFull, kmin, o), b = __shfl_xor_sync(kFull, kmax, o);
-    kmin = a < kmin ? a : kmin;
-    kmax = b > kmax ? b : kmax;
-  }
+  kmin = __reduce_min_sync(kFull, kmin);
+  kmax = __reduce_max_sync(kFull, kmax);
   if (lane == 0) {
-    wmin[warp] = kmin;
-    wmax[warp] = kmax;
+    S.wmin[warp] = kmin;
+    S.wmax[warp] = kmax;
   }
-  if (tid == 0) s_cnt = 0;
+  if (tid == 0) S.s_cnt = 0;
   __syncthreads();
   const uint32_t self_key = keys[i];
-#pragma unroll
-  for (int w = 0; w < BW; ++w) {
-    kmin = wmin[w] < kmin ? wmin[w] : kmin;
-    kmax = wmax[w] > kmax ? wmax[w] : kmax;
-  }
+  kmin = __reduce_min_sync(kFull, S.wmin[lane]);
+  kmax = __reduce_max_sync(kFull, S.wmax[lane]);
 
   if (K > 0) {
     // ---- radix select on rel = key - kmin, 11 bits at a time from the top of the occupied range:
@@ -298,13 +301,12 @@ __global__ void __launch_bounds__(BT) lantern_knn_row_kernel(BuildParams P, int 
     int hi = range ? 32 - __clz(range) : 0;
     uint32_t prefix = 0;
     int need = K, ties_total = V - 1;
-    bool first_pass = true;
     while (hi > 0) {
       const int lo = hi > HB ? hi - HB : 0;
       const uint32_t dmask = (1u << (hi - lo)) - 1u;
-      for (int t = tid; t < HBINS / 2; t += BT) hist[t] = 0u;
+      for (int t = tid; t < HBINS / 2; t += KT) hist[t] = 0u;
       __syncthreads();
-      for (int j = tid; j < V; j += BT) {
+      for (int j = tid; j < V; j += KT) {
         const uint32_t rel = keys[j] - kmin;
         if (j != i && (hi >= 32 || (rel >> hi) == (prefix >> hi))) {
           const uint32_t b = (rel >> lo) & dmask;
@@ -312,10 +314,10 @@ __global__ void __launch_bounds__(BT) lantern_knn_row_kernel(BuildParams P, int 
         }
       }
       __syncthreads();
-      int loc[HBINS / BT], s = 0;
+      int loc[HBINS / KT], s = 0;
 #pragma unroll
-      for (int q = 0; q < HBINS / BT; ++q) {
-        loc[q] = bin_count(tid * (HBINS / BT) + q);
+      for (int q = 0; q < HBINS / KT; ++q) {
+        loc[q] = bin_count(tid * (HBINS / KT) + q);
         s += loc[q];
       }
       int incl = s;
@@ -324,79 +326,26 @@ __global__ void __launch_bounds__(BT) lantern_knn_row_kernel(BuildParams P, int 
         const int t = __shfl_up_sync(kFull, incl, o);
         if (lane >= o) incl += t;
       }
-      if (lane == 31) wcnt[warp] = incl;
+      if (lane == 31) S.wcnt[warp] = incl;
       __syncthreads();
       int excl = incl - s;
-#pragma unroll
-      for (int w = 0; w < BW; ++w)
-        if (w < warp) excl += wcnt[w];
+      for (int w = 0; w < warp; ++w) excl += S.wcnt[w];
       if (excl < need && need <= excl + s) {   // exactly one thread
         int run = excl;
 #pragma unroll
-        for (int q = 0; q < HBINS / BT; ++q) {
+        for (int q = 0; q < HBINS / KT; ++q) {
           if (run < need && need <= run + loc[q]) {
-            s_digit = tid * (HBINS / BT) + q;
-            s_below = run;
-            s_ties = loc[q];
+            S.s_digit = tid * (HBINS / KT) + q;
+            S.s_below = run;
+            S.s_ties = loc[q];
           }
           run += loc[q];
         }
       }
       __syncthreads();
-      if (first_pass) {
-        // Common case: no bin up to the one that holds the K-th key is crowded.  The prefix sums of the
-        // histogram are then the places of a counting sort by bin: scatter the indices of those keys,
-        // rank every key inside its bin by (key, index), and store it at its final place.
-        first_pass = false;
-        const int digit = s_digit, n_cand = s_below + s_ties;
-        bool crowded = false;
-#pragma unroll
-        for (int q = 0; q < HBINS / BT; ++q) crowded |= (tid * (HBINS / BT) + q <= digit) && loc[q] > FAST_POP;
-        if (!__syncthreads_or(crowded)) {
-          // own words only: each counter becomes its bin's cursor (offsets stay below 65536; bins past `digit`
-          // are never advanced)
-          static_assert(HBINS / BT == 4, "a thread owns two words of counters");
-          hist[2 * tid] = static_cast<unsigned>(excl) | (static_cast<unsigned>(excl + loc[0]) << 16);
-          hist[2 * tid + 1] = static_cast<unsigned>(excl + loc[0] + loc[1]) |
-                              (static_cast<unsigned>(excl + loc[0] + loc[1] + loc[2]) << 16);
-          __syncthreads();
-          for (int j = tid; j < V; j += BT) {
-            const int b = static_cast<int>((keys[j] - kmin) >> lo);
-            if (j != i && b <= digit) {
-              const int sh = (b & 1) << 4;
-              const unsigned old = atomicAdd(&hist[b >> 1], 1u << sh);
-              list16[(old >> sh) & 0xffffu] = static_cast<unsigned short>(j);
-            }
-          }
-          __syncthreads();   // every cursor now holds the end of its bin = the start of the next
-          int32_t* irow = P.idx + static_cast<size_t>(i) * P.k;
-          float* drow = P.dist ? P.dist + static_cast<size_t>(i) * P.k : nullptr;
-          if (tid == 0) {
-            irow[0] = i;
-            if (drow) drow[0] = __uint_as_float(self_key);
-          }
-          for (int t = tid; t < n_cand; t += BT) {
-            const unsigned j = list16[t];
-            const uint32_t key = keys[j];
-            const int b = static_cast<int>((key - kmin) >> lo);
-            const int start = b ? bin_count(b - 1) : 0, end = bin_count(b);
-            const unsigned long long comp = (static_cast<unsigned long long>(key) << 32) | j;
-            int rank = start;
-            for (int u = start; u < end; ++u) {
-              const unsigned ju = list16[u];
-              rank += ((static_cast<unsigned long long>(keys[ju]) << 32) | ju) < comp;
-            }
-            if (rank < K) {   // in the last bin: the `need` smallest, ties by smaller index
-              irow[1 + rank] = static_cast<int32_t>(j);
-              if (drow) drow[1 + rank] = __uint_as_float(key);
-            }
-          }
-          return;
-        }
-      }
-      need -= s_below;
-      ties_total = s_ties;
-      prefix |= static_cast<uint32_t>(s_digit) << lo;
+      need -= S.s_below;
+      ties_total = S.s_ties;
+      prefix |= static_cast<uint32_t>(S.s_digit) << lo;
       hi = lo;
     }
     __syncthreads();   // the histogram's storage becomes the list
@@ -405,33 +354,28 @@ __global__ void __launch_bounds__(BT) lantern_knn_row_kernel(BuildParams P, int 
 
     // ---- compaction (one counter update per warp) ----
     const bool all_ties = (ties_total == need);
-    for (int base = 0; base < V; base += BT) {
+    for (int base = 0; base < V; base += KT) {
       const int j = base + tid;
       const uint32_t key = j < V ? keys[j] : 0u;
       const bool sel = j < V && j != i && (key < tau || (all_ties && key == tau));
       const unsigned bal = __ballot_sync(kFull, sel);
       if (bal) {
         int pos = 0;
-        if (lane == 0) pos = atomicAdd(&s_cnt, __popc(bal));
+        if (lane == 0) pos = atomicAdd(&S.s_cnt, __popc(bal));
         pos = __shfl_sync(kFull, pos, 0) + __popc(bal & ((1u << lane) - 1u));
         if (sel) list[pos] = (static_cast<unsigned long long>(key) << 32) | static_cast<unsigned>(j);
       }
     }
     if (!all_ties) {   // more ties than places: take them in index order
       int run = 0;
-      for (int base = 0; base < V && run < need; base += BT) {
+      for (int base = 0; base < V && run < need; base += KT) {
         const int j = base + tid;
         const bool flag = j < V && j != i && keys[j] == tau;
         const unsigned bal = __ballot_sync(kFull, flag);
-        if (lane == 0) wcnt[warp] = __popc(bal);
+        if (lane == 0) S.wcnt[warp] = __popc(bal);
         __syncthreads();
-        int before = 0, chunk = 0;
-#pragma unroll
-        for (int w = 0; w < BW; ++w) {
-          const int c = wcnt[w];
-          if (w < warp) before += c;
-          chunk += c;
-        }
+        const int c = S.wcnt[lane];
+        const int before = __reduce_add_sync(kFull, lane < warp ? c : 0), chunk = __reduce_add_sync(kFull, c);
         const int rank = run + before + __popc(bal & ((1u << lane) - 1u));
         if (flag && rank < need)
           list[n_less + rank] = (static_cast<unsigned long long>(tau) << 32) | static_cast<unsigned>(j);
@@ -439,16 +383,16 @@ __global__ void __launch_bounds__(BT) lantern_knn_row_kernel(BuildParams P, int 
         __syncthreads();
       }
     }
-    for (int t = K + tid; t < P2; t += BT) list[t] = ~0ull;
+    for (int t = K + tid; t < P2; t += KT) list[t] = ~0ull;
     __syncthreads();
 
     // ---- bitonic sort of (key, index) composites: strides below 64 in registers by shuffles ----
     const int nblk = P2 >> 6;
-    for (int blk = warp; blk < nblk; blk += BW) bitonic_block64(list, blk, lane, 2, 64);
+    for (int blk = warp; blk < nblk; blk += KW) bitonic_block64(list, blk, lane, 2, 64);
     __syncthreads();
     for (int size = 128; size <= P2; size <<= 1) {
       for (int stride = size >> 1; stride >= 64; stride >>= 1) {
-        for (int t = tid; t < (P2 >> 1); t += BT) {
+        for (int t = tid; t < (P2 >> 1); t += KT) {
           const int lo = ((t & ~(stride - 1)) << 1) | (t & (stride - 1));
           const int hi2 = lo | stride;
           const bool up = (lo & size) == 0;
@@ -460,7 +404,7 @@ __global__ void __launch_bounds__(BT) lantern_knn_row_kernel(BuildParams P, int 
         }
         __syncthreads();
       }
-      for (int blk = warp; blk < nblk; blk += BW) bitonic_block64(list, blk, lane, size, size);
+      for (int blk = warp; blk < nblk; blk += KW) bitonic_block64(list, blk, lane, size, size);
       __syncthreads();
     }
   }
@@ -472,11 +416,301 @@ __global__ void __launch_bounds__(BT) lantern_knn_row_kernel(BuildParams P, int 
     irow[0] = i;
     if (drow) drow[0] = __uint_as_float(self_key);
   }
-  for (int t = tid; t < K; t += BT) {
+  for (int t = tid; t < K; t += KT) {
     const unsigned long long c = list[t];
     irow[1 + t] = static_cast<int32_t>(c & 0xffffffffu);
     if (drow) drow[1 + t] = __uint_as_float(static_cast<uint32_t>(c >> 32));
   }
+  __syncthreads();
+}
+
+// bytes of shared memory per row: keep list, order of the list entries by bin, bins
+static __host__ __device__ constexpr size_t row_bytes(int cap) {
+  return ((static_cast<size_t>(cap) * 10 + 15) & ~size_t(15)) + NBINS * 4;
+}
+
+// R rows per CTA; KT / R threads rank a row.
+template <int R, bool SCRATCH>
+__global__ void __launch_bounds__(KT, 1) lantern_knn_rows_kernel(BuildParams P, int P2) {
+  constexpr int RT = KT / R;       // threads of a row's team
+  constexpr int RW = RT / 32;
+  constexpr int U = 2;             // codes per thread and step of the key pass
+  constexpr int OWN = NBINS / RT;  // bins per thread of a team
+  extern __shared__ __align__(16) unsigned char dsm[];
+  __shared__ __align__(16) float As[SMALL_D][R];
+  __shared__ GeneralShared S;
+  __shared__ int s_cnt[R], s_wsum[R][RW], s_slow[R];
+  __shared__ float s_t[R], s_lo[R], s_scale[R];
+  const int tid = threadIdx.x, lane = tid & 31;
+  const int V = P.V, D = P.D, k = P.k, cap = P.cap;
+  const int row0 = blockIdx.x * R;
+  const bool vec = (D & 3) == 0;
+  const size_t per_row = row_bytes(cap);
+  auto list_of = [&](int r) { return reinterpret_cast<unsigned long long*>(dsm + r * per_row); };
+  auto bins_of = [&](int r) { return reinterpret_cast<unsigned*>(dsm + (r + 1) * per_row - NBINS * 4); };
+
+  if (!SCRATCH) {
+    for (int t = tid; t < SMALL_D * R; t += KT) {
+      const int d = t / R, r = t % R;
+      As[d][r] = (d < D && row0 + r < V) ? P.codebook[static_cast<size_t>(row0 + r) * D + d] : 0.0f;
+    }
+  }
+  if (tid < R) s_cnt[tid] = 0, s_slow[tid] = 0;
+  __syncthreads();
+
+  const int r = tid / RT, rt = tid % RT;   // this thread's team and its place in it
+  const int i = row0 + r;
+  // ---- 1. the bound, from SAMPLE keys spread over the codebook by the golden ratio (so that no period of the
+  // code order is sampled in step) ----
+  {
+    float* smp = reinterpret_cast<float*>(bins_of(r));
+    for (int s = rt; s < SAMPLE; s += RT) {
+      const int j = static_cast<int>((static_cast<unsigned long long>(static_cast<uint32_t>(s) * 2654435769u) * static_cast<unsigned>(V)) >> 32);
+      float key = 0.0f;
+      if (SCRATCH) {
+        if (i < V) key = __uint_as_float(P.scratch[static_cast<size_t>(i) * V + j]);
+      } else {
+        const float* b = P.codebook + static_cast<size_t>(j) * D;
+        for (int d = 0; d < D; ++d) {
+          const float t = __fsub_rn(As[d][r], __ldg(b + d));
+          key = __fmaf_rn(t, t, key);
+        }
+      }
+      smp[s] = key;
+    }
+    __syncthreads();
+    if (rt < 32) {   // one warp per row: bisection on the sampled values
+      uint32_t key[SAMPLE / 32], least = 0xffffffffu, most = 0u;
+#pragma unroll
+      for (int q = 0; q < SAMPLE / 32; ++q) {
+        key[q] = __float_as_uint(smp[q * 32 + lane]);
+        least = key[q] < least ? key[q] : least;
+        most = key[q] > most ? key[q] : most;
+      }
+      most = __reduce_max_sync(kFull, most);
+      uint32_t low = 0;
+      for (int q = 0; q < 3; ++q) {   // third smallest of the lanes' minima: where the bins start
+        low = __reduce_min_sync(kFull, least);
+        if (least == low) least = 0xffffffffu;
+      }
+      if (low > most) low = most;     // (fewer than three different minima)
+      uint32_t t = 0x7f800000u;
+      if (P.want > 0) {
+        // count(key <= hi) >= want > count(key <= lo); a few more than wanted will do
+        const int room = P.want / 16 + 2;
+        uint32_t lo = 0u, hi = most;
+        for (int pass = 0; pass < 48 && hi - lo > 1u; ++pass) {
+          uint32_t m = __float_as_uint(0.5f * __uint_as_float(lo) + 0.5f * __uint_as_float(hi));
+          if (!(m > lo && m < hi)) m = lo + ((hi - lo) >> 1);
+          int c0 = 0, c1 = 0;
+#pragma unroll
+          for (int q = 0; q < SAMPLE / 32; q += 2) {
+            c0 += key[q] <= m;
+            c1 += key[q + 1] <= m;
+          }
+          const int c = __reduce_add_sync(kFull, c0 + c1);
+          if (c >= P.want) hi = m;
+          else lo = m;
+          if (c >= P.want && c <= P.want + room) break;
+        }
+        t = hi;
+      }
+      if (lane == 0) {
+        const float lo_f = __uint_as_float(low), hi_f = __uint_as_float(t < most ? t : most);
+        s_t[r] = __uint_as_float(t);
+        s_lo[r] = lo_f;
+        s_scale[r] = hi_f > lo_f ? static_cast<float>(NBINS) / (hi_f - lo_f) : 0.0f;
+      }
+    }
+    __syncthreads();
+  }
+
+  // ---- 2. all keys; those within the bound go to their row's list ----
+  const unsigned below = (1u << lane) - 1u;
+  if (!SCRATCH) {
+    float t_row[R];
+#pragma unroll
+    for (int q = 0; q < R; ++q) t_row[q] = s_t[q];
+    for (int base = 0; base < V; base += U * KT) {
+      unsigned long long acc[U][R / 2];
+      const float* b[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const int j = base + u * KT + tid;
+        b[u] = P.codebook + static_cast<size_t>(j < V ? j : 0) * D;
+#pragma unroll
+        for (int q = 0; q < R / 2; ++q) acc[u][q] = 0ull;
+      }
+      for (int d0 = 0; d0 < D; d0 += 4) {
+        float4 v[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          if (vec) {
+            v[u] = __ldg(reinterpret_cast<const float4*>(b[u] + d0));
+          } else {   // zero padding (As is zero there too) adds fma(0, 0, acc) = acc exactly
+            v[u].x = __ldg(b[u] + d0);
+            v[u].y = d0 + 1 < D ? __ldg(b[u] + d0 + 1) : 0.0f;
+            v[u].z = d0 + 2 < D ? __ldg(b[u] + d0 + 2) : 0.0f;
+            v[u].w = d0 + 3 < D ? __ldg(b[u] + d0 + 3) : 0.0f;
+          }
+        }
+#pragma unroll
+        for (int dd = 0; dd < 4; ++dd) {
+          unsigned long long a2[R / 2];
+#pragma unroll
+          for (int q = 0; q < R / 2; ++q) a2[q] = *reinterpret_cast<const unsigned long long*>(&As[d0 + dd][2 * q]);
+#pragma unroll
+          for (int u = 0; u < U; ++u) {
+            const unsigned long long bb = dup2(dd == 0 ? v[u].x : (dd == 1 ? v[u].y : (dd == 2 ? v[u].z : v[u].w)));
+#pragma unroll
+            for (int q = 0; q < R / 2; ++q) {
+              const unsigned long long t = sub2(a2[q], bb);
+              acc[u][q] = fma2(t, t, acc[u][q]);
+            }
+          }
+        }
+      }
+      // one counter update per row and warp
+      unsigned bal[U][R];
+      int mine = 0;
+#pragma unroll
+      for (int q = 0; q < R; ++q) {
+        int n = 0;
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          const uint32_t key = static_cast<uint32_t>(q & 1 ? acc[u][q / 2] >> 32 : acc[u][q / 2]);
+          bal[u][q] = __ballot_sync(kFull, base + u * KT + tid < V && __uint_as_float(key) <= t_row[q]);
+          n += __popc(bal[u][q]);
+        }
+        if (lane == q) mine = n;
+      }
+      int start = 0;
+      if (lane < R && mine) start = atomicAdd(&s_cnt[lane], mine);
+#pragma unroll
+      for (int q = 0; q < R; ++q) {
+        int pos = __shfl_sync(kFull, start, q);
+        unsigned long long* list = list_of(q);
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          const uint32_t key = static_cast<uint32_t>(q & 1 ? acc[u][q / 2] >> 32 : acc[u][q / 2]);
+          const int at = pos + __popc(bal[u][q] & below);
+          if (((bal[u][q] >> lane) & 1u) && at < cap)
+            list[at] = (static_cast<unsigned long long>(key) << 32) | static_cast<unsigned>(base + u * KT + tid + 1);
+          pos += __popc(bal[u][q]);
+        }
+      }
+    }
+  } else if (i < V) {   // each team reads its own row of keys
+    const uint32_t* src = P.scratch + static_cast<size_t>(i) * V;
+    const float t = s_t[r];
+    unsigned long long* list = list_of(r);
+    const bool vec4 = (V & 3) == 0;
+    for (int base = 0; base < V; base += 4 * RT) {
+      const int j0 = base + 4 * rt;
+      uint32_t key[4] = {0x7fffffffu, 0x7fffffffu, 0x7fffffffu, 0x7fffffffu};   // NaN: never kept
+      if (vec4) {
+        if (j0 < V) {
+          const uint4 v = __ldcs(reinterpret_cast<const uint4*>(src + j0));
+          key[0] = v.x, key[1] = v.y, key[2] = v.z, key[3] = v.w;
+        }
+      } else {
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+          if (j0 + u < V) key[u] = __ldcs(src + j0 + u);
+      }
+      unsigned bal[4];
+      int n = 0;
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        bal[u] = __ballot_sync(kFull, __uint_as_float(key[u]) <= t);
+        n += __popc(bal[u]);
+      }
+      int pos = 0;
+      if (lane == 0 && n) pos = atomicAdd(&s_cnt[r], n);
+      pos = __shfl_sync(kFull, pos, 0);
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int at = pos + __popc(bal[u] & below);
+        if (((bal[u] >> lane) & 1u) && at < cap)
+          list[at] = (static_cast<unsigned long long>(key[u]) << 32) | static_cast<unsigned>(j0 + u + 1);
+        pos += __popc(bal[u]);
+      }
+    }
+  }
+  __syncthreads();
+
+  // ---- 3. counting sort and ranking, a team per row ----
+  if (i < V) {
+    auto team = [&]() { asm volatile("bar.sync %0, %1;" ::"r"(1 + r), "n"(RT) : "memory"); };
+    unsigned long long* list = list_of(r);
+    unsigned* bins = bins_of(r);
+    unsigned short* order = reinterpret_cast<unsigned short*>(list + cap);
+    const int n = s_cnt[r];
+    const float lo = s_lo[r], scale = s_scale[r];
+    auto bin_of = [&](unsigned long long c) {   // monotone in the key
+      const float x = (__uint_as_float(static_cast<uint32_t>(c >> 32)) - lo) * scale;
+      return x > 0.0f ? min(static_cast<int>(x), NBINS - 1) : 0;
+    };
+    if (n < k || n > cap) {
+      if (rt == 0) s_slow[r] = 1;
+    } else {
+#pragma unroll
+      for (int q = 0; q < OWN; ++q) bins[q * RT + rt] = 0u;
+      team();
+      for (int e = rt; e < n; e += RT) {
+        unsigned long long c = list[e];
+        if (static_cast<uint32_t>(c) == static_cast<uint32_t>(i + 1)) list[e] = c = 0ull;   // the code itself comes first
+        atomicAdd(&bins[bin_of(c)], 1u);
+      }
+      team();
+      int loc[OWN], s = 0;
+#pragma unroll
+      for (int q = 0; q < OWN; ++q) {
+        loc[q] = static_cast<int>(bins[rt * OWN + q]);
+        s += loc[q];
+      }
+      int incl = s;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int t = __shfl_up_sync(kFull, incl, o);
+        if (lane >= o) incl += t;
+      }
+      if (lane == 31) s_wsum[r][rt >> 5] = incl;
+      team();
+      int at = incl - s;
+#pragma unroll
+      for (int w = 0; w < RW; ++w)
+        if (w < (rt >> 5)) at += s_wsum[r][w];
+#pragma unroll
+      for (int q = 0; q < OWN; ++q) {
+        bins[rt * OWN + q] = static_cast<unsigned>(at);   // every count becomes its bin's cursor
+        if (loc[q] > CROWD && at < k) s_slow[r] = 1;
+        at += loc[q];
+      }
+      team();
+      if (!s_slow[r]) {
+        for (int e = rt; e < n; e += RT) order[atomicAdd(&bins[bin_of(list[e])], 1u)] = static_cast<unsigned short>(e);
+        team();   // every cursor now holds the end of its bin = the start of the next
+        int32_t* irow = P.idx + static_cast<size_t>(i) * k;
+        float* drow = P.dist ? P.dist + static_cast<size_t>(i) * k : nullptr;
+        for (int p = rt; p < n; p += RT) {
+          const unsigned long long c = list[order[p]];
+          const int b = bin_of(c);
+          const int start = b ? static_cast<int>(bins[b - 1]) : 0, end = static_cast<int>(bins[b]);
+          if (start >= k) break;
+          int rank = start;
+          for (int u = start; u < end; ++u) rank += list[order[u]] < c;
+          if (rank < k) {
+            irow[rank] = c ? static_cast<int32_t>(static_cast<uint32_t>(c)) - 1 : i;
+            if (drow) drow[rank] = __uint_as_float(static_cast<uint32_t>(c >> 32));
+          }
+        }
+      }
+    }
+  }
+  __syncthreads();
+  for (int q = 0; q < R; ++q)
+    if (s_slow[q]) knn_row_general(P, row0 + q, P2, dsm, S);
 }
 
 static int next_pow2(int x) {
@@ -485,11 +719,15 @@ static int next_pow2(int x) {
   return p;
 }
 
-// Rows whose keys are held in scratch at a time: 64 MB at V = 16384, which the per-row kernel still finds
-// in L2 (1152 rows, which would fill the distance kernel's last wave of CTAs, measured slower).
-static int rows_per_block(int V) {
-  int r = V < 1024 ? V : 1024;
-  return (r + TM - 1) / TM * TM;
+constexpr size_t kRowSmem = 216 * 1024;   // dynamic shared memory of the row kernel, at most
+
+template <int R>
+static cudaError_t launch_rows(const BuildParams& P, int P2, size_t smem, cudaStream_t st) {
+  auto kk = P.scratch ? lantern_knn_rows_kernel<R, true> : lantern_knn_rows_kernel<R, false>;
+  const cudaError_t e = cudaFuncSetAttribute(kk, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+  if (e != cudaSuccess) return e;
+  kk<<<(P.V + R - 1) / R, KT, smem, st>>>(P, P2);
+  return cudaGetLastError();
 }
 
 }  // namespace lantern
@@ -500,7 +738,7 @@ extern "C" size_t lantern_build_workspace_bytes(int V, int D, int k) {
   (void)k;
   if (V < 1 || D < 1) return 0;
   if (D <= SMALL_D) return 0;
-  return static_cast<size_t>(rows_per_block(V)) * V * 4;
+  return static_cast<size_t>(V) * V * 4;   // the keys of all pairs
 }
 
 extern "C" lantern_status lantern_build_neighbors(const float* codebook, int V, int D, int k, int32_t* idx,
@@ -513,40 +751,40 @@ extern "C" lantern_status lantern_build_neighbors(const float* codebook, int V, 
   if (need_ws && (!workspace || workspace_bytes < need_ws || (reinterpret_cast<uintptr_t>(workspace) & 15)))
     return LANTERN_E_WORKSPACE;
   cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
-  const int P2 = next_pow2(k - 1 < 64 ? 64 : k - 1);   // the sort works on whole 64-element blocks
-  const size_t fast_bytes = HBINS * 2 + ((static_cast<size_t>(k - 1 + FAST_POP) * 2 + 15) & ~size_t(15));
-  const size_t list_bytes = static_cast<size_t>(P2) * 8 > fast_bytes ? static_cast<size_t>(P2) * 8 : fast_bytes;
-  const size_t smem = ((static_cast<size_t>(V) * 4 + 15) & ~size_t(15)) + list_bytes;
-  if (smem > 220 * 1024) return LANTERN_E_SHAPE;
-  if (cudaFuncSetAttribute(lantern_knn_row_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024) !=
-      cudaSuccess)
-    return LANTERN_E_CUDA;
+  const int P2 = next_pow2(k - 1 < 64 ? 64 : k - 1);   // the general path's sort works on whole 64-element blocks
+  const size_t list_bytes = static_cast<size_t>(P2) * 8 > HBINS * 2 ? static_cast<size_t>(P2) * 8 : HBINS * 2;
+  const size_t general = ((static_cast<size_t>(V) * 4 + 15) & ~size_t(15)) + list_bytes;
   BuildParams P;
   P.codebook = codebook;
+  P.scratch = D > SMALL_D ? static_cast<const uint32_t*>(workspace) : nullptr;
   P.idx = idx;
   P.dist = dist;
   P.V = V;
   P.D = D;
   P.k = k;
-  if (D <= SMALL_D) {
-    P.scratch = nullptr;
-    P.row0 = 0;
-    lantern_knn_row_kernel<<<V, BT, smem, st>>>(P, P2);
-    return cudaGetLastError() == cudaSuccess ? LANTERN_OK : LANTERN_E_CUDA;
+  // The k-th smallest of V keys has rank k SAMPLE / V in the sample, with a binomial spread; 3.5 standard deviations
+  // above that the bound fails one row in some thousands, and the list is as long as the kept keys may be with the same
+  // margin.  Few codes: the bound would keep most of them anyway.
+  const double f = static_cast<double>(SAMPLE) / V, mean = k * f, sd = sqrt(mean * (1.0 - static_cast<double>(k) / V));
+  const int want = static_cast<int>(mean + 3.5 * sd) + 3, most = want + want / 16 + 2;
+  const double kept = (most + 3.5 * sqrt(static_cast<double>(most))) / f;
+  P.want = (V <= 2 * SAMPLE || kept >= V) ? 0 : want;
+  P.cap = P.want ? (static_cast<int>(kept) + 7) & ~7 : V;
+  // As many rows per CTA as their lists leave room for (eight rows share every load of a code).  The longest list,
+  // 7264 entries at V = 32768 and k = 4097, leaves room for two.
+  const size_t per_row = row_bytes(P.cap);
+  const int R = 8 * per_row <= kRowSmem ? 8 : (4 * per_row <= kRowSmem ? 4 : 2);
+  const size_t smem = R * per_row > general ? R * per_row : general;
+  if (smem > kRowSmem) return LANTERN_E_SHAPE;
+  cudaError_t e = cudaSuccess;
+  if (D > SMALL_D) {
+    const int t = (V + TM - 1) / TM;
+    lantern_distance_tile_kernel<<<t * (t + 1) / 2, 256, 0, st>>>(codebook, static_cast<uint32_t*>(workspace), V, D);
+    e = cudaGetLastError();
+    if (e != cudaSuccess) return LANTERN_E_CUDA;
   }
-  const int rb = rows_per_block(V);
-  uint32_t* scratch = static_cast<uint32_t*>(workspace);
-  for (int row0 = 0; row0 < V; row0 += rb) {
-    const int rows = V - row0 < rb ? V - row0 : rb;
-    dim3 grid((V + TM - 1) / TM, (rows + TM - 1) / TM);
-    lantern_distance_tile_kernel<<<grid, 256, 0, st>>>(codebook, scratch, V, D, row0, rows);
-    if (cudaGetLastError() != cudaSuccess) return LANTERN_E_CUDA;
-    P.scratch = scratch;
-    P.row0 = row0;
-    lantern_knn_row_kernel<<<rows, BT, smem, st>>>(P, P2);
-    if (cudaGetLastError() != cudaSuccess) return LANTERN_E_CUDA;
-  }
-  return LANTERN_OK;
+  e = R == 8 ? launch_rows<8>(P, P2, smem, st) : (R == 4 ? launch_rows<4>(P, P2, smem, st) : launch_rows<2>(P, P2, smem, st));
+  return e == cudaSuccess ? LANTERN_OK : LANTERN_E_CUDA;
 }
 
 // ---------------------------------------------------------------------------------------
