@@ -11,10 +11,9 @@
 //
 // Selection per row.  Only about k of the V keys matter, so no pass but the first looks at the others:
 //   1. a sample of 1024 keys gives a bound t below which, with room to spare, the k smallest lie;
-//   2. one pass over all keys keeps those <= t (composites key << 32 | index + 1; the code itself, 0);
-//   3. the keep list -- some 1.5 k entries -- is counting-sorted into 1024 bins of equal width, every entry
-//      ranked inside its bin by (key, index) and stored at its final position, so that ties are taken
-//      by smaller index.
+//   2. one pass over all keys keeps those <= t (composites key << 32 | index + 1; the code itself: 0);
+//   3. the keep list -- some 1.5 k entries -- is counting-sorted into 2048 bins, in place through registers, every
+//      entry ranked inside its bin and stored at its final position, so that ties are taken by smaller index.
 // A row whose sample misled (fewer than k kept, or more than fit) or whose keys crowd a bin (massive ties)
 // takes the general path: radix select down to the exact threshold key over all V keys, compaction, bitonic
 // sort of the composites.
@@ -27,17 +26,16 @@
 
 namespace lantern {
 
-constexpr int KT = 1024;         // threads of the row kernel: one CTA per SM
-constexpr int KW = KT / 32;
 constexpr int SMALL_D = 32;
 constexpr int TM = 128;          // distance tile edge (rows and columns of one CTA)
 constexpr int DK = 16;           // dimensions staged per step
 constexpr int HB = 11;           // general path: radix-select digit, 2048 bins, kept in the (still unused) list area
 constexpr int HBINS = 1 << HB;
 constexpr int SAMPLE = 1024;     // keys sampled per row
-constexpr int NBINS = 1024;      // bins of the counting sort
-constexpr int CROWD = 256;       // largest bin that is ranked by pairwise comparison
-static_assert(SAMPLE <= NBINS, "the sample is kept where the bins will be");
+constexpr int NBINS = 2048;      // bins of the counting sort, 16-bit counters, two to a word
+constexpr int CROWD = 255;       // largest bin that is ranked by pairwise comparison
+constexpr int KEEP = 18;         // list entries per thread of a row's team, at most
+static_assert(SAMPLE <= NBINS / 2, "the sample is kept where the bins will be");
 
 struct BuildParams {
   const float* codebook;
@@ -75,7 +73,8 @@ __device__ __forceinline__ unsigned long long fma2(unsigned long long a, unsigne
 //
 // (a - b)^2 and (b - a)^2 round alike, so key(j, i) = key(i, j) to the bit: only the tiles on and above the
 // diagonal are computed, and every tile is stored a second time transposed.  The kernel is bound by the fp32
-// pipes (two operations per pair and dimension).
+// pipes (two operations per pair and dimension): 2.19 ms at V = 16384, D = 256 against 1.85 ms at their full rate (all
+// tiles, a block of 1024 rows per launch: 4.6 ms).
 // ---------------------------------------------------------------------------------------
 __device__ __forceinline__ float4 fetch_quad(const float* __restrict__ cb, int row, int row_end, int D, int d, bool vec) {
   float4 v = make_float4(0.0f, 0.0f, 0.0f, 0.0f);   // zero padding adds fma(0, 0, acc) = acc exactly
@@ -253,13 +252,14 @@ __device__ __forceinline__ float key_of(const float* ai, const float* __restrict
 }
 
 struct GeneralShared {
-  int wcnt[KW];
-  uint32_t wmin[KW], wmax[KW];
+  int wcnt[32];
+  uint32_t wmin[32], wmax[32];
   float ai[SMALL_D];
   int s_digit, s_below, s_ties, s_cnt;
 };
 
 // The general path for row i, by the whole CTA: dsm = V keys, then the list of P2 composites.
+template <int KT>
 __device__ __noinline__ void knn_row_general(const BuildParams& P, int i, int P2, unsigned char* dsm, GeneralShared& S) {
   uint32_t* keys = reinterpret_cast<uint32_t*>(dsm);                                  // [V]
   unsigned long long* list =
@@ -268,6 +268,7 @@ __device__ __noinline__ void knn_row_general(const BuildParams& P, int i, int P2
   auto bin_count = [hist](int b) { return static_cast<int>((hist[b >> 1] >> ((b & 1) << 4)) & 0xffffu); };
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int V = P.V, D = P.D, K = P.k - 1;
+  constexpr int KW = KT / 32;
 
   // ---- keys (and their range over j != i) ----
   uint32_t kmin = 0xffffffffu, kmax = 0u;
@@ -291,8 +292,8 @@ __device__ __noinline__ void knn_row_general(const BuildParams& P, int i, int P2
   if (tid == 0) S.s_cnt = 0;
   __syncthreads();
   const uint32_t self_key = keys[i];
-  kmin = __reduce_min_sync(kFull, S.wmin[lane]);
-  kmax = __reduce_max_sync(kFull, S.wmax[lane]);
+  kmin = __reduce_min_sync(kFull, S.wmin[lane & (KW - 1)]);
+  kmax = __reduce_max_sync(kFull, S.wmax[lane & (KW - 1)]);
 
   if (K > 0) {
     // ---- radix select on rel = key - kmin, 11 bits at a time from the top of the occupied range:
@@ -374,7 +375,7 @@ __device__ __noinline__ void knn_row_general(const BuildParams& P, int i, int P2
         const unsigned bal = __ballot_sync(kFull, flag);
         if (lane == 0) S.wcnt[warp] = __popc(bal);
         __syncthreads();
-        const int c = S.wcnt[lane];
+        const int c = lane < KW ? S.wcnt[lane] : 0;
         const int before = __reduce_add_sync(kFull, lane < warp ? c : 0), chunk = __reduce_add_sync(kFull, c);
         const int rank = run + before + __popc(bal & ((1u << lane) - 1u));
         if (flag && rank < need)
@@ -424,30 +425,38 @@ __device__ __noinline__ void knn_row_general(const BuildParams& P, int i, int P2
   __syncthreads();
 }
 
-// bytes of shared memory per row: keep list, order of the list entries by bin, bins
+// bytes of shared memory per row: keep list (and two entries that take what does not fit), bins
 static __host__ __device__ constexpr size_t row_bytes(int cap) {
-  return ((static_cast<size_t>(cap) * 10 + 15) & ~size_t(15)) + NBINS * 4;
+  return ((static_cast<size_t>(cap + 2) * 8 + 15) & ~size_t(15)) + NBINS * 2;
 }
 
-// R rows per CTA; KT / R threads rank a row.
-template <int R, bool SCRATCH>
-__global__ void __launch_bounds__(KT, 1) lantern_knn_rows_kernel(BuildParams P, int P2) {
-  constexpr int RT = KT / R;       // threads of a row's team
+// R rows per CTA of KT threads; KT / R threads rank a row.
+//
+// What bounds it (V = 16384, k = 1000, cycles of a CTA of eight rows, D = 8): the key pass 40 k, of which the fp32
+// pipes need 16 k and instruction issue 24 k; sample and bound 9 k; counting sort 13 k; ranking 11 k.
+// 0.55 ms per table; 1.20 ms when a CTA selected from all keys of one row (73 k warp instructions per row, now 26 k).
+// With scratch keys, D = 256: 0.55 ms, against 0.16 ms that reading the keys takes.
+template <int KT, int R, bool SCRATCH>
+__global__ void __launch_bounds__(KT, 1024 / KT) lantern_knn_rows_kernel(BuildParams P, int P2) {
+  constexpr int RT = KT / R;         // threads of a row's team
   constexpr int RW = RT / 32;
-  constexpr int U = 2;             // codes per thread and step of the key pass
-  constexpr int OWN = NBINS / RT;  // bins per thread of a team
+  constexpr int U = 2;               // codes per thread and step of the key pass
+  constexpr int OWN = NBINS / 2 / RT;   // words of bins per thread of a team
+  constexpr int SMP = SAMPLE / RT;   // sampled keys per thread of a team
   extern __shared__ __align__(16) unsigned char dsm[];
   __shared__ __align__(16) float As[SMALL_D][R];
   __shared__ GeneralShared S;
   __shared__ int s_cnt[R], s_wsum[R][RW], s_slow[R];
   __shared__ float s_t[R], s_lo[R], s_scale[R];
+  __shared__ int s_vote[2][R][RW];
+  __shared__ uint32_t s_low[R][3 * RW], s_most[R][RW];
   const int tid = threadIdx.x, lane = tid & 31;
   const int V = P.V, D = P.D, k = P.k, cap = P.cap;
   const int row0 = blockIdx.x * R;
   const bool vec = (D & 3) == 0;
   const size_t per_row = row_bytes(cap);
   auto list_of = [&](int r) { return reinterpret_cast<unsigned long long*>(dsm + r * per_row); };
-  auto bins_of = [&](int r) { return reinterpret_cast<unsigned*>(dsm + (r + 1) * per_row - NBINS * 4); };
+  auto bins_of = [&](int r) { return reinterpret_cast<unsigned*>(dsm + (r + 1) * per_row - NBINS * 2); };
 
   if (!SCRATCH) {
     for (int t = tid; t < SMALL_D * R; t += KT) {
@@ -460,74 +469,107 @@ __global__ void __launch_bounds__(KT, 1) lantern_knn_rows_kernel(BuildParams P, 
 
   const int r = tid / RT, rt = tid % RT;   // this thread's team and its place in it
   const int i = row0 + r;
+  auto team = [&]() { asm volatile("bar.sync %0, %1;" ::"r"(1 + r), "n"(RT) : "memory"); };
   // ---- 1. the bound, from SAMPLE keys spread over the codebook by the golden ratio (so that no period of the
   // code order is sampled in step) ----
   {
-    float* smp = reinterpret_cast<float*>(bins_of(r));
-    for (int s = rt; s < SAMPLE; s += RT) {
-      const int j = static_cast<int>((static_cast<unsigned long long>(static_cast<uint32_t>(s) * 2654435769u) * static_cast<unsigned>(V)) >> 32);
-      float key = 0.0f;
-      if (SCRATCH) {
-        if (i < V) key = __uint_as_float(P.scratch[static_cast<size_t>(i) * V + j]);
-      } else {
-        const float* b = P.codebook + static_cast<size_t>(j) * D;
-        for (int d = 0; d < D; ++d) {
-          const float t = __fsub_rn(As[d][r], __ldg(b + d));
-          key = __fmaf_rn(t, t, key);
-        }
-      }
-      smp[s] = key;
-    }
-    __syncthreads();
-    if (rt < 32) {   // one warp per row: bisection on the sampled values
-      uint32_t key[SAMPLE / 32], least = 0xffffffffu, most = 0u;
+    auto sampled = [&](int s) {
+      return static_cast<int>((static_cast<unsigned long long>(static_cast<uint32_t>(s) * 2654435769u) * static_cast<unsigned>(V)) >> 32);
+    };
+    uint32_t key[SMP];
+    if constexpr (SCRATCH) {
+      const uint32_t* src = P.scratch + static_cast<size_t>(i < V ? i : 0) * V;
 #pragma unroll
-      for (int q = 0; q < SAMPLE / 32; ++q) {
-        key[q] = __float_as_uint(smp[q * 32 + lane]);
-        least = key[q] < least ? key[q] : least;
-        most = key[q] > most ? key[q] : most;
+      for (int q = 0; q < SMP; ++q) key[q] = __ldg(src + sampled(q * RT + rt));
+    } else {   // every thread takes codes of the sample against all rows of the CTA
+      for (int s = tid; s < SAMPLE; s += KT) {
+        const float* b = P.codebook + static_cast<size_t>(sampled(s)) * D;
+        float acc[R];
+#pragma unroll
+        for (int q = 0; q < R; ++q) acc[q] = 0.0f;
+        auto dim = [&](int d, float v) {
+#pragma unroll
+          for (int q = 0; q < R; ++q) {
+            const float t = __fsub_rn(As[d][q], v);
+            acc[q] = __fmaf_rn(t, t, acc[q]);
+          }
+        };
+        if (vec) {
+          for (int d = 0; d < D; d += 4) {
+            const float4 v = __ldg(reinterpret_cast<const float4*>(b + d));
+            dim(d, v.x), dim(d + 1, v.y), dim(d + 2, v.z), dim(d + 3, v.w);
+          }
+        } else {
+          for (int d = 0; d < D; ++d) dim(d, __ldg(b + d));
+        }
+#pragma unroll
+        for (int q = 0; q < R; ++q) reinterpret_cast<uint32_t*>(bins_of(q))[s] = __float_as_uint(acc[q]);
       }
-      most = __reduce_max_sync(kFull, most);
-      uint32_t low = 0;
-      for (int q = 0; q < 3; ++q) {   // third smallest of the lanes' minima: where the bins start
-        low = __reduce_min_sync(kFull, least);
-        if (least == low) least = 0xffffffffu;
+      __syncthreads();
+#pragma unroll
+      for (int q = 0; q < SMP; ++q) key[q] = bins_of(r)[q * RT + rt];
+    }
+    // where the bins start: about the third smallest of the sample (of the warps' three smallest lane minima)
+    const int wv = rt >> 5;
+    uint32_t least = 0xffffffffu, most = 0u;
+#pragma unroll
+    for (int q = 0; q < SMP; ++q) {
+      least = key[q] < least ? key[q] : least;
+      most = key[q] > most ? key[q] : most;
+    }
+    most = __reduce_max_sync(kFull, most);
+    if (lane == 0) s_most[r][wv] = most;
+    for (int q = 0; q < 3; ++q) {
+      const uint32_t low = __reduce_min_sync(kFull, least);
+      if (lane == 0) s_low[r][3 * wv + q] = low;
+      if (least == low) least = 0xffffffffu;
+    }
+    team();
+    most = 0u;
+#pragma unroll
+    for (int w = 0; w < RW; ++w) most = s_most[r][w] > most ? s_most[r][w] : most;
+    uint32_t t = 0x7f800000u;
+    if (P.want > 0) {
+      // bisection on the sampled values: count(key <= hi) >= want > count(key <= lo); a few more than wanted will do
+      const int room = P.want / 16 + 2;
+      uint32_t lo = 0u, hi = most;
+      for (int pass = 0; pass < 48 && hi - lo > 1u; ++pass) {
+        uint32_t m = __float_as_uint(0.5f * __uint_as_float(lo) + 0.5f * __uint_as_float(hi));
+        if (!(m > lo && m < hi)) m = lo + ((hi - lo) >> 1);
+        int c = 0;
+#pragma unroll
+        for (int q = 0; q < SMP; ++q) c += key[q] <= m;
+        c = __reduce_add_sync(kFull, c);
+        if (lane == 0) s_vote[pass & 1][r][wv] = c;
+        team();
+        c = 0;
+#pragma unroll
+        for (int w = 0; w < RW; ++w) c += s_vote[pass & 1][r][w];
+        if (c >= P.want) hi = m;
+        else lo = m;
+        if (c >= P.want && c <= P.want + room) break;
+      }
+      t = hi;
+    }
+    if (rt < 32) {
+      uint32_t low = 0u, mine = lane < 3 * RW ? s_low[r][lane] : 0xffffffffu;
+      for (int q = 0; q < 3; ++q) {
+        low = __reduce_min_sync(kFull, mine);
+        if (mine == low) mine = 0xffffffffu;
       }
       if (low > most) low = most;     // (fewer than three different minima)
-      uint32_t t = 0x7f800000u;
-      if (P.want > 0) {
-        // count(key <= hi) >= want > count(key <= lo); a few more than wanted will do
-        const int room = P.want / 16 + 2;
-        uint32_t lo = 0u, hi = most;
-        for (int pass = 0; pass < 48 && hi - lo > 1u; ++pass) {
-          uint32_t m = __float_as_uint(0.5f * __uint_as_float(lo) + 0.5f * __uint_as_float(hi));
-          if (!(m > lo && m < hi)) m = lo + ((hi - lo) >> 1);
-          int c0 = 0, c1 = 0;
-#pragma unroll
-          for (int q = 0; q < SAMPLE / 32; q += 2) {
-            c0 += key[q] <= m;
-            c1 += key[q + 1] <= m;
-          }
-          const int c = __reduce_add_sync(kFull, c0 + c1);
-          if (c >= P.want) hi = m;
-          else lo = m;
-          if (c >= P.want && c <= P.want + room) break;
-        }
-        t = hi;
-      }
       if (lane == 0) {
         const float lo_f = __uint_as_float(low), hi_f = __uint_as_float(t < most ? t : most);
         s_t[r] = __uint_as_float(t);
         s_lo[r] = lo_f;
-        s_scale[r] = hi_f > lo_f ? static_cast<float>(NBINS) / (hi_f - lo_f) : 0.0f;
+        s_scale[r] = hi_f > lo_f ? 1.0f / (hi_f - lo_f) : 0.0f;
       }
     }
     __syncthreads();
   }
 
   // ---- 2. all keys; those within the bound go to their row's list ----
-  const unsigned below = (1u << lane) - 1u;
-  if (!SCRATCH) {
+  if constexpr (!SCRATCH) {
     float t_row[R];
 #pragma unroll
     for (int q = 0; q < R; ++q) t_row[q] = s_t[q];
@@ -557,8 +599,15 @@ __global__ void __launch_bounds__(KT, 1) lantern_knn_rows_kernel(BuildParams P, 
 #pragma unroll
         for (int dd = 0; dd < 4; ++dd) {
           unsigned long long a2[R / 2];
+          if (R >= 4) {
 #pragma unroll
-          for (int q = 0; q < R / 2; ++q) a2[q] = *reinterpret_cast<const unsigned long long*>(&As[d0 + dd][2 * q]);
+            for (int q = 0; q < R / 2; q += 2) {
+              const ulonglong2 a = *reinterpret_cast<const ulonglong2*>(&As[d0 + dd][2 * q]);
+              a2[q] = a.x, a2[(q + 1) % (R / 2)] = a.y;
+            }
+          } else {
+            a2[0] = *reinterpret_cast<const unsigned long long*>(&As[d0 + dd][0]);
+          }
 #pragma unroll
           for (int u = 0; u < U; ++u) {
             const unsigned long long bb = dup2(dd == 0 ? v[u].x : (dd == 1 ? v[u].y : (dd == 2 ? v[u].z : v[u].w)));
@@ -570,104 +619,147 @@ __global__ void __launch_bounds__(KT, 1) lantern_knn_rows_kernel(BuildParams P, 
           }
         }
       }
-      // one counter update per row and warp
-      unsigned bal[U][R];
-      int mine = 0;
+      if (base + U * KT > V) {   // codes past the end: NaN, never kept
 #pragma unroll
-      for (int q = 0; q < R; ++q) {
-        int n = 0;
+        for (int u = 0; u < U; ++u)
+          if (base + u * KT + tid >= V) {
 #pragma unroll
-        for (int u = 0; u < U; ++u) {
-          const uint32_t key = static_cast<uint32_t>(q & 1 ? acc[u][q / 2] >> 32 : acc[u][q / 2]);
-          bal[u][q] = __ballot_sync(kFull, base + u * KT + tid < V && __uint_as_float(key) <= t_row[q]);
-          n += __popc(bal[u][q]);
-        }
-        if (lane == q) mine = n;
+            for (int q = 0; q < R / 2; ++q) acc[u][q] = 0x7fffffff7fffffffull;
+          }
       }
+      // How many of this thread's keys each row keeps, four rows to a word (at most U each, 32 U per warp), and a
+      // prefix over the warp; then one counter update per row and warp.  (Ballots and population counts in
+      // their place kept the XU pipe busy for 24 of the pass's 51 thousand cycles.)
+      constexpr int NW = (R + 3) / 4;
+      auto key_of_row = [&](int u, int q) {
+        return __uint_as_float(static_cast<uint32_t>(q & 1 ? acc[u][q / 2] >> 32 : acc[u][q / 2]));
+      };
+      uint32_t cnt[NW] = {}, incl[NW], tot[NW];
+#pragma unroll
+      for (int q = 0; q < R; ++q)
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+          if (key_of_row(u, q) <= t_row[q]) cnt[q / 4] += 1u << (8 * (q % 4));
+#pragma unroll
+      for (int w = 0; w < NW; ++w) {
+        incl[w] = cnt[w];
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+          const uint32_t v = __shfl_up_sync(kFull, incl[w], o);
+          if (lane >= o) incl[w] += v;
+        }
+        tot[w] = __shfl_sync(kFull, incl[w], 31);
+        incl[w] -= cnt[w];
+      }
+      const int mine = ((NW > 1 && (lane & 4) ? tot[NW - 1] : tot[0]) >> (8 * (lane & 3))) & 0xffu;
       int start = 0;
       if (lane < R && mine) start = atomicAdd(&s_cnt[lane], mine);
 #pragma unroll
       for (int q = 0; q < R; ++q) {
-        int pos = __shfl_sync(kFull, start, q);
-        unsigned long long* list = list_of(q);
+        int at = __shfl_sync(kFull, start, q) + static_cast<int>((incl[q / 4] >> (8 * (q % 4))) & 0xffu);
+        at = at < cap ? at : cap;                        // (the list has room for U more)
+        unsigned long long* to = list_of(q) + at;
 #pragma unroll
         for (int u = 0; u < U; ++u) {
-          const uint32_t key = static_cast<uint32_t>(q & 1 ? acc[u][q / 2] >> 32 : acc[u][q / 2]);
-          const int at = pos + __popc(bal[u][q] & below);
-          if (((bal[u][q] >> lane) & 1u) && at < cap)
-            list[at] = (static_cast<unsigned long long>(key) << 32) | static_cast<unsigned>(base + u * KT + tid + 1);
-          pos += __popc(bal[u][q]);
+          const float key = key_of_row(u, q);
+          if (key <= t_row[q]) {
+            *to = (static_cast<unsigned long long>(__float_as_uint(key)) << 32) | static_cast<unsigned>(base + u * KT + tid + 1);
+            ++to;
+          }
         }
       }
     }
-  } else if (i < V) {   // each team reads its own row of keys
+  } else if (i < V) {   // each team reads its own row of keys, W groups of four per thread at a time
+    constexpr int W = 4;
     const uint32_t* src = P.scratch + static_cast<size_t>(i) * V;
     const float t = s_t[r];
     unsigned long long* list = list_of(r);
     const bool vec4 = (V & 3) == 0;
-    for (int base = 0; base < V; base += 4 * RT) {
-      const int j0 = base + 4 * rt;
-      uint32_t key[4] = {0x7fffffffu, 0x7fffffffu, 0x7fffffffu, 0x7fffffffu};   // NaN: never kept
-      if (vec4) {
-        if (j0 < V) {
-          const uint4 v = __ldcs(reinterpret_cast<const uint4*>(src + j0));
-          key[0] = v.x, key[1] = v.y, key[2] = v.z, key[3] = v.w;
+    for (int base = 0; base < V; base += W * 4 * RT) {
+      uint4 key[W];
+#pragma unroll
+      for (int w = 0; w < W; ++w) {
+        const int j0 = base + w * 4 * RT + 4 * rt;
+        key[w] = make_uint4(0x7fffffffu, 0x7fffffffu, 0x7fffffffu, 0x7fffffffu);   // NaN: never kept
+        if (vec4) {
+          if (j0 < V) key[w] = __ldcs(reinterpret_cast<const uint4*>(src + j0));
+        } else {
+          if (j0 < V) key[w].x = __ldcs(src + j0);
+          if (j0 + 1 < V) key[w].y = __ldcs(src + j0 + 1);
+          if (j0 + 2 < V) key[w].z = __ldcs(src + j0 + 2);
+          if (j0 + 3 < V) key[w].w = __ldcs(src + j0 + 3);
         }
-      } else {
-#pragma unroll
-        for (int u = 0; u < 4; ++u)
-          if (j0 + u < V) key[u] = __ldcs(src + j0 + u);
       }
-      unsigned bal[4];
-      int n = 0;
+      // thread by thread: how many of the sixteen are kept, where they go, then the entries
+      int c = 0;
 #pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        bal[u] = __ballot_sync(kFull, __uint_as_float(key[u]) <= t);
-        n += __popc(bal[u]);
+      for (int w = 0; w < W; ++w) {
+        const uint32_t kk[4] = {key[w].x, key[w].y, key[w].z, key[w].w};
+#pragma unroll
+        for (int u = 0; u < 4; ++u) c += __uint_as_float(kk[u]) <= t;
       }
-      int pos = 0;
-      if (lane == 0 && n) pos = atomicAdd(&s_cnt[r], n);
-      pos = __shfl_sync(kFull, pos, 0);
+      int incl = c;
 #pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const int at = pos + __popc(bal[u] & below);
-        if (((bal[u] >> lane) & 1u) && at < cap)
-          list[at] = (static_cast<unsigned long long>(key[u]) << 32) | static_cast<unsigned>(j0 + u + 1);
-        pos += __popc(bal[u]);
+      for (int o = 1; o < 32; o <<= 1) {
+        const int v = __shfl_up_sync(kFull, incl, o);
+        if (lane >= o) incl += v;
+      }
+      int at = 0;
+      if (lane == 31) at = atomicAdd(&s_cnt[r], incl);
+      at = __shfl_sync(kFull, at, 31) + incl - c;
+#pragma unroll
+      for (int w = 0; w < W; ++w) {
+        const uint32_t kk[4] = {key[w].x, key[w].y, key[w].z, key[w].w};
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          if (__uint_as_float(kk[u]) <= t) {
+            if (at < cap) list[at] = (static_cast<unsigned long long>(kk[u]) << 32) | static_cast<unsigned>(base + w * 4 * RT + 4 * rt + u + 1);
+            ++at;
+          }
+        }
       }
     }
   }
   __syncthreads();
 
-  // ---- 3. counting sort and ranking, a team per row ----
+  // ---- 3. counting sort (in place, through registers) and ranking, a team per row ----
   if (i < V) {
-    auto team = [&]() { asm volatile("bar.sync %0, %1;" ::"r"(1 + r), "n"(RT) : "memory"); };
     unsigned long long* list = list_of(r);
     unsigned* bins = bins_of(r);
-    unsigned short* order = reinterpret_cast<unsigned short*>(list + cap);
     const int n = s_cnt[r];
     const float lo = s_lo[r], scale = s_scale[r];
-    auto bin_of = [&](unsigned long long c) {   // monotone in the key
-      const float x = (__uint_as_float(static_cast<uint32_t>(c >> 32)) - lo) * scale;
-      return x > 0.0f ? min(static_cast<int>(x), NBINS - 1) : 0;
+    auto bin_of = [&](uint32_t key) {   // monotone in the key
+      // the square: near the bound the keys lie closer together (distances in D dimensions grow like the D/2-th root)
+      const float x = fmaxf(__uint_as_float(key) - lo, 0.0f) * scale;
+      return min(static_cast<int>(x * x * static_cast<float>(NBINS)), NBINS - 1);
     };
+    auto bin_at = [&](int b) { return static_cast<int>((bins[b >> 1] >> ((b & 1) << 4)) & 0xffffu); };
     if (n < k || n > cap) {
       if (rt == 0) s_slow[r] = 1;
     } else {
 #pragma unroll
       for (int q = 0; q < OWN; ++q) bins[q * RT + rt] = 0u;
       team();
-      for (int e = rt; e < n; e += RT) {
-        unsigned long long c = list[e];
-        if (static_cast<uint32_t>(c) == static_cast<uint32_t>(i + 1)) list[e] = c = 0ull;   // the code itself comes first
-        atomicAdd(&bins[bin_of(c)], 1u);
+      uint32_t key[KEEP], who[KEEP];    // this thread's entries: the key; index + 1 and place of arrival in its bin
+#pragma unroll
+      for (int q = 0; q < KEEP; ++q) {
+        const int e = q * RT + rt;
+        if (e < n) {
+          const unsigned long long c = list[e];
+          key[q] = static_cast<uint32_t>(c >> 32);
+          who[q] = static_cast<uint32_t>(c);
+          if (who[q] == static_cast<uint32_t>(i + 1)) key[q] = who[q] = 0u;   // the code itself comes first
+          const int b = bin_of(key[q]), sh = (b & 1) << 4;
+          who[q] |= ((atomicAdd(&bins[b >> 1], 1u << sh) >> sh) & 0xffffu) << 16;
+        }
       }
       team();
-      int loc[OWN], s = 0;
+      unsigned loc[OWN];
+      int s = 0;
 #pragma unroll
       for (int q = 0; q < OWN; ++q) {
-        loc[q] = static_cast<int>(bins[rt * OWN + q]);
-        s += loc[q];
+        loc[q] = bins[rt * OWN + q];
+        s += static_cast<int>((loc[q] & 0xffffu) + (loc[q] >> 16));
       }
       int incl = s;
 #pragma unroll
@@ -677,29 +769,34 @@ __global__ void __launch_bounds__(KT, 1) lantern_knn_rows_kernel(BuildParams P, 
       }
       if (lane == 31) s_wsum[r][rt >> 5] = incl;
       team();
-      int at = incl - s;
+      unsigned at = static_cast<unsigned>(incl - s);
 #pragma unroll
       for (int w = 0; w < RW; ++w)
-        if (w < (rt >> 5)) at += s_wsum[r][w];
+        if (w < (rt >> 5)) at += static_cast<unsigned>(s_wsum[r][w]);
 #pragma unroll
-      for (int q = 0; q < OWN; ++q) {
-        bins[rt * OWN + q] = static_cast<unsigned>(at);   // every count becomes its bin's cursor
-        if (loc[q] > CROWD && at < k) s_slow[r] = 1;
-        at += loc[q];
+      for (int q = 0; q < OWN; ++q) {   // every count becomes the place where its bin starts
+        const unsigned c0 = loc[q] & 0xffffu, c1 = loc[q] >> 16;
+        bins[rt * OWN + q] = at | ((at + c0) << 16);
+        if ((c0 > CROWD && at < static_cast<unsigned>(k)) || (c1 > CROWD && at + c0 < static_cast<unsigned>(k))) s_slow[r] = 1;
+        at += c0 + c1;
       }
       team();
       if (!s_slow[r]) {
-        for (int e = rt; e < n; e += RT) order[atomicAdd(&bins[bin_of(list[e])], 1u)] = static_cast<unsigned short>(e);
-        team();   // every cursor now holds the end of its bin = the start of the next
+#pragma unroll
+        for (int q = 0; q < KEEP; ++q) {
+          if (q * RT + rt < n)
+            list[bin_at(bin_of(key[q])) + (who[q] >> 16)] = (static_cast<unsigned long long>(key[q]) << 32) | (who[q] & 0xffffu);
+        }
+        team();
         int32_t* irow = P.idx + static_cast<size_t>(i) * k;
         float* drow = P.dist ? P.dist + static_cast<size_t>(i) * k : nullptr;
         for (int p = rt; p < n; p += RT) {
-          const unsigned long long c = list[order[p]];
-          const int b = bin_of(c);
-          const int start = b ? static_cast<int>(bins[b - 1]) : 0, end = static_cast<int>(bins[b]);
+          const unsigned long long c = list[p];
+          const int b = bin_of(static_cast<uint32_t>(c >> 32));
+          const int start = bin_at(b), end = b + 1 < NBINS ? bin_at(b + 1) : n;
           if (start >= k) break;
           int rank = start;
-          for (int u = start; u < end; ++u) rank += list[order[u]] < c;
+          for (int u = start; u < end; ++u) rank += list[u] < c;
           if (rank < k) {
             irow[rank] = c ? static_cast<int32_t>(static_cast<uint32_t>(c)) - 1 : i;
             if (drow) drow[rank] = __uint_as_float(static_cast<uint32_t>(c >> 32));
@@ -710,7 +807,7 @@ __global__ void __launch_bounds__(KT, 1) lantern_knn_rows_kernel(BuildParams P, 
   }
   __syncthreads();
   for (int q = 0; q < R; ++q)
-    if (s_slow[q]) knn_row_general(P, row0 + q, P2, dsm, S);
+    if (s_slow[q]) knn_row_general<KT>(P, row0 + q, P2, dsm, S);
 }
 
 static int next_pow2(int x) {
@@ -719,11 +816,11 @@ static int next_pow2(int x) {
   return p;
 }
 
-constexpr size_t kRowSmem = 216 * 1024;   // dynamic shared memory of the row kernel, at most
+constexpr size_t kRowSmem = 216 * 1024;   // dynamic shared memory of an SM that the row kernel counts on
 
-template <int R>
+template <int KT, int R, bool SCRATCH>
 static cudaError_t launch_rows(const BuildParams& P, int P2, size_t smem, cudaStream_t st) {
-  auto kk = P.scratch ? lantern_knn_rows_kernel<R, true> : lantern_knn_rows_kernel<R, false>;
+  auto kk = lantern_knn_rows_kernel<KT, R, SCRATCH>;
   const cudaError_t e = cudaFuncSetAttribute(kk, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
   if (e != cudaSuccess) return e;
   kk<<<(P.V + R - 1) / R, KT, smem, st>>>(P, P2);
@@ -770,12 +867,16 @@ extern "C" lantern_status lantern_build_neighbors(const float* codebook, int V, 
   const double kept = (most + 3.5 * sqrt(static_cast<double>(most))) / f;
   P.want = (V <= 2 * SAMPLE || kept >= V) ? 0 : want;
   P.cap = P.want ? (static_cast<int>(kept) + 7) & ~7 : V;
-  // As many rows per CTA as their lists leave room for (eight rows share every load of a code).  The longest list,
-  // 7264 entries at V = 32768 and k = 4097, leaves room for two.
+  // As many rows per CTA as their lists leave room for (and a team's registers hold): eight rows share every load of a
+  // code.  The longest list, 7264 entries at V = 32768 and k = 4097, leaves room for two.  Rows read from
+  // scratch share nothing: two CTAs of half the size then overlap one another's phases.
   const size_t per_row = row_bytes(P.cap);
-  const int R = 8 * per_row <= kRowSmem ? 8 : (4 * per_row <= kRowSmem ? 4 : 2);
-  const size_t smem = R * per_row > general ? R * per_row : general;
-  if (smem > kRowSmem) return LANTERN_E_SHAPE;
+  const int kt = P.scratch ? 512 : 1024;
+  auto fits = [&](int R) { return R * per_row <= kRowSmem && P.cap <= KEEP * (1024 / R); };
+  const int R = fits(8) ? 8 : (fits(4) ? 4 : 2);   // per 1024 threads
+  const size_t rows_smem = R * per_row * kt / 1024;
+  const size_t smem = rows_smem > general ? rows_smem : general;
+  if (smem > kRowSmem || P.cap > KEEP * (1024 / R)) return LANTERN_E_SHAPE;
   cudaError_t e = cudaSuccess;
   if (D > SMALL_D) {
     const int t = (V + TM - 1) / TM;
@@ -783,7 +884,12 @@ extern "C" lantern_status lantern_build_neighbors(const float* codebook, int V, 
     e = cudaGetLastError();
     if (e != cudaSuccess) return LANTERN_E_CUDA;
   }
-  e = R == 8 ? launch_rows<8>(P, P2, smem, st) : (R == 4 ? launch_rows<4>(P, P2, smem, st) : launch_rows<2>(P, P2, smem, st));
+  if (P.scratch)
+    e = R == 8 ? launch_rows<512, 4, true>(P, P2, smem, st)
+               : (R == 4 ? launch_rows<512, 2, true>(P, P2, smem, st) : launch_rows<512, 1, true>(P, P2, smem, st));
+  else
+    e = R == 8 ? launch_rows<1024, 8, false>(P, P2, smem, st)
+               : (R == 4 ? launch_rows<1024, 4, false>(P, P2, smem, st) : launch_rows<1024, 2, false>(P, P2, smem, st));
   return e == cudaSuccess ? LANTERN_OK : LANTERN_E_CUDA;
 }
 

@@ -97,3 +97,25 @@ def test_argument_errors():
         lt.build_neighbors(cb, 0)
     with pytest.raises(ValueError):
         lt.build_neighbors(cb.cpu(), 4)
+
+
+@pytest.mark.parametrize("V,D,k,kind", [
+    (2048, 8, 1000, "gauss"), (2049, 8, 1000, "gauss"), (2049, 8, 1, "gauss"),      # the sampled bound starts at 2049 codes
+    (4096, 8, 1000, "period"), (4096, 4, 300, "ties"),                              # codes of one cluster 512 apart; ties
+    (6000, 8, 2500, "gauss"), (9001, 8, 4097, "gauss"),                             # four, two rows per CTA
+    (2500, 40, 700, "period"), (5001, 33, 1500, "period"), (8193, 33, 4097, "gauss")])   # keys read from scratch
+def test_selection_paths_exact(V, D, k, kind):
+    if kind == "ties":
+        cb = li.codebook_integer(V, D, lo=-2, hi=3, seed=9)
+    elif kind == "period":
+        cb = li.codebook_clustered(V, D, centres=512, seed=10)
+    else:
+        cb = li.codebook_gaussian(V, D, seed=11)
+    gi, gd = _gpu(cb, k)
+    rows = np.unique(np.concatenate([np.arange(20), np.arange(V - 20, V), np.random.default_rng(1).integers(0, V, 24)])).astype(np.int32)
+    oi, od = oracle.build_neighbors(cb, k, rows=rows)
+    assert np.array_equal(gi[rows], oi)
+    assert np.array_equal(gd[rows].view(np.uint32), od.view(np.uint32))
+    assert np.array_equal(gi[:, 0], np.arange(V))
+    srt = np.sort(gi, axis=1)
+    assert np.all(srt[:, 1:] != srt[:, :-1])
