@@ -79,8 +79,7 @@ const char* lantern_status_string(lantern_status s);
  *   V, D, k    1 <= k <= V <= 32768, 1 <= D <= 4096, k <= 4097
  *   idx        out [V, k] int32; idx[i,0] == i
  *   dist       out [V, k] fp32 squared distances, dist[i,0] == 0; may be NULL
- *   workspace  lantern_build_workspace_bytes(V, D, k) bytes (0 for D <= 32: may then be NULL; else 4 V^2, the
- *              distances of all pairs)
+ *   workspace  lantern_build_workspace_bytes(V, D, k) bytes (0 for D <= 32: may then be NULL)
  * ---------------------------------------------------------------------------------------- */
 size_t lantern_build_workspace_bytes(int V, int D, int k);
 

@@ -6,7 +6,7 @@
 //
 // Small D (<= 32): a CTA takes R codes (rows of the table) at once and computes their keys against the
 // whole codebook, two rows to a packed fp32 instruction.  Large D: a tiled SIMT kernel writes the keys
-// of all pairs to global scratch first (each (i, j) accumulator still runs over d in order), and the same row
+// of a block of rows to global scratch first (each (i, j) accumulator still runs over d in order), and the same row
 // kernel reads them from there.
 //
 // Selection per row.  Only about k of the V keys matter, so no pass but the first looks at the others:
@@ -39,10 +39,11 @@ static_assert(SAMPLE <= NBINS / 2, "the sample is kept where the bins will be");
 
 struct BuildParams {
   const float* codebook;
-  const uint32_t* scratch;       // [V, V] key bits of all pairs (large-D path), else null
+  const uint32_t* scratch;       // [rows, V] key bits of rows row0.. (large-D path), else null
   int32_t* idx;
   float* dist;
   int V, D, k;
+  int row0, row_end;             // the rows of this launch
   int cap;                       // entries of a row's keep list
   int want;                      // rank in the sample that bounds the k smallest keys; 0 = keep everything (cap = V)
 };
@@ -66,15 +67,10 @@ __device__ __forceinline__ unsigned long long fma2(unsigned long long a, unsigne
 }
 
 // ---------------------------------------------------------------------------------------
-// keys of all pairs, large D: a 128 x 128 tile per CTA, 8 x 8 accumulators per thread
+// keys of a block of rows, large D: a 128 x 128 tile per CTA, 8 x 8 accumulators per thread
 // (rows ty*4.. and 64+ty*4.., columns tx*4.. and 64+tx*4.., so that every shared-memory read is
 // one conflict-free 16-byte load), the next 16 dimensions fetched into registers while the
 // current ones are used.  Every (i, j) accumulator still runs over d in order.
-//
-// (a - b)^2 and (b - a)^2 round alike, so key(j, i) = key(i, j) to the bit: only the tiles on and above the
-// diagonal are computed, and every tile is stored a second time transposed.  The kernel is bound by the fp32
-// pipes (two operations per pair and dimension): 2.19 ms at V = 16384, D = 256 against 1.85 ms at their full rate (all
-// tiles, a block of 1024 rows per launch: 4.6 ms).
 // ---------------------------------------------------------------------------------------
 __device__ __forceinline__ float4 fetch_quad(const float* __restrict__ cb, int row, int row_end, int D, int d, bool vec) {
   float4 v = make_float4(0.0f, 0.0f, 0.0f, 0.0f);   // zero padding adds fma(0, 0, acc) = acc exactly
@@ -93,16 +89,12 @@ __device__ __forceinline__ float4 fetch_quad(const float* __restrict__ cb, int r
 }
 
 __global__ void __launch_bounds__(256, 2) lantern_distance_tile_kernel(const float* __restrict__ cb, uint32_t* out, int V,
-                                                                       int D) {
+                                                                       int D, int row0, int rows) {
   __shared__ __align__(16) float As[DK][TM];
   __shared__ __align__(16) float Bs[DK][TM];
   const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
-  // tile (tr, tc) with tr <= tc, numbered column by column: tc (tc + 1) / 2 + tr
-  int tc = static_cast<int>((sqrtf(8.0f * static_cast<float>(blockIdx.x) + 1.0f) - 1.0f) * 0.5f);
-  while (tc * (tc + 1) / 2 > static_cast<int>(blockIdx.x)) --tc;
-  while ((tc + 1) * (tc + 2) / 2 <= static_cast<int>(blockIdx.x)) ++tc;
-  const int tr = blockIdx.x - tc * (tc + 1) / 2;
-  const int rbase = tr * TM, cbase = tc * TM;
+  const int rbase = row0 + blockIdx.y * TM, cbase = blockIdx.x * TM;
+  const int row_end = (row0 + rows < V) ? row0 + rows : V;
   const bool vec = (D & 3) == 0;
   unsigned long long acc[8][4];
 #pragma unroll
@@ -114,7 +106,7 @@ __global__ void __launch_bounds__(256, 2) lantern_distance_tile_kernel(const flo
   float4 ra[2], rb[2];
 #pragma unroll
   for (int l = 0; l < 2; ++l) {
-    ra[l] = fetch_quad(cb, rbase + srow, V, D, 4 * (squad + 2 * l), vec);
+    ra[l] = fetch_quad(cb, rbase + srow, row_end, D, 4 * (squad + 2 * l), vec);
     rb[l] = fetch_quad(cb, cbase + srow, V, D, 4 * (squad + 2 * l), vec);
   }
   for (int d0 = 0; d0 < D; d0 += DK) {
@@ -134,7 +126,7 @@ __global__ void __launch_bounds__(256, 2) lantern_distance_tile_kernel(const flo
     if (d0 + DK < D) {
 #pragma unroll
       for (int l = 0; l < 2; ++l) {
-        ra[l] = fetch_quad(cb, rbase + srow, V, D, d0 + DK + 4 * (squad + 2 * l), vec);
+        ra[l] = fetch_quad(cb, rbase + srow, row_end, D, d0 + DK + 4 * (squad + 2 * l), vec);
         rb[l] = fetch_quad(cb, cbase + srow, V, D, d0 + DK + 4 * (squad + 2 * l), vec);
       }
     }
@@ -159,36 +151,25 @@ __global__ void __launch_bounds__(256, 2) lantern_distance_tile_kernel(const flo
     __syncthreads();
   }
   const bool vec_out = (V & 3) == 0;
-  auto store4 = [&](int row, int col, uint32_t w0, uint32_t w1, uint32_t w2, uint32_t w3) {
-    if (row >= V) return;
-    uint32_t* o = out + static_cast<size_t>(row) * V + col;
-    if (vec_out && col + 3 < V) {
-      *reinterpret_cast<uint4*>(o) = make_uint4(w0, w1, w2, w3);
-    } else {
-      if (col < V) o[0] = w0;
-      if (col + 1 < V) o[1] = w1;
-      if (col + 2 < V) o[2] = w2;
-      if (col + 3 < V) o[3] = w3;
-    }
-  };
-  auto lo = [](unsigned long long v) { return static_cast<uint32_t>(v); };
-  auto hi = [](unsigned long long v) { return static_cast<uint32_t>(v >> 32); };
 #pragma unroll
   for (int r = 0; r < 8; ++r) {
-    const int row = rbase + (r < 4 ? ty * 4 + r : 64 + ty * 4 + (r - 4));
+    const int gr = rbase + (r < 4 ? ty * 4 + r : 64 + ty * 4 + (r - 4));
+    if (gr >= row_end) continue;
+    uint32_t* orow = out + static_cast<size_t>(gr - row0) * V;
 #pragma unroll
-    for (int h = 0; h < 2; ++h)
-      store4(row, cbase + 64 * h + tx * 4, lo(acc[r][2 * h]), hi(acc[r][2 * h]), lo(acc[r][2 * h + 1]), hi(acc[r][2 * h + 1]));
-  }
-  if (tr != tc) {   // the mirror image: the two rows of threads of a warp fill one 32-byte sector per column
+    for (int h = 0; h < 2; ++h) {
+      const int gc = cbase + 64 * h + tx * 4;
+      const unsigned long long p0 = acc[r][2 * h], p1 = acc[r][2 * h + 1];
+      const uint32_t w[4] = {static_cast<uint32_t>(p0), static_cast<uint32_t>(p0 >> 32), static_cast<uint32_t>(p1),
+                             static_cast<uint32_t>(p1 >> 32)};
+      if (vec_out && gc + 3 < V) {
+        *reinterpret_cast<uint4*>(orow + gc) = make_uint4(w[0], w[1], w[2], w[3]);
+      } else {
 #pragma unroll
-    for (int c = 0; c < 4; ++c)
-#pragma unroll
-      for (int g = 0; g < 2; ++g) {
-        const int col = rbase + 64 * g + ty * 4, row = cbase + (c < 2 ? tx * 4 + 2 * c : 64 + tx * 4 + 2 * (c - 2));
-        store4(row, col, lo(acc[4 * g][c]), lo(acc[4 * g + 1][c]), lo(acc[4 * g + 2][c]), lo(acc[4 * g + 3][c]));
-        store4(row + 1, col, hi(acc[4 * g][c]), hi(acc[4 * g + 1][c]), hi(acc[4 * g + 2][c]), hi(acc[4 * g + 3][c]));
+        for (int c = 0; c < 4; ++c)
+          if (gc + c < V) orow[gc + c] = w[c];
       }
+    }
   }
 }
 
@@ -275,7 +256,7 @@ __device__ __noinline__ void knn_row_general(const BuildParams& P, int i, int P2
   if (!P.scratch && tid < D) S.ai[tid] = P.codebook[static_cast<size_t>(i) * D + tid];
   __syncthreads();
   for (int j = tid; j < V; j += KT) {
-    const uint32_t key = P.scratch ? P.scratch[static_cast<size_t>(i) * V + j]
+    const uint32_t key = P.scratch ? P.scratch[static_cast<size_t>(i - P.row0) * V + j]
                                    : __float_as_uint(key_of(S.ai, P.codebook + static_cast<size_t>(j) * D, D, (D & 3) == 0));
     keys[j] = key;
     if (j != i) {
@@ -435,7 +416,6 @@ static __host__ __device__ constexpr size_t row_bytes(int cap) {
 // What bounds it (V = 16384, k = 1000, cycles of a CTA of eight rows, D = 8): the key pass 40 k, of which the fp32
 // pipes need 16 k and instruction issue 24 k; sample and bound 9 k; counting sort 13 k; ranking 11 k.
 // 0.55 ms per table; 1.20 ms when a CTA selected from all keys of one row (73 k warp instructions per row, now 26 k).
-// With scratch keys, D = 256: 0.55 ms, against 0.16 ms that reading the keys takes.
 template <int KT, int R, bool SCRATCH>
 __global__ void __launch_bounds__(KT, 1024 / KT) lantern_knn_rows_kernel(BuildParams P, int P2) {
   constexpr int RT = KT / R;         // threads of a row's team
@@ -452,7 +432,7 @@ __global__ void __launch_bounds__(KT, 1024 / KT) lantern_knn_rows_kernel(BuildPa
   __shared__ uint32_t s_low[R][3 * RW], s_most[R][RW];
   const int tid = threadIdx.x, lane = tid & 31;
   const int V = P.V, D = P.D, k = P.k, cap = P.cap;
-  const int row0 = blockIdx.x * R;
+  const int row0 = P.row0 + blockIdx.x * R, row_end = P.row_end;
   const bool vec = (D & 3) == 0;
   const size_t per_row = row_bytes(cap);
   auto list_of = [&](int r) { return reinterpret_cast<unsigned long long*>(dsm + r * per_row); };
@@ -461,7 +441,7 @@ __global__ void __launch_bounds__(KT, 1024 / KT) lantern_knn_rows_kernel(BuildPa
   if (!SCRATCH) {
     for (int t = tid; t < SMALL_D * R; t += KT) {
       const int d = t / R, r = t % R;
-      As[d][r] = (d < D && row0 + r < V) ? P.codebook[static_cast<size_t>(row0 + r) * D + d] : 0.0f;
+      As[d][r] = (d < D && row0 + r < row_end) ? P.codebook[static_cast<size_t>(row0 + r) * D + d] : 0.0f;
     }
   }
   if (tid < R) s_cnt[tid] = 0, s_slow[tid] = 0;
@@ -478,7 +458,7 @@ __global__ void __launch_bounds__(KT, 1024 / KT) lantern_knn_rows_kernel(BuildPa
     };
     uint32_t key[SMP];
     if constexpr (SCRATCH) {
-      const uint32_t* src = P.scratch + static_cast<size_t>(i < V ? i : 0) * V;
+      const uint32_t* src = P.scratch + static_cast<size_t>(i < row_end ? i - P.row0 : 0) * V;
 #pragma unroll
       for (int q = 0; q < SMP; ++q) key[q] = __ldg(src + sampled(q * RT + rt));
     } else {   // every thread takes codes of the sample against all rows of the CTA
@@ -669,9 +649,9 @@ __global__ void __launch_bounds__(KT, 1024 / KT) lantern_knn_rows_kernel(BuildPa
         }
       }
     }
-  } else if (i < V) {   // each team reads its own row of keys, W groups of four per thread at a time
+  } else if (i < row_end) {   // each team reads its own row of keys, W groups of four per thread at a time
     constexpr int W = 4;
-    const uint32_t* src = P.scratch + static_cast<size_t>(i) * V;
+    const uint32_t* src = P.scratch + static_cast<size_t>(i - P.row0) * V;
     const float t = s_t[r];
     unsigned long long* list = list_of(r);
     const bool vec4 = (V & 3) == 0;
@@ -723,7 +703,7 @@ __global__ void __launch_bounds__(KT, 1024 / KT) lantern_knn_rows_kernel(BuildPa
   __syncthreads();
 
   // ---- 3. counting sort (in place, through registers) and ranking, a team per row ----
-  if (i < V) {
+  if (i < row_end) {
     unsigned long long* list = list_of(r);
     unsigned* bins = bins_of(r);
     const int n = s_cnt[r];
@@ -818,12 +798,19 @@ static int next_pow2(int x) {
 
 constexpr size_t kRowSmem = 216 * 1024;   // dynamic shared memory of an SM that the row kernel counts on
 
+// Rows whose keys are held in scratch at a time: 64 MB at V = 16384, which the row kernel still finds
+// in L2 (1152 rows, which would fill the distance kernel's last wave of CTAs, measured slower).
+static int rows_per_block(int V) {
+  int r = V < 1024 ? V : 1024;
+  return (r + TM - 1) / TM * TM;
+}
+
 template <int KT, int R, bool SCRATCH>
 static cudaError_t launch_rows(const BuildParams& P, int P2, size_t smem, cudaStream_t st) {
   auto kk = lantern_knn_rows_kernel<KT, R, SCRATCH>;
   const cudaError_t e = cudaFuncSetAttribute(kk, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
   if (e != cudaSuccess) return e;
-  kk<<<(P.V + R - 1) / R, KT, smem, st>>>(P, P2);
+  kk<<<(P.row_end - P.row0 + R - 1) / R, KT, smem, st>>>(P, P2);
   return cudaGetLastError();
 }
 
@@ -835,7 +822,7 @@ extern "C" size_t lantern_build_workspace_bytes(int V, int D, int k) {
   (void)k;
   if (V < 1 || D < 1) return 0;
   if (D <= SMALL_D) return 0;
-  return static_cast<size_t>(V) * V * 4;   // the keys of all pairs
+  return static_cast<size_t>(rows_per_block(V)) * V * 4;
 }
 
 extern "C" lantern_status lantern_build_neighbors(const float* codebook, int V, int D, int k, int32_t* idx,
@@ -877,20 +864,25 @@ extern "C" lantern_status lantern_build_neighbors(const float* codebook, int V, 
   const size_t rows_smem = R * per_row * kt / 1024;
   const size_t smem = rows_smem > general ? rows_smem : general;
   if (smem > kRowSmem || P.cap > KEEP * (1024 / R)) return LANTERN_E_SHAPE;
-  cudaError_t e = cudaSuccess;
-  if (D > SMALL_D) {
-    const int t = (V + TM - 1) / TM;
-    lantern_distance_tile_kernel<<<t * (t + 1) / 2, 256, 0, st>>>(codebook, static_cast<uint32_t*>(workspace), V, D);
-    e = cudaGetLastError();
-    if (e != cudaSuccess) return LANTERN_E_CUDA;
+  auto select = [&]() {
+    if (P.scratch)
+      return R == 8 ? launch_rows<512, 4, true>(P, P2, smem, st)
+                    : (R == 4 ? launch_rows<512, 2, true>(P, P2, smem, st) : launch_rows<512, 1, true>(P, P2, smem, st));
+    return R == 8 ? launch_rows<1024, 8, false>(P, P2, smem, st)
+                  : (R == 4 ? launch_rows<1024, 4, false>(P, P2, smem, st) : launch_rows<1024, 2, false>(P, P2, smem, st));
+  };
+  const int rb = P.scratch ? rows_per_block(V) : V;
+  for (P.row0 = 0; P.row0 < V; P.row0 += rb) {
+    P.row_end = V - P.row0 < rb ? V : P.row0 + rb;
+    if (P.scratch) {
+      const int rows = P.row_end - P.row0;
+      const dim3 grid((V + TM - 1) / TM, (rows + TM - 1) / TM);
+      lantern_distance_tile_kernel<<<grid, 256, 0, st>>>(codebook, static_cast<uint32_t*>(workspace), V, D, P.row0, rows);
+      if (cudaGetLastError() != cudaSuccess) return LANTERN_E_CUDA;
+    }
+    if (select() != cudaSuccess) return LANTERN_E_CUDA;
   }
-  if (P.scratch)
-    e = R == 8 ? launch_rows<512, 4, true>(P, P2, smem, st)
-               : (R == 4 ? launch_rows<512, 2, true>(P, P2, smem, st) : launch_rows<512, 1, true>(P, P2, smem, st));
-  else
-    e = R == 8 ? launch_rows<1024, 8, false>(P, P2, smem, st)
-               : (R == 4 ? launch_rows<1024, 4, false>(P, P2, smem, st) : launch_rows<1024, 2, false>(P, P2, smem, st));
-  return e == cudaSuccess ? LANTERN_OK : LANTERN_E_CUDA;
+  return LANTERN_OK;
 }
 
 // ---------------------------------------------------------------------------------------
