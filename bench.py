@@ -107,6 +107,12 @@ def method_work(parents, accept_len, accept_path, N: int):
 NCU_TRAFFIC = {"kernel_revision": 18, "workload": "batch_chain", "traffic_over_algorithmic": 564017408 / 548656352}
 
 
+def stream_operations(greedy: bool, top_k_active: bool) -> int:
+    """Kernels and memsets of one verification call: memset, plan and the fused pass; greedy decoding and the logit
+    filter keep walk and bonus draw as kernels of their own, the filter one for thresholds."""
+    return 6 if top_k_active else (5 if greedy else 3)
+
+
 def ncu_traffic(workload, alg_bytes):
     import paper_2410_03355_b200 as lt
     if NCU_TRAFFIC["traffic_over_algorithmic"] is None or workload != NCU_TRAFFIC["workload"]:
@@ -713,7 +719,7 @@ def main():
         lit_cold, _ = lit.timed(50, 3, flush=flush)
         chain["literal_call"] = {"sequences_per_call": lit.B, "us_per_call_back_to_back": 1e3 * lit_total / 200,
                                  "us_per_call_l2_flushed": 1e3 * lit_cold / 50, "fused_kernel_us": 1e3 * lit_fused,
-                                 "stream_operations_per_call": lt.verify_launch_count(False, False),
+                                 "stream_operations_per_call": stream_operations(False, False),
                                  "note": "back to back the 23 MB of rows stay in L2; flushed they come from HBM"}
         del lit
         # the same call under the paper's other settings (same inputs, same table): greedy decoding (tau = 0), the
@@ -780,7 +786,7 @@ def main():
                          "note": "algorithmic bytes = rows of the contexts the kernel evaluated + neighbour rows of the "
                                  "nodes it tested; method_* counts only what Algorithm 1's loop reaches"},
             "cpu_baseline": cpu, "e2e": e2e,
-            "gpu_launches": (lt.verify_launch_count(args.greedy, top_active) - 1) * args.steps, "clocks": clocks,
+            "gpu_launches": (stream_operations(args.greedy, top_active) - 1) * args.steps, "clocks": clocks,
             "neighbor_build": {"ms": build_ms, "V": V, "D": cfg["D"], "k": k, "pairs_per_s": V * V / (build_ms * 1e-3)},
             "outputs": {"mean_accept_len": accept_mean, "sequences_with_status_bits": status_bad},
             "configs": configs,

@@ -287,10 +287,11 @@ lantern_status lantern_verify_static(const void* target_logits, const void* draf
  * stored profiler counters can be matched to the code they were taken on. */
 int lantern_kernel_revision(void);
 
-/* Number of kernels (and memsets) one verification call enqueues: memset, plan, fused pass or greedy
+/* Number of kernels (and memsets) that one verification call enqueues, at most: memset, plan, fused pass or greedy
  * pass, walk, bonus; a call whose top-k filter is active (0 < top_k < V) enqueues one threshold kernel
  * more (ahead of the greedy pass; in sampling ahead of the bonus draw -- the fused pass finds the
- * thresholds of its own contexts).  For launch accounting. */
+ * thresholds of its own contexts).  Sampling without the filter enqueues fewer: its fused pass walks and
+ * draws the bonus tokens itself. */
 int lantern_verify_launch_count(int greedy, int top_k_active);
 
 /* ------------------------------------------------------------------------------------------

@@ -1,20 +1,19 @@
-// LANTERN relaxed verification step on sm_100a: plan -> fused context pass -> walk -> bonus.
+// LANTERN relaxed verification step on sm_100a: plan -> fused context pass, which walks and draws as well.
 //
-// One "context" is a row of logits that has at least one drafted child.  The fused pass is
-// a persistent kernel, one CTA per SM: a bulk asynchronous copy (TMA, completion on an
-// mbarrier) brings the context's two target rows and its drafter row into shared memory
-// while the CTA is still working on the previous context; the rows are then read ONCE into
-// registers, guidance-combined, turned into softmax numerators, and every child of the
-// context is tested on chip:
+// One "context" is a row of logits that has at least one drafted child.  The fused pass (verify_context.cuh) is
+// a persistent kernel: bulk asynchronous copies (TMA, completion on an mbarrier) bring a context's target rows
+// into shared memory; the rows are read ONCE into registers, guidance-combined, turned into softmax numerators,
+// and every child of the context is tested on chip:
 //     A_{k,delta}(x~)  : gather of the target numerators at the token's neighbour row and a
-//                        block-wide prefix scan with the strict bound (Algorithm 2, 2nd block)
+//                        prefix scan with the strict bound (Algorithm 2, 2nd block)
 //     accept test      : r * p(x~) < sum_A q                     (Section 4.3, final rule)
 //     on rejection     : residual [q_{k,delta}(.|D=x~) - p]_+ over all V tokens, its total,
 //                        and either the next sibling's test on the renormalised residual or
 //                        the inverse-CDF draw of the replacement token   (Section 4.3, Alg. 1)
-// Each context leaves a 16-byte record; a tiny walk kernel follows the records from the root
-// (Algorithm 1's loop), and a last kernel draws the bonus token where the walk ended on a
-// context without children (Algorithm 1, line after the loop).
+// Algorithm 1's loop over the decided contexts and the draw of the bonus token happen inside the same pass.
+// Two paths keep the older split into passes, plan -> contexts -> walk -> bonus: greedy decoding (verify_greedy.cuh) and
+// sampling with the top-k logit filter (verify_context_filtered.cuh, verify_bonus.cuh); their contexts leave 16-byte
+// records, which a small walk kernel follows from the root.
 //
 // Precision: processed logits are fp32 (difference, fused multiply-add, division, each
 // rounded once); exponentials come from the fp32 ex2 unit (about 3e-7 relative); every sum over more
@@ -90,9 +89,17 @@ __global__ void __launch_bounds__(PLAN_WARPS * 32) lantern_plan_kernel(VerifyPar
   for (int c = lane; c < R; c += 32) P.dead[static_cast<size_t>(b) * R + c] = 0;
   status = __reduce_or_sync(kFull, status);
   __syncwarp();
-  if (lane == 0) P.seq_status[b] = status;
+  if (lane == 0) {
+    P.seq_status[b] = status;
+    if (P.walk_inline) {   // what stands if the fused pass never gets to the end of this sequence
+      P.out_len[b] = 0;
+      P.out_tok[b] = -1;
+      if (P.out_status) P.out_status[b] = status ? status : LANTERN_ST_INTERNAL;
+      if (status) atomicOr(&P.counters->status_or, status);
+    }
+  }
   if (status) {   // the walk reports the fault; no work is queued for this sequence
-    for (int r = lane; r < N; r += 32) P.work[static_cast<size_t>(r) * B + b].item = -1;
+    for (int r = lane; r < max(N, 1); r += 32) P.work[static_cast<size_t>(r) * B + b].item = -1;
     return;
   }
 
@@ -247,6 +254,7 @@ __global__ void __launch_bounds__(PLAN_WARPS * 32) lantern_plan_kernel(VerifyPar
       n_ctx += __popc(bal);
     }
   }
+  if (N == 0 && P.walk_inline) n_ctx = 1;
   // (thousands of warps would otherwise queue up on one address: most find the maximum already there)
   if (lane == 0 && n_ctx > *reinterpret_cast<volatile int*>(&P.counters->n_rank)) atomicMax(&P.counters->n_rank, n_ctx);
   __syncwarp();         // the shared arrays are complete
@@ -271,12 +279,16 @@ __global__ void __launch_bounds__(PLAN_WARPS * 32) lantern_plan_kernel(VerifyPar
     lb = __shfl_sync(kFull, lb, 0);
     const unsigned below = (1u << lane) - 1u;
     if (c < R) {
-      if (n == 0) {
-        Record leaf = {kLeaf, -1, 0, 0};
-        P.records[static_cast<size_t>(b) * R + c] = leaf;
+      Record* rec = P.records + static_cast<size_t>(b) * R + c;
+      if (P.walk_inline) {
+        *reinterpret_cast<unsigned long long*>(rec) = n == 0 ? kWalkLeaf : (c == 0 ? kWalkWaiting : kWalkPending);
+      } else if (n == 0) {
+        *rec = {kLeaf, -1, 0, 0};
       } else {
-        Record pending = {-1, -1, LANTERN_ST_INTERNAL, 0};   // stands until the fused pass has evaluated the context
-        P.records[static_cast<size_t>(b) * R + c] = pending;
+        *rec = {-1, -1, LANTERN_ST_INTERNAL, 0};   // stands until the fused pass has evaluated the context
+      }
+      if (n == 0 && N == 0) P.work[b] = {b, 0, 0, 0, 0, 0.0f, u_final, b};   // no drafts: one draw from the root's q
+      if (n > 0) {
         const int start = cur[c] - n;
         const int f = s_first[c];             // the context's first child (smallest node index)
         WorkItem w = {b * R + c, b * N + start, (n << 16) | f, (din[f + 1] << 16) | siz[f + 1], s_tok[f],
@@ -291,8 +303,7 @@ __global__ void __launch_bounds__(PLAN_WARPS * 32) lantern_plan_kernel(VerifyPar
 
 }  // namespace lantern
 
-// kernel 2: the fused context pass
-#include "verify_context.cuh"
+// (kernel 2, the fused context pass, is compiled in files of its own: see verify_common.cuh)
 // greedy decoding (temperature 0)
 #include "verify_greedy.cuh"
 #include "verify_bonus.cuh"
@@ -404,28 +415,28 @@ static cudaError_t launch_topk(const VerifyParams& P, int mode, long long jobs, 
 
 // the variants of the fused context kernel live in verify_context_v<tone + 2 jsd + 4 topk>.cu
 #define LANTERN_DECLARE_VARIANT(n) \
-  cudaError_t launch_context_v##n(const VerifyParams&, int, bool, bool, int, size_t, cudaStream_t);
+  cudaError_t launch_context_v##n(const VerifyParams&, bool, bool, long long, int, cudaStream_t);
 LANTERN_DECLARE_VARIANT(0) LANTERN_DECLARE_VARIANT(1) LANTERN_DECLARE_VARIANT(2) LANTERN_DECLARE_VARIANT(3)
 LANTERN_DECLARE_VARIANT(4) LANTERN_DECLARE_VARIANT(5) LANTERN_DECLARE_VARIANT(6) LANTERN_DECLARE_VARIANT(7)
 #undef LANTERN_DECLARE_VARIANT
 
-cudaError_t launch_context_kernel(const VerifyParams& P, int CH, bool bf16, bool uncond, bool tone, bool jsd, bool topk,
-                                  int grid, size_t smem_bytes, cudaStream_t st) {
+cudaError_t launch_context_kernel(const VerifyParams& P, bool bf16, bool uncond, bool tone, bool jsd, bool topk,
+                                  long long items, int sms, cudaStream_t st) {
   switch ((tone ? 1 : 0) | (jsd ? 2 : 0) | (topk ? 4 : 0)) {
-    case 0: return launch_context_v0(P, CH, bf16, uncond, grid, smem_bytes, st);
-    case 1: return launch_context_v1(P, CH, bf16, uncond, grid, smem_bytes, st);
-    case 2: return launch_context_v2(P, CH, bf16, uncond, grid, smem_bytes, st);
-    case 3: return launch_context_v3(P, CH, bf16, uncond, grid, smem_bytes, st);
-    case 4: return launch_context_v4(P, CH, bf16, uncond, grid, smem_bytes, st);
-    case 5: return launch_context_v5(P, CH, bf16, uncond, grid, smem_bytes, st);
-    case 6: return launch_context_v6(P, CH, bf16, uncond, grid, smem_bytes, st);
-    default: return launch_context_v7(P, CH, bf16, uncond, grid, smem_bytes, st);
+    case 0: return launch_context_v0(P, bf16, uncond, items, sms, st);
+    case 1: return launch_context_v1(P, bf16, uncond, items, sms, st);
+    case 2: return launch_context_v2(P, bf16, uncond, items, sms, st);
+    case 3: return launch_context_v3(P, bf16, uncond, items, sms, st);
+    case 4: return launch_context_v4(P, bf16, uncond, items, sms, st);
+    case 5: return launch_context_v5(P, bf16, uncond, items, sms, st);
+    case 6: return launch_context_v6(P, bf16, uncond, items, sms, st);
+    default: return launch_context_v7(P, bf16, uncond, items, sms, st);
   }
 }
 
-template <bool BF16, bool UNC, bool TOPK>
+template <bool BF16, bool UNC>
 static cudaError_t launch_bonus(const VerifyParams& P, int sms, cudaStream_t st) {
-  auto kb = lantern_bonus_stream_kernel<BF16, UNC, TOPK>;
+  auto kb = lantern_bonus_stream_kernel<BF16, UNC>;
   const size_t smem = static_cast<size_t>(P.V) * (UNC ? 2 : 1) * (BF16 ? 2 : 4);   // one context's raw target rows
   cudaError_t e = cudaFuncSetAttribute(kb, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
   if (e != cudaSuccess) return e;
@@ -439,22 +450,23 @@ static cudaError_t launch_bonus(const VerifyParams& P, int sms, cudaStream_t st)
   return cudaGetLastError();
 }
 
-template <bool BF16, bool UNC, bool TOPK>
-static cudaError_t launch_verify(const VerifyParams& P, int CH, bool tone, bool jsd, long long items, int sms,
-                                 int grid_ctx, size_t smem_bytes, cudaStream_t st) {
-  cudaError_t e;   // (with the top-k filter the fused pass finds the thresholds of its contexts itself)
+// Sampling.  Without the logit filter the fused pass walks the contexts and draws the bonus tokens as well; with it
+// (the fused pass finds the thresholds of its contexts itself) walk, thresholds of the bonus rows and bonus draw follow.
+template <bool BF16, bool UNC>
+static cudaError_t launch_verify(const VerifyParams& P, bool tone, bool jsd, long long items, int sms, cudaStream_t st) {
+  const bool topk = P.top_k > 0;
+  cudaError_t e;
   if (g_ev_before && g_ev_after) cudaEventRecord(g_ev_before, st);
-  e = launch_context_kernel(P, CH, BF16, UNC, tone, jsd, TOPK, grid_ctx, smem_bytes, st);
+  e = launch_context_kernel(P, BF16, UNC, tone, jsd, topk, items, sms, st);
   if (e != cudaSuccess) return e;
   if (g_ev_before && g_ev_after) cudaEventRecord(g_ev_after, st);
+  if (!topk) return cudaSuccess;
   lantern_walk_kernel<<<(P.B + 127) / 128, 128, 0, st>>>(P);
   e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  if (TOPK) {
-    e = launch_topk<BF16, UNC>(P, 1, P.B, sms, st);
-    if (e != cudaSuccess) return e;
-  }
-  return launch_bonus<BF16, UNC, TOPK>(P, sms, st);
+  e = launch_topk<BF16, UNC>(P, 1, P.B, sms, st);
+  if (e != cudaSuccess) return e;
+  return launch_bonus<BF16, UNC>(P, sms, st);
 }
 
 template <bool BF16, bool UNC, bool TOPK>
@@ -506,8 +518,8 @@ extern "C" size_t lantern_verify_workspace_bytes(int B, int N, int V, int k, int
 }
 
 extern "C" int lantern_verify_launch_count(int greedy, int top_k_active) {
-  // memset, plan, fused pass (or greedy pass), walk, bonus; with the filter one threshold kernel more: ahead
-  // of the greedy pass, or ahead of the bonus draw in sampling (the fused pass finds its own thresholds)
+  // greedy decoding: memset, plan, greedy pass, walk, bonus, and the threshold kernel with the filter; sampling with the
+  // filter the same, without it memset, plan and the fused pass, which walks and draws by itself
   (void)greedy;
   return 5 + (top_k_active ? 1 : 0);
 }
@@ -613,13 +625,8 @@ static lantern_status verify_impl(const void* target_logits, const void* draft_l
   if (!(T >= 0.0f) || !(delta >= 0.0f) || !isfinite(T) || !isfinite(delta)) return LANTERN_E_PARAM;
   if (has_uncond && !isfinite(cfg_scale)) return LANTERN_E_PARAM;
   const bool greedy = T == 0.0f;   // Section 4.3, last sentence: no drafter distribution, no random numbers
-  const int esize = dtype == LANTERN_BF16 ? 2 : 4;
-  const int nrows = has_uncond ? 3 : 2;
-  const int CH = V > 4 * GT * 8 ? 8 : (V > 2 * GT * 8 ? 4 : (V > GT * 8 ? 2 : 1));   // 8-token chunks per thread
-  // one staging area of three row slots per consumer group; the numerators are kept over the rows they came from
-  const size_t smem_bytes = NGRP * ((static_cast<size_t>(3) * V * esize + 127) & ~static_cast<size_t>(127));
-  (void)nrows;
-  if (!greedy && (smem_bytes > 192 * 1024 || (dtype == LANTERN_F32 && V > 8192))) return LANTERN_E_SHAPE;   // plus the kernel's static part: within the 227 KB of a CTA
+  // sampling keeps a context's numerators (4 bytes per token) and rows on chip: fp32 rows only up to 8192 tokens
+  if (!greedy && dtype == LANTERN_F32 && V > 8192) return LANTERN_E_SHAPE;
   if (B == 0) return LANTERN_OK;
   if (!target_logits || !neighbor_idx || !out_accept_len || !out_next_token) return LANTERN_E_NULL;
   if (!greedy && !uniforms) return LANTERN_E_NULL;
@@ -669,6 +676,7 @@ static lantern_status verify_impl(const void* target_logits, const void* draft_l
   // only the threshold kernel of greedy decoding with the logit filter walks the compact list
   P.ctx_slots = (greedy && topk) ? reinterpret_cast<int32_t*>(ws + L.slots) : nullptr;
   P.dead = ws + L.dead;
+  P.walk_inline = !greedy && !topk;
   P.wait_tries = g_wait_tries;
   P.withhold_item = g_withhold_item;
 
@@ -687,8 +695,6 @@ static lantern_status verify_impl(const void* target_logits, const void* draft_l
   if (cudaGetLastError() != cudaSuccess) return LANTERN_E_CUDA;
 
   const long long items = static_cast<long long>(B) * (N > 0 ? N : 1);   // upper bound of contexts with children
-  const long long ctas = (items + NGRP - 1) / NGRP;   // every CTA runs NGRP contexts at a time
-  const int grid_ctx = static_cast<int>(ctas < sms ? ctas : sms);
   const int grid_bonus = B < 4 * sms ? B : 4 * sms;   // greedy bonus: 256-thread CTAs
   cudaError_t e;
   const bool bf = dtype == LANTERN_BF16, un = has_uncond != 0;
@@ -702,13 +708,8 @@ static lantern_status verify_impl(const void* target_logits, const void* draft_l
   }
   // every combination of the compile-time variants exists: T = 1 never meets the division code
   const bool tone = T == 1.0f, jsd = divergence == LANTERN_DIV_JSD;
-#define LANTERN_DISPATCH2(KV)                                                                        \
-  (bf ? (un ? launch_verify<true, true, KV>(P, CH, tone, jsd, items, sms, grid_ctx, smem_bytes, st)   \
-            : launch_verify<true, false, KV>(P, CH, tone, jsd, items, sms, grid_ctx, smem_bytes, st)) \
-      : (un ? launch_verify<false, true, KV>(P, CH, tone, jsd, items, sms, grid_ctx, smem_bytes, st)  \
-            : launch_verify<false, false, KV>(P, CH, tone, jsd, items, sms, grid_ctx, smem_bytes, st)))
-  e = topk ? LANTERN_DISPATCH2(true) : LANTERN_DISPATCH2(false);
-#undef LANTERN_DISPATCH2
+  e = bf ? (un ? launch_verify<true, true>(P, tone, jsd, items, sms, st) : launch_verify<true, false>(P, tone, jsd, items, sms, st))
+         : (un ? launch_verify<false, true>(P, tone, jsd, items, sms, st) : launch_verify<false, false>(P, tone, jsd, items, sms, st));
   return e == cudaSuccess ? LANTERN_OK : LANTERN_E_CUDA;
 }
 

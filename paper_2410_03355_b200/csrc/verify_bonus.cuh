@@ -1,4 +1,5 @@
-// Bonus draw (Algorithm 1, line after the verification loop): where the walk ends on a context
+// Bonus draw (Algorithm 1, line after the verification loop) of calls with the top-k logit filter (the other
+// sampling calls draw inside the fused pass): where the walk ends on a context
 // without children, the next token is drawn from that context's target distribution by inverse
 // CDF at the sequence's last uniform.  Included by verify.cu after verify_greedy.cuh, whose row
 // staging helpers it shares.
@@ -29,7 +30,7 @@ struct BonusShared {
   unsigned long long bar_full;
 };
 
-template <bool BF16, bool UNC, bool TOPK>
+template <bool BF16, bool UNC>
 __global__ void __launch_bounds__(BNT, 3) lantern_bonus_stream_kernel(VerifyParams P) {
   extern __shared__ __align__(128) unsigned char bsm[];
   __shared__ BonusShared S;
@@ -51,12 +52,10 @@ __global__ void __launch_bounds__(BNT, 3) lantern_bonus_stream_kernel(VerifyPara
       z.z = __fdiv_rn(z.z, P.T);
       z.w = __fdiv_rn(z.w, P.T);
     }
-    if (TOPK) {   // below the row's top-k threshold: -inf (a NaN stays, to be reported)
-      z.x = z.x < tq ? NEG_INF : z.x;
-      z.y = z.y < tq ? NEG_INF : z.y;
-      z.z = z.z < tq ? NEG_INF : z.z;
-      z.w = z.w < tq ? NEG_INF : z.w;
-    }
+    z.x = z.x < tq ? NEG_INF : z.x;   // below the row's top-k threshold: -inf (a NaN stays, to be reported)
+    z.y = z.y < tq ? NEG_INF : z.y;
+    z.z = z.z < tq ? NEG_INF : z.z;
+    z.w = z.w < tq ? NEG_INF : z.w;
     return z;
   };
 
@@ -89,8 +88,7 @@ __global__ void __launch_bounds__(BNT, 3) lantern_bonus_stream_kernel(VerifyPara
     const int item = b * R + P.bonus_ctx[i];
     const int i_next = i + G < count ? i + G : i;
     const int item_next = item_of(i_next);   // used when the rows have been read twice: nothing selects on it before
-    float tq = 0.0f;
-    if (TOPK) tq = __ldg(P.thr_q + item);
+    const float tq = __ldg(P.thr_q + item);
     const double u = static_cast<double>(P.uniforms[static_cast<size_t>(b) * R + N]);
     const bool ok = mbar_wait(bar, it & 1, P.wait_tries);
     const int q0 = tid * Q;                  // this thread's quads: q0 .. q0 + Q - 1, as far as the row goes

@@ -7,10 +7,14 @@
 #include <math.h>
 #include <stdint.h>
 
+#include <type_traits>
+
 #include "lantern.h"
 #include "lantern_device.cuh"
 
 namespace lantern {
+
+#define LANTERN_CONTEXT_KERNEL_REVISION 19   // bump on every change to the fused context kernel
 
 constexpr int MAX_N = 1024;
 
@@ -92,8 +96,25 @@ struct VerifyParams {
   float* thr_q;                 // [B, R] top_k-th largest processed target logit of a context row
   float* thr_p;                 // [B, R] the same for the drafter row
   uint32_t wait_tries;          // limit of every bounded mbarrier wait, in tries
+  int walk_inline;              // the fused pass walks and draws the bonus tokens itself: records hold walk words
   int withhold_item;            // self-test only: the copies of this context are never issued (-1 = none)
 };
+
+constexpr int kNone = 0x7fffffff;
+// A residual whose total weight is at most this fraction of the current target's mass defines no
+// distribution to draw from (the single-precision residual pass resolves totals to a few 1e-7 of that
+// mass): the walk stops there and the next token comes from the context's own target.
+constexpr double kDegenerate = 1e-5;
+
+// The walk over the contexts of a sequence, where the fused pass does it itself (verify_context.cuh): one word per
+// context, exchanged by whoever decides the context and by the walk when it gets there.
+//   bits 0..1 state; walk waiting: bits 8..15 status so far, bits 16..31 drafts accepted so far;
+//   decided: bits 8..15 status, bits 16..31 accepted node + 1 (0 = none), bits 32..63 replacement token
+enum : unsigned { kWalkPending = 0, kWalkWaiting = 1, kWalkDecided = 2, kWalkLeaf = 3 };
+__device__ __forceinline__ unsigned long long walk_word(unsigned state, unsigned status, unsigned count, int token = 0) {
+  return state | (status << 8) | (static_cast<unsigned long long>(count) << 16) |
+         (static_cast<unsigned long long>(static_cast<unsigned>(token)) << 32);
+}
 
 __device__ __forceinline__ float sum8(const float* v) {
   return ((v[0] + v[1]) + (v[2] + v[3])) + ((v[4] + v[5]) + (v[6] + v[7]));
@@ -103,7 +124,8 @@ __device__ __forceinline__ float sum8(const float* v) {
 // Launch of the fused context kernel (verify_context.cuh).  Its variants -- temperature 1 compiled
 // out or not (TONE), TVD or JSD bound, top-k thresholds applied or not -- are compiled in separate
 // translation units (verify_context_v*.cu) so that they build in parallel; this function picks one.
-cudaError_t launch_context_kernel(const VerifyParams& P, int CH, bool bf16, bool uncond, bool tone, bool jsd, bool topk,
-                                  int grid, size_t smem_bytes, cudaStream_t st);
+// `items` = upper bound of the contexts with children in the call, `sms` = SMs of the device.
+cudaError_t launch_context_kernel(const VerifyParams& P, bool bf16, bool uncond, bool tone, bool jsd, bool topk,
+                                  long long items, int sms, cudaStream_t st);
 
 }  // namespace lantern

@@ -1,54 +1,85 @@
-// Fused context pass of the LANTERN verification step (included by verify.cu).
+// Fused context pass of the LANTERN verification step.
 //
-// Persistent kernel, one CTA per SM.  The CTA holds TWO independent consumer groups of eight
-// warps, each working on its own context in its own staging area of shared memory, and two
-// producer warps (one thread each) that hand out contexts and issue the bulk asynchronous
-// copies (TMA, completion on an mbarrier, no multicast) of a group's next rows as soon as the
-// group releases its area.  The two groups drift apart in phase, so the latency-bound deciding
-// part of one context overlaps the issue-bound streaming part of the other and the copy of a
-// third: the SM is rarely idle although every context is a chain of dependent steps.
+// Persistent kernel, one CTA per SM.  The CTA holds one or more independent consumer groups, each
+// working on its own context in its own staging area of shared memory, and one producer warp per group
+// that hands out contexts, issues the bulk asynchronous copies (TMA, completion on an mbarrier, no
+// multicast) of a context's target rows, and walks the decided contexts (see below).  The groups
+// drift apart in phase, so the latency-bound deciding part of one context overlaps the issue-bound
+// streaming parts of the others.
 //
-// Streaming part (per thread, on its own tokens, in passes of at most 32 tokens): guidance
-// combine, the thread's own maximum, numerators 2^((z - max) log2 e) through the hardware ex2
-// unit, partial sums -- no cross-thread step at all, so the warps stream at full rate.  The
-// numerators E are stored over the context's own raw target rows (every thread overwrites only
-// bytes that it alone has read) and stay in the units of their (pass, thread) slice; a
-// per-slice factor, tabulated once the common maximum is known, brings them to common units
-// when they are used.  Sums
-// over many numerators average the ex2 unit's ~1e-7 rounding out; the two single probabilities
-// that decide a position, q(x~) and p(x~), are recomputed by one thread in double precision.
+// Three shapes (CtxNarrow, CtxPair, CtxWide below): three groups of eight warps per SM where there are sequences enough
+// to fill the GPU, two or one of sixteen warps where there are not.
+//
+// The area of a group holds the two target rows only (64 KB at V = 16384, bf16): the drafter row, of
+// which the common case needs nothing but its maximum, its sum and one entry, is read straight from
+// global memory (it was asked into L2 one context ahead) into registers while the target rows are
+// still being copied.
+//
+// Streaming part (per thread, on its own tokens): guidance combine, the maximum of a slice of at most
+// 16 tokens, numerators 2^(z log2 e - n) through the hardware ex2 unit with the slice's own integer
+// shift n = ceil(max * log2 e), partial sums -- no cross-thread step at all.  The numerators E
+// are stored over the context's own raw target rows (every thread overwrites only bytes that it alone has
+// read) and stay in the units of their slice; the shifts are tabulated, and because they are integers
+// a numerator comes to common units by an exact power of two.  One group barrier then publishes E,
+// the table and the per-warp maxima and sums.  Sums over many numerators average the ex2 unit's ~1e-7
+// rounding out; the two single probabilities that decide a position, q(x~) and p(x~), are formed by one
+// thread in double precision.
 //
 // Deciding part, per child (Section 4.3 / Algorithm 2, second block): gather of the neighbour
-// row's numerators, double-precision scan against the strict bound, accept test; on rejection
-// the residual [q_{k,delta}(.|D = x~) - p]_+ in one register pass (drafter numerators are
-// recomputed from the raw drafter row, which stays in shared memory), its total, and either the
-// inverse-CDF draw or the write-back for the next sibling.
-#pragma once
-
+// row's numerators, double-precision scan against the strict bound (the per-warp totals tell every warp
+// which warp the bound falls into; only that one looks for the slot), accept test; on rejection
+// the residual [q_{k,delta}(.|D = x~) - p]_+ in one register pass (the drafter logits are read
+// again, normally from L2), its total, and either the inverse-CDF draw or the write-back for the
+// next sibling.
+//
 // Which contexts are evaluated.  Algorithm 1 stops at the first rejection, so a context behind a
 // rejected node is never tested by the method.  Work items come in breadth-first order per sequence
-// (see the plan kernel); when a context has been decided, its group marks the contexts behind every
-// child it did not accept as dead (a sequence's contexts are numbered in pre-order for this, so that a
-// subtree is one contiguous range of marks), and a producer that meets a dead context leaves it out.  A context whose parent is still undecided when its turn comes is
-// evaluated anyway: with few sequences per call that keeps every SM busy (all contexts of a tree run
-// side by side), with many sequences it is rare, and the walk kernel reads only records on the
-// accepted path either way, so the result never depends on what was speculated.
-#define LANTERN_CONTEXT_KERNEL_REVISION 18   // bump on every change to this file
+// (see the plan kernel); when a context has been decided, its producer marks the contexts behind every
+// child that was not accepted as dead (a sequence's contexts are numbered in pre-order for this, so that a
+// subtree is one contiguous range of marks), and a producer that meets a dead context leaves it out.  A context whose
+// parent is still undecided when its turn comes is evaluated anyway: with few sequences per call that keeps every SM
+// busy (all contexts of a tree run side by side), with many sequences it is rare, and the walk reads only results on the
+// accepted path either way, so the outcome never depends on what was speculated.
+//
+// The walk (Algorithm 1's loop) needs no pass of its own.  Every context has a word that two parties exchange, each
+// once: the producer whose group has decided the context, and the walk when it gets there (from the root, which starts
+// as "walk waiting").  Whichever comes second goes on: along the accepted child, to the next word.  So a sequence
+// is walked by whoever completes the next piece of its path, nobody waits, and where the walk ends on
+// a context without children (or on one whose residual had no weight) the draw from that context's q
+// is the next thing the same group does.
+#pragma once
+
+#include "verify_common.cuh"
 
 namespace lantern {
 
-constexpr int GT = 256;         // threads of one consumer group
-constexpr int GW = GT / 32;     // warps of one consumer group
-constexpr int LOG_GT = 8;
-constexpr int NGRP = 2;         // consumer groups per CTA
-constexpr int MAXU = 16;        // (pass, warp) slices of a context, at most
-constexpr int kNone = 0x7fffffff;
-// A residual whose total weight is at most this fraction of the current target's mass defines no
-// distribution to draw from (the single-precision residual pass resolves totals to a few 1e-7 of that
-// mass): the walk stops there and the next token comes from the context's own target.
-constexpr double kDegenerate = 1e-5;
-constexpr int CTX_THREADS = NGRP * GT + NGRP * 32;   // consumers, then one producer warp per group
+// GT = threads of one consumer group (8 warps or more), NGRP = groups per CTA, AREAS = staging areas per group,
+// CTAS = CTAs per SM.
+template <int GT_, int NGRP_, int AREAS_, int CTAS_>
+struct CtxShape {
+  static constexpr int GT = GT_, NGRP = NGRP_, AREAS = AREAS_, CTAS = CTAS_;
+  static constexpr int THREADS = NGRP * (GT + 32);
+};
+using CtxNarrow = CtxShape<256, 3, 1, 1>;   // 27 warps of 72 registers
+using CtxPair = CtxShape<512, 1, 1, 2>;     // 2 * 17 warps of 56 registers
+using CtxWide = CtxShape<512, 1, 2, 1>;     // 17 warps
+// Which shape.  A context is a chain of dependent steps; sixteen warps get through it in two thirds of the time eight
+// need, but three contexts per SM hide one another's latencies.  With few sequences per call the path through each
+// is what takes the time (and fewer contexts in flight mean fewer evaluated for nothing), with many the throughput.
+// V = 16384, us per call narrow / pair / wide: 8 trees 50 / 46 / 44, 128 trees 116 / 100 / 98, 300 trees 155 / 147 / 138,
+// 900 trees 254 / 243 / 270, 1500 trees 334 / 327 / 398; chains of 7: 200 sequences 82 / 69 / 71, 500 113 / 112 / 134,
+// 1024 172 / 181 / 233, 8192 981 / 1152 / 1450.  Rows of 8192 tokens and less give sixteen warps too little to do
+// (128 trees of 8192 tokens 78 / 78 / 88).
+static inline int ctx_shape(const VerifyParams& P, int sms) {   // 0 = narrow, 1 = pair, 2 = wide
+  if (P.V <= 8192) return 0;
+  if (P.B <= 2 * sms) return 2;
+  return P.B <= (P.parents ? 10 : 3) * sms ? 1 : 0;
+}
 
+// bytes of one staging area: 4 bytes per token for the numerators, which replace the raw target rows
+static inline __host__ __device__ size_t ctx_area_bytes(int V, bool bf16, bool uncond) {
+  return (static_cast<size_t>(V) * ((bf16 || !uncond) ? 4 : 8) + 127) & ~static_cast<size_t>(127);
+}
 // Thread t of a group owns, for chunk c, the eight consecutive tokens [(c*GT + t)*8, +8), i.e. 16-byte
 // group g = c*GT + t of a bf16 row.  E is laid over the context's own raw target rows: with bf16 logits
 // the low four numerators of g replace g's bytes in row slot 0 and the high four replace g's bytes in
@@ -59,53 +90,59 @@ __device__ __forceinline__ int ephys(int x, int row_floats) {
   if (BF16) return ((x >> 2) & 1) * row_floats + ((x >> 3) << 2) + (x & 3);
   return x;
 }
-// index of the (pass, thread) slice that owns token x in the factor table; LOG_CP = log2(chunks per pass)
-template <int LOG_CP>
-__device__ __forceinline__ int owner_slice(int x) {
-  const int g = x >> 3;
-  return ((g >> (LOG_GT + LOG_CP)) << LOG_GT) | (g & (GT - 1));
+
+// 2^(z log2 e) = y * 2^n for one value, n an integer, to about 1.5e-7: the exponent is formed in double precision,
+// its fraction split into an fp32 head for the ex2 unit and a tail that is applied to first order.
+struct Exp2Split {
+  double y, n;
+};
+__device__ __forceinline__ Exp2Split exp2_split(float z) {
+  Exp2Split r = {0.0, 0.0};
+  if (z > -1.0e30f) {   // (-inf stays zero)
+    const double x = static_cast<double>(z) * 1.4426950408889634074;
+    r.n = rint(x);
+    const double f = x - r.n;
+    const float fh = static_cast<float>(f);
+    const float fl = static_cast<float>(f - static_cast<double>(fh));
+    const float y = ex2_approx(fh);
+    r.y = static_cast<double>(__fmaf_rn(y, fl * 0.693147182464599609375f, y));
+  }
+  return r;
+}
+// 2^d for an integer d <= 0 held in a float, 0 below -126: exact, three instructions, no conversion
+__device__ __forceinline__ float exp2_int(float d) {
+  return __int_as_float(__float_as_int(fmaxf(d, -127.0f) + 12583039.0f) << 23);   // 1.5 * 2^23 + 127
+}
+// 2^d for an integer d held in a double, 0 far below the range of what it is compared with
+__device__ __forceinline__ double exp2_int_d(double d) {
+  const int e = static_cast<int>(fmin(fmax(d, -1000.0), 1000.0));
+  return e <= -1000 ? 0.0 : __hiloint2double((1023 + e) << 20, 0);
 }
 
-__device__ __forceinline__ void gbar(int grp);   // barrier among the threads of one consumer group (below)
-
-}  // namespace lantern
-#include "verify_context_topk.cuh"
-namespace lantern {
-
-struct GroupShared {
-  double wzq[GW], wzp[GW];      // per-warp sums of numerators, common units
-  double wt[8 * GW];            // per-(chunk, warp) totals for scans and block sums
-  double sbefore[GW];           // prefix sum just before a warp's first failing neighbour
-  double acc_e, acc_p;          // double-precision numerators of the tested x~, common units
-  double hist[32];              // drafter/target scale ratio of each earlier rejection round of this context
-  float fqt[2 * GT];            // factor of every (pass, thread) slice: its units -> common units
-  float wmq[GW], wmp[GW];       // per-warp maxima of the slices' shift constants
-  int first[GW];                // a warp's first failing neighbour slot
-  int badslot[GW];              // a warp's first neighbour slot with an entry outside [0, V)
-  int cand[GW];
-  int acc_valid;                // acc_e / acc_p are usable for the current child
-  int tok;
-  int fail;                     // a bounded wait for the target rows ran out (sticky)
-  GroupTopk tk;                 // scratch of the top-k threshold search (TOPK variants)
-  GroupItem work[2];            // descriptor of context i in work[i & 1]: the next one is published while the current one runs
+struct CtxResult {              // what a group hands back to its producer
+  int accepted;                 // accepted child, -1 if there is none
+  int token;                    // token drawn, -1 if none
+  int status;
 };
 
-__device__ __forceinline__ float ex2_approx(float x) {
-  float y;
-  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-  return y;
-}
-
-// 2^(z log2(e) - shift) for one value, to about 1.5e-7: the exponent is formed in double precision,
-// split into an fp32 head for the ex2 unit and a tail that is applied to first order.
-__device__ __forceinline__ double exp2_single(float z, float shift) {
-  const double x = static_cast<double>(z) * 1.4426950408889634074 - static_cast<double>(shift);
-  const float xh = static_cast<float>(x);
-  if (xh < -1000.0f) return 0.0;   // far below the flush-to-zero range; also keeps -inf from turning into inf - inf
-  const float xl = static_cast<float>(x - static_cast<double>(xh));
-  const float y = ex2_approx(xh);
-  return static_cast<double>(__fmaf_rn(y, xl * 0.693147182464599609375f, y));
-}
+template <int GW>
+struct alignas(16) GroupShared {
+  alignas(16) double wz[GW][2]; // per-warp sums of numerators (target, drafter), in the warp's units
+  double wt[64];                // per-(chunk, warp) totals for scans and block sums
+  Exp2Split single[2];          // q(x~), p(x~) of the next child to test, not yet in common units (thread 0's own note)
+  double acc_e, acc_p;          // double-precision numerators of the tested x~, common units
+  double cut_sum;               // moved mass of A where the bound fell into a warp's slots
+  double jsd_mass;              // the JSD bound as a mass, common units
+  double hist[32];              // drafter/target scale ratio of each earlier rejection round of this context
+  alignas(8) float wn[GW][2];   // the warps' units: their largest shifts
+  float slice[1024];            // shift of every (slice, thread)
+  int cut_m;                    // |A| - 1 that goes with cut_sum
+  int badslot[3];               // first neighbour slot with an entry outside [0, V), by scan round (mod 3)
+  int tok;
+  int fail;                     // a bounded wait for the target rows ran out (sticky)
+  GroupItem work[2];            // descriptor of context i in work[i & 1]: the next one is published while the current one runs
+  CtxResult result[2];          // result of context i in result[i & 1]
+};
 
 // one row of a context into one row slot of a staging area, in bulk copies of at most 16 KB
 __device__ __forceinline__ void ctx_issue_row(unsigned char* dst, const unsigned char* src, int rowbytes, uint64_t* bar) {
@@ -113,13 +150,6 @@ __device__ __forceinline__ void ctx_issue_row(unsigned char* dst, const unsigned
     const int n = min(16384, rowbytes - off);
     bulk_load(dst + off, src + off, static_cast<uint32_t>(n), bar);
   }
-}
-// the drafter row of a context, into row slot 2
-__device__ __forceinline__ void ctx_issue_drafter(const VerifyParams& P, int item, unsigned char* stage, int rowbytes,
-                                                  uint64_t* bar) {
-  mbar_expect_tx(bar, static_cast<uint32_t>(rowbytes));
-  ctx_issue_row(stage + 2 * rowbytes, static_cast<const unsigned char*>(P.draft) + static_cast<size_t>(item) * rowbytes,
-                rowbytes, bar);
 }
 // the target rows of a context (conditional, and unconditional if there is one), into row slots 0 and 1
 template <bool UNC>
@@ -132,17 +162,21 @@ __device__ __forceinline__ void ctx_issue_target(const VerifyParams& P, int item
   if (UNC) ctx_issue_row(stage + rowbytes, t + static_cast<size_t>(P.B) * P.R * rowbytes, rowbytes, bar);
 }
 
-// Ask L2 for the rows of a context ahead of time: the bulk copy that later brings them into shared
-// memory (it cannot start before the group has released its staging area) then finds them on chip.
-template <bool BF16, bool UNC>
+// Ask L2 for rows of a context ahead of time: the drafter row, which the group reads itself, always; the target rows
+// where a bulk copy is issued long before its context's turn (two staging areas) -- with one area the copy starts as soon as
+// rows that are on their way to the same SM have arrived, and prefetching them as well measured slower (8192 chains
+// 1.056 against 1.028 ms; with two areas 128 trees 98 against 103 us the other way round).
+template <bool UNC, bool TARGET>
 __device__ __forceinline__ void ctx_prefetch_rows(const VerifyParams& P, int item, int rowbytes) {
   const size_t row_off = static_cast<size_t>(item) * rowbytes;
-  const size_t branch = static_cast<size_t>(P.B) * P.R * rowbytes;
-  const unsigned char* t = static_cast<const unsigned char*>(P.target) + row_off;
   const unsigned char* d = static_cast<const unsigned char*>(P.draft) + row_off;
-  asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(t), "r"(rowbytes) : "memory");
-  if (UNC) asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(t + branch), "r"(rowbytes) : "memory");
-  asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(d), "r"(rowbytes) : "memory");
+  if (P.draft) asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(d), "r"(rowbytes) : "memory");
+  if (TARGET) {
+    const unsigned char* t = static_cast<const unsigned char*>(P.target) + row_off;
+    const size_t branch = static_cast<size_t>(P.B) * P.R * rowbytes;
+    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(t), "r"(rowbytes) : "memory");
+    if (UNC) asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(t + branch), "r"(rowbytes) : "memory");
+  }
 }
 
 // one logit of a row in global memory, widened to fp32
@@ -152,115 +186,145 @@ __device__ __forceinline__ float ctx_raw_logit(const void* base, size_t elem) {
   return __ldg(static_cast<const float*>(base) + elem);
 }
 
-// Packed pairs of fp32 values (Blackwell's two-wide fp32 instructions): each lane is rounded exactly
-// like the scalar instruction, so results do not depend on the packing.
-__device__ __forceinline__ uint64_t pack2(float lo, float hi) {
-  uint64_t r;
-  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
-  return r;
+// eight raw logits of one 16-byte group (bf16) or 32 bytes (fp32) of a row in global memory
+template <bool BF16>
+struct Raw8 {
+  uint4 a, b;   // b: second half of an fp32 group
+};
+template <bool BF16>
+__device__ __forceinline__ Raw8<BF16> load_raw8(const unsigned char* row, int g) {
+  Raw8<BF16> d;
+  if (BF16) {
+    d.a = ld_stream(row + static_cast<size_t>(g) * 16);
+  } else {
+    d.a = ld_stream(row + static_cast<size_t>(g) * 32);
+    d.b = ld_stream(row + static_cast<size_t>(g) * 32 + 16);
+  }
+  return d;
 }
-__device__ __forceinline__ void unpack2(uint64_t v, float& lo, float& hi) {
-  asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
+// the same as four packed pairs of fp32 values
+template <bool BF16>
+__device__ __forceinline__ void raw8_pairs(const Raw8<BF16>& d, uint64_t (&o)[4]) {
+  if (BF16) {
+    const uint32_t w[4] = {d.a.x, d.a.y, d.a.z, d.a.w};
+#pragma unroll
+    for (int i = 0; i < 4; ++i) o[i] = pack2(__uint_as_float(w[i] << 16), __uint_as_float(w[i] & 0xffff0000u));
+  } else {
+    o[0] = pack2(__uint_as_float(d.a.x), __uint_as_float(d.a.y));
+    o[1] = pack2(__uint_as_float(d.a.z), __uint_as_float(d.a.w));
+    o[2] = pack2(__uint_as_float(d.b.x), __uint_as_float(d.b.y));
+    o[3] = pack2(__uint_as_float(d.b.z), __uint_as_float(d.b.w));
+  }
 }
-__device__ __forceinline__ uint64_t sub2(uint64_t a, uint64_t b) {
-  uint64_t r;
-  asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-  return r;
-}
-__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
-  uint64_t r;
-  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-  return r;
-}
-__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
-  uint64_t r;
-  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
-  return r;
-}
-__device__ __forceinline__ float max3(float a, float b, float c) {
-  float r;
-  asm("max.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
-  return r;
-}
-
-// barrier among the 256 threads of consumer group `grp` (hardware barrier 1 + grp)
-__device__ __forceinline__ void gbar(int grp) { asm volatile("bar.sync %0, %1;" ::"r"(1 + grp), "n"(GT) : "memory"); }
-// the same barrier, returning the AND of every thread's predicate
-__device__ __forceinline__ bool gbar_and(int grp, bool pred) {
-  uint32_t r;
-  asm volatile(
-      "{\n\t.reg .pred p, q;\n\t"
-      "setp.ne.u32 p, %1, 0;\n\t"
-      "bar.red.and.pred q, %2, %3, p;\n\t"
-      "selp.u32 %0, 1, 0, q;\n\t}"
-      : "=r"(r)
-      : "r"(static_cast<uint32_t>(pred)), "r"(1 + grp), "n"(GT)
-      : "memory");
-  return r != 0;
-}
-// a load that stays where it is written (issued early on purpose; the value is used much later)
-__device__ __forceinline__ int ld_nc_here(const int32_t* p) {
-  int v;
-  asm volatile("ld.global.nc.s32 %0, [%1];" : "=r"(v) : "l"(p));
-  return v;
-}
-__device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
-  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_addr(bar)) : "memory");
+// maximum of eight raw logits and m (bf16: two running maxima, one per half word)
+template <bool BF16>
+__device__ __forceinline__ uint32_t raw8_max(const Raw8<BF16>& d, uint32_t m) {
+  if (BF16) return bf16x2_max(bf16x2_max(bf16x2_max(d.a.x, d.a.y), bf16x2_max(d.a.z, d.a.w)), m);
+  const float v = max3(max3(__uint_as_float(d.a.x), __uint_as_float(d.a.y), __uint_as_float(m)),
+                       max3(__uint_as_float(d.a.z), __uint_as_float(d.a.w), __uint_as_float(d.b.x)),
+                       max3(__uint_as_float(d.b.y), __uint_as_float(d.b.z), __uint_as_float(d.b.w)));
+  return __float_as_uint(v);
 }
 
-// CH = 8-token chunks per thread (1, 2, 4 or 8); a thread streams them in NP passes of CP chunks.
+// Totals over the warp of N per-thread values at once: every exchange halves the values a lane still carries, so
+// N values cost N - 1 exchanges plus the rest of the butterfly instead of 5 N.  Lane l ends with the total of
+// value l / (32 / N).
+template <int N>
+__device__ __forceinline__ double warp_transposed_sum(const float (&v)[N], int lane) {
+  double d[N];
+  int o = 16;
+  if constexpr (N > 1) {
+    const bool up = lane & 16;
+#pragma unroll
+    for (int i = 0; i < N / 2; ++i) {
+      const float send = up ? v[i] : v[i + N / 2], keep = up ? v[i + N / 2] : v[i];
+      d[i] = static_cast<double>(keep) + static_cast<double>(__shfl_xor_sync(kFull, send, 16));
+    }
+    o = 8;
+#pragma unroll
+    for (int n = N / 2; n > 1; n >>= 1) {
+      const bool u = lane & o;
+#pragma unroll
+      for (int i = 0; i < n / 2; ++i) {
+        const double send = u ? d[i] : d[i + n / 2], keep = u ? d[i + n / 2] : d[i];
+        d[i] = keep + __shfl_xor_sync(kFull, send, o);
+      }
+      o >>= 1;
+    }
+  } else {
+    d[0] = static_cast<double>(v[0]);
+  }
+#pragma unroll
+  for (; o > 0; o >>= 1) d[0] += __shfl_xor_sync(kFull, d[0], o);
+  return d[0];
+}
+
+// Exchange of a walk word.  The word carries everything its receiver needs and what the two sides store besides does
+// not depend on order, so no fence is paid for (with acquire and release the producers became the bottleneck: 1.12
+// instead of 1.07 ms on 8192 chains).
+__device__ __forceinline__ unsigned long long walk_exchange(Record* rec, unsigned long long v) {
+  unsigned long long old;
+  asm volatile("atom.relaxed.gpu.global.exch.b64 %0, [%1], %2;" : "=l"(old) : "l"(rec), "l"(v) : "memory");
+  return old;
+}
+
+// CH = 8-token chunks per thread (1, 2, 4 or 8); the target's numerators come in slices of CP chunks.
 // TONE = the temperature is exactly 1 (the paper's sampling setting): no division is compiled in.
 // JSD selects the Section 5.3.2 bound at compile time, so that the default path carries none of its code.
-// TOPK applies the per-row thresholds of the top-k logit filter (Appendix B.2; written by
-// lantern_topk_kernel): processed logits below a row's threshold count as -inf.
-template <int CH, bool BF16, bool UNC, bool TONE, bool JSD, bool TOPK>
-__global__ void __launch_bounds__(CTX_THREADS, 1) lantern_context_kernel(VerifyParams P) {
-  constexpr int NP = CH > 4 ? 2 : 1;          // passes
-  constexpr int CP = CH / NP;                 // chunks per pass
-  constexpr int LOG_CP = CP == 4 ? 2 : (CP == 2 ? 1 : 0);
+template <class SHAPE, int CH, bool BF16, bool UNC, bool TONE, bool JSD>
+__global__ void __launch_bounds__(SHAPE::THREADS, SHAPE::CTAS) lantern_context_kernel(VerifyParams P) {
+  constexpr int GT = SHAPE::GT, GW = GT / 32, NGRP = SHAPE::NGRP, AREAS = SHAPE::AREAS;
+  constexpr int LOG_GT = GT == 1024 ? 10 : (GT == 512 ? 9 : 8);
+  static_assert((1 << LOG_GT) == GT, "256, 512 or 1024 threads per group");
+  constexpr int SLOTS = 1024 / GT;            // neighbour slots per thread and scan round
+  constexpr int CP = CH > 2 ? 2 : CH;         // chunks per slice
+  constexpr int NP = CH / CP;                 // slices per thread
+  constexpr int LOG_CP = CP == 2 ? 1 : 0;
+  constexpr int AHEAD = BF16 ? (CH < 4 ? CH : 4) : (CH < 2 ? CH : 2);   // drafter groups in flight in a residual pass
+  static_assert(NP * GT <= 1024 && CH * GW <= 64, "tables of slices and blocks");
   extern __shared__ __align__(128) unsigned char smem[];
-  __shared__ GroupShared SG[NGRP];
-  // per group: drafter row landed / target rows landed / drafter slot free / target slots (E) free
-  __shared__ __align__(8) uint64_t bar_full_d[NGRP], bar_full_t[NGRP], bar_empty_d[NGRP], bar_empty_t[NGRP];
+  __shared__ GroupShared<GW> SG[NGRP];
+  // Per group: next context published / the next context may be chosen / context i finished (by i mod 2: the producer may
+  // look for context i - 1 when context i has been finished too); per area: rows landed
+  __shared__ __align__(8) uint64_t bar_item[NGRP], bar_next[NGRP], bar_done[NGRP][2], bar_rows[NGRP][AREAS];
 
   const int tid = threadIdx.x, lane = tid & 31;
   const int V = P.V, N = P.N, R = P.R, k = P.k;
   const int rowbytes = V * (BF16 ? 2 : 4);
-  const int stage_bytes = (3 * rowbytes + 127) & ~127;   // row slots: conditional, unconditional, drafter
-  const int row_floats = rowbytes >> 2;
-  auto EI = [&](int x) { return ephys<BF16>(x, row_floats); };
-  const float L_hi = 1.44269502162933349609375f;   // fl32(log2 e)
+  const int area_bytes = static_cast<int>(ctx_area_bytes(V, BF16, UNC));
+  const float L2E = 1.44269502162933349609375f;   // fl32(log2 e)
   const float ninf = __int_as_float(0xff800000);
 
   if (tid == 0) {
     for (int g = 0; g < NGRP; ++g) {
-      mbar_init(&bar_full_d[g], 1);
-      mbar_init(&bar_full_t[g], 1);
-      mbar_init(&bar_empty_d[g], GW);
-      mbar_init(&bar_empty_t[g], GW);
+      mbar_init(&bar_item[g], 1);
+      mbar_init(&bar_next[g], GW);
+      mbar_init(&bar_done[g][0], GW);
+      mbar_init(&bar_done[g][1], GW);
+      for (int a = 0; a < AREAS; ++a) mbar_init(&bar_rows[g][a], 1);
       SG[g].fail = 0;
-      SG[g].tk.n_list[0] = SG[g].tk.n_list[1] = 0;
+      SG[g].badslot[0] = SG[g].badslot[1] = SG[g].badslot[2] = kNone;
     }
     fence_mbar_init();
     fence_proxy_async();
   }
-  if (TOPK && tid < NGRP * GT) SG[tid >> LOG_GT].tk.hist[0][tid & (GT - 1)] = SG[tid >> LOG_GT].tk.hist[1][tid & (GT - 1)] = 0;
   __syncthreads();
 
   // ======================= producer warps =======================
-  // One warp per consumer group hands out work and keeps that group's copies going.  Its 32 lanes look
+  // One warp per consumer group hands out work, keeps that group's copies going and walks.  Its 32 lanes look
   // at up to 32 consecutive work slots at a time (a batch: the first one dealt statically, later ones
   // from a global counter, in sizes that shrink towards the end of the list so that the groups finish
   // together), drop the empty and the dead ones, and lane 0 feeds the rest to the group one by one:
-  // the drafter row as soon as the group has streamed the previous one, the target rows as soon as the
-  // group releases its staging area.  The next batch is loaded while the current one is being worked
-  // on, so that no round trip to the work list is on the critical path.
+  // the context is chosen, and published, when the group has streamed the one before (so that it can go on to
+  // the next drafter row without asking), and its target rows are copied as soon as a staging area is free.  The
+  // next batch is loaded while the current one is being worked on, so that no round trip to the work list is
+  // on the critical path.
   if (tid >= NGRP * GT) {
     const int grp = (tid - NGRP * GT) >> 5;
-    GroupShared& S = SG[grp];
+    GroupShared<GW>& S = SG[grp];
     const int total = P.counters->n_rank * P.B;  // occupied part of the slot array
     const int G = gridDim.x * NGRP;              // producers in the grid
-    const int me = blockIdx.x * NGRP + grp;
+    const int me = grp * gridDim.x + blockIdx.x; // few contexts: one to an SM before any SM gets a second one
     const uint32_t tries = P.wait_tries;
     // Slots per batch.  Few live contexts per batch (two; one towards the end of the list, so that the groups
     // finish together): a batch is worked through in order, and the longer that takes the more of its
@@ -274,28 +338,22 @@ __global__ void __launch_bounds__(CTX_THREADS, 1) lantern_context_kernel(VerifyP
       const int s = live * ((slots_seen + 1) / (live_seen + 1));
       return s < 1 ? 1 : (s > 32 ? 32 : s);
     };
+    // what a lane keeps of a candidate: its slot, its context and its dead mark (the rest is read when it is taken)
     struct Cand {
-      int item, cbase, nchild_node0, span0, tok0, mark;
-      float r0, u_final;
+      int slot, item, mark;
     };
     auto load_cand = [&](int start, int size) -> Cand {
-      Cand c;
-      c.item = -1;
-      c.cbase = c.nchild_node0 = c.span0 = c.tok0 = c.mark = 0;
-      c.r0 = c.u_final = 0.0f;
-      const int w = start + lane;
-      if (lane < size && w < total) {
-        const int4 lo = __ldg(reinterpret_cast<const int4*>(P.work + w));
-        const int4 hi = __ldg(reinterpret_cast<const int4*>(P.work + w) + 1);
-        c.item = lo.x, c.cbase = lo.y, c.nchild_node0 = lo.z, c.span0 = lo.w;
-        c.tok0 = hi.x, c.r0 = __int_as_float(hi.y), c.u_final = __int_as_float(hi.z), c.mark = hi.w;
+      Cand c = {start + lane, -1, 0};
+      if (lane < size && c.slot < total) {
+        c.item = __ldg(&P.work[c.slot].item);
+        c.mark = __ldg(&P.work[c.slot].mark);
       }
       return c;
     };
     auto is_dead = [&](int mark) -> bool {
       return *reinterpret_cast<const volatile unsigned char*>(P.dead + mark) != 0;
     };
-    int n_eval = 0, n_skip = 0;
+    int n_eval = 0, n_skip = 0, n_draw = 0;
     // live candidates of a batch, as a lane mask
     auto filter = [&](const Cand& c) -> unsigned {
       const bool has = c.item >= 0;
@@ -305,98 +363,146 @@ __global__ void __launch_bounds__(CTX_THREADS, 1) lantern_context_kernel(VerifyP
       live_seen += __popc(live);
       return live;
     };
+    // Tickets for the dynamic batches are asked for two batches ahead and the candidates of a batch are read one batch
+    // ahead, so that a producer waits for neither.
     const int b0 = batch_size(0);
-    Cand cur = load_cand(me * b0, b0);
-    bool cur_end = me * b0 >= total;
-    int seen = G * b0;
-    // start of the next dynamic batch (lane 0 asks, everybody hears)
-    auto grab = [&](int& size) -> int {
-      size = batch_size(seen < total ? seen : total);
-      int st = 0;
-      if (lane == 0) st = G * b0 + atomicAdd(&P.counters->work_next, size);
-      st = __shfl_sync(kFull, st, 0);
-      seen = st;
-      slots_seen += size;
-      return st;
+    Cand cur = load_cand(me * b0, b0), nxt;
+    bool cur_end = me * b0 >= total, nxt_end = false, primed = false;
+    int ticket = 0, ticket_size = 0, seen = G * b0;
+    auto ask = [&]() {       // (lane 0 holds the answer)
+      ticket_size = batch_size(seen < total ? seen : total);
+      if (lane == 0) ticket = atomicAdd(&P.counters->work_next, ticket_size);
+      slots_seen += ticket_size;
     };
-    int nsize = 0;
-    int nstart = grab(nsize);
-    Cand nxt = load_cand(nstart, nsize);
-    bool nxt_end = nstart >= total;
+    auto load_next = [&]() {
+      seen = G * b0 + __shfl_sync(kFull, ticket, 0);
+      nxt = load_cand(seen, ticket_size);
+      nxt_end = seen >= total;
+      ask();
+    };
+    ask();
     unsigned mask = filter(cur);
-    int i = 0;        // contexts handed to the group so far
-    bool clean = true;
     auto next_batch = [&]() {   // make `mask` non-empty if any live context is left
+      if (!primed) {
+        primed = true;
+        load_next();
+      }
       while (mask == 0 && !cur_end) {
         cur = nxt;
         cur_end = nxt_end;
-        if (!cur_end) {
-          nstart = grab(nsize);
-          nxt = load_cand(nstart, nsize);
-          nxt_end = nstart >= total;
-        }
+        if (!cur_end) load_next();
         mask = filter(cur);
       }
     };
-    for (;;) {
-      next_batch();
-      if (mask == 0) break;
-      const int l = __ffs(mask) - 1;
-      mask &= mask - 1;
-      // Top-k filter: where the two thresholds of this context lie, from a sample of its rows in global memory
-      // (they have been asked into L2 already) -- found now, while the group is busy with the context before.
-      float br_d[4] = {0.0f, 0.0f, 0.0f, 0.0f}, br_t[4] = {0.0f, 0.0f, 0.0f, 0.0f};
-      if (TOPK) {
-        const int item_l = __shfl_sync(kFull, cur.item, l);
-        const size_t row = static_cast<size_t>(item_l) * V;
-        const size_t branch = static_cast<size_t>(P.B) * R * V;
-        auto raw8 = [&](const void* base, size_t elem, float (&z)[8]) {
-          if (BF16) {
-            const uint4 x = __ldg(reinterpret_cast<const uint4*>(static_cast<const unsigned short*>(base) + elem));
-            const uint32_t xw[4] = {x.x, x.y, x.z, x.w};
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-              z[2 * q] = __uint_as_float(xw[q] << 16);
-              z[2 * q + 1] = __uint_as_float(xw[q] & 0xffff0000u);
-            }
-          } else {
-            const float4 x0 = __ldg(reinterpret_cast<const float4*>(static_cast<const float*>(base) + elem));
-            const float4 x1 = __ldg(reinterpret_cast<const float4*>(static_cast<const float*>(base) + elem) + 1);
-            z[0] = x0.x, z[1] = x0.y, z[2] = x0.z, z[3] = x0.w, z[4] = x1.x, z[5] = x1.y, z[6] = x1.z, z[7] = x1.w;
-          }
-        };
-        auto zd_g = [&](int g, float (&z)[8]) {      // the same operations as the streaming loop, lane by lane
-          raw8(P.draft, row + static_cast<size_t>(g) * 8, z);
-          if (!TONE) {
-#pragma unroll
-            for (int e = 0; e < 8; ++e) z[e] = __fdiv_rn(z[e], P.T);
-          }
-        };
-        auto zt_g = [&](int g, float (&z)[8]) {
-          raw8(P.target, row + static_cast<size_t>(g) * 8, z);
-          if (UNC) {
-            float u[8];
-            raw8(P.target, branch + row + static_cast<size_t>(g) * 8, u);
-#pragma unroll
-            for (int e = 0; e < 8; ++e) z[e] = __fmaf_rn(P.cfg_scale, __fsub_rn(z[e], u[e]), u[e]);
-          }
-          if (!TONE) {
-#pragma unroll
-            for (int e = 0; e < 8; ++e) z[e] = __fdiv_rn(z[e], P.T);
-          }
-        };
-        tkg_warp_bracket(zd_g, P.top_k, V, lane, br_d);
-        tkg_warp_bracket(zt_g, P.top_k, V, lane, br_t);
+    // A sequence's final outcome.  (Its status stood at INTERNAL until now, see the plan kernel.)
+    auto finish = [&](int b, int token, int status) {
+      P.out_tok[b] = token;
+      if (P.out_status) P.out_status[b] = status;
+      if (status) atomicOr(&P.counters->status_or, status);
+    };
+    // Lane 0: a pending draw from a context's own q, and the context handed out last (everything its result needs;
+    // nc0 = nchild << 16 | node0, 0 for a draw).  `open`: that context's result has not been taken yet.
+    int draw_item = -1, draw_status = 0;
+    float draw_u = 0.0f;
+    int p_item = 0, p_cbase = 0, p_nc0 = 0, p_span0 = 0, p_status = 0;
+    float p_u = 0.0f;
+    bool open = false;
+    // Takes the group's result for context j, the one handed out last.  Returns false if the group never delivered.
+    auto take_result = [&](int j) -> bool {
+      if (!mbar_wait(&bar_done[grp][j & 1], (j >> 1) & 1, tries)) return false;
+      open = false;
+      const CtxResult res = S.result[j & 1];
+      const int item = __shfl_sync(kFull, p_item, 0), nc0 = __shfl_sync(kFull, p_nc0, 0);
+      const int b = item / R;
+      if (nc0 == 0) {
+        if (lane == 0) finish(b, res.token, p_status | res.status);
+        return true;
       }
-      // The drafter slot is free once every warp of the group has streamed the previous context's
-      // drafter row (nothing reads it afterwards), i.e. while that context is still being decided:
-      // the next drafter row travels early, and the group streams it while its target rows are copied.
-      if (i >= 1 && !mbar_wait(&bar_empty_d[grp], (i - 1) & 1, tries)) {
-        clean = false;   // the group never released its slot: it has given up, and so does its producer
+      // Algorithm 1 goes on from the accepted child only: every context behind another child is dead.  In
+      // pre-order those are one contiguous range per child.
+      const int cbase = __shfl_sync(kFull, p_cbase, 0), span0 = __shfl_sync(kFull, p_span0, 0), nchild = nc0 >> 16;
+      unsigned char* marks = P.dead + static_cast<size_t>(b) * R;
+      for (int c = 0; c < nchild; ++c) {
+        int node_c = nc0 & 0xffff, span_c = span0;
+        if (c > 0) {
+          const int4 kid = __ldg(reinterpret_cast<const int4*>(P.children + cbase + c));
+          node_c = kid.x, span_c = kid.w;
+        }
+        if (node_c != res.accepted)
+          for (int o = lane; o < (span_c & 0xffff); o += 32) marks[(span_c >> 16) + o] = 1;
+      }
+      if (lane == 0) {
+        Record* recs = P.records + static_cast<size_t>(b) * R;
+        int at = item - b * R, accepted = res.accepted, token = res.token, status = res.status;
+        unsigned long long w = walk_exchange(recs + at, walk_word(kWalkDecided, status, accepted + 1, token));
+        if ((w & 3u) == kWalkWaiting) {   // the walk stands here already: go on with it
+          int st = static_cast<int>(w >> 8) & 0xff, len = static_cast<int>(w >> 16) & 0xffff;
+          for (;;) {
+            st |= status;
+            if (status & (LANTERN_ST_NONFINITE | LANTERN_ST_INTERNAL)) {
+              finish(b, -1, st);
+              break;
+            }
+            bool from_q = (status & LANTERN_ST_DEGENERATE) != 0;   // a residual without weight: draw from the context's own target
+            if (!from_q) {
+              if (accepted < 0) {
+                finish(b, token, st);
+                break;
+              }
+              if (P.out_path) P.out_path[static_cast<size_t>(b) * N + len] = accepted;
+              atomicMax(&P.out_len[b], ++len);   // (pieces of the path may be stored out of order)
+              at = accepted + 1;
+              w = walk_exchange(recs + at, walk_word(kWalkWaiting, st, len));
+              from_q = (w & 3u) == kWalkLeaf;                      // no drafts left on this path: bonus token from q
+            }
+            if (from_q) {
+              draw_item = b * R + at;
+              draw_status = st;
+              draw_u = p_u;
+              break;
+            }
+            if ((w & 3u) != kWalkDecided) break;                   // whoever decides that context goes on
+            status = static_cast<int>(w >> 8) & 0xff;
+            accepted = static_cast<int>(w >> 16 & 0xffff) - 1;
+            token = static_cast<int>(w >> 32);
+          }
+        }
+      }
+      __syncwarp();
+      return true;
+    };
+    int i = 0;        // contexts handed to the group so far
+    bool clean = true;
+    for (;;) {
+      const bool drawing = __shfl_sync(kFull, draw_item, 0) >= 0;
+      if (!drawing) {
+        if (mask == 0) next_batch();
+        if (mask == 0) {   // nothing left but what the group is working on, which may end in a draw
+          if (!open) break;
+          if (!take_result(i - 1)) {
+            clean = false;
+            break;
+          }
+          continue;
+        }
+      }
+      int l = 0;
+      int4 lo = make_int4(0, 0, 0, 0), hi = make_int4(0, 0, 0, 0);
+      if (!drawing) {
+        l = __ffs(mask) - 1;
+        mask &= mask - 1;
+        const int slot = __shfl_sync(kFull, cur.slot, l);
+        if (lane == 0) {   // its description, in flight while the group is waited for
+          lo = __ldg(reinterpret_cast<const int4*>(P.work + slot));
+          hi = __ldg(reinterpret_cast<const int4*>(P.work + slot) + 1);
+        }
+      }
+      if (i >= 1 && !mbar_wait(&bar_next[grp], (i - 1) & 1, tries)) {
+        clean = false;   // the group never came this far: it has given up, and so does its producer
         break;
       }
       // as late as possible: has the context died meanwhile, has the call been given up?
-      const int gone = (lane == l && is_dead(cur.mark)) ? 1 : 0;
+      const int gone = (!drawing && lane == l && is_dead(cur.mark)) ? 1 : 0;
       const int stop = *reinterpret_cast<const volatile int*>(&P.counters->abort);
       if (__any_sync(kFull, stop != 0)) break;
       if (__any_sync(kFull, gone)) {
@@ -404,32 +510,44 @@ __global__ void __launch_bounds__(CTX_THREADS, 1) lantern_context_kernel(VerifyP
         continue;
       }
       GroupItem it;
-      it.item = __shfl_sync(kFull, cur.item, l);
-      it.cbase = __shfl_sync(kFull, cur.cbase, l);
-      const int nn0 = __shfl_sync(kFull, cur.nchild_node0, l);
-      it.nchild = nn0 >> 16;
-      it.node0 = nn0 & 0xffff;
-      it.span0 = __shfl_sync(kFull, cur.span0, l);
-      it.tok0 = __shfl_sync(kFull, cur.tok0, l);
-      it.r0 = __shfl_sync(kFull, cur.r0, l);
-      it.u_final = __shfl_sync(kFull, cur.u_final, l);
-#pragma unroll
-      for (int q = 0; q < 4; ++q) it.bracket[0][q] = br_d[q], it.bracket[1][q] = br_t[q];
-      bool ok = true;
+      int it_status = 0;
+      if (drawing) {
+        it.item = draw_item, it.cbase = 0, it.nchild = 0, it.node0 = 0, it.span0 = 0, it.tok0 = 0, it.r0 = 0.0f, it.u_final = draw_u;
+        it_status = draw_status;
+        draw_item = -1;
+      } else {   // (a work slot without children is a draw from the outset: a call without drafts)
+        it.item = lo.x, it.cbase = lo.y, it.nchild = lo.z >> 16, it.node0 = lo.z & 0xffff, it.span0 = lo.w;
+        it.tok0 = hi.x, it.r0 = __int_as_float(hi.y), it.u_final = __int_as_float(hi.z);
+      }
       if (lane == 0) {
-        S.work[i & 1] = it;                   // published by the mbarrier operation of the copy below
-        const bool withheld = it.item == P.withhold_item;   // self-test of the bounded waits: nothing is copied
-        fence_proxy_async();
-        if (!withheld) ctx_issue_drafter(P, it.item, smem + grp * stage_bytes, rowbytes, &bar_full_d[grp]);
-        // the target slots (later E) are free once every warp of the group has finished the previous context
-        if (i >= 1 && !mbar_wait(&bar_empty_t[grp], (i - 1) & 1, tries)) ok = false;
-        if (ok && !withheld) {
+        S.work[i & 1] = it;
+        mbar_arrive(&bar_item[grp]);
+      }
+      const int area = i % AREAS;
+      auto issue = [&]() {
+        if (lane == 0 && it.item != P.withhold_item) {   // (self-test of the bounded waits: nothing is copied)
           fence_proxy_async();
-          ctx_issue_target<UNC>(P, it.item, smem + grp * stage_bytes, rowbytes, &bar_full_t[grp]);
+          ctx_issue_target<UNC>(P, it.item, smem + (grp * AREAS + area) * area_bytes, rowbytes, &bar_rows[grp][area]);
+        }
+      };
+      bool ok = true;
+      if (AREAS > 1) {
+        issue();           // (the area's last context has been taken back already)
+        if (open) ok = take_result(i - 1);
+      } else {
+        // the area is free once every warp of the group has finished the previous context
+        if (i >= 1) ok = mbar_wait(&bar_done[grp][(i - 1) & 1], ((i - 1) >> 1) & 1, tries);
+        if (ok) {
+          issue();
+          if (open) take_result(i - 1);
         }
       }
-      ok = __shfl_sync(kFull, ok ? 1 : 0, 0) != 0;
-      ++n_eval;
+      const bool draw_now = __shfl_sync(kFull, it.nchild, 0) == 0;
+      n_draw += draw_now ? 1 : 0;
+      n_eval += draw_now ? 0 : 1;
+      p_item = it.item, p_cbase = it.cbase, p_nc0 = draw_now ? 0 : (it.nchild << 16 | it.node0), p_span0 = it.span0;
+      p_status = it_status, p_u = it.u_final;
+      open = true;
       ++i;
       if (!ok) {
         clean = false;
@@ -439,21 +557,21 @@ __global__ void __launch_bounds__(CTX_THREADS, 1) lantern_context_kernel(VerifyP
       // nothing waits for it) and an L2 prefetch of its rows -- of a context that has passed the dead check,
       // so that hardly any prefetched row goes unused.
       next_batch();
-      if (mask) {
+      if (mask && __shfl_sync(kFull, draw_item, 0) < 0) {
         const int item_ahead = __shfl_sync(kFull, cur.item, __ffs(mask) - 1);
-        if (lane == 0) ctx_prefetch_rows<BF16, UNC>(P, item_ahead, rowbytes);
+        if (lane == 0) ctx_prefetch_rows<UNC, (AREAS > 1)>(P, item_ahead, rowbytes);
       }
     }
     if (lane == 0) {
       if (clean) {   // the group is waiting for its next context: hand it the terminator
-        if (i == 0 || mbar_wait(&bar_empty_d[grp], (i - 1) & 1, tries)) {
+        if (i == 0 || mbar_wait(&bar_next[grp], (i - 1) & 1, tries)) {
           S.work[i & 1].item = -1;
-          __threadfence_block();
-          mbar_arrive(&bar_full_d[grp]);
+          mbar_arrive(&bar_item[grp]);
         }
       }
       if (n_eval) atomicAdd(&P.counters->n_evaluated, n_eval);
       if (n_skip) atomicAdd(&P.counters->n_skipped, n_skip);
+      if (n_draw) atomicAdd(&P.counters->n_bonus, n_draw);
     }
     return;
   }
@@ -462,468 +580,385 @@ __global__ void __launch_bounds__(CTX_THREADS, 1) lantern_context_kernel(VerifyP
   const int grp = tid >> LOG_GT;        // which group
   const int gt = tid & (GT - 1);        // thread within the group
   const int gw = gt >> 5;               // warp within the group
-  GroupShared& S = SG[grp];
-  unsigned char* stage = smem + grp * stage_bytes;    // this group's rows, later its E
-  float* E = reinterpret_cast<float*>(stage);
-  // staging rows: 0 = conditional target, 1 = unconditional target (if any), 2 = drafter
-  const unsigned char* rc = stage;
-  const unsigned char* ru = stage + rowbytes;
-  unsigned char* rd = stage + 2 * rowbytes;
-  constexpr bool T_is_one = TONE;
-  // The eight raw drafter logits of 16-byte group g of a row in global memory (a rejection reads the
-  // drafter row again from there -- normally from L2 -- because its slot already belongs to the next context)
-  struct DraftRaw {
-    uint4 a, b;   // b: second half of an fp32 group
+  GroupShared<GW>& S = SG[grp];
+  const int row_floats = rowbytes >> 2;
+  auto EI = [&](int x) { return ephys<BF16>(x, row_floats); };
+  // index of the slice that owns token x in the table of shifts
+  auto owner_slice = [&](int x) {
+    const int g = x >> 3;
+    return ((g >> (LOG_GT + LOG_CP)) << LOG_GT) | (g & (GT - 1));
   };
-  auto draft_fetch = [&](const unsigned char* row, int g) {
-    DraftRaw d;
-    d.b = make_uint4(0, 0, 0, 0);
-    if (BF16) {
-      d.a = __ldg(reinterpret_cast<const uint4*>(row + static_cast<size_t>(g) * 16));
-    } else {
-      d.a = __ldg(reinterpret_cast<const uint4*>(row + static_cast<size_t>(g) * 32));
-      d.b = __ldg(reinterpret_cast<const uint4*>(row + static_cast<size_t>(g) * 32 + 16));
-    }
-    return d;
-  };
-  // the same eight as processed logits (z_p = l_d / T)
-  auto draft_chunk = [&](const DraftRaw& d, float (&out)[8]) {
-    if (BF16) {
-      const uint32_t dw[4] = {d.a.x, d.a.y, d.a.z, d.a.w};
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        out[2 * i] = __uint_as_float(dw[i] << 16);
-        out[2 * i + 1] = __uint_as_float(dw[i] & 0xffff0000u);
-      }
-    } else {
-      const uint32_t dw[8] = {d.a.x, d.a.y, d.a.z, d.a.w, d.b.x, d.b.y, d.b.z, d.b.w};
-#pragma unroll
-      for (int e = 0; e < 8; ++e) out[e] = __uint_as_float(dw[e]);
-    }
-    if (!T_is_one) {
-#pragma unroll
-      for (int e = 0; e < 8; ++e) out[e] = __fdiv_rn(out[e], P.T);
-    }
-  };
+  const bool full = V == CH * GT * 8;                 // every thread owns CH whole chunks: no bounds to check
+  const bool nbr_vec = SLOTS == 4 && (k & 3) == 0 && (reinterpret_cast<uintptr_t>(P.nbr) & 15) == 0;
+  const size_t branch = static_cast<size_t>(P.B) * R * V;   // elements from a conditional row to its unconditional one
   const uint32_t tries = P.wait_tries;
-  // A bounded wait that runs out ends the group: the context keeps the "not evaluated" record the plan
-  // gave it (the walk reports INTERNAL for a sequence that reaches it), the call is given up (no producer
-  // hands out further work), and one thread gives the copies that may still be on their way into this
-  // group's staging area the same bounded wait before the group leaves.
-  auto give_up = [&](int iter, bool drafter_too) {
-    if (gt == 0) {
-      *reinterpret_cast<volatile int*>(&P.counters->abort) = 1;
-      if (drafter_too) mbar_wait(&bar_full_d[grp], iter & 1, tries);
-      mbar_wait(&bar_full_t[grp], iter & 1, tries);
-      if (!drafter_too) mbar_wait(&bar_full_d[grp], (iter + 1) & 1, tries);   // the next drafter row may be under way
+  auto gbar = [&]() { asm volatile("bar.sync %0, %1;" ::"r"(1 + grp), "n"(GT) : "memory"); };   // the group's threads
+  auto divide_T = [&](uint64_t v) {
+    float lo, hi;
+    unpack2(v, lo, hi);
+    return pack2(__fdiv_rn(lo, P.T), __fdiv_rn(hi, P.T));
+  };
+  // this thread's slots SLOTS gt .. of a neighbour row, from slot `base` on (slot 0 is the token itself,
+  // entries past the row are not looked at)
+  auto load_slots = [&](int token, int base, int (&n)[SLOTS]) {
+    const int32_t* row = P.nbr + static_cast<size_t>(token) * k + base + SLOTS * gt;
+    if (nbr_vec) {
+      int4 v = make_int4(0, 0, 0, 0);
+      if (base + SLOTS * gt < k) v = ld_nc_here4(row);   // k % 4 == 0: all four slots exist
+      n[0] = v.x, n[1 % SLOTS] = v.y, n[2 % SLOTS] = v.z, n[3 % SLOTS] = v.w;
+    } else {
+#pragma unroll
+      for (int i = 0; i < SLOTS; ++i) n[i] = base + SLOTS * gt + i < k ? ld_nc_here(row + i) : 0;
     }
   };
+  // Scan rounds of this group so far, mod 2 and mod 3: a round's totals are not overwritten, and its bad-slot word is
+  // not cleared, before every warp has read them.
+  int round2 = 0, round3 = 0;
   for (int iter = 0;; ++iter) {
-    // One warp watches the copy's mbarrier (bounded wait); the group barrier then releases everybody
-    // at once and tells every thread alike whether the rows have landed.
-    bool landed = true;
-    if (gw == 0) landed = mbar_wait(&bar_full_d[grp], iter & 1, tries);
-    const bool arrived = gbar_and(grp, landed);
-    if (!arrived) {   // the drafter row did not land within the limit
-      give_up(iter, true);
-      break;
-    }
-    const GroupItem cur = S.work[iter & 1];
-    const int item = cur.item;
-    if (item < 0) break;
-    float tq = 0.0f, tp = 0.0f;   // top-k thresholds of this context's target and drafter rows (found below)
-    const int b = item / R;
-    const ChildInfo* kids = P.children + cur.cbase;
-    const int nchild = cur.nchild;
+    const int area = iter % AREAS;
+    // A bounded wait that runs out ends the group: the context keeps its undecided word, so the sequences that need it
+    // keep INTERNAL; the call is given up (no producer hands out further work), and one thread gives
+    // the copies that may still be on their way into this group's staging areas the same bounded wait before the group
+    // leaves.
+    auto give_up = [&]() {
+      if (gt == 0) {
+        *reinterpret_cast<volatile int*>(&P.counters->abort) = 1;
+        atomicOr(&P.counters->status_or, LANTERN_ST_INTERNAL);
+        mbar_wait(&bar_rows[grp][area], (iter / AREAS) & 1, tries);
+        if (AREAS > 1) mbar_wait(&bar_rows[grp][(iter + 1) % AREAS], ((iter + 1) / AREAS) & 1, tries);
+      }
+    };
+    // Every warp waits for the next context by itself and may run ahead of slower ones: whatever it overwrites
+    // before the next group barrier they have finished with (with one staging area because the target rows land only when
+    // all warps have released it; with two areas a barrier sees to it).  A wait that runs out is reported behind that
+    // barrier, where every thread sees it alike.
+    if (AREAS > 1) gbar();
+    const bool there = mbar_wait(&bar_item[grp], iter & 1, tries);
+    if (!there) S.fail = 1;
+    const GroupItem& cur = S.work[iter & 1];
+    const int item = there ? cur.item : -1;
+    unsigned char* stage = smem + (grp * AREAS + area) * area_bytes;   // this context's target rows, later its E
+    float* E = reinterpret_cast<float*>(stage);
+    const int nchild = item < 0 ? 0 : cur.nchild;                      // 0: nothing but a draw from q
+    const unsigned char* drow = static_cast<const unsigned char*>(P.draft) + static_cast<size_t>(item) * rowbytes;
 
-    // first child: its neighbour row (four slots per thread) and, for thread 0, its raw logits; issued
-    // now, used after the streaming part
+    // first child: its neighbour row and, for thread 0, its raw logits; issued now, used after the streaming part
     int node = cur.node0;
     int xt = cur.tok0;
-    float r = cur.r0;
-    int nb[4];
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const int j = 4 * gt + 1 + i;
-      nb[i] = (j < k) ? ld_nc_here(P.nbr + static_cast<size_t>(xt) * k + j) : -1;
-    }
-    // (the drafter logit of x~ goes to every thread: the drafter row does not stay in shared memory)
-    float raw_c = 0.0f, raw_u = 0.0f;
-    float raw_d = ctx_raw_logit<BF16>(P.draft, static_cast<size_t>(item) * V + xt);
-    if (gt == 0) {
+    int nb[SLOTS];
+    float raw_c = 0.0f, raw_u = 0.0f, raw_d = 0.0f;
+    auto fetch_single = [&]() {
       const size_t e = static_cast<size_t>(item) * V + xt;
+      raw_d = ctx_raw_logit<BF16>(P.draft, e);
       raw_c = ctx_raw_logit<BF16>(P.target, e);
-      if (UNC) raw_u = ctx_raw_logit<BF16>(P.target, static_cast<size_t>(P.B) * R * V + e);
-    }
+      if (UNC) raw_u = ctx_raw_logit<BF16>(P.target, branch + e);
+    };
+    auto note_single = [&]() {
+      float z = raw_c;
+      if (UNC) z = __fmaf_rn(P.cfg_scale, __fsub_rn(raw_c, raw_u), raw_u);
+      S.single[0] = exp2_split(TONE ? z : __fdiv_rn(z, P.T));
+      S.single[1] = exp2_split(TONE ? raw_d : __fdiv_rn(raw_d, P.T));
+    };
 
-    // ---------------- streaming part, thread-local, NP passes of CP chunks ----------------
+    // ---------------- streaming part, thread-local ----------------
     // values travel as packed pairs (tokens 2i, 2i+1 of a chunk)
-    uint64_t a2[CP * 4];
-    float mlq_mine[NP], mlp_mine[NP];   // this thread's shift constants fl(max * log2 e), per pass
-    float tq_mine[NP], tp_mine[NP];     // and its sums of numerators, in its own units
-    const uint64_t L2 = pack2(L_hi, L_hi);
-    // four packed pairs of processed logits of 16-byte group g of a row
-    auto pairs_of = [&](const unsigned char* row, int g, uint64_t (&o)[4]) {
-      if (BF16) {
-        const uint4 x = *reinterpret_cast<const uint4*>(row + g * 16);
-        const uint32_t xw[4] = {x.x, x.y, x.z, x.w};
+    const uint64_t L2 = pack2(L2E, L2E);
+    float nd = 0.0f, td = 1.0f;   // drafter: this thread's shift and its sum of numerators, in its own units
+    float nq[NP <= 2 ? NP : 1] = {};  // target: the shifts of the slices, where they are few (else in S.slice)
+    auto shift_of = [&](int p) { return NP <= 2 ? nq[NP <= 2 ? p : 0] : S.slice[p * GT + gt]; };
+    float nq_max = 0.0f, tq = 1.0f;   // target: the largest shift of the slices; the sum, in its units
+    auto stream_drafter = [&](auto whole) {
+      Raw8<BF16> raw[CH];
 #pragma unroll
-        for (int i = 0; i < 4; ++i) o[i] = pack2(__uint_as_float(xw[i] << 16), __uint_as_float(xw[i] & 0xffff0000u));
-      } else {
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          const float4 x = *reinterpret_cast<const float4*>(row + g * 32 + h * 16);
-          o[2 * h] = pack2(x.x, x.y);
-          o[2 * h + 1] = pack2(x.z, x.w);
-        }
-      }
-    };
-    auto divide_T = [&](uint64_t v) {
-      float lo, hi;
-      unpack2(v, lo, hi);
-      return pack2(__fdiv_rn(lo, P.T), __fdiv_rn(hi, P.T));
-    };
-    if (TOPK) {   // the drafter row's top-k threshold, from the staged row (the row came early)
-      auto zd = [&](int g, float (&z)[8]) {
-        uint64_t d2[4];
-        pairs_of(rd, g, d2);
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          uint64_t l2 = d2[i];
-          if (!T_is_one) l2 = divide_T(l2);
-          unpack2(l2, z[2 * i], z[2 * i + 1]);
-        }
-      };
-      tp = tkg_kth_largest(zd, cur.bracket[0], P.top_k, V, CH, S.tk, 0, grp, gt, &P.counters->n_slow_topk);
-    }
-    // --- drafter first (its row came early): slice maximum and partial sum of numerators ---
-#pragma unroll
-    for (int p = 0; p < NP; ++p) {
-      float mp = ninf;
-#pragma unroll
-      for (int c = 0; c < CP; ++c) {
-        const int g = (p * CP + c) * GT + gt;
-        if (g * 8 < V) {
-          uint64_t d2[4];
-          pairs_of(rd, g, d2);
-#pragma unroll
-          for (int i = 0; i < 4; ++i) {
-            uint64_t l2 = d2[i];
-            if (!T_is_one) l2 = divide_T(l2);
-            float lo, hi;
-            unpack2(l2, lo, hi);
-            if (TOPK) {   // below the row's top-k threshold: -inf
-              lo = lo < tp ? ninf : lo, hi = hi < tp ? ninf : hi;
-              l2 = pack2(lo, hi);
-            }
-            a2[c * 4 + i] = l2;
-            mp = max3(mp, lo, hi);
-          }
+      for (int c = 0; c < CH; ++c) {
+        const int g = c * GT + gt;
+        if (decltype(whole)::value || g * 8 < V) {
+          raw[c] = load_raw8<BF16>(drow, g);
         } else {
-#pragma unroll
-          for (int i = 0; i < 4; ++i) a2[c * 4 + i] = pack2(ninf, ninf);
+          const uint32_t w = BF16 ? 0xff80ff80u : 0xff800000u;
+          raw[c].a = raw[c].b = make_uint4(w, w, w, w);
         }
       }
-      mp = fmaxf(mp, -1.0e37f);
-      const float mlp_w = mp * L_hi;
-      mlp_mine[p] = mlp_w;
-      const uint64_t nml2 = pack2(-mlp_w, -mlp_w);
+      uint32_t mw = BF16 ? 0xff80ff80u : 0xff800000u;
+#pragma unroll
+      for (int c = 0; c < CH; ++c) mw = raw8_max<BF16>(raw[c], mw);
+      float m = BF16 ? fmaxf(__uint_as_float(mw << 16), __uint_as_float(mw & 0xffff0000u)) : __uint_as_float(mw);
+      if (!TONE) m = __fdiv_rn(m, P.T);           // division is monotone: the maximum of the quotients
+      // a slice without any finite logit (padding, masked tokens) still needs a finite shift
+      nd = ceilf(fmaxf(m, -1.0e37f) * L2E);
+      const uint64_t nn2 = pack2(-nd, -nd);
       uint64_t t2 = pack2(0.0f, 0.0f);
 #pragma unroll
-      for (int c = 0; c < CP; ++c) {
-        uint64_t e2[4];
+      for (int c = 0; c < CH; ++c) {
+        uint64_t z2[4];
+        raw8_pairs<BF16>(raw[c], z2);
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
+          if (!TONE) z2[i] = divide_T(z2[i]);
           float lo, hi;
-          unpack2(fma2(a2[c * 4 + i], L2, nml2), lo, hi);
-          e2[i] = pack2(ex2_approx(lo), ex2_approx(hi));
+          unpack2(fma2(z2[i], L2, nn2), lo, hi);
+          z2[i] = pack2(ex2_approx(lo), ex2_approx(hi));
         }
-        t2 = add2(t2, add2(add2(e2[0], e2[1]), add2(e2[2], e2[3])));
+        t2 = add2(t2, add2(add2(z2[0], z2[1]), add2(z2[2], z2[3])));
       }
-      float tlo, thi;
-      unpack2(t2, tlo, thi);
-      tp_mine[p] = tlo + thi;
-    }
-
-    // The drafter slot is not read again for this context (a rejection fetches the drafter logits from
-    // global memory): hand it back, so that the next context's drafter row is copied while this one is decided.
-    __syncwarp();
-    if (lane == 0) mbar_arrive(&bar_empty_d[grp]);
-    // The target rows were issued when the previous context was released; they arrive while the drafter
-    // row is streamed.  Every thread waits for itself (bounded); a wait that runs out is reported after
-    // the next group barrier, where every thread sees it alike.
-    if (!mbar_wait(&bar_full_t[grp], iter & 1, tries)) S.fail = 1;
-    if (TOPK) {   // the target row's threshold, on the guided (and tempered) logits the streaming loop forms
+      float lo, hi;
+      unpack2(t2, lo, hi);
+      td = lo + hi;
+    };
+    // target: guidance combine, slice maximum, numerators, partial sum; E replaces the raw rows
+    auto stream_target = [&](auto whole) {
+      const unsigned char* rc = stage;
+      const unsigned char* ru = stage + rowbytes;
       const uint64_t s2 = pack2(P.cfg_scale, P.cfg_scale);
-      auto zt = [&](int g, float (&z)[8]) {
-        uint64_t c2[4], u2[4];
-        pairs_of(rc, g, c2);
-        if (UNC) pairs_of(ru, g, u2);
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          uint64_t l2 = c2[i];
-          if (UNC) l2 = fma2(s2, sub2(c2[i], u2[i]), u2[i]);
-          if (!T_is_one) l2 = divide_T(l2);
-          unpack2(l2, z[2 * i], z[2 * i + 1]);
+      auto pairs_of = [&](const unsigned char* row, int g, uint64_t (&o)[4]) {
+        Raw8<BF16> d;
+        if (BF16) {
+          d.a = *reinterpret_cast<const uint4*>(row + g * 16);
+        } else {
+          d.a = *reinterpret_cast<const uint4*>(row + g * 32);
+          d.b = *reinterpret_cast<const uint4*>(row + g * 32 + 16);
         }
+        raw8_pairs<BF16>(d, o);
       };
-      tq = tkg_kth_largest(zt, cur.bracket[1], P.top_k, V, CH, S.tk, 1, grp, gt, &P.counters->n_slow_topk);
-    }
-    // --- target: guidance combine, slice maximum, numerators, partial sum; E replaces the raw rows ---
+      float n_run = -3.0e37f;
+      tq = 0.0f;
+#pragma unroll (NP > 2 ? 1 : NP)
+      for (int p = 0; p < NP; ++p) {   // (rolled where there are many: three groups in different phases fill the instruction cache)
+        uint64_t a2[CP * 4];
+        float m = ninf;
 #pragma unroll
-    for (int p = 0; p < NP; ++p) {
-      const uint64_t s2 = pack2(P.cfg_scale, P.cfg_scale);
-      float mq = ninf;
+        for (int c = 0; c < CP; ++c) {
+          const int g = (p * CP + c) * GT + gt;
+          if (decltype(whole)::value || g * 8 < V) {
+            uint64_t c2[4], u2[4];
+            pairs_of(rc, g, c2);
+            if (UNC) pairs_of(ru, g, u2);
 #pragma unroll
-      for (int c = 0; c < CP; ++c) {
-        const int g = (p * CP + c) * GT + gt;
-        if (g * 8 < V) {
-          uint64_t c2[4], u2[4];
-          pairs_of(rc, g, c2);
-          if (UNC) pairs_of(ru, g, u2);
-#pragma unroll
-          for (int i = 0; i < 4; ++i) {
-            uint64_t l2 = c2[i];
-            if (UNC) l2 = fma2(s2, sub2(c2[i], u2[i]), u2[i]);   // l_u + s (l_c - l_u)
-            if (!T_is_one) l2 = divide_T(l2);
-            if (TOPK) {   // below the row's top-k threshold: -inf (a NaN stays, to be reported)
+            for (int i = 0; i < 4; ++i) {
+              uint64_t l2 = c2[i];
+              if (UNC) l2 = fma2(s2, sub2(c2[i], u2[i]), u2[i]);   // l_u + s (l_c - l_u)
+              if (!TONE) l2 = divide_T(l2);
+              a2[c * 4 + i] = l2;
               float lo, hi;
               unpack2(l2, lo, hi);
-              l2 = pack2(lo < tq ? ninf : lo, hi < tq ? ninf : hi);
+              m = max3(m, lo, hi);
             }
-            a2[c * 4 + i] = l2;
-            float lo, hi;
-            unpack2(l2, lo, hi);
-            mq = max3(mq, lo, hi);
+          } else {
+#pragma unroll
+            for (int i = 0; i < 4; ++i) a2[c * 4 + i] = pack2(ninf, ninf);
           }
-        } else {
-#pragma unroll
-          for (int i = 0; i < 4; ++i) a2[c * 4 + i] = pack2(ninf, ninf);
         }
+        const float n_p = ceilf(fmaxf(m, -1.0e37f) * L2E);
+        const uint64_t nn2 = pack2(-n_p, -n_p);
+        uint64_t t2 = pack2(0.0f, 0.0f);
+#pragma unroll
+        for (int c = 0; c < CP; ++c) {
+          uint64_t e2[4];
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            float lo, hi;
+            unpack2(fma2(a2[c * 4 + i], L2, nn2), lo, hi);
+            e2[i] = pack2(ex2_approx(lo), ex2_approx(hi));
+          }
+          t2 = add2(t2, add2(add2(e2[0], e2[1]), add2(e2[2], e2[3])));
+          const int g = (p * CP + c) * GT + gt;
+          if (decltype(whole)::value || g * 8 < V) {
+            *reinterpret_cast<ulonglong2*>(E + EI(g * 8)) = make_ulonglong2(e2[0], e2[1]);
+            *reinterpret_cast<ulonglong2*>(E + EI(g * 8 + 4)) = make_ulonglong2(e2[2], e2[3]);
+          }
+        }
+        float lo, hi;
+        unpack2(t2, lo, hi);
+        S.slice[p * GT + gt] = n_p;
+        if (NP <= 2) nq[NP <= 2 ? p : 0] = n_p;
+        const float n_new = fmaxf(n_run, n_p);
+        tq = __fmaf_rn(tq, exp2_int(n_run - n_new), (lo + hi) * exp2_int(n_p - n_new));
+        n_run = n_new;
       }
-      // a slice without any finite logit (padding, masked tokens) still needs a finite shift
-      mq = fmaxf(mq, -1.0e37f);
-      const float mlq_w = mq * L_hi;
-      mlq_mine[p] = mlq_w;
-      const uint64_t nml2 = pack2(-mlq_w, -mlq_w);
-      uint64_t t2 = pack2(0.0f, 0.0f);
-#pragma unroll
-      for (int c = 0; c < CP; ++c) {
-        float e[8];
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          float lo, hi;
-          unpack2(fma2(a2[c * 4 + i], L2, nml2), lo, hi);
-          e[2 * i] = ex2_approx(lo);
-          e[2 * i + 1] = ex2_approx(hi);
-        }
-        t2 = add2(t2, add2(add2(pack2(e[0], e[1]), pack2(e[2], e[3])), add2(pack2(e[4], e[5]), pack2(e[6], e[7]))));
-        const int g = (p * CP + c) * GT + gt;
-        if (g * 8 < V) {
-          *reinterpret_cast<float4*>(E + EI(g * 8)) = make_float4(e[0], e[1], e[2], e[3]);
-          *reinterpret_cast<float4*>(E + EI(g * 8 + 4)) = make_float4(e[4], e[5], e[6], e[7]);
-        }
-      }
-      float tlo, thi;
-      unpack2(t2, tlo, thi);
-      tq_mine[p] = tlo + thi;
+      nq_max = n_run;
+    };
+    if (nchild > 0) {
+      load_slots(xt, 0, nb);
+      if (gt == 0) fetch_single();
+      if (full) stream_drafter(std::true_type{});
+      else stream_drafter(std::false_type{});
+      if (gt == 0) note_single();
     }
+    // The target rows were issued when the staging area fell free; they arrive while the drafter
+    // row is streamed.  Every thread waits for itself (bounded); a wait that runs out is reported after
+    // the next group barrier, where every thread sees it alike.
+    if (item >= 0) {
+      if (!mbar_wait(&bar_rows[grp][area], (iter / AREAS) & 1, tries)) S.fail = 1;
+      if (full) stream_target(std::true_type{});
+      else stream_target(std::false_type{});
+    }
+
     // ---------------- group statistics ----------------
-    // common maxima first (one warp reduction, then eight values read by everybody), then the slices'
-    // factors and the normalisers
-    float mlq_g, mlp_g;
+    // per warp: the largest shift and the sum in its units, for target and drafter; then one barrier, and every
+    // warp combines the partials for itself (lane l: warp l % GW)
     {
-      float mq_t = mlq_mine[0], mp_t = mlp_mine[0];
+      const float n = nq_max;
+      const float wnq = redux_max(n), wnd = redux_max(nd);
+      const double zq = static_cast<double>(tq * exp2_int(n - wnq));
+      const double zp = static_cast<double>(td * exp2_int(nd - wnd));
+      // both sums in one butterfly: after the first exchange the lower half of the warp carries one, the upper the other
+      const bool up = lane & 16;
+      double z = (up ? zp : zq) + __shfl_xor_sync(kFull, up ? zq : zp, 16);
 #pragma unroll
-      for (int p = 1; p < NP; ++p) {
-        mq_t = fmaxf(mq_t, mlq_mine[p]);
-        mp_t = fmaxf(mp_t, mlp_mine[p]);
-      }
-      mq_t = warp_max(mq_t);
-      mp_t = warp_max(mp_t);
-      if (lane == 0) {
-        S.wmq[gw] = mq_t;
-        S.wmp[gw] = mp_t;
+      for (int o = 8; o > 0; o >>= 1) z += __shfl_xor_sync(kFull, z, o);
+      if ((lane & 15) == 0) {
+        S.wz[gw][up] = z;
+        S.wn[gw][up] = up ? wnd : wnq;
       }
     }
-    gbar(grp);   // [stats 1] per-warp maxima, and E, are visible
-    if (S.fail) {   // the target rows did not land within the limit
-      give_up(iter, false);
+    gbar();   // E, the slices' shifts and the per-warp partials are visible
+    if (S.fail) {   // no context was published, or its target rows did not land, within the limit
+      give_up();
       break;
     }
-    mlq_g = S.wmq[0];
-    mlp_g = S.wmp[0];
+    if (item < 0) break;
+    // the producer may choose (and publish) the next context
+    if (lane == 0) mbar_arrive(&bar_next[grp]);
+    float Nq, Np;                // common units
+    double Zq, Zp;
+    {
+      const float2 n = *reinterpret_cast<const float2*>(S.wn[lane & (GW - 1)]);
+      const double2 z = *reinterpret_cast<const double2*>(S.wz[lane & (GW - 1)]);
+      Nq = redux_max(n.x);
+      Np = redux_max(n.y);
+      Zq = z.x * static_cast<double>(exp2_int(n.x - Nq));
+      Zp = z.y * static_cast<double>(exp2_int(n.y - Np));
 #pragma unroll
-    for (int w = 1; w < GW; ++w) {
-      mlq_g = fmaxf(mlq_g, S.wmq[w]);
-      mlp_g = fmaxf(mlp_g, S.wmp[w]);
-    }
-    float fq_mine[NP], fp_mine[NP];
-    double Zq = 0.0, Zp = 0.0;
-#pragma unroll
-    for (int p = 0; p < NP; ++p) {
-      fq_mine[p] = ex2_approx(mlq_mine[p] - mlq_g);
-      fp_mine[p] = ex2_approx(mlp_mine[p] - mlp_g);
-      S.fqt[p * GT + gt] = fq_mine[p];
-      Zq += static_cast<double>(fq_mine[p]) * static_cast<double>(tq_mine[p]);
-      Zp += static_cast<double>(fp_mine[p]) * static_cast<double>(tp_mine[p]);
-    }
-    Zq = warp_sum(Zq);
-    Zp = warp_sum(Zp);
-    if (lane == 0) {
-      S.wzq[gw] = Zq;
-      S.wzp[gw] = Zp;
-    }
-    gbar(grp);   // [stats 2] factor table and per-warp sums are visible
-    Zq = 0.0;
-    Zp = 0.0;
-#pragma unroll
-    for (int w = 0; w < GW; ++w) {
-      Zq += S.wzq[w];
-      Zp += S.wzp[w];
+      for (int o = GW / 2; o > 0; o >>= 1) {
+        Zq += __shfl_xor_sync(kFull, Zq, o);
+        Zp += __shfl_xor_sync(kFull, Zp, o);
+      }
     }
 
     int status = 0;              // bits every thread sets alike
     int accepted = -1;
-    bool record_written = false;
+    bool drawn = false;
+    // normalisers: q'(x) = E(x) * 2^(slice shift - Nq) / Zq_c, and p' likewise
+    // (Zp_c = 0 stands for a drafter distribution that has no mass left).  Comparisons are written on
+    // the unnormalised sums, so that no thread divides on the way to a decision.
+    double Zq_c = Zq, Zp_c = Zp;
     if (!(Zq > 0.0 && Zq < 1e300 && Zp > 0.0 && Zp < 1e300)) {
       status |= LANTERN_ST_NONFINITE;
     } else {
-      // current normalisers: q'(x) = E(x) * fq[slice of x] / Zq_c,  p'(x) = ep(x) * fp[slice of x] / Zp_c
-      // (Zp_c = 0 stands for a drafter distribution that has no mass left).  Comparisons are written on
-      // the unnormalised sums, so that no thread divides on the way to a decision.
-      double Zq_c = Zq, Zp_c = Zp;
       const double delta = static_cast<double>(P.delta);
-      if (gt == 0) {   // the two single probabilities of the first child, in double precision
-        float zq = raw_c;
-        if (UNC) zq = __fmaf_rn(P.cfg_scale, __fsub_rn(raw_c, raw_u), raw_u);
-        float zp = raw_d;
-        if (!T_is_one) {
-          zq = __fdiv_rn(zq, P.T);
-          zp = __fdiv_rn(zp, P.T);
-        }
-        if (TOPK) {   // these come from global memory, unfiltered
-          zq = zq < tq ? ninf : zq;
-          zp = zp < tp ? ninf : zp;
-        }
-        S.acc_e = exp2_single(zq, mlq_g);
-        S.acc_p = exp2_single(zp, mlp_g);
-        S.acc_valid = 1;
-      }
+      const ChildInfo* kids = P.children + cur.cbase;
+      float r = cur.r0;
+      auto mass = [&](int n) { return E[EI(n)] * exp2_int(S.slice[owner_slice(n)] - Nq); };   // common units
 
       for (int ci = 0; ci < nchild; ++ci) {
-        if (gt == 0) atomicAdd(&P.counters->n_tested, 1);   // work accounting (a fire-and-forget reduction)
-        const int32_t* nrow = P.nbr + static_cast<size_t>(xt) * k;
         // the next sibling's description, wanted only after a rejection: in flight meanwhile
-        ChildInfo sib = {0, 0, 0.0f, 0};
-        if (ci + 1 < nchild) {
-          const int4 v = __ldg(reinterpret_cast<const int4*>(kids + ci + 1));
-          sib.node = v.x, sib.token = v.y, sib.r = __int_as_float(v.z);
-        }
-        // bulk numerators of x~ itself, common units (drafter: from its raw logit; no mass is left once x~
-        // was rejected as an earlier sibling of this context, or where the top-k filter cut it)
-        float px_bulk, e_xt_bulk;
-        {
-          float dz = raw_d;
-          if (!T_is_one) dz = __fdiv_rn(dz, P.T);
-          if (TOPK) dz = dz < tp ? ninf : dz;
-          for (int j = 0; j < ci; ++j)
-            if (__ldg(&kids[j].token) == xt) dz = ninf;
-          px_bulk = ex2_approx(__fmaf_rn(dz, L_hi, -mlp_g));
-          e_xt_bulk = E[EI(xt)] * S.fqt[owner_slice<LOG_CP>(xt)];
+        int4 sib = make_int4(0, 0, 0, 0);
+        if (ci + 1 < nchild) sib = __ldg(reinterpret_cast<const int4*>(kids + ci + 1));
+        if (gt == 0) {
+          // The tested token's two numerators in common units, in double precision from its raw logits, carried
+          // through every rejection round so far (E <- max(0, E - ratio_i * ep)); the sums they are compared
+          // with are sums of thousands of terms and do not suffer from cancellation.  A token that has lost its
+          // mass (it lay in an earlier A, or was itself rejected before) has none.
+          const Exp2Split q = S.single[0], p = S.single[1];
+          double e = q.y * exp2_int_d(q.n - static_cast<double>(Nq));
+          double pe = p.y * exp2_int_d(p.n - static_cast<double>(Np));
+          if (ci > 0) {
+            const float bulk = mass(xt);
+            if (ci <= 32) {
+              for (int i = 0; i < ci; ++i) e = fmax(0.0, e - S.hist[i] * pe);
+              if (bulk == 0.0f) e = 0.0;
+            } else {
+              e = static_cast<double>(bulk);
+            }
+            for (int j = 0; j < ci; ++j)
+              if (__ldg(&kids[j].token) == xt) pe = 0.0;
+          }
+          S.acc_e = e;
+          S.acc_p = pe;
+          atomicAdd(&P.counters->n_tested, 1);   // work accounting (a fire-and-forget reduction)
         }
 
         // ---- A_{k,delta}(x~): gather + prefix scan with the strict bound ----
         double thr = delta * Zq_c;   // the bound in the units of the unnormalised sums
-        // Section 5.3.2: the mass whose JSD is delta; the group's last warp finds it together, published by
-        // [scan 1] through the last slot of wt[], which nothing else touches between the start of a child and
-        // its [scan 2]
+        // Section 5.3.2: the mass whose JSD is delta; the group's last warp finds it together
         if (JSD && gw == GW - 1) {
-          const double sstar = jsd_mass_bound_warp(delta, static_cast<double>(e_xt_bulk) / Zq_c, lane) * Zq_c;
-          if (lane == 0) S.wt[8 * GW - 1] = sstar;
+          const double mine = jsd_mass_bound_warp(delta, static_cast<double>(mass(xt)) / Zq_c, lane) * Zq_c;
+          if (lane == 0) S.jsd_mass = mine;
         }
         double carry = 0.0, sm = 0.0;
         int m = k - 1;
         bool cut = false;
-        for (int base = 0; base < k - 1 && !cut; base += 4 * GT) {
-          double pre4[4];       // inclusive prefix over this thread's four slots
-          bool val4[4];
+        for (int base = 0; !cut && base < k; base += SLOTS * GT) {
+          if (base > 0) load_slots(xt, base, nb);
+          const int j0 = base + SLOTS * gt;
+          double pre[SLOTS];    // inclusive prefix over this thread's slots
           double run = 0.0;
-          int my_bad = kNone;   // first of this thread's slots whose entry lies outside [0, V): it carries no mass
 #pragma unroll
-          for (int i = 0; i < 4; ++i) {
-            const int j = base + 4 * gt + 1 + i;
-            val4[i] = j < k;
-            const int n = base == 0 ? nb[i] : (val4[i] ? __ldg(nrow + j) : -1);
-            const bool inr = val4[i] && static_cast<unsigned>(n) < static_cast<unsigned>(V);
-            if (val4[i] && !inr && my_bad == kNone) my_bad = j;
-            run += inr ? static_cast<double>(E[EI(n)] * S.fqt[owner_slice<LOG_CP>(n)]) : 0.0;
-            pre4[i] = run;
+          for (int i = 0; i < SLOTS; ++i) {
+            const int j = j0 + i, n = nb[i];
+            if (j >= 1 && j < k) {
+              if (static_cast<unsigned>(n) < static_cast<unsigned>(V)) run += static_cast<double>(mass(n));
+              else atomicMin(&S.badslot[round3], j);   // carries no mass
+            }
+            pre[i] = run;
           }
           const double incl = warp_incl_scan(run, lane);
-          if (lane == 31) S.wt[gw] = incl;
-          gbar(grp);   // [scan 1]
-          if (JSD && base == 0) thr = S.wt[8 * GW - 1];
-          double pre = 0.0, tot = 0.0;
+          if (lane == 31) S.wt[round2 * GW + gw] = incl;
+          gbar();   // [scan 1]
+          if (JSD && base == 0) thr = S.jsd_mass;
+          // every warp: running totals of the warps (lane l: warp l % GW), the first one that reaches the bound
+          double tot = S.wt[round2 * GW + (lane & (GW - 1))];
 #pragma unroll
-          for (int w = 0; w < GW; ++w) {
-            const double t = S.wt[w];
-            if (w < gw) pre += t;
-            tot += t;
+          for (int o = 1; o < GW; o <<= 1) {
+            const double t = __shfl_up_sync(kFull, tot, o);
+            if ((lane & (GW - 1)) >= o) tot += t;
           }
-          const double before = carry + pre + (incl - run);   // prefix before this thread's first slot
-          int my_first = kNone;
-          double my_before = 0.0;
-#pragma unroll
-          for (int i = 3; i >= 0; --i) {
-            const double Sj = before + pre4[i];
-            if (val4[i] && !(Sj < thr)) {
-              my_first = base + 4 * gt + 1 + i;
-              my_before = i > 0 ? before + pre4[i > 0 ? i - 1 : 0] : before;
-            }
-          }
-          const int wfirst = __reduce_min_sync(kFull, my_first);
-          if (wfirst != kNone && my_first == wfirst) {
-            S.first[gw] = wfirst;
-            S.sbefore[gw] = my_before;
-          } else if (wfirst == kNone && lane == 0) {
-            S.first[gw] = kNone;
-          }
-          const int wbad = __reduce_min_sync(kFull, my_bad);
-          if (lane == 0) S.badslot[gw] = wbad;
-          gbar(grp);   // [scan 2]
-          int gfirst = kNone, src = 0, gbad = kNone;
-#pragma unroll
-          for (int w = GW - 1; w >= 0; --w) {
-            const int f = S.first[w];
-            if (f != kNone && f <= gfirst) {
-              gfirst = f;
-              src = w;
-            }
-            gbad = min(gbad, S.badslot[w]);
-          }
-          // a bad entry is reported where Algorithm 2's loop meets it, i.e. ahead of the slot that ends the set
-          if (gbad < gfirst) status |= LANTERN_ST_BAD_TABLE;
-          if (gfirst != kNone) {
-            m = gfirst - 1;
-            sm = S.sbefore[src];
-            cut = true;
-          } else {
-            carry += tot;
+          const unsigned over = __ballot_sync(kFull, !(carry + tot < thr));
+          const int bad = S.badslot[round3];
+          const int after = round3 < 2 ? round3 + 1 : 0, clear = after < 2 ? after + 1 : 0;
+          if (gt == 0) S.badslot[clear] = kNone;   // last read before [scan 1], next written behind the next one
+          const double carry_in = carry;
+          round2 ^= 1;
+          round3 = after;
+          if (over == 0) {
+            if (bad != kNone) status |= LANTERN_ST_BAD_TABLE;
+            carry += __shfl_sync(kFull, tot, GW - 1);
             sm = carry;
+          } else {
+            cut = true;
+            const int wc = __ffs(over) - 1;   // (the first GW lanes come first)
+            if (gw == wc) {
+              const double below = __shfl_sync(kFull, tot, (wc + GW - 1) & (GW - 1));
+              const double before = carry_in + (wc > 0 ? below : 0.0) + (incl - run);   // prefix before this thread's first slot
+              int first = kNone;
+              double moved = 0.0;
+#pragma unroll
+              for (int i = SLOTS - 1; i >= 0; --i) {
+                if (j0 + i >= 1 && j0 + i < k && !(before + pre[i] < thr)) {
+                  first = j0 + i;
+                  moved = i > 0 ? before + pre[i > 0 ? i - 1 : 0] : before;
+                }
+              }
+              const unsigned who = __ballot_sync(kFull, first != kNone);
+              if (who ? lane == __ffs(who) - 1 : lane == 31) {
+                // (no slot: the total reached the bound by rounding alone; the set ends with this warp's slots)
+                S.cut_m = who ? first - 1 : min(j0 + SLOTS - 1, k - 1);
+                S.cut_sum = who ? moved : before + run;
+              }
+            }
+            gbar();   // [scan 2]
+            m = S.cut_m;
+            sm = S.cut_sum;
+            // a bad entry is reported where Algorithm 2's loop meets it, i.e. ahead of the slot that ends the set
+            if (bad <= m) status |= LANTERN_ST_BAD_TABLE;
           }
         }
-        if (k == 1) gbar(grp);   // publish S.acc_* when the scan loop did not run
-        // the two single probabilities: thread 0's double-precision values where it has them; a bulk
-        // value of exactly zero (token inside an earlier A, or rejected before) stays zero
-        const bool acc = S.acc_valid != 0;
-        const double e_xt = (acc && e_xt_bulk != 0.0f) ? S.acc_e : static_cast<double>(e_xt_bulk);
-        const double p_xt = (acc && px_bulk != 0.0f) ? S.acc_p : static_cast<double>(px_bulk);
         // Section 4.3: accept iff r p(x~) < sum_A q, i.e. r p_xt / Zp_c < (e_xt + sm) / Zq_c, both sides times Zq_c Zp_c
-        const double qa_un = e_xt + sm;
+        const double p_xt = S.acc_p;
+        const double qa_un = S.acc_e + sm;
         const bool accept = Zp_c > 0.0 ? static_cast<double>(r) * p_xt * Zq_c < qa_un * Zp_c : 0.0 < qa_un;
         if (gt == 0 && (P.out_qa || P.out_px || P.out_m)) {
-          const size_t o = static_cast<size_t>(b) * N + node;
+          const size_t o = static_cast<size_t>(item / R) * N + node;
           if (P.out_qa) P.out_qa[o] = static_cast<float>(qa_un / Zq_c);
           if (P.out_px) P.out_px[o] = Zp_c > 0.0 ? static_cast<float>(p_xt / Zp_c) : 0.0f;
           if (P.out_m) P.out_m[o] = m;
@@ -933,23 +968,20 @@ __global__ void __launch_bounds__(CTX_THREADS, 1) lantern_context_kernel(VerifyP
           break;
         }
         // ---- rejected: residual [q_{k,delta}(.|D = x~) - p]_+ ----
-        // the drafter logits of the first pass: asked for at once, in flight while A is flagged and across the barrier
-        const unsigned char* drow = static_cast<const unsigned char*>(P.draft) + static_cast<size_t>(item) * rowbytes;
-        DraftRaw dnext[CP];
+        // the first drafter logits: asked for at once, in flight while A is flagged and across the barrier
+        Raw8<BF16> ahead[AHEAD];
 #pragma unroll
-        for (int c = 0; c < CP; ++c) {
+        for (int c = 0; c < AHEAD; ++c) {
           const int g = c * GT + gt;
-          dnext[c] = draft_fetch(drow, g * 8 < V ? g : gt);
+          ahead[c] = load_raw8<BF16>(drow, g * 8 < V ? g : 0);
         }
         // members of A (x~ included) leave no residual mass: flag them with a negative sign
-        for (int base = 0; base < m; base += 4 * GT) {
+        for (int base = 0; base <= m; base += SLOTS * GT) {
+          if (base > 0 || m >= SLOTS * GT - 1) load_slots(xt, base, nb);   // (a longer scan has replaced the first slots)
 #pragma unroll
-          for (int i = 0; i < 4; ++i) {
-            const int j = base + 4 * gt + 1 + i;
-            if (j <= m) {
-              const int n = base == 0 ? nb[i] : __ldg(nrow + j);
-              if (static_cast<unsigned>(n) < static_cast<unsigned>(V)) E[EI(n)] = -fabsf(E[EI(n)]);
-            }
+          for (int i = 0; i < SLOTS; ++i) {
+            const int j = base + SLOTS * gt + i;
+            if (j >= 1 && j <= m && static_cast<unsigned>(nb[i]) < static_cast<unsigned>(V)) E[EI(nb[i])] = -fabsf(E[EI(nb[i])]);
           }
         }
         if (gt == 0) E[EI(xt)] = -fabsf(E[EI(xt)]);
@@ -962,236 +994,187 @@ __global__ void __launch_bounds__(CTX_THREADS, 1) lantern_context_kernel(VerifyP
           if (((t >> 3) & (GT - 1)) == gt) struck |= 1u << (t >> (3 + LOG_GT));
         }
         const bool last = (ci + 1 == nchild);
-        if (!last) {   // next sibling's neighbour row, in flight during the residual pass
-          node = sib.node;
-          xt = sib.token;
-          r = sib.r;
-#pragma unroll
-          for (int i = 0; i < 4; ++i) {
-            const int j = 4 * gt + 1 + i;
-            nb[i] = (j < k) ? ld_nc_here(P.nbr + static_cast<size_t>(xt) * k + j) : -1;
-          }
-          raw_d = ctx_raw_logit<BF16>(P.draft, static_cast<size_t>(item) * V + xt);
-          if (gt == 0) {   // its raw target logits, for the double-precision replay below
-            const size_t e = static_cast<size_t>(item) * V + xt;
-            raw_c = ctx_raw_logit<BF16>(P.target, e);
-            if (UNC) raw_u = ctx_raw_logit<BF16>(P.target, static_cast<size_t>(P.B) * R * V + e);
-          }
+        if (!last) {   // next sibling's neighbour row and raw logits, in flight during the residual pass
+          node = sib.x;
+          xt = sib.y;
+          r = __int_as_float(sib.z);
+          load_slots(xt, 0, nb);
+          if (gt == 0) fetch_single();
         }
-        gbar(grp);   // [flags]
+        gbar();   // [flags]
         // w = E - (p'/q' scale ratio) * ep in common units, i.e. E - ratio * ep in the slice's own units
         // of E; the residual replaces E (it is the next sibling's target, or what the draw reads)
         const float ratio_g = Zp_c > 0.0 ? static_cast<float>(Zq_c / Zp_c) : 0.0f;
-        float cs[CH];
-        double wsum = 0.0, psum = 0.0;
+        const float fd = exp2_int(nd - Np);   // this thread's drafter units -> common units
+        float wsum = 0.0f, psum = 0.0f;       // common units; the thread's own units
 #pragma unroll
         for (int p = 0; p < NP; ++p) {
           // (a slice whose numerators are all negligible has factor 0; nothing of it survives anyway)
-          const float ratio = fq_mine[p] > 0.0f ? ratio_g * (fp_mine[p] / fq_mine[p]) : 0.0f;
-          float wp_ = 0.0f, pp_ = 0.0f;
-          DraftRaw dcur[CP];
+          const float fq = exp2_int(shift_of(p) - Nq);
+          const float ratio = fq > 0.0f ? ratio_g * (fd / fq) : 0.0f;
+          const uint64_t nr2 = pack2(-ratio, -ratio), nn2 = pack2(-nd, -nd);
 #pragma unroll
-          for (int c = 0; c < CP; ++c) {
-            dcur[c] = dnext[c];
-            if (p + 1 < NP) {   // the next pass's logits travel during this pass
-              const int g = ((p + 1) * CP + c) * GT + gt;
-              dnext[c] = draft_fetch(drow, g * 8 < V ? g : gt);
+          for (int c = p * CP; c < (p + 1) * CP; ++c) {
+            const Raw8<BF16> raw = ahead[c % AHEAD];
+            if (c + AHEAD < CH) {   // the next groups travel during this one
+              const int g = (c + AHEAD) * GT + gt;
+              ahead[c % AHEAD] = load_raw8<BF16>(drow, g * 8 < V ? g : 0);
             }
-          }
+            const int g = c * GT + gt;
+            if (full || g * 8 < V) {
+              float z[8];
+              {
+                uint64_t z2[4];
+                raw8_pairs<BF16>(raw, z2);
 #pragma unroll
-          for (int c = 0; c < CP; ++c) {
-            const int g = (p * CP + c) * GT + gt;
-            float w8[8];
-            if (g * 8 < V) {
-              const float4 lo = *reinterpret_cast<const float4*>(E + EI(g * 8));
-              const float4 hi = *reinterpret_cast<const float4*>(E + EI(g * 8 + 4));
-              const float e8[8] = {lo.x, lo.y, lo.z, lo.w, hi.x, hi.y, hi.z, hi.w};
-              float ep8[8];
-              draft_chunk(dcur[c], ep8);
-              if (TOPK) {   // below the row's top-k threshold: -inf
-#pragma unroll
-                for (int e = 0; e < 8; ++e) ep8[e] = ep8[e] < tp ? ninf : ep8[e];
+                for (int i = 0; i < 4; ++i) {
+                  if (!TONE) z2[i] = divide_T(z2[i]);
+                  unpack2(z2[i], z[2 * i], z[2 * i + 1]);
+                }
               }
-              if ((struck >> (p * CP + c)) & 1u) {   // a token rejected in this context sits in this chunk
+              if ((struck >> c) & 1u) {   // a token rejected in this context sits in this chunk
                 for (int j = 0; j <= ci; ++j) {
                   const int t = __ldg(&kids[j].token);
                   if ((t >> 3) == g) {
 #pragma unroll
-                    for (int e = 0; e < 8; ++e) ep8[e] = (t & 7) == e ? ninf : ep8[e];
+                    for (int e = 0; e < 8; ++e) z[e] = (t & 7) == e ? ninf : z[e];
                   }
                 }
               }
+              const ulonglong2 ea = *reinterpret_cast<const ulonglong2*>(E + EI(g * 8));
+              const ulonglong2 eb = *reinterpret_cast<const ulonglong2*>(E + EI(g * 8 + 4));
+              const uint64_t e2[4] = {ea.x, ea.y, eb.x, eb.y};
+              uint64_t w2[4], ps2 = pack2(0.0f, 0.0f);
 #pragma unroll
-              for (int e = 0; e < 8; ++e) {
-                ep8[e] = ex2_approx(__fmaf_rn(ep8[e], L_hi, -mlp_mine[p]));
-                w8[e] = fmaxf(0.0f, __fmaf_rn(-ratio, ep8[e], e8[e]));
+              for (int i = 0; i < 4; ++i) {
+                float lo, hi;
+                unpack2(fma2(pack2(z[2 * i], z[2 * i + 1]), L2, nn2), lo, hi);
+                const uint64_t ep = pack2(ex2_approx(lo), ex2_approx(hi));
+                ps2 = add2(ps2, ep);
+                unpack2(fma2(nr2, ep, e2[i]), lo, hi);
+                w2[i] = pack2(fmaxf(0.0f, lo), fmaxf(0.0f, hi));
               }
-              pp_ += sum8(ep8);
-              *reinterpret_cast<float4*>(E + EI(g * 8)) = make_float4(w8[0], w8[1], w8[2], w8[3]);
-              *reinterpret_cast<float4*>(E + EI(g * 8 + 4)) = make_float4(w8[4], w8[5], w8[6], w8[7]);
-            } else {
-#pragma unroll
-              for (int e = 0; e < 8; ++e) w8[e] = 0.0f;
-            }
-            cs[p * CP + c] = sum8(w8);
-            wp_ += cs[p * CP + c];
-          }
-          wsum += static_cast<double>(wp_) * static_cast<double>(fq_mine[p]);
-          psum += static_cast<double>(pp_) * static_cast<double>(fp_mine[p]);
-        }
-        double W, Sp;
-        if (!last) {
-          const double ww = warp_sum(wsum);
-          const double wp = warp_sum(psum);
-          if (lane == 0) {
-            S.wt[gw] = ww;
-            S.wt[GW + gw] = wp;
-          }
-          gbar(grp);   // [totals] also publishes the written-back residual
-          W = 0.0;
-          Sp = 0.0;
-#pragma unroll
-          for (int w = 0; w < GW; ++w) {
-            W += S.wt[w];
-            Sp += S.wt[GW + w];
-          }
-          if (!(W > kDegenerate * Zq_c)) {
-            status |= LANTERN_ST_DEGENERATE;
-            break;
-          }
-          if (gt == 0) {
-            // The next sibling's own two probabilities in double precision: its numerators from the raw
-            // logits, carried through every rejection round so far (E <- max(0, E - ratio_i * ep)); the
-            // totals W, Sp are sums of thousands of terms and do not suffer from cancellation.
-            if (ci < 32) {
-              S.hist[ci] = static_cast<double>(ratio_g);
-              float zq = raw_c;
-              if (UNC) zq = __fmaf_rn(P.cfg_scale, __fsub_rn(raw_c, raw_u), raw_u);
-              float zp = raw_d;
-              if (!T_is_one) {
-                zq = __fdiv_rn(zq, P.T);
-                zp = __fdiv_rn(zp, P.T);
-              }
-              if (TOPK) {   // these come from global memory, unfiltered
-                zq = zq < tq ? ninf : zq;
-                zp = zp < tp ? ninf : zp;
-              }
-              double e = exp2_single(zq, mlq_g);
-              const double pe = exp2_single(zp, mlp_g);
-              for (int i = 0; i <= ci; ++i) e = fmax(0.0, e - S.hist[i] * pe);
-              S.acc_e = e;
-              S.acc_p = pe;
-              S.acc_valid = 1;
-            } else {
-              S.acc_valid = 0;
+              *reinterpret_cast<ulonglong2*>(E + EI(g * 8)) = make_ulonglong2(w2[0], w2[1]);
+              *reinterpret_cast<ulonglong2*>(E + EI(g * 8 + 4)) = make_ulonglong2(w2[2], w2[3]);
+              float lo, hi;
+              unpack2(ps2, lo, hi);
+              psum += lo + hi;
+              unpack2(add2(add2(w2[0], w2[1]), add2(w2[2], w2[3])), lo, hi);
+              wsum = __fmaf_rn(lo + hi, fq, wsum);
             }
           }
-          Zq_c = W;
-          Zp_c = Sp > 0.0 ? Sp : 0.0;
-          continue;
         }
-        // ---- last child rejected: draw the replacement token from the residual (Algorithm 1) ----
-        double csd[CH], incl[CH], excl[CH] = {};
+        if (last) break;   // the draw below takes it from here
+        const float both[2] = {wsum, psum * fd};
+        const double z = warp_transposed_sum<2>(both, lane);
+        if ((lane & 15) == 0) S.wz[gw][lane >> 4] = z;
+        if (gt == 0) note_single();
+        gbar();   // [totals] also publishes the written-back residual
+        const double2 z2 = *reinterpret_cast<const double2*>(S.wz[lane & (GW - 1)]);
+        double W = z2.x, Sp = z2.y;
 #pragma unroll
-        for (int c = 0; c < CH; ++c) {
-          csd[c] = static_cast<double>(cs[c]) * static_cast<double>(fq_mine[c / CP]);
-          incl[c] = warp_incl_scan(csd[c], lane);
-          if (lane == 31) S.wt[c * GW + gw] = incl[c];
-        }
-        gbar(grp);   // [draw 1]
-        {
-          // exclusive prefix over (chunk, warp) in chunk-major order; 32 entries per round
-          double carry2 = 0.0;
-#pragma unroll
-          for (int half = 0; half < (CH * GW + 31) / 32; ++half) {
-            const int e = half * 32 + lane;
-            const double t = e < CH * GW ? S.wt[e] : 0.0;
-            const double in = warp_incl_scan(t, lane);
-            const double ex = carry2 + in - t;
-#pragma unroll
-            for (int c = 0; c < CH; ++c) {
-              const int want = c * GW + gw;
-              const double got = __shfl_sync(kFull, ex, want & 31);
-              if ((want >> 5) == half) excl[c] = got + incl[c] - csd[c];
-            }
-            carry2 += __shfl_sync(kFull, in, 31);
-          }
-          W = carry2;
+        for (int o = GW / 2; o > 0; o >>= 1) {
+          W += __shfl_xor_sync(kFull, W, o);
+          Sp += __shfl_xor_sync(kFull, Sp, o);
         }
         if (!(W > kDegenerate * Zq_c)) {
           status |= LANTERN_ST_DEGENERATE;
           break;
         }
-        const double target = static_cast<double>(cur.u_final) * W;
-        int cand = kNone;
+        if (gt == 0 && ci < 32) S.hist[ci] = static_cast<double>(ratio_g);
+        Zq_c = W;
+        Zp_c = Sp > 0.0 ? Sp : 0.0;
+      }
+
+      // ---- the draw, by inverse CDF over E in token order: the replacement token from the residual where the last
+      // child was rejected (Algorithm 1), the bonus token from q itself where there are no children ----
+      if (accepted < 0 && !(status & LANTERN_ST_DEGENERATE)) {
+        {
+          float cs[CH];        // weight of each of this thread's chunks, common units
 #pragma unroll
-        for (int c = CH - 1; c >= 0; --c)
-          if (excl[c] + csd[c] > target) cand = c * GT + gt;
-        const int wmin = __reduce_min_sync(kFull, cand);
-        if (lane == 0) S.cand[gw] = wmin;
-        if (gt == 0) S.tok = -1;
-        gbar(grp);   // [draw 2]
-        const int win = __reduce_min_sync(kFull, lane < GW ? S.cand[lane] : kNone);
-        if (win == kNone) {
-          // rounding left no slot above the target: the largest token of positive weight
+          for (int c = 0; c < CH; ++c) {
+            const int g = c * GT + gt;
+            cs[c] = 0.0f;
+            if (full || g * 8 < V) {
+              const ulonglong2 ea = *reinterpret_cast<const ulonglong2*>(E + EI(g * 8));
+              const ulonglong2 eb = *reinterpret_cast<const ulonglong2*>(E + EI(g * 8 + 4));
+              float lo, hi;
+              unpack2(add2(add2(ea.x, ea.y), add2(eb.x, eb.y)), lo, hi);
+              cs[c] = (lo + hi) * exp2_int(shift_of(c / CP) - Nq);
+            }
+          }
+          const double t = warp_transposed_sum<CH>(cs, lane);
+          if ((lane & (32 / CH - 1)) == 0) S.wt[(lane / (32 / CH)) * GW + gw] = t;
+          if (gt == 0) S.tok = -1;
+        }
+        gbar();   // [draw 1] totals of the (chunk, warp) blocks, in token order chunk by chunk
+        double before, W;
+        int blk;
+        {
+          // every warp: the block in which the cumulative weight first exceeds the target (two blocks per lane)
+          const double t0 = 2 * lane < CH * GW ? S.wt[2 * lane] : 0.0, t1 = 2 * lane < CH * GW ? S.wt[2 * lane + 1] : 0.0;
+          const double incl = warp_incl_scan(t0 + t1, lane);
+          W = __shfl_sync(kFull, incl, 31);
+          const double target = static_cast<double>(cur.u_final) * W;
+          const unsigned over = __ballot_sync(kFull, incl > target);
+          const double ex = incl - (t0 + t1);
+          const bool second = !(ex + t0 > target);
+          blk = over ? __shfl_sync(kFull, 2 * lane + (second ? 1 : 0), __ffs(over) - 1) : -1;
+          before = __shfl_sync(kFull, second ? ex + t0 : ex, over ? __ffs(over) - 1 : 0);
+        }
+        const double target = static_cast<double>(cur.u_final) * W;
+        if (!(W > kDegenerate * Zq_c)) {
+          status |= LANTERN_ST_DEGENERATE;
+        } else if (blk < 0) {
+          // rounding left no block above the target: the largest token of positive weight
           int lastp = -1;
           for (int c = 0; c < CH; ++c) {
             const int g = c * GT + gt;
-            if (g * 8 < V && cs[c] > 0.0f)
+            if (g * 8 < V)
               for (int e = 0; e < 8; ++e)
                 if (E[EI(g * 8 + e)] > 0.0f) lastp = g * 8 + e;
           }
           if (lastp >= 0) atomicMax(&S.tok, lastp);
-          gbar(grp);
-          if (gt == 0) {
-            Record rec = {-1, S.tok, status | (S.tok < 0 ? LANTERN_ST_DEGENERATE : 0), 0};
-            P.records[item] = rec;
-          }
-        } else if ((win & (GT - 1)) == gt) {
-          const int wc = win >> LOG_GT;
-          const int g = wc * GT + gt;
-          double ex_c = 0.0, fqd = 0.0;
-#pragma unroll
-          for (int c = 0; c < CH; ++c)
-            if (c == wc) {
-              ex_c = excl[c];
-              fqd = static_cast<double>(fq_mine[c / CP]);
+          gbar();
+          drawn = true;
+          if (gt == 0) S.result[iter & 1] = {-1, S.tok, status | (S.tok < 0 ? LANTERN_ST_DEGENERATE : 0)};
+        } else {
+          drawn = true;
+          if ((blk & (GW - 1)) == gw) {   // the block's own warp: the thread, then the token
+            const int c = blk / GW, g = c * GT + gt;
+            float w8[8] = {};
+            float fq = 0.0f;
+            if (g * 8 < V) {
+              const float4 a = *reinterpret_cast<const float4*>(E + EI(g * 8));
+              const float4 b = *reinterpret_cast<const float4*>(E + EI(g * 8 + 4));
+              w8[0] = a.x, w8[1] = a.y, w8[2] = a.z, w8[3] = a.w, w8[4] = b.x, w8[5] = b.y, w8[6] = b.z, w8[7] = b.w;
+              fq = exp2_int(S.slice[(c / CP) * GT + gt] - Nq);
             }
-          int tok = -1, lastpos = -1;
-          double cum = ex_c;
-          for (int e = 0; e < 8; ++e) {
-            const float wv = E[EI(g * 8 + e)];
-            cum += static_cast<double>(wv) * fqd;
-            if (wv > 0.0f) lastpos = e;
-            if (tok < 0 && cum > target) tok = e;
+            const double mine = static_cast<double>(sum8(w8) * fq);
+            const double incl = warp_incl_scan(mine, lane);
+            const unsigned over = __ballot_sync(kFull, before + incl > target);
+            const unsigned some = __ballot_sync(kFull, mine > 0.0);
+            const int who = over ? __ffs(over) - 1 : 31 - __clz(some);   // (rounding: its last thread with weight)
+            if (lane == who) {
+              int tok = -1, lastpos = -1;
+              double cum = before + (incl - mine);
+#pragma unroll
+              for (int e = 0; e < 8; ++e) {
+                cum += static_cast<double>(w8[e]) * static_cast<double>(fq);
+                if (w8[e] > 0.0f) lastpos = e;
+                if (tok < 0 && cum > target) tok = e;
+              }
+              if (tok < 0) tok = lastpos;
+              S.result[iter & 1] = {-1, g * 8 + tok, status};
+            }
           }
-          if (tok < 0) tok = lastpos;
-          Record rec = {-1, g * 8 + tok, status, 0};
-          P.records[item] = rec;
         }
-        record_written = true;
       }
     }
-    if (!record_written && gt == 0) {
-      Record rec = {accepted, -1, status, 0};
-      P.records[item] = rec;
-    }
-    // Algorithm 1 goes on from the accepted child only: every context behind another child is dead.  In
-    // pre-order those are one contiguous range per child.
-    for (int j = 0; j < nchild; ++j) {
-      int node_j = cur.node0, span_j = cur.span0;
-      if (j > 0) {
-        const int4 kid = __ldg(reinterpret_cast<const int4*>(kids + j));
-        node_j = kid.x, span_j = kid.w;
-      }
-      if (node_j != accepted) {
-        unsigned char* first = P.dead + static_cast<size_t>(b) * R + (span_j >> 16);
-        for (int o = gt; o < (span_j & 0xffff); o += GT) first[o] = 1;
-      }
-    }
-    // this context's staging area (rows and E) is no longer needed by this warp
+    if (!drawn && gt == 0) S.result[iter & 1] = {accepted, -1, status};
+    // this context's staging area (rows and E) is no longer needed by this warp, and its result is there
     __syncwarp();
-    if (lane == 0) mbar_arrive(&bar_empty_t[grp]);
+    if (lane == 0) mbar_arrive(&bar_done[grp][iter & 1]);
   }
 }
 

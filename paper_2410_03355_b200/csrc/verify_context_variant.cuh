@@ -1,31 +1,63 @@
 // One compile-time variant (TONE, JSD, TOPK) of the fused context kernel for every row layout:
 // included by verify_context_v*.cu after defining LANTERN_VARIANT_{TONE,JSD,TOPK,NAME}.
 #include "verify_common.cuh"
+#if LANTERN_VARIANT_TOPK
+#include "verify_context_filtered.cuh"
+#else
 #include "verify_context.cuh"
+#endif
 
 namespace lantern {
 
+#if LANTERN_VARIANT_TOPK
 template <int CHC, bool BF16, bool UNC>
-static cudaError_t launch_one(const VerifyParams& P, int grid, size_t smem_bytes, cudaStream_t st) {
-  auto kc = lantern_context_kernel<CHC, BF16, UNC, LANTERN_VARIANT_TONE, LANTERN_VARIANT_JSD, LANTERN_VARIANT_TOPK>;
+static cudaError_t launch_one(const VerifyParams& P, long long items, int sms, cudaStream_t st) {
+  auto kc = lantern_context_topk_kernel<CHC, BF16, UNC, LANTERN_VARIANT_TONE, LANTERN_VARIANT_JSD, true>;
+  // one staging area of three row slots per consumer group; the numerators are kept over the rows they came from
+  const size_t smem_bytes = NGRP * ((static_cast<size_t>(3) * P.V * (BF16 ? 2 : 4) + 127) & ~static_cast<size_t>(127));
+  const long long ctas = (items + NGRP - 1) / NGRP;   // every CTA runs NGRP contexts at a time
+  const int grid = static_cast<int>(ctas < sms ? ctas : sms);
   cudaError_t e = cudaFuncSetAttribute(kc, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem_bytes));
   if (e != cudaSuccess) return e;
   kc<<<grid, CTX_THREADS, smem_bytes, st>>>(P);
   return cudaGetLastError();
 }
+#else
+template <class SHAPE, int CHC, bool BF16, bool UNC>
+static cudaError_t launch_shape(const VerifyParams& P, long long items, int sms, cudaStream_t st) {
+  auto kc = lantern_context_kernel<SHAPE, CHC, BF16, UNC, LANTERN_VARIANT_TONE, LANTERN_VARIANT_JSD>;
+  const size_t smem_bytes = SHAPE::NGRP * SHAPE::AREAS * ctx_area_bytes(P.V, BF16, UNC);
+  const int ctas = sms * SHAPE::CTAS;
+  const int grid = static_cast<int>(items < ctas ? items : ctas);
+  cudaError_t e = cudaFuncSetAttribute(kc, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem_bytes));
+  if (e != cudaSuccess) return e;
+  kc<<<grid, SHAPE::THREADS, smem_bytes, st>>>(P);
+  return cudaGetLastError();
+}
+template <int CHC, bool BF16, bool UNC>
+static cudaError_t launch_one(const VerifyParams& P, long long items, int sms, cudaStream_t st) {
+  if constexpr (CHC == 8 && BF16) {   // rows beyond 8192 tokens
+    const int shape = ctx_shape(P, sms);
+    if (shape == 2) return launch_shape<CtxWide, CHC / 2, BF16, UNC>(P, items, sms, st);
+    if (shape == 1) return launch_shape<CtxPair, CHC / 2, BF16, UNC>(P, items, sms, st);
+  }
+  return launch_shape<CtxNarrow, CHC, BF16, UNC>(P, items, sms, st);
+}
+#endif
 
 template <int CHC>
-static cudaError_t launch_layout(const VerifyParams& P, bool bf, bool un, int grid, size_t smem_bytes, cudaStream_t st) {
-  return bf ? (un ? launch_one<CHC, true, true>(P, grid, smem_bytes, st) : launch_one<CHC, true, false>(P, grid, smem_bytes, st))
-            : (un ? launch_one<CHC, false, true>(P, grid, smem_bytes, st) : launch_one<CHC, false, false>(P, grid, smem_bytes, st));
+static cudaError_t launch_layout(const VerifyParams& P, bool bf, bool un, long long items, int sms, cudaStream_t st) {
+  return bf ? (un ? launch_one<CHC, true, true>(P, items, sms, st) : launch_one<CHC, true, false>(P, items, sms, st))
+            : (un ? launch_one<CHC, false, true>(P, items, sms, st) : launch_one<CHC, false, false>(P, items, sms, st));
 }
 
-cudaError_t LANTERN_VARIANT_NAME(const VerifyParams& P, int CH, bool bf, bool un, int grid, size_t smem_bytes,
-                                 cudaStream_t st) {
-  return CH == 8 ? launch_layout<8>(P, bf, un, grid, smem_bytes, st)
-                 : (CH == 4 ? launch_layout<4>(P, bf, un, grid, smem_bytes, st)
-                            : (CH == 2 ? launch_layout<2>(P, bf, un, grid, smem_bytes, st)
-                                       : launch_layout<1>(P, bf, un, grid, smem_bytes, st)));
+cudaError_t LANTERN_VARIANT_NAME(const VerifyParams& P, bool bf, bool un, long long items, int sms, cudaStream_t st) {
+  // 8-token chunks per thread of a 256-thread group: the smallest power of two that covers the row
+  const int chunks = (P.V + 2047) / 2048;
+  return chunks > 4 ? launch_layout<8>(P, bf, un, items, sms, st)
+                    : (chunks > 2 ? launch_layout<4>(P, bf, un, items, sms, st)
+                                  : (chunks > 1 ? launch_layout<2>(P, bf, un, items, sms, st)
+                                                : launch_layout<1>(P, bf, un, items, sms, st)));
 }
 
 }  // namespace lantern

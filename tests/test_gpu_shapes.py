@@ -1,0 +1,49 @@
+"""The fused pass runs in one of three shapes, chosen by row length and number of sequences; its walk over the decided
+contexts is done by whoever completes the next piece of a path.  Calls on both sides of every line against the oracle."""
+import numpy as np
+import pytest
+import torch
+
+import lantern_inputs as li
+import paper_2410_03355_b200 as lt
+from parity import assert_parity, compare, near_ceiling, run_gpu, tables
+
+pytestmark = pytest.mark.gpu
+
+
+def _sms():
+    return torch.cuda.get_device_properties(0).multi_processor_count
+
+
+@pytest.mark.parametrize("V,per_sm,extra,N,tree", [
+    (16384, 2, 0, 2, False), (16384, 2, 1, 2, False), (16384, 3, 0, 2, False), (16384, 3, 1, 2, False),   # wide | pair | narrow
+    (16384, 2, 1, 9, True), (8200, 0, 5, 14, True), (8200, 2, 1, 2, False), (8192, 0, 5, 14, True)])
+def test_shapes_against_oracle(V, per_sm, extra, N, tree):
+    B = per_sm * _sms() + extra
+    seed = 90 + V % 97 + B + N
+    par = li.tree_parents(B, N, depth=4, seed=seed) if tree else None
+    inp = li.verify_inputs(B, N, V, dtype=li.BF16, has_uncond=True, cfg_scale=4.0, rho=0.9, sigma_draft=0.8, parents=par, seed=seed)
+    host, dev = tables(li.codebook_gaussian(V, 8, seed=14), 100, inp.draft_tokens)
+    res = compare(inp, host, 0.2, run_gpu(inp, dev, 0.2))
+    assert_parity(res)
+    assert res["near"] <= near_ceiling(B)
+
+
+def test_calls_without_drafts():
+    """N = 0: one draw per sequence from the root's target, for one sequence and for more than the groups of the GPU."""
+    V = 1024
+    host, dev = tables(li.codebook_gaussian(V, 8, seed=15), 16, np.zeros(1, np.int32))
+    for B in (1, 7 * _sms() + 3):
+        inp = li.verify_inputs(B, 0, V, dtype=li.F32, has_uncond=False, cfg_scale=1.0, seed=B)
+        d = torch.from_numpy(inp.target_logits).cuda()
+        out = lt.verify(d, None, 1.0, 1.0, None, None, dev, 0.2, torch.from_numpy(inp.uniforms).cuda())
+        torch.cuda.synchronize()
+        z = inp.target_logits[0, :, 0].astype(np.float64)
+        e = np.exp(z - z.max(axis=1, keepdims=True))
+        cdf = np.cumsum(e, axis=1)
+        u = inp.uniforms[:, 0].astype(np.float64) * cdf[:, -1]
+        want = (cdf <= u[:, None]).sum(axis=1)
+        # a draw within 1e-6 of an edge of the distribution may go either way
+        edge = np.abs(cdf - u[:, None]).min(axis=1) / cdf[:, -1] < 1e-6
+        assert np.array_equal(out.next_token.cpu().numpy()[~edge], want[~edge]) and edge.sum() <= max(1, B // 50)
+        assert not out.status.any() and not out.accept_len.any()
