@@ -96,12 +96,11 @@ def _ptr(t: Optional[torch.Tensor], dtype=None, name: str = "tensor"):
         raise ValueError(f"{name} must be contiguous")
     if dtype is not None and t.dtype != dtype:
         raise ValueError(f"{name} must have dtype {dtype}, got {t.dtype}")
-    return ctypes.c_void_p(t.data_ptr())
+    return t.data_ptr()
 
 
 def _stream_ptr(stream: Optional[torch.cuda.Stream]):
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return ctypes.c_void_p(s.cuda_stream)
+    return (stream if stream is not None else torch.cuda.current_stream()).cuda_stream
 
 
 def build_workspace_bytes(V: int, D: int, k: int) -> int:
@@ -214,27 +213,27 @@ def verify(target_logits: torch.Tensor, draft_logits: Optional[torch.Tensor], cf
     k = neighbor_idx.shape[1]
     if neighbor_idx.shape[0] != V:
         raise ValueError("neighbor_idx must have V rows")
-    with torch.cuda.device(dev):
-        if out is None:
-            i32 = dict(dtype=torch.int32, device=dev)
-            out = VerifyOutputs(
-                accept_len=torch.empty(B, **i32), next_token=torch.empty(B, **i32),
-                accept_path=torch.empty((B, N), **i32), status=torch.empty(B, **i32),
-                node_qa=torch.empty((B, N), dtype=torch.float32, device=dev) if trace else None,
-                node_px=torch.empty((B, N), dtype=torch.float32, device=dev) if trace else None,
-                node_m=torch.empty((B, N), **i32) if trace else None)
-        need = verify_workspace_bytes(B, N, V, int(k), dtype, top_k)
-        if workspace is None:
-            workspace = torch.empty(max(need, 256), dtype=torch.uint8, device=dev)
-        rc = lib.lantern_verify_ex(
-            _ptr(target_logits, None, "target_logits"), _ptr(draft_logits, target_logits.dtype, "draft_logits"),
-            dtype, float(cfg_scale), int(C == 2), float(T), _ptr(draft_tokens, torch.int32, "draft_tokens"),
-            _ptr(tree_parents, torch.int32, "tree_parents"), _ptr(neighbor_idx, torch.int32, "neighbor_idx"),
-            int(k), float(delta), DIVERGENCES[divergence], int(top_k), _ptr(uniforms, torch.float32, "uniforms"),
-            B, N, V, _ptr(out.accept_len, torch.int32), _ptr(out.next_token, torch.int32),
-            _ptr(out.accept_path, torch.int32), _ptr(out.status, torch.int32), _ptr(out.node_qa, torch.float32),
-            _ptr(out.node_px, torch.float32), _ptr(out.node_m, torch.int32), _ptr(workspace),
-            workspace.numel(), _stream_ptr(stream))
+    if dev.type == "cuda" and dev.index != torch.cuda.current_device():
+        with torch.cuda.device(dev):
+            return verify(target_logits, draft_logits, cfg_scale, T, draft_tokens, tree_parents, neighbor_idx, delta, uniforms,
+                          out=out, trace=trace, workspace=workspace, stream=stream, divergence=divergence, top_k=top_k)
+    i32, f32 = torch.int32, torch.float32
+    if out is None:
+        def new(shape, dt):
+            return torch.empty(shape, dtype=dt, device=dev)
+        out = VerifyOutputs(accept_len=new(B, i32), next_token=new(B, i32), accept_path=new((B, N), i32), status=new(B, i32),
+                            node_qa=new((B, N), f32) if trace else None, node_px=new((B, N), f32) if trace else None,
+                            node_m=new((B, N), i32) if trace else None)
+    if workspace is None:
+        workspace = torch.empty(max(verify_workspace_bytes(B, N, V, int(k), dtype, top_k), 256), dtype=torch.uint8, device=dev)
+    rc = lib.lantern_verify_ex(
+        _ptr(target_logits, None, "target_logits"), _ptr(draft_logits, target_logits.dtype, "draft_logits"),
+        dtype, float(cfg_scale), int(C == 2), float(T), _ptr(draft_tokens, i32, "draft_tokens"),
+        _ptr(tree_parents, i32, "tree_parents"), _ptr(neighbor_idx, i32, "neighbor_idx"),
+        int(k), float(delta), DIVERGENCES[divergence], int(top_k), _ptr(uniforms, f32, "uniforms"),
+        B, N, V, _ptr(out.accept_len, i32), _ptr(out.next_token, i32), _ptr(out.accept_path, i32), _ptr(out.status, i32),
+        _ptr(out.node_qa, f32), _ptr(out.node_px, f32), _ptr(out.node_m, i32), _ptr(workspace),
+        workspace.numel(), _stream_ptr(stream))
     if rc != 0:
         raise LanternError(rc, "lantern_verify_ex")
     return out

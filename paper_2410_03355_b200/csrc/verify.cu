@@ -37,15 +37,12 @@ namespace lantern {
 // Every context with children starts with a record that says "not evaluated" (INTERNAL), which
 // the fused pass overwrites; contexts without children are marked as leaves.
 // ---------------------------------------------------------------------------------------
-constexpr int PLAN_WARPS = 4;
 constexpr int kPlanArrays = 13;  // per-warp arrays of N + 2 ints in shared memory
 
-__global__ void __launch_bounds__(PLAN_WARPS * 32) lantern_plan_kernel(VerifyParams P) {
-  extern __shared__ int plan_smem[];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int b = blockIdx.x * PLAN_WARPS + warp;
-  if (b >= P.B) return;
+// One sequence, by one warp; returns the number of its contexts with children, or its fault bits << 16.
+__device__ __forceinline__ int plan_sequence(const VerifyParams& P, int* plan_smem, int b, int warp, int lane) {
   const int N = P.N, R = P.R, B = P.B;
+  if (b >= B) return 0;
   int* cnt = plan_smem + warp * kPlanArrays * (R + 1);   // cnt[c]: number of children of context c
   int* cur = cnt + (R + 1);                    // fill cursor, ends as the end offset of context c
   int* dep = cur + (R + 1);                    // depth of context c (root = 0), later its breadth-first rank
@@ -95,12 +92,11 @@ __global__ void __launch_bounds__(PLAN_WARPS * 32) lantern_plan_kernel(VerifyPar
       P.out_len[b] = 0;
       P.out_tok[b] = -1;
       if (P.out_status) P.out_status[b] = status ? status : LANTERN_ST_INTERNAL;
-      if (status) atomicOr(&P.counters->status_or, status);
     }
   }
   if (status) {   // the walk reports the fault; no work is queued for this sequence
     for (int r = lane; r < max(N, 1); r += 32) P.work[static_cast<size_t>(r) * B + b].item = -1;
-    return;
+    return status << 16;
   }
 
   ChildInfo* kids = P.children + static_cast<size_t>(b) * N;
@@ -255,8 +251,6 @@ __global__ void __launch_bounds__(PLAN_WARPS * 32) lantern_plan_kernel(VerifyPar
     }
   }
   if (N == 0 && P.walk_inline) n_ctx = 1;
-  // (thousands of warps would otherwise queue up on one address: most find the maximum already there)
-  if (lane == 0 && n_ctx > *reinterpret_cast<volatile int*>(&P.counters->n_rank)) atomicMax(&P.counters->n_rank, n_ctx);
   __syncwarp();         // the shared arrays are complete
   for (int i = lane; i < N; i += 32) {   // the child lists, written by all lanes
     ChildInfo ci = {i, s_tok[i], __int_as_float(s_uni[i]), (din[i + 1] << 16) | siz[i + 1]};
@@ -298,6 +292,24 @@ __global__ void __launch_bounds__(PLAN_WARPS * 32) lantern_plan_kernel(VerifyPar
         if (P.ctx_slots) P.ctx_slots[n >= 2 ? hb + __popc(heavy & below) : cap - 1 - (lb + __popc(light & below))] = slot;
       }
     }
+  }
+  return n_ctx;
+}
+
+__global__ void __launch_bounds__(PLAN_WARPS * 32) lantern_plan_kernel(VerifyParams P) {
+  extern __shared__ int plan_smem[];
+  __shared__ int s_words[PLAN_WARPS];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  grid_dependency_wait();
+  grid_dependents_launch();
+  if (P.clear_counters && blockIdx.x == 0 && threadIdx.x < 64) reinterpret_cast<int*>(P.counters)[threadIdx.x] = 0;
+  const int word = plan_sequence(P, plan_smem, blockIdx.x * PLAN_WARPS + warp, warp, lane);
+  if (lane == 0) s_words[warp] = word;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    int ranks = 0, bits = 0;
+    for (int w = 0; w < PLAN_WARPS; ++w) ranks = max(ranks, s_words[w] & 0xffff), bits |= s_words[w] >> 16;
+    P.block_words[blockIdx.x] = bits << 16 | ranks;
   }
 }
 
@@ -386,6 +398,17 @@ static WsLayout ws_layout(int B, int N, bool topk = false) {
   L.thrp = o;     o += topk ? align_up(b * R * 4, 256) : 0;
   L.total = o;
   return L;
+}
+
+// SMs of the current device (asked for once per device: it does not change), 0 if there is none
+static int sm_count() {
+  static std::atomic<int> known[64];
+  int dev = -1, n = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0) return 0;
+  if (dev < 64 && (n = known[dev].load(std::memory_order_relaxed)) > 0) return n;
+  if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 0;
+  if (dev < 64) known[dev].store(n, std::memory_order_relaxed);
+  return n;
 }
 
 static thread_local cudaEvent_t g_ev_before = nullptr, g_ev_after = nullptr;
@@ -676,23 +699,23 @@ static lantern_status verify_impl(const void* target_logits, const void* draft_l
   // only the threshold kernel of greedy decoding with the logit filter walks the compact list
   P.ctx_slots = (greedy && topk) ? reinterpret_cast<int32_t*>(ws + L.slots) : nullptr;
   P.dead = ws + L.dead;
+  P.block_words = P.bonus_seq;
+  P.clear_counters = P.ctx_slots == nullptr;   // (the compact list is counted while the plan is made)
   P.walk_inline = !greedy && !topk;
   P.wait_tries = g_wait_tries;
   P.withhold_item = g_withhold_item;
 
-  int dev = 0, sms = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess) return LANTERN_E_CUDA;
-  if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return LANTERN_E_CUDA;
+  const int sms = sm_count();
   if (sms < 1) return LANTERN_E_CUDA;
 
-  if (cudaMemsetAsync(P.counters, 0, 256, st) != cudaSuccess) return LANTERN_E_CUDA;
+  if (!P.clear_counters && cudaMemsetAsync(P.counters, 0, 256, st) != cudaSuccess) return LANTERN_E_CUDA;
   const size_t plan_smem = static_cast<size_t>(PLAN_WARPS) * kPlanArrays * (N + 2) * sizeof(int);
+  static DeviceFlags plan_ready;
   if (plan_smem > 48 * 1024 &&
-      cudaFuncSetAttribute(lantern_plan_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           static_cast<int>(plan_smem)) != cudaSuccess)
+      allow_shared_memory(lantern_plan_kernel, PLAN_WARPS * kPlanArrays * (MAX_N + 2) * sizeof(int), plan_ready) != cudaSuccess)
     return LANTERN_E_CUDA;
-  lantern_plan_kernel<<<(B + PLAN_WARPS - 1) / PLAN_WARPS, PLAN_WARPS * 32, plan_smem, st>>>(P);
-  if (cudaGetLastError() != cudaSuccess) return LANTERN_E_CUDA;
+  if (launch_dependent(lantern_plan_kernel, (B + PLAN_WARPS - 1) / PLAN_WARPS, PLAN_WARPS * 32, plan_smem, st, P) != cudaSuccess)
+    return LANTERN_E_CUDA;
 
   const long long items = static_cast<long long>(B) * (N > 0 ? N : 1);   // upper bound of contexts with children
   const int grid_bonus = B < 4 * sms ? B : 4 * sms;   // greedy bonus: 256-thread CTAs

@@ -7,6 +7,7 @@
 #include <math.h>
 #include <stdint.h>
 
+#include <atomic>
 #include <type_traits>
 
 #include "lantern.h"
@@ -18,12 +19,11 @@ namespace lantern {
 
 constexpr int MAX_N = 1024;
 
-struct Counters {               // first 256 bytes of the workspace, zeroed per call
+struct Counters {               // first 256 bytes of the workspace, zeroed per call (by the plan kernel, or ahead of it, see clear_counters)
   int work_next;                // dynamic part of the work counter
   int n_heavy;                  // contexts with >= 2 children (first in the compact list)
   int n_light;                  // contexts with exactly 1 child
   int n_bonus;                  // sequences whose next token is drawn from a context's own target
-  int n_rank;                   // largest number of contexts with children in one sequence
   int n_evaluated;              // contexts the fused pass evaluated
   int n_skipped;                // contexts it left out because the walk cannot reach them
   int n_tested;                 // drafted nodes it tested
@@ -96,6 +96,9 @@ struct VerifyParams {
   float* thr_q;                 // [B, R] top_k-th largest processed target logit of a context row
   float* thr_p;                 // [B, R] the same for the drafter row
   uint32_t wait_tries;          // limit of every bounded mbarrier wait, in tries
+  int32_t* block_words;         // one word per block of the plan kernel: largest number of contexts with children in one of
+                                //     its sequences, and its sequences' fault bits << 16 (read before bonus_seq, whose storage it is, is written)
+  int clear_counters;           // the plan kernel zeroes the counters (nothing in it counts then)
   int walk_inline;              // the fused pass walks and draws the bonus tokens itself: records hold walk words
   int withhold_item;            // self-test only: the copies of this context are never issued (-1 = none)
 };
@@ -116,10 +119,65 @@ __device__ __forceinline__ unsigned long long walk_word(unsigned state, unsigned
          (static_cast<unsigned long long>(static_cast<unsigned>(token)) << 32);
 }
 
+constexpr int PLAN_WARPS = 4;   // sequences per block of the plan kernel
+
+// The plan's summary, by a whole warp: slots in the occupied part of the work list, and the fault bits of all sequences.
+__device__ __forceinline__ int plan_slots(const VerifyParams& P, int lane, int& faults) {
+  int ranks = P.parents ? 0 : (P.N > 0 ? P.N : (P.walk_inline ? 1 : 0)), bits = 0;
+  const int blocks = (P.B + PLAN_WARPS - 1) / PLAN_WARPS;
+#pragma unroll 4
+  for (int i = lane; i < blocks; i += 32) {
+    const int w = __ldg(P.block_words + i);
+    ranks = max(ranks, w & 0xffff);
+    bits |= w >> 16;
+  }
+  faults = __reduce_or_sync(kFull, bits);
+  return __reduce_max_sync(kFull, ranks) * P.B;
+}
+// The same without the fault bits: a chain has a context with a child for every draft.
+__device__ __forceinline__ int plan_slots(const VerifyParams& P, int lane) {
+  if (!P.parents) return (P.N > 0 ? P.N : (P.walk_inline ? 1 : 0)) * P.B;
+  int faults;
+  return plan_slots(P, lane, faults);
+}
+
 __device__ __forceinline__ float sum8(const float* v) {
   return ((v[0] + v[1]) + (v[2] + v[3])) + ((v[4] + v[5]) + (v[6] + v[7]));
 }
 
+
+// ---- host side ----
+// Which devices a kernel's shared-memory limit has been raised on (ordinals 0..63; beyond that it is raised every time).
+struct DeviceFlags {
+  std::atomic<unsigned long long> bits{0};
+};
+template <class K>
+static inline cudaError_t allow_shared_memory(K kernel, size_t bytes, DeviceFlags& ready) {
+  int dev = -1;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  const unsigned long long bit = dev >= 0 && dev < 64 ? 1ull << dev : 0ull;
+  if (ready.bits.load(std::memory_order_acquire) & bit) return cudaSuccess;
+  e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(bytes));
+  if (e == cudaSuccess) ready.bits.fetch_or(bit, std::memory_order_release);
+  return e;
+}
+// Launch that lets the kernel be put in place while the one before it in the stream still runs (it waits for it by
+// grid_dependency_wait before it touches anything).
+template <class K>
+static inline cudaError_t launch_dependent(K kernel, int grid, int threads, size_t smem, cudaStream_t st, const VerifyParams& P) {
+  cudaLaunchAttribute attr = {};
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t c = {};
+  c.gridDim = dim3(grid);
+  c.blockDim = dim3(threads);
+  c.dynamicSmemBytes = smem;
+  c.stream = st;
+  c.attrs = &attr;
+  c.numAttrs = 1;
+  return cudaLaunchKernelEx(&c, kernel, P);
+}
 
 // Launch of the fused context kernel (verify_context.cuh).  Its variants -- temperature 1 compiled
 // out or not (TONE), TVD or JSD bound, top-k thresholds applied or not -- are compiled in separate

@@ -309,6 +309,7 @@ __global__ void __launch_bounds__(SHAPE::THREADS, SHAPE::CTAS) lantern_context_k
     fence_proxy_async();
   }
   __syncthreads();
+  grid_dependency_wait();   // the plan, and whatever made the inputs
 
   // ======================= producer warps =======================
   // One warp per consumer group hands out work, keeps that group's copies going and walks.  Its 32 lanes look
@@ -322,7 +323,7 @@ __global__ void __launch_bounds__(SHAPE::THREADS, SHAPE::CTAS) lantern_context_k
   if (tid >= NGRP * GT) {
     const int grp = (tid - NGRP * GT) >> 5;
     GroupShared<GW>& S = SG[grp];
-    const int total = P.counters->n_rank * P.B;  // occupied part of the slot array
+    const int total = plan_slots(P, lane);       // occupied part of the slot array
     const int G = gridDim.x * NGRP;              // producers in the grid
     const int me = grp * gridDim.x + blockIdx.x; // few contexts: one to an SM before any SM gets a second one
     const uint32_t tries = P.wait_tries;
@@ -572,6 +573,11 @@ __global__ void __launch_bounds__(SHAPE::THREADS, SHAPE::CTAS) lantern_context_k
       if (n_eval) atomicAdd(&P.counters->n_evaluated, n_eval);
       if (n_skip) atomicAdd(&P.counters->n_skipped, n_skip);
       if (n_draw) atomicAdd(&P.counters->n_bonus, n_draw);
+    }
+    if (me == 0) {   // sequences that the plan found at fault
+      int faults;
+      plan_slots(P, lane, faults);
+      if (faults && lane == 0) atomicOr(&P.counters->status_or, faults);
     }
     return;
   }

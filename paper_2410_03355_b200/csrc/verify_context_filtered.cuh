@@ -209,7 +209,7 @@ __global__ void __launch_bounds__(CTX_THREADS, 1) lantern_context_topk_kernel(Ve
   if (tid >= NGRP * GT) {
     const int grp = (tid - NGRP * GT) >> 5;
     GroupShared& S = SG[grp];
-    const int total = P.counters->n_rank * P.B;  // occupied part of the slot array
+    const int total = plan_slots(P, lane);       // occupied part of the slot array
     const int G = gridDim.x * NGRP;              // producers in the grid
     const int me = blockIdx.x * NGRP + grp;
     const uint32_t tries = P.wait_tries;

@@ -26,13 +26,13 @@ static cudaError_t launch_one(const VerifyParams& P, long long items, int sms, c
 template <class SHAPE, int CHC, bool BF16, bool UNC>
 static cudaError_t launch_shape(const VerifyParams& P, long long items, int sms, cudaStream_t st) {
   auto kc = lantern_context_kernel<SHAPE, CHC, BF16, UNC, LANTERN_VARIANT_TONE, LANTERN_VARIANT_JSD>;
-  const size_t smem_bytes = SHAPE::NGRP * SHAPE::AREAS * ctx_area_bytes(P.V, BF16, UNC);
+  const size_t groups = SHAPE::NGRP * SHAPE::AREAS;
   const int ctas = sms * SHAPE::CTAS;
-  const int grid = static_cast<int>(items < ctas ? items : ctas);
-  cudaError_t e = cudaFuncSetAttribute(kc, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem_bytes));
+  const int grid = static_cast<int>(items < ctas ? items : ctas);   // a few contexts get an SM each
+  static DeviceFlags ready;
+  const cudaError_t e = allow_shared_memory(kc, groups * (64 << 10), ready);   // the longest rows need 64 KB per area
   if (e != cudaSuccess) return e;
-  kc<<<grid, SHAPE::THREADS, smem_bytes, st>>>(P);
-  return cudaGetLastError();
+  return launch_dependent(kc, grid, SHAPE::THREADS, groups * ctx_area_bytes(P.V, BF16, UNC), st, P);
 }
 template <int CHC, bool BF16, bool UNC>
 static cudaError_t launch_one(const VerifyParams& P, long long items, int sms, cudaStream_t st) {

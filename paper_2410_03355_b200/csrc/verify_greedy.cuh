@@ -233,7 +233,7 @@ __global__ void __launch_bounds__(GCT, 3) lantern_greedy_context_kernel(VerifyPa
   const uint32_t area_bytes = (UNC ? 2 : 1) * rowbytes;   // a multiple of 16: V % 8 == 0
   const float L_hi = 1.44269502162933349609375f;
   const float NEG_INF = __int_as_float(0xff800000);
-  const int total = P.counters->n_rank * P.B;   // occupied part of the slot array (breadth-first order per sequence)
+  const int total = warp == 0 ? plan_slots(P, lane) : 0;   // occupied part of the slot array (breadth-first order per sequence)
   const int quads = V >> 2;
   const int G = gridDim.x;
   int n_eval = 0, n_skip = 0, n_test = 0;       // thread 0: work accounting
