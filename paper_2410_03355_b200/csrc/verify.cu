@@ -11,9 +11,8 @@
 //                        and either the next sibling's test on the renormalised residual or
 //                        the inverse-CDF draw of the replacement token   (Section 4.3, Alg. 1)
 // Algorithm 1's loop over the decided contexts and the draw of the bonus token happen inside the same pass.
-// Two paths keep the older split into passes, plan -> contexts -> walk -> bonus: greedy decoding (verify_greedy.cuh) and
-// sampling with the top-k logit filter (verify_context_filtered.cuh, verify_bonus.cuh); their contexts leave 16-byte
-// records, which a small walk kernel follows from the root.
+// Greedy decoding (verify_greedy.cuh) has passes of its own, plan -> contexts -> walk -> next tokens; its contexts leave
+// 16-byte records, which a small walk kernel follows from the root.
 //
 // Precision: processed logits are fp32 (difference, fused multiply-add, division, each
 // rounded once); exponentials come from the fp32 ex2 unit (about 3e-7 relative); every sum over more
@@ -318,7 +317,6 @@ __global__ void __launch_bounds__(PLAN_WARPS * 32) lantern_plan_kernel(VerifyPar
 // (kernel 2, the fused context pass, is compiled in files of its own: see verify_common.cuh)
 // greedy decoding (temperature 0)
 #include "verify_greedy.cuh"
-#include "verify_bonus.cuh"
 #include "verify_topk.cuh"
 
 namespace lantern {
@@ -418,10 +416,9 @@ constexpr uint32_t kDefaultWaitTries = 1u << 21;
 static thread_local uint32_t g_wait_tries = kDefaultWaitTries;
 static thread_local int g_withhold_item = -1;
 
-// thresholds of the top-k filter: mode 0 = rows of the contexts with children (after the plan),
-// mode 1 = rows of the bonus draws (after the walk)
+// thresholds of the top-k filter for greedy decoding: target rows of the contexts with children (after the plan)
 template <bool BF16, bool UNC>
-static cudaError_t launch_topk(const VerifyParams& P, int mode, long long jobs, int sms, cudaStream_t st) {
+static cudaError_t launch_topk(const VerifyParams& P, long long jobs, int sms, cudaStream_t st) {
   auto kt = lantern_topk_kernel<BF16, UNC>;
   const size_t smem = static_cast<size_t>(P.V) * (UNC ? 2 : 1) * (BF16 ? 2 : 4);   // one job's raw rows
   cudaError_t e = cudaFuncSetAttribute(kt, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
@@ -432,7 +429,7 @@ static cudaError_t launch_topk(const VerifyParams& P, int mode, long long jobs, 
   if (per_sm < 1) return cudaErrorInvalidConfiguration;
   const long long slots = static_cast<long long>(sms) * per_sm;
   const int grid = static_cast<int>(jobs < slots ? (jobs > 0 ? jobs : 1) : slots);
-  kt<<<grid, TKT, smem, st>>>(P, mode);
+  kt<<<grid, TKT, smem, st>>>(P);
   return cudaGetLastError();
 }
 
@@ -457,39 +454,14 @@ cudaError_t launch_context_kernel(const VerifyParams& P, bool bf16, bool uncond,
   }
 }
 
-template <bool BF16, bool UNC>
-static cudaError_t launch_bonus(const VerifyParams& P, int sms, cudaStream_t st) {
-  auto kb = lantern_bonus_stream_kernel<BF16, UNC>;
-  const size_t smem = static_cast<size_t>(P.V) * (UNC ? 2 : 1) * (BF16 ? 2 : 4);   // one context's raw target rows
-  cudaError_t e = cudaFuncSetAttribute(kb, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
-  if (e != cudaSuccess) return e;
-  int per_sm = 0;
-  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kb, BNT, smem);
-  if (e != cudaSuccess) return e;
-  if (per_sm < 1) return cudaErrorInvalidConfiguration;
-  const long long slots = static_cast<long long>(sms) * per_sm;
-  const int grid = static_cast<int>(P.B < slots ? P.B : slots);
-  kb<<<grid, BNT, smem, st>>>(P);
-  return cudaGetLastError();
-}
-
-// Sampling.  Without the logit filter the fused pass walks the contexts and draws the bonus tokens as well; with it
-// (the fused pass finds the thresholds of its contexts itself) walk, thresholds of the bonus rows and bonus draw follow.
-template <bool BF16, bool UNC>
-static cudaError_t launch_verify(const VerifyParams& P, bool tone, bool jsd, long long items, int sms, cudaStream_t st) {
-  const bool topk = P.top_k > 0;
-  cudaError_t e;
+// Sampling: the fused pass finds its contexts' thresholds, walks the contexts and draws the bonus tokens itself.
+static cudaError_t launch_verify(const VerifyParams& P, bool bf16, bool uncond, bool tone, bool jsd, long long items, int sms,
+                                 cudaStream_t st) {
   if (g_ev_before && g_ev_after) cudaEventRecord(g_ev_before, st);
-  e = launch_context_kernel(P, BF16, UNC, tone, jsd, topk, items, sms, st);
+  const cudaError_t e = launch_context_kernel(P, bf16, uncond, tone, jsd, P.top_k > 0, items, sms, st);
   if (e != cudaSuccess) return e;
   if (g_ev_before && g_ev_after) cudaEventRecord(g_ev_after, st);
-  if (!topk) return cudaSuccess;
-  lantern_walk_kernel<<<(P.B + 127) / 128, 128, 0, st>>>(P);
-  e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  e = launch_topk<BF16, UNC>(P, 1, P.B, sms, st);
-  if (e != cudaSuccess) return e;
-  return launch_bonus<BF16, UNC>(P, sms, st);
+  return cudaSuccess;
 }
 
 template <bool BF16, bool UNC, bool TOPK>
@@ -510,7 +482,7 @@ static cudaError_t launch_greedy(const VerifyParams& P, long long items, int sms
   const long long slots = static_cast<long long>(sms) * per_sm;
   const int grid_ctx = static_cast<int>(items < slots ? items : slots);
   if (TOPK) {
-    e = launch_topk<BF16, UNC>(P, 0, items, sms, st);
+    e = launch_topk<BF16, UNC>(P, items, sms, st);
     if (e != cudaSuccess) return e;
   }
   if (g_ev_before && g_ev_after) cudaEventRecord(g_ev_before, st);
@@ -541,8 +513,8 @@ extern "C" size_t lantern_verify_workspace_bytes(int B, int N, int V, int k, int
 }
 
 extern "C" int lantern_verify_launch_count(int greedy, int top_k_active) {
-  // greedy decoding: memset, plan, greedy pass, walk, bonus, and the threshold kernel with the filter; sampling with the
-  // filter the same, without it memset, plan and the fused pass, which walks and draws by itself
+  // greedy decoding: plan, greedy pass, walk, next tokens; with the filter also a memset and the threshold kernel.
+  // sampling: plan and the fused pass, which does the rest by itself
   (void)greedy;
   return 5 + (top_k_active ? 1 : 0);
 }
@@ -695,13 +667,12 @@ static lantern_status verify_impl(const void* target_logits, const void* draft_l
   P.divergence = divergence;
   P.top_k = topk ? top_k : 0;
   P.thr_q = topk ? reinterpret_cast<float*>(ws + L.thrq) : nullptr;
-  P.thr_p = topk ? reinterpret_cast<float*>(ws + L.thrp) : nullptr;
   // only the threshold kernel of greedy decoding with the logit filter walks the compact list
   P.ctx_slots = (greedy && topk) ? reinterpret_cast<int32_t*>(ws + L.slots) : nullptr;
   P.dead = ws + L.dead;
   P.block_words = P.bonus_seq;
   P.clear_counters = P.ctx_slots == nullptr;   // (the compact list is counted while the plan is made)
-  P.walk_inline = !greedy && !topk;
+  P.walk_inline = !greedy;
   P.wait_tries = g_wait_tries;
   P.withhold_item = g_withhold_item;
 
@@ -731,8 +702,7 @@ static lantern_status verify_impl(const void* target_logits, const void* draft_l
   }
   // every combination of the compile-time variants exists: T = 1 never meets the division code
   const bool tone = T == 1.0f, jsd = divergence == LANTERN_DIV_JSD;
-  e = bf ? (un ? launch_verify<true, true>(P, tone, jsd, items, sms, st) : launch_verify<true, false>(P, tone, jsd, items, sms, st))
-         : (un ? launch_verify<false, true>(P, tone, jsd, items, sms, st) : launch_verify<false, false>(P, tone, jsd, items, sms, st));
+  e = launch_verify(P, bf, un, tone, jsd, items, sms, st);
   return e == cudaSuccess ? LANTERN_OK : LANTERN_E_CUDA;
 }
 

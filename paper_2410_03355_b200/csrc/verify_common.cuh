@@ -61,7 +61,6 @@ struct WorkItem {               // one context with children: everything its CTA
 struct GroupItem {              // the same, as a producer hands it to its consumer group through shared memory
   int item, cbase, nchild, node0, tok0, span0;
   float r0, u_final;
-  float bracket[2][4];          // top-k filter only: where the thresholds of the drafter row [0] and the target row [1] lie
 };
 
 struct VerifyParams {
@@ -92,9 +91,8 @@ struct VerifyParams {
   int B, N, R, V, k;
   float cfg_scale, T, delta;
   int divergence;               // LANTERN_DIV_TVD or LANTERN_DIV_JSD: what delta bounds
-  int top_k;                    // logit filter; 0 = off (then thr_q, thr_p are null)
-  float* thr_q;                 // [B, R] top_k-th largest processed target logit of a context row
-  float* thr_p;                 // [B, R] the same for the drafter row
+  int top_k;                    // logit filter; 0 = off
+  float* thr_q;                 // greedy decoding with the filter: [B, R] top_k-th largest target logit of a context row, else null
   uint32_t wait_tries;          // limit of every bounded mbarrier wait, in tries
   int32_t* block_words;         // one word per block of the plan kernel: largest number of contexts with children in one of
                                 //     its sequences, and its sequences' fault bits << 16 (read before bonus_seq, whose storage it is, is written)

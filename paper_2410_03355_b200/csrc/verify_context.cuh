@@ -119,13 +119,32 @@ __device__ __forceinline__ double exp2_int_d(double d) {
   return e <= -1000 ? 0.0 : __hiloint2double((1023 + e) << 20, 0);
 }
 
+constexpr int TOPK_LIST = 2080; // values inside the bracket of a threshold search, at most
+constexpr int TOPK_BINS = 128;  // bins of its sample
+constexpr int TOPK_FINE = 256;  // bins of the bracket
+constexpr int TOPK_TINY = 32;   // values of the wanted bin that a warp ranks
+
 struct CtxResult {              // what a group hands back to its producer
   int accepted;                 // accepted child, -1 if there is none
   int token;                    // token drawn, -1 if none
   int status;
 };
 
+// scratch of the top-k threshold search (verify_context_topk.cuh)
+template <int GW, bool TOPK>
+struct GroupTopk {};
 template <int GW>
+struct GroupTopk<GW, true> {
+  alignas(16) int hist[TOPK_BINS];   // the sample, by value; zero between searches
+  float range[GW][2];           // per warp: smallest and largest finite value of the sample
+  int count[GW][2];             // per warp: values above the bracket, values inside it
+  int fine[TOPK_FINE];          // the listed values, by value; zero between searches
+  float tiny[TOPK_TINY];        // the values of the wanted bin
+  int listed[3], picked[3];     // entries of the list and of tiny, by search (mod 3)
+  float threshold;
+};
+
+template <int GW, bool TOPK>
 struct alignas(16) GroupShared {
   alignas(16) double wz[GW][2]; // per-warp sums of numerators (target, drafter), in the warp's units
   double wt[64];                // per-(chunk, warp) totals for scans and block sums
@@ -135,14 +154,19 @@ struct alignas(16) GroupShared {
   double jsd_mass;              // the JSD bound as a mass, common units
   double hist[32];              // drafter/target scale ratio of each earlier rejection round of this context
   alignas(8) float wn[GW][2];   // the warps' units: their largest shifts
-  float slice[1024];            // shift of every (slice, thread)
+  float slice[TOPK ? TOPK_LIST : 1024];   // shift of every (slice, thread); before that the list of a threshold search
   int cut_m;                    // |A| - 1 that goes with cut_sum
   int badslot[3];               // first neighbour slot with an entry outside [0, V), by scan round (mod 3)
   int tok;
   int fail;                     // a bounded wait for the target rows ran out (sticky)
   GroupItem work[2];            // descriptor of context i in work[i & 1]: the next one is published while the current one runs
   CtxResult result[2];          // result of context i in result[i & 1]
+  GroupTopk<GW, TOPK> tk;
 };
+
+}  // namespace lantern
+#include "verify_context_topk.cuh"
+namespace lantern {
 
 // one row of a context into one row slot of a staging area, in bulk copies of at most 16 KB
 __device__ __forceinline__ void ctx_issue_row(unsigned char* dst, const unsigned char* src, int rowbytes, uint64_t* bar) {
@@ -216,6 +240,18 @@ __device__ __forceinline__ void raw8_pairs(const Raw8<BF16>& d, uint64_t (&o)[4]
     o[3] = pack2(__uint_as_float(d.b.z), __uint_as_float(d.b.w));
   }
 }
+// four pairs of 16-byte (bf16) or 32-byte group g of a staged row
+template <bool BF16>
+__device__ __forceinline__ void staged_pairs(const unsigned char* row, int g, uint64_t (&o)[4]) {
+  Raw8<BF16> d;
+  if (BF16) {
+    d.a = *reinterpret_cast<const uint4*>(row + g * 16);
+  } else {
+    d.a = *reinterpret_cast<const uint4*>(row + g * 32);
+    d.b = *reinterpret_cast<const uint4*>(row + g * 32 + 16);
+  }
+  raw8_pairs<BF16>(d, o);
+}
 // maximum of eight raw logits and m (bf16: two running maxima, one per half word)
 template <bool BF16>
 __device__ __forceinline__ uint32_t raw8_max(const Raw8<BF16>& d, uint32_t m) {
@@ -271,7 +307,8 @@ __device__ __forceinline__ unsigned long long walk_exchange(Record* rec, unsigne
 // CH = 8-token chunks per thread (1, 2, 4 or 8); the target's numerators come in slices of CP chunks.
 // TONE = the temperature is exactly 1 (the paper's sampling setting): no division is compiled in.
 // JSD selects the Section 5.3.2 bound at compile time, so that the default path carries none of its code.
-template <class SHAPE, int CH, bool BF16, bool UNC, bool TONE, bool JSD>
+// TOPK = the logit filter is on (Appendix B.2): processed logits below the top_k-th largest of their row count as -inf.
+template <class SHAPE, int CH, bool BF16, bool UNC, bool TONE, bool JSD, bool TOPK>
 __global__ void __launch_bounds__(SHAPE::THREADS, SHAPE::CTAS) lantern_context_kernel(VerifyParams P) {
   constexpr int GT = SHAPE::GT, GW = GT / 32, NGRP = SHAPE::NGRP, AREAS = SHAPE::AREAS;
   constexpr int LOG_GT = GT == 1024 ? 10 : (GT == 512 ? 9 : 8);
@@ -283,7 +320,7 @@ __global__ void __launch_bounds__(SHAPE::THREADS, SHAPE::CTAS) lantern_context_k
   constexpr int AHEAD = BF16 ? (CH < 4 ? CH : 4) : (CH < 2 ? CH : 2);   // drafter groups in flight in a residual pass
   static_assert(NP * GT <= 1024 && CH * GW <= 64, "tables of slices and blocks");
   extern __shared__ __align__(128) unsigned char smem[];
-  __shared__ GroupShared<GW> SG[NGRP];
+  __shared__ GroupShared<GW, TOPK> SG[NGRP];
   // Per group: next context published / the next context may be chosen / context i finished (by i mod 2: the producer may
   // look for context i - 1 when context i has been finished too); per area: rows landed
   __shared__ __align__(8) uint64_t bar_item[NGRP], bar_next[NGRP], bar_done[NGRP][2], bar_rows[NGRP][AREAS];
@@ -304,9 +341,16 @@ __global__ void __launch_bounds__(SHAPE::THREADS, SHAPE::CTAS) lantern_context_k
       for (int a = 0; a < AREAS; ++a) mbar_init(&bar_rows[g][a], 1);
       SG[g].fail = 0;
       SG[g].badslot[0] = SG[g].badslot[1] = SG[g].badslot[2] = kNone;
+      if constexpr (TOPK) {
+        for (int q = 0; q < 3; ++q) SG[g].tk.listed[q] = SG[g].tk.picked[q] = 0;
+      }
     }
     fence_mbar_init();
     fence_proxy_async();
+  }
+  if constexpr (TOPK) {
+    for (int q = tid; q < NGRP * TOPK_FINE; q += SHAPE::THREADS) SG[q / TOPK_FINE].tk.fine[q % TOPK_FINE] = 0;
+    for (int q = tid; q < NGRP * TOPK_BINS; q += SHAPE::THREADS) SG[q / TOPK_BINS].tk.hist[q % TOPK_BINS] = 0;
   }
   __syncthreads();
   grid_dependency_wait();   // the plan, and whatever made the inputs
@@ -322,7 +366,7 @@ __global__ void __launch_bounds__(SHAPE::THREADS, SHAPE::CTAS) lantern_context_k
   // on the critical path.
   if (tid >= NGRP * GT) {
     const int grp = (tid - NGRP * GT) >> 5;
-    GroupShared<GW>& S = SG[grp];
+    GroupShared<GW, TOPK>& S = SG[grp];
     const int total = plan_slots(P, lane);       // occupied part of the slot array
     const int G = gridDim.x * NGRP;              // producers in the grid
     const int me = grp * gridDim.x + blockIdx.x; // few contexts: one to an SM before any SM gets a second one
@@ -586,7 +630,7 @@ __global__ void __launch_bounds__(SHAPE::THREADS, SHAPE::CTAS) lantern_context_k
   const int grp = tid >> LOG_GT;        // which group
   const int gt = tid & (GT - 1);        // thread within the group
   const int gw = gt >> 5;               // warp within the group
-  GroupShared<GW>& S = SG[grp];
+  GroupShared<GW, TOPK>& S = SG[grp];
   const int row_floats = rowbytes >> 2;
   auto EI = [&](int x) { return ephys<BF16>(x, row_floats); };
   // index of the slice that owns token x in the table of shifts
@@ -620,6 +664,7 @@ __global__ void __launch_bounds__(SHAPE::THREADS, SHAPE::CTAS) lantern_context_k
   // Scan rounds of this group so far, mod 2 and mod 3: a round's totals are not overwritten, and its bad-slot word is
   // not cleared, before every warp has read them.
   int round2 = 0, round3 = 0;
+  int search3 = 0;                      // threshold searches so far, mod 3
   for (int iter = 0;; ++iter) {
     const int area = iter % AREAS;
     // A bounded wait that runs out ends the group: the context keeps its undecided word, so the sequences that need it
@@ -636,10 +681,22 @@ __global__ void __launch_bounds__(SHAPE::THREADS, SHAPE::CTAS) lantern_context_k
     };
     // Every warp waits for the next context by itself and may run ahead of slower ones: whatever it overwrites
     // before the next group barrier they have finished with (with one staging area because the target rows land only when
-    // all warps have released it; with two areas a barrier sees to it).  A wait that runs out is reported behind that
+    // all warps have released it; with two areas, or a threshold search, a barrier sees to it).  A wait that runs out is reported behind that
     // barrier, where every thread sees it alike.
-    if (AREAS > 1) gbar();
-    const bool there = mbar_wait(&bar_item[grp], iter & 1, tries);
+    if (AREAS > 1 && !TOPK) gbar();
+    bool there = mbar_wait(&bar_item[grp], iter & 1, tries);
+    if (TOPK) {   // (every thread has to take the same path to the barriers of a threshold search)
+      uint32_t all;
+      asm volatile(
+          "{\n\t.reg .pred p, q;\n\t"
+          "setp.ne.u32 p, %1, 0;\n\t"
+          "bar.red.and.pred q, %2, %3, p;\n\t"
+          "selp.u32 %0, 1, 0, q;\n\t}"
+          : "=r"(all)
+          : "r"(static_cast<uint32_t>(there)), "r"(1 + grp), "n"(GT)
+          : "memory");
+      there = all != 0;
+    }
     if (!there) S.fail = 1;
     const GroupItem& cur = S.work[iter & 1];
     const int item = there ? cur.item : -1;
@@ -659,11 +716,14 @@ __global__ void __launch_bounds__(SHAPE::THREADS, SHAPE::CTAS) lantern_context_k
       raw_c = ctx_raw_logit<BF16>(P.target, e);
       if (UNC) raw_u = ctx_raw_logit<BF16>(P.target, branch + e);
     };
+    float tq = ninf, tp = ninf;   // top-k thresholds of the target and the drafter row
     auto note_single = [&]() {
-      float z = raw_c;
-      if (UNC) z = __fmaf_rn(P.cfg_scale, __fsub_rn(raw_c, raw_u), raw_u);
-      S.single[0] = exp2_split(TONE ? z : __fdiv_rn(z, P.T));
-      S.single[1] = exp2_split(TONE ? raw_d : __fdiv_rn(raw_d, P.T));
+      float zq = raw_c, zp = raw_d;
+      if (UNC) zq = __fmaf_rn(P.cfg_scale, __fsub_rn(raw_c, raw_u), raw_u);
+      if (!TONE) zq = __fdiv_rn(zq, P.T), zp = __fdiv_rn(zp, P.T);
+      if (TOPK) zq = zq < tq ? ninf : zq, zp = zp < tp ? ninf : zp;
+      S.single[0] = exp2_split(zq);
+      S.single[1] = exp2_split(zp);
     };
 
     // ---------------- streaming part, thread-local ----------------
@@ -672,9 +732,9 @@ __global__ void __launch_bounds__(SHAPE::THREADS, SHAPE::CTAS) lantern_context_k
     float nd = 0.0f, td = 1.0f;   // drafter: this thread's shift and its sum of numerators, in its own units
     float nq[NP <= 2 ? NP : 1] = {};  // target: the shifts of the slices, where they are few (else in S.slice)
     auto shift_of = [&](int p) { return NP <= 2 ? nq[NP <= 2 ? p : 0] : S.slice[p * GT + gt]; };
-    float nq_max = 0.0f, tq = 1.0f;   // target: the largest shift of the slices; the sum, in its units
-    auto stream_drafter = [&](auto whole) {
-      Raw8<BF16> raw[CH];
+    float nq_max = 0.0f, sq = 1.0f;   // target: the largest shift of the slices; the sum, in its units
+    Raw8<BF16> raw[CH];           // the drafter row (dead after the reduction below)
+    auto load_drafter = [&](auto whole) {
 #pragma unroll
       for (int c = 0; c < CH; ++c) {
         const int g = c * GT + gt;
@@ -685,6 +745,8 @@ __global__ void __launch_bounds__(SHAPE::THREADS, SHAPE::CTAS) lantern_context_k
           raw[c].a = raw[c].b = make_uint4(w, w, w, w);
         }
       }
+    };
+    auto reduce_drafter = [&]() {
       uint32_t mw = BF16 ? 0xff80ff80u : 0xff800000u;
 #pragma unroll
       for (int c = 0; c < CH; ++c) mw = raw8_max<BF16>(raw[c], mw);
@@ -702,6 +764,10 @@ __global__ void __launch_bounds__(SHAPE::THREADS, SHAPE::CTAS) lantern_context_k
         for (int i = 0; i < 4; ++i) {
           if (!TONE) z2[i] = divide_T(z2[i]);
           float lo, hi;
+          if (TOPK) {
+            unpack2(z2[i], lo, hi);
+            z2[i] = pack2(lo < tp ? ninf : lo, hi < tp ? ninf : hi);
+          }
           unpack2(fma2(z2[i], L2, nn2), lo, hi);
           z2[i] = pack2(ex2_approx(lo), ex2_approx(hi));
         }
@@ -716,18 +782,8 @@ __global__ void __launch_bounds__(SHAPE::THREADS, SHAPE::CTAS) lantern_context_k
       const unsigned char* rc = stage;
       const unsigned char* ru = stage + rowbytes;
       const uint64_t s2 = pack2(P.cfg_scale, P.cfg_scale);
-      auto pairs_of = [&](const unsigned char* row, int g, uint64_t (&o)[4]) {
-        Raw8<BF16> d;
-        if (BF16) {
-          d.a = *reinterpret_cast<const uint4*>(row + g * 16);
-        } else {
-          d.a = *reinterpret_cast<const uint4*>(row + g * 32);
-          d.b = *reinterpret_cast<const uint4*>(row + g * 32 + 16);
-        }
-        raw8_pairs<BF16>(d, o);
-      };
       float n_run = -3.0e37f;
-      tq = 0.0f;
+      sq = 0.0f;
 #pragma unroll (NP > 2 ? 1 : NP)
       for (int p = 0; p < NP; ++p) {   // (rolled where there are many: three groups in different phases fill the instruction cache)
         uint64_t a2[CP * 4];
@@ -737,16 +793,26 @@ __global__ void __launch_bounds__(SHAPE::THREADS, SHAPE::CTAS) lantern_context_k
           const int g = (p * CP + c) * GT + gt;
           if (decltype(whole)::value || g * 8 < V) {
             uint64_t c2[4], u2[4];
-            pairs_of(rc, g, c2);
-            if (UNC) pairs_of(ru, g, u2);
+            if (TOPK) {   // (processed already)
+              const ulonglong2 ea = *reinterpret_cast<const ulonglong2*>(E + EI(g * 8));
+              const ulonglong2 eb = *reinterpret_cast<const ulonglong2*>(E + EI(g * 8 + 4));
+              c2[0] = ea.x, c2[1] = ea.y, c2[2] = eb.x, c2[3] = eb.y;
+            } else {
+              staged_pairs<BF16>(rc, g, c2);
+              if (UNC) staged_pairs<BF16>(ru, g, u2);
+            }
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
               uint64_t l2 = c2[i];
-              if (UNC) l2 = fma2(s2, sub2(c2[i], u2[i]), u2[i]);   // l_u + s (l_c - l_u)
-              if (!TONE) l2 = divide_T(l2);
-              a2[c * 4 + i] = l2;
+              if (UNC && !TOPK) l2 = fma2(s2, sub2(c2[i], u2[i]), u2[i]);   // l_u + s (l_c - l_u)
+              if (!TONE && !TOPK) l2 = divide_T(l2);
               float lo, hi;
               unpack2(l2, lo, hi);
+              if (TOPK) {   // (a NaN stays, to be reported)
+                lo = lo < tq ? ninf : lo, hi = hi < tq ? ninf : hi;
+                l2 = pack2(lo, hi);
+              }
+              a2[c * 4 + i] = l2;
               m = max3(m, lo, hi);
             }
           } else {
@@ -778,7 +844,7 @@ __global__ void __launch_bounds__(SHAPE::THREADS, SHAPE::CTAS) lantern_context_k
         S.slice[p * GT + gt] = n_p;
         if (NP <= 2) nq[NP <= 2 ? p : 0] = n_p;
         const float n_new = fmaxf(n_run, n_p);
-        tq = __fmaf_rn(tq, exp2_int(n_run - n_new), (lo + hi) * exp2_int(n_p - n_new));
+        sq = __fmaf_rn(sq, exp2_int(n_run - n_new), (lo + hi) * exp2_int(n_p - n_new));
         n_run = n_new;
       }
       nq_max = n_run;
@@ -786,15 +852,60 @@ __global__ void __launch_bounds__(SHAPE::THREADS, SHAPE::CTAS) lantern_context_k
     if (nchild > 0) {
       load_slots(xt, 0, nb);
       if (gt == 0) fetch_single();
-      if (full) stream_drafter(std::true_type{});
-      else stream_drafter(std::false_type{});
-      if (gt == 0) note_single();
+      if (full) load_drafter(std::true_type{});
+      else load_drafter(std::false_type{});
+      if constexpr (TOPK) {   // the drafter row's threshold, from the registers that hold the row
+        auto own = [&](int c, float (&z)[8]) {
+          uint64_t z2[4];
+          raw8_pairs<BF16>(raw[c], z2);
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            if (!TONE) z2[i] = divide_T(z2[i]);
+            unpack2(z2[i], z[2 * i], z[2 * i + 1]);
+          }
+        };
+        auto again = [&](int c, float (&z)[8]) {
+          row_logits<BF16, TONE>(P, P.draft, static_cast<size_t>(item) * V, c * GT + gt, z);
+        };
+        tp = group_kth_largest<SHAPE, CH, CH>(P, own, own, own, again, V, S, grp, gt, search3);
+      }
+      reduce_drafter();
+      if (!TOPK && gt == 0) note_single();
     }
     // The target rows were issued when the staging area fell free; they arrive while the drafter
     // row is streamed.  Every thread waits for itself (bounded); a wait that runs out is reported after
     // the next group barrier, where every thread sees it alike.
     if (item >= 0) {
       if (!mbar_wait(&bar_rows[grp][area], (iter / AREAS) & 1, tries)) S.fail = 1;
+      if constexpr (TOPK) {   // the target row's threshold; the processed logits replace the raw ones they came from
+        auto guided = [&](int c, float (&z)[8]) {
+          const int g = c * GT + gt;
+          uint64_t c2[4], u2[4];
+          staged_pairs<BF16>(stage, g, c2);
+          if (UNC) staged_pairs<BF16>(stage + rowbytes, g, u2);
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            uint64_t l2 = c2[i];
+            if (UNC) l2 = fma2(pack2(P.cfg_scale, P.cfg_scale), sub2(c2[i], u2[i]), u2[i]);
+            if (!TONE) l2 = divide_T(l2);
+            unpack2(l2, z[2 * i], z[2 * i + 1]);
+          }
+        };
+        auto guided_in_place = [&](int c, float (&z)[8]) {
+          const int g = c * GT + gt;
+          guided(c, z);
+          *reinterpret_cast<float4*>(E + EI(g * 8)) = make_float4(z[0], z[1], z[2], z[3]);
+          *reinterpret_cast<float4*>(E + EI(g * 8 + 4)) = make_float4(z[4], z[5], z[6], z[7]);
+        };
+        auto processed = [&](int c, float (&z)[8]) {
+          const int g = c * GT + gt;
+          const float4 a = *reinterpret_cast<const float4*>(E + EI(g * 8));
+          const float4 b = *reinterpret_cast<const float4*>(E + EI(g * 8 + 4));
+          z[0] = a.x, z[1] = a.y, z[2] = a.z, z[3] = a.w, z[4] = b.x, z[5] = b.y, z[6] = b.z, z[7] = b.w;
+        };
+        tq = group_kth_largest<SHAPE, CH, (NP > 2 ? 2 : CH)>(P, guided, guided_in_place, processed, processed, V, S, grp, gt, search3);
+        if (gt == 0 && nchild > 0) note_single();
+      }
       if (full) stream_target(std::true_type{});
       else stream_target(std::false_type{});
     }
@@ -805,7 +916,7 @@ __global__ void __launch_bounds__(SHAPE::THREADS, SHAPE::CTAS) lantern_context_k
     {
       const float n = nq_max;
       const float wnq = redux_max(n), wnd = redux_max(nd);
-      const double zq = static_cast<double>(tq * exp2_int(n - wnq));
+      const double zq = static_cast<double>(sq * exp2_int(n - wnq));
       const double zp = static_cast<double>(td * exp2_int(nd - wnd));
       // both sums in one butterfly: after the first exchange the lower half of the warp carries one, the upper the other
       const bool up = lane & 16;
@@ -1036,6 +1147,10 @@ __global__ void __launch_bounds__(SHAPE::THREADS, SHAPE::CTAS) lantern_context_k
                 for (int i = 0; i < 4; ++i) {
                   if (!TONE) z2[i] = divide_T(z2[i]);
                   unpack2(z2[i], z[2 * i], z[2 * i + 1]);
+                  if (TOPK) {
+                    z[2 * i] = z[2 * i] < tp ? ninf : z[2 * i];
+                    z[2 * i + 1] = z[2 * i + 1] < tp ? ninf : z[2 * i + 1];
+                  }
                 }
               }
               if ((struck >> c) & 1u) {   // a token rejected in this context sits in this chunk

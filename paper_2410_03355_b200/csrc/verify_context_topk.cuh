@@ -1,328 +1,329 @@
-// Top-k threshold of one staged row, found by the consumer group that is about to stream the row
-// (Appendix B.2: logits below the K-th largest of their row count as -inf; ties at that value are kept).
-// Included by verify_context.cuh; used by the TOPK variants of the fused kernel only.
+// Top-k threshold of one row of a context (Appendix B.2: logits below the K-th largest of their row count as -inf; ties at
+// that value are kept).  Included by verify_context.cuh.
 //
-// The row sits in shared memory as raw logits; `zchunk(g, z)` turns 16-byte group g into its eight
-// processed logits (guidance combine, temperature) with exactly the roundings of the streaming loop.
-// Steps, all exact in the end (the sample only decides where to look):
-//   1. the group's producer warp, while the group is still busy with the context before, takes a
-//      512-value sample spread over the row (from global memory) and finds, by bisection with warp-wide
-//      counts, two values (lo, hi) whose sample ranks lie three standard deviations to either side of
-//      the rank the K-th largest is expected to have in the sample; they travel with the work item;
-//   2. every thread goes over its 64 values once, without a branch: it counts those >= hi and notes
-//      down, one byte each, which of its values lie in [lo, hi); the notes of all threads are then
-//      gathered into one list (one counter update per warp), so that what follows is evenly spread;
-//   3. if the K-th largest does lie in [lo, hi) -- count(>= hi) < K <= count(>= lo) -- the listed values go
-//      into a 256-bin histogram over [lo, hi) (a monotone map, so bins are ordered like the values),
-//      every warp finds the bin holding the wanted rank by a suffix scan of its own, the values of
-//      that bin (a handful) are put side by side, and every warp ranks them with shuffles;
-//   4. otherwise (a sample that misleads, more notes than fit, a crowded bin) the value is found by plain
-//      bisection on the order-preserving bit patterns, one pass over the row per step: slow, exact,
-//      and bounded by 32 passes.  lantern_verify_counts reports how many rows needed it.
+// Found by the group that holds the row, on processed logits (guidance combine, temperature) with exactly the roundings of
+// the streaming part.  Exact in the end; the sample only decides where to look:
+//   1. four values per thread, spread over the row, go into a histogram of 128 bins between the smallest and
+//      the largest of them; two bin edges whose sample ranks lie three standard deviations to either side of the rank
+//      the K-th largest is expected to have give a bracket [lo, hi);
+//   2. every thread goes over its values twice: it counts those >= hi and those inside the bracket, and, knowing its place by
+//      one counter update per warp, puts the latter on a list;
+//   3. if the K-th largest does lie in [lo, hi) -- count(>= hi) < K <= count(>= lo) -- the listed values go into a histogram of 256
+//      bins over the bracket, every warp finds the bin that holds the wanted rank by a suffix scan of its own, and ranks
+//      the handful of values of that bin; a crowded bin (ties) is left to one warp, which searches the
+//      list by two pivots per pass, set where the rank should lie if the values were spread evenly;
+//   4. otherwise (a sample that misleads, a list too long) by plain bisection on the order-preserving bit patterns,
+//      one pass over the row per step: slow, exact, and bounded by 34 passes.  lantern_verify_counts reports how many rows
+//      needed it.
 #pragma once
 
 namespace lantern {
 
-constexpr int TKG_OWN = 24;         // bracket values a thread can note down (about five are expected)
-constexpr int TKG_LIST = 2048;      // bracket values of the whole row
-constexpr int TKG_BINS = 256;
-constexpr int TKG_TINY = 32;        // values of the wanted bin that one warp can rank
-static_assert(TKG_BINS == GT, "every thread of a group clears one bin");
-
-struct GroupTopk {
-  // During the pass: code[i * GT + t] = which of its 64 values thread t found inside the bracket as its i-th.
-  // Afterwards the same bytes hold, per entry of `list`, the bin its value fell into.
-  unsigned char code[TKG_OWN * GT];
-  unsigned short list[TKG_LIST];    // (thread << 8) | code of every bracket value, in no particular order
-  int hist[2][TKG_BINS];            // [0] serves the drafter row of a context, [1] its target row: a call never
-  float tiny[2][TKG_TINY];          //     clears what a slow warp may still be reading from the call before
-  int n_tiny[2], n_list[2];
-  int wsum[GW][2];
-};
-
 // order-preserving bit pattern of a processed logit: NaN lowest, -0 as +0
-__device__ __forceinline__ uint32_t tkg_key(float z) {
+__device__ __forceinline__ uint32_t topk_order(float z) {
   if (z != z) return 0u;
   if (z == 0.0f) z = 0.0f;
   const uint32_t u = __float_as_uint(z);
   return (u & 0x80000000u) ? ~u : (u | 0x80000000u);
 }
-__device__ __forceinline__ float tkg_value(uint32_t key) {
+__device__ __forceinline__ float topk_from_order(uint32_t key) {
   return __uint_as_float((key & 0x80000000u) ? (key & 0x7fffffffu) : ~key);
 }
+constexpr uint32_t TOPK_ORDER_NINF = 0x007fffffu;
 
-// Two values whose ranks among the warp's sample values (16 per lane, NaN = absent) are within `slack` of
-// r_hi and r_lo: both searches advance in the same passes.  Where a search finds no such value (equal
-// sample values) it ends on the side that widens the bracket.
-__device__ __forceinline__ void tkg_sample_bracket(const float (&s)[16], uint32_t kmin, uint32_t kmax, int r_hi, int r_lo,
-                                                   int slack, bool want_hi, bool want_lo, float& lo, float& hi) {
-  uint32_t Lh = kmin, Hh = kmax + 1u, Ll = kmin, Hl = kmax + 1u;   // count(>= L) = everything, count(>= H) = 0
-  bool done_h = !want_hi, done_l = !want_lo;
-  for (int pass = 0; pass < 40 && !(done_h && done_l); ++pass) {
-    uint32_t ph = tkg_key(0.5f * tkg_value(Lh) + 0.5f * tkg_value(Hh - 1u));
-    if (!(ph > Lh && ph < Hh)) ph = Lh + ((Hh - Lh) >> 1);
-    uint32_t pl = tkg_key(0.5f * tkg_value(Ll) + 0.5f * tkg_value(Hl - 1u));
-    if (!(pl > Ll && pl < Hl)) pl = Ll + ((Hl - Ll) >> 1);
-    const float vh = tkg_value(ph), vl = tkg_value(pl);
-    int ch0 = 0, ch1 = 0, cl0 = 0, cl1 = 0;
+// eight processed logits of 16-byte group g of a row in global memory (no guidance)
+template <bool BF16, bool TONE>
+__device__ __forceinline__ void row_logits(const VerifyParams& P, const void* base, size_t row, int g, float (&z)[8]) {
+  const size_t elem = row + static_cast<size_t>(g) * 8;
+  if (BF16) {
+    const uint4 x = __ldg(reinterpret_cast<const uint4*>(static_cast<const unsigned short*>(base) + elem));
+    const uint32_t w[4] = {x.x, x.y, x.z, x.w};
 #pragma unroll
-    for (int i = 0; i < 16; i += 2) {
-      ch0 += s[i] >= vh;
-      ch1 += s[i + 1] >= vh;
-      cl0 += s[i] >= vl;
-      cl1 += s[i + 1] >= vl;
+    for (int q = 0; q < 4; ++q) {
+      z[2 * q] = __uint_as_float(w[q] << 16);
+      z[2 * q + 1] = __uint_as_float(w[q] & 0xffff0000u);
     }
-    const int both = __reduce_add_sync(kFull, ((ch0 + ch1) << 16) | (cl0 + cl1));   // 512 values at most: no carry
-    const int ch = both >> 16, cl = both & 0xffff;
-    if (!done_h) {
-      if (ch > r_hi + slack) Lh = ph;
-      else if (ch < r_hi - slack) Hh = ph;
-      else hi = vh, done_h = true;
-      if (!done_h && Hh - Lh <= 1u) hi = tkg_value(Hh), done_h = true;   // fewer above it: a wider bracket
-    }
-    if (!done_l) {
-      if (cl > r_lo + slack) Ll = pl;
-      else if (cl < r_lo - slack) Hl = pl;
-      else lo = vl, done_l = true;
-      if (!done_l && Hl - Ll <= 1u) lo = tkg_value(Ll), done_l = true;   // more above it: a wider bracket
-    }
+  } else {
+    const float4 a = __ldg(reinterpret_cast<const float4*>(static_cast<const float*>(base) + elem));
+    const float4 b = __ldg(reinterpret_cast<const float4*>(static_cast<const float*>(base) + elem) + 1);
+    z[0] = a.x, z[1] = a.y, z[2] = a.z, z[3] = a.w, z[4] = b.x, z[5] = b.y, z[6] = b.z, z[7] = b.w;
   }
-  if (!done_h) hi = tkg_value(Hh);
-  if (!done_l) lo = tkg_value(Ll);
-}
-
-// sum of two per-thread counts over the group (every thread gets both sums); one group barrier
-__device__ __forceinline__ void tkg_group_sum2(GroupTopk& T, int grp, int gw, int lane, int& a, int& b) {
-  a = __reduce_add_sync(kFull, a);
-  b = __reduce_add_sync(kFull, b);
-  gbar(grp);            // the previous readers of wsum are done
-  if (lane == 0) {
-    T.wsum[gw][0] = a;
-    T.wsum[gw][1] = b;
-  }
-  gbar(grp);
-  a = b = 0;
+  if (!TONE) {
 #pragma unroll
-  for (int w = 0; w < GW; ++w) {
-    a += T.wsum[w][0];
-    b += T.wsum[w][1];
+    for (int e = 0; e < 8; ++e) z[e] = __fdiv_rn(z[e], P.T);
   }
 }
 
-// Step 4 of the header comment: the K-th largest by bisection on bit patterns, one pass over the row per step.
-// Invariant: count(key >= L) >= K > count(key >= H).  If fewer than K values lie above -inf the answer is
-// -inf (nothing is cut).
-template <class ZF>
-__device__ __forceinline__ float tkg_exact_by_passes(ZF& zchunk, int K, int V, int CH, GroupTopk& T, int grp, int gt) {
-  const int gw = gt >> 5, lane = gt & 31;
-  const uint32_t KNINF = 0x007fffffu;
-  uint32_t L = KNINF, H = 0xff800001u;          // -inf .. just above +inf
-  {
-    int c = 0, dummy = 0;
-    for (int ch = 0; ch < CH; ++ch) {
-      const int g = ch * GT + gt;
-      if (g * 8 < V) {
-        float z[8];
-        zchunk(g, z);
-#pragma unroll
-        for (int e = 0; e < 8; ++e) c += tkg_key(z[e]) > KNINF;
-      }
-    }
-    tkg_group_sum2(T, grp, gw, lane, c, dummy);
-    if (c < K) return __int_as_float(0xff800000);
-    L = KNINF + 1u;
-  }
-  for (int pass = 0; pass < 34 && H - L > 1u; ++pass) {
-    const uint32_t p = L + ((H - L) >> 1);
-    int c = 0, dummy = 0;
-    for (int ch = 0; ch < CH; ++ch) {
-      const int g = ch * GT + gt;
-      if (g * 8 < V) {
-        float z[8];
-        zchunk(g, z);
-#pragma unroll
-        for (int e = 0; e < 8; ++e) c += tkg_key(z[e]) >= p;
-      }
-    }
-    tkg_group_sum2(T, grp, gw, lane, c, dummy);
-    if (c >= K) L = p;
-    else H = p;
-  }
-  return tkg_value(L);
-}
-
-// Step 1 of the header comment, run by one warp (all 32 lanes call it and get the same values): the
-// bracket of a row from a 512-value sample.  `zchunk(g, z)` gives the eight processed logits of 16-byte
-// group g, from wherever the caller keeps the row.  out = {lo, hi, base, scale}.
-template <class ZF>
-__device__ __forceinline__ void tkg_warp_bracket(ZF& zchunk, int K, int V, int lane, float (&out)[4]) {
-  const float qnan = __int_as_float(0x7fc00000);
+// Step 3, by one warp: the rank-th largest of the n values in `list` (1 <= rank <= n, no NaN).
+__device__ __forceinline__ float topk_listed(const float* list, int n, int rank, int lane) {
   const float pinf = __int_as_float(0x7f800000), ninf = __int_as_float(0xff800000);
-  const int groups = V >> 3;
-  const int take = groups < 64 ? groups : 64;            // sampled 16-byte groups, spread evenly
-  float s[16];
-  uint32_t kmin = 0xffffffffu, kmax = 0u;
-#pragma unroll
-  for (int h = 0; h < 2; ++h) {
-    const int j = lane + 32 * h;
-    float z[8];
-    if (j < take) zchunk(j * groups / take, z);           // j < 64 and groups <= 2048: no overflow
-#pragma unroll
-    for (int e = 0; e < 8; ++e) {
-      const float v = j < take ? z[e] : qnan;
-      s[8 * h + e] = v;
-      const uint32_t kk = tkg_key(v);
-      if (kk > 0x007fffffu) {                             // above -inf
-        kmin = kk < kmin ? kk : kmin;
-        kmax = kk > kmax ? kk : kmax;
-      }
+  float vmin = pinf, vmax = ninf;
+  for (int i = lane; i < n; i += 32) {
+    const float v = list[i];
+    vmin = fminf(vmin, v);
+    vmax = fmaxf(vmax, v);
+  }
+  uint32_t L = __reduce_min_sync(kFull, topk_order(vmin)), H = __reduce_max_sync(kFull, topk_order(vmax)) + 1u;
+  int cL = n, cH = 0;                       // count(>= L) >= rank > count(>= H), on order-preserving bit patterns
+  bool even = true;                         // the last pass took enough away: go on with interpolation
+  for (int pass = 0; pass < 64 && H - L > 1u && cL > rank && cH < rank - 1; ++pass) {
+    uint32_t p1, p2;                        // L < p1 <= p2 < H
+    p1 = p2 = L + ((H - L) >> 1);
+    if (even) {
+      const float a = topk_from_order(L), b = topk_from_order(H - 1u);
+      const float in = static_cast<float>(cL - cH), pos = (static_cast<float>(rank - cH) - 0.5f) / in;   // from the top
+      const float half = 0.8f / sqrtf(in);
+      const uint32_t q1 = topk_order(b - (b - a) * fminf(pos + half, 1.0f)), q2 = topk_order(b - (b - a) * fmaxf(pos - half, 0.0f));
+      if (q1 > L && q1 < H) p1 = q1;
+      if (q2 > L && q2 < H) p2 = q2;
+      if (p1 > p2) p1 = p2;
     }
+    const float v1 = topk_from_order(p1), v2 = topk_from_order(p2);
+    int c1 = 0, c2 = 0;
+    for (int i = lane; i < n; i += 32) {
+      const float v = list[i];
+      c1 += v >= v1;
+      c2 += v >= v2;
+    }
+    const int both = __reduce_add_sync(kFull, (c1 << 16) | c2);
+    c1 = both >> 16, c2 = both & 0xffff;
+    const int before = cL - cH;
+    if (c2 >= rank) {
+      L = p2, cL = c2;
+    } else if (c1 >= rank) {
+      L = p1, cL = c1, H = p2, cH = c2;
+    } else {
+      H = p1, cH = c1;
+    }
+    even = 2 * (cL - cH) <= before;
   }
-  kmin = __reduce_min_sync(kFull, kmin);
-  kmax = __reduce_max_sync(kFull, kmax);
-  float lo = ninf, hi = pinf, base = 0.0f, scale = 0.0f;
-  if (kmax >= kmin) {                                     // the sample holds a finite value
-    const float ns = static_cast<float>(take * 8);
-    const float mean = static_cast<float>(K) * ns / static_cast<float>(V);
-    const float sd = sqrtf(mean * (1.0f - static_cast<float>(K) / static_cast<float>(V)));
-    const int slack = static_cast<int>(0.25f * sd) + 1;
-    const int r_hi = static_cast<int>(mean - 3.0f * sd) - slack - 1;
-    const int r_lo = static_cast<int>(mean + 3.0f * sd) + slack + 2;
-    tkg_sample_bracket(s, kmin, kmax, r_hi, r_lo, slack, r_hi > slack, r_lo < static_cast<int>(ns) - slack, lo, hi);
-    // bins: over [lo, hi) where both are finite, else over the sample's own range (values beyond it are clamped)
-    const float b0 = lo > ninf ? lo : tkg_value(kmin), b1 = hi < pinf ? hi : tkg_value(kmax);
-    base = b0;
-    scale = b1 > b0 ? static_cast<float>(TKG_BINS) / (b1 - b0) : 0.0f;
+  // the answer is the smallest value >= L where exactly `rank` values are, the largest below H where rank - 1 are not below
+  // it, and L itself where the interval has closed
+  const float vL = topk_from_order(L), vH = topk_from_order(H);
+  uint32_t up = 0xffffffffu, down = 0u;
+  for (int i = lane; i < n; i += 32) {
+    const float v = list[i];
+    const uint32_t key = topk_order(v);
+    if (v >= vL) up = key < up ? key : up;
+    if (H == 0xff800001u || v < vH) down = key > down ? key : down;
   }
-  out[0] = lo, out[1] = hi, out[2] = base, out[3] = scale;
+  up = __reduce_min_sync(kFull, up);
+  down = __reduce_max_sync(kFull, down);
+  return topk_from_order(cL == rank ? up : (cH == rank - 1 ? down : L));
 }
 
-// Steps 2-4: the K-th largest processed logit of the row behind `zchunk` (0 < K < V), given the bracket
-// br = {lo, hi, base, scale}; every thread of the group calls it and gets the same value.  CH = 16-byte
-// groups per thread.  `which` = 0 for a context's drafter row, 1 for its target row (see GroupTopk).  The
-// histogram and the list counter of `which` are zero on entry and left zero on exit.
-template <class ZF>
-__device__ __forceinline__ float tkg_kth_largest(ZF& zchunk, const float (&br)[4], int K, int V, int CH, GroupTopk& T,
-                                                 int which, int grp, int gt, int* slow_count) {
-  const int gw = gt >> 5, lane = gt & 31;
-  if (gt == 0) T.n_tiny[which] = 0;                       // next touched behind two group barriers
-  const float lo = br[0], hi = br[1], base = br[2], scale = br[3];
-  auto bin_of = [&](float v) {
-    const float x = (v - base) * scale;
-    return x < 0.0f ? 0 : (x >= static_cast<float>(TKG_BINS) ? TKG_BINS - 1 : static_cast<int>(x));
-  };
-  // the value behind a list entry, recomputed from the staged row
-  auto value_of = [&](int entry) {
+// sum of a per-thread count over the group (every thread gets it); two group barriers
+template <int GW, class BAR>
+__device__ __forceinline__ int topk_group_sum(GroupTopk<GW, true>& T, int gw, int lane, int a, BAR& gbar) {
+  a = __reduce_add_sync(kFull, a);
+  gbar();               // the previous readers of count[] are done
+  if (lane == 0) T.count[gw][0] = a;
+  gbar();
+  return __reduce_add_sync(kFull, lane < GW ? T.count[lane][0] : 0);
+}
+
+// The K-th largest processed logit of a row (0 < K < V); every thread of the group calls it and gets the same value.
+// The callables give the eight values of this thread's chunk c: for the sample, for the first and the second sweep (loops
+// unrolled UNROLL times), and for the slow path (in a rolled loop).  search3 = searches of this group so far, mod 3: its list
+// counter is zero on entry, and the one after the next is cleared here.
+template <class SHAPE, int CH, int UNROLL, class Z0, class Z1, class Z2, class Z3, class SH>
+__device__ __forceinline__ float group_kth_largest(const VerifyParams& P, Z0& sampled, Z1& first, Z2& second, Z3& slow, int V, SH& S,
+                                                   int grp, int gt, int& search3) {
+  constexpr int GT = SHAPE::GT, GW = GT / 32;
+  const float pinf = __int_as_float(0x7f800000), ninf = __int_as_float(0xff800000);
+  auto gbar = [&]() { asm volatile("bar.sync %0, %1;" ::"r"(1 + grp), "n"(GT) : "memory"); };
+  auto& T = S.tk;
+  float* list = S.slice;
+  const int K = P.top_k, gw = gt >> 5, lane = gt & 31;
+  auto here = [&](int c) { return (c * GT + gt) * 8 < V; };
+  // ---- 1. ----
+  float smp[4];
+  constexpr int FROM = CH < 4 ? CH : 4;               // chunks the sample is taken from, 4 / FROM values of each
+#pragma unroll
+  for (int q = 0; q < FROM; ++q) {
+    const int c = q * (CH / FROM);
     float z[8];
-    zchunk(((entry >> 3) & 7) * GT + (entry >> 8), z);
-    const int e = entry & 7;
-    const float a0 = (e & 1) ? z[1] : z[0], a1 = (e & 1) ? z[3] : z[2], a2 = (e & 1) ? z[5] : z[4], a3 = (e & 1) ? z[7] : z[6];
-    const float b0 = (e & 2) ? a1 : a0, b1 = (e & 2) ? a3 : a2;
-    return (e & 4) ? b1 : b0;
-  };
-  // ---- 2. one pass, thread-local and free of branches: count the values >= hi, note those in [lo, hi) ----
+    const bool on = here(c);
+    if (on) sampled(c, z);
+#pragma unroll
+    for (int e = 0; e < 4 / FROM; ++e) smp[q * (4 / FROM) + e] = on ? z[e * (2 * FROM)] : __int_as_float(0x7fc00000);
+  }
+  float vmin = pinf, vmax = ninf;
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    if (smp[q] > ninf) vmin = fminf(vmin, smp[q]);
+    vmax = fmaxf(vmax, smp[q]);                        // (a NaN is passed over)
+  }
+  vmin = -redux_max(-vmin);
+  vmax = redux_max(vmax);
+  if (lane == 0) T.range[gw][0] = vmin, T.range[gw][1] = vmax;
+  gbar();
+  vmin = -redux_max(lane < GW ? -T.range[lane][0] : ninf);
+  vmax = redux_max(lane < GW ? T.range[lane][1] : ninf);
+  const float width = (vmax - vmin) * (1.0f / TOPK_BINS);
+  const float scale = width > 0.0f && width < pinf ? 1.0f / width : 0.0f;
+#pragma unroll
+  for (int q = 0; q < 4; ++q)
+    if (smp[q] == smp[q]) atomicAdd(&T.hist[min(static_cast<int>(fmaxf((smp[q] - vmin) * scale, 0.0f)), TOPK_BINS - 1)], 1);
+  gbar();
+  float lo = ninf, hi = pinf;
+  {
+    constexpr int PER = TOPK_BINS / 32;
+    static_assert(PER == 4, "a lane reads four bins");
+    const int4 h = *reinterpret_cast<const int4*>(&T.hist[lane * PER]);
+    int incl = h.x + h.y + h.z + h.w;                  // suffix sum over the lanes
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int v = __shfl_down_sync(kFull, incl, o);
+      if (lane + o < 32) incl += v;
+    }
+    const int s0 = incl, s1 = s0 - h.x, s2 = s1 - h.y, s3 = s2 - h.z;   // sample values in this bin and above
+    const float ns = static_cast<float>(__shfl_sync(kFull, incl, 0)), share = static_cast<float>(K) / static_cast<float>(V);
+    const float mean = share * ns, sd = sqrtf(mean * (1.0f - share));
+    const int r_hi = static_cast<int>(floorf(mean - 3.0f * sd)) - 1, r_lo = static_cast<int>(mean + 3.0f * sd) + 2;
+    const int over = (s0 > r_hi) + (s1 > r_hi) + (s2 > r_hi) + (s3 > r_hi);
+    const int cover = (s0 >= r_lo) + (s1 >= r_lo) + (s2 >= r_lo) + (s3 >= r_lo);
+    const int both = __reduce_add_sync(kFull, over << 16 | cover);
+    const int b_hi = both >> 16, b_lo = (both & 0xffff) - 1;
+    if (r_hi >= 0 && b_hi < TOPK_BINS) hi = vmin + width * static_cast<float>(b_hi);
+    if (b_lo > 0) lo = vmin + width * static_cast<float>(b_lo);
+  }
+  // ---- 2. ----
   int c_hi = 0, n_in = 0;
-  for (int ch = 0; ch < CH; ++ch) {
-    const int g = ch * GT + gt;
-    if (g * 8 < V) {
+#pragma unroll UNROLL
+  for (int c = 0; c < CH; ++c) {
+    if (here(c)) {
       float z[8];
-      zchunk(g, z);
+      first(c, z);
 #pragma unroll
       for (int e = 0; e < 8; ++e) {
-        const float v = z[e];
-        c_hi += v >= hi;
-        const bool in = v >= lo && v < hi;
-        if (in) T.code[(n_in < TKG_OWN ? n_in : TKG_OWN - 1) * GT + gt] = static_cast<unsigned char>(ch * 8 + e);
-        n_in += in;
+        c_hi += z[e] >= hi;
+        n_in += z[e] >= lo;
       }
     }
   }
-  // the notes of all threads as one list (one counter update per warp), so that the next steps are balanced
-  const int n_own = n_in < TKG_OWN ? n_in : TKG_OWN;
+  n_in -= c_hi;
   {
-    int incl = n_own;
+    int incl = n_in;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
       const int v = __shfl_up_sync(kFull, incl, o);
       if (lane >= o) incl += v;
     }
     int start = 0;
-    if (lane == 31) start = atomicAdd(&T.n_list[which], incl);
-    const int pos = __shfl_sync(kFull, start, 31) + incl - n_own;
-    for (int i = 0; i < n_own; ++i)
-      if (pos + i < TKG_LIST) T.list[pos + i] = static_cast<unsigned short>((gt << 8) | T.code[i * GT + gt]);
-  }
-  int c_in = n_in + (n_in > TKG_OWN ? (1 << 20) : 0);     // bit 20 and up: threads whose notes overflowed
-  tkg_group_sum2(T, grp, gw, lane, c_hi, c_in);           // its barriers also publish the list
-  const bool overflow = (c_in >> 20) != 0 || (c_in & 0xfffff) > TKG_LIST;   // (no overflowing thread: c_in = listed values)
-  c_in &= 0xfffff;
-  if (gt == 0) T.n_list[which] = 0;                       // everybody has read it (the sum above went through two barriers)
-  if (overflow || !(c_hi < K && K <= c_hi + c_in)) {
-    if (gt == 0) atomicAdd(slow_count, 1);
-    return tkg_exact_by_passes(zchunk, K, V, CH, T, grp, gt);
-  }
-  // ---- 3. histogram of the bracket values; the bin that holds rank K - c_hi counted from the top ----
-  for (int i = gt; i < c_in; i += GT) {
-    const int b = bin_of(value_of(T.list[i]));
-    T.code[i] = static_cast<unsigned char>(b);            // (the per-thread notes are no longer needed)
-    atomicAdd(&T.hist[which][b], 1);
-  }
-  gbar(grp);
-  int bin, rank;
-  {                                                       // every warp for itself: no barrier to publish the result
-    const int* h = T.hist[which] + lane * (TKG_BINS / 32);
-    int mine = 0;
+    if (lane == 31) start = atomicAdd(&T.listed[search3], incl);
+    int pos = __shfl_sync(kFull, start, 31) + incl - n_in;
+    if (lane == 31) T.count[gw][1] = incl;
+    const bool room = __all_sync(kFull, pos + n_in <= TOPK_LIST);
+    if (room) {
+      float* to = list + pos;
+#pragma unroll UNROLL
+      for (int c = 0; c < CH; ++c) {
+        if (here(c)) {
+          float z[8];
+          second(c, z);
 #pragma unroll
-    for (int i = 0; i < TKG_BINS / 32; ++i) mine += h[i];
-    int suffix = mine;                                    // inclusive suffix sum over the lanes
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const int v = __shfl_down_sync(kFull, suffix, o);
-      if (lane + o < 32) suffix += v;
-    }
-    const int above = suffix - mine;                      // values in the bins of higher lanes
-    const int want = K - c_hi;                            // 1 <= want <= c_in
-    const bool here = above < want && want <= above + mine;
-    int b = TKG_BINS / 32 - 1, acc = above;
-    if (here) {
-      for (; b > 0; --b) {
-        if (acc + h[b] >= want) break;
-        acc += h[b];
+          for (int e = 0; e < 8; ++e)
+            if (z[e] >= lo && z[e] < hi) *to++ = z[e];
+        }
       }
     }
-    const int src = __ffs(__ballot_sync(kFull, here)) - 1;   // exactly one lane holds the rank
-    bin = __shfl_sync(kFull, lane * (TKG_BINS / 32) + b, src);
-    rank = __shfl_sync(kFull, want - acc, src);           // rank inside that bin, from its top
   }
-  // the values of that bin, for one warp to rank
-  for (int i = gt; i < c_in; i += GT) {
-    if (T.code[i] == bin) {
-      const int pos = atomicAdd(&T.n_tiny[which], 1);
-      if (pos < TKG_TINY) T.tiny[which][pos] = value_of(T.list[i]);
+  const int w_hi = __reduce_add_sync(kFull, c_hi);
+  if (lane == 0) T.count[gw][0] = w_hi;
+  gbar();
+  c_hi = __reduce_add_sync(kFull, lane < GW ? T.count[lane][0] : 0);
+  const int c_in = __reduce_add_sync(kFull, lane < GW ? T.count[lane][1] : 0);
+  const int now = search3;
+  search3 = now < 2 ? now + 1 : 0;
+  if (gt == 0) T.listed[now > 0 ? now - 1 : 2] = T.picked[now > 0 ? now - 1 : 2] = 0;   // (the one before the current one comes after the next)
+  if (gt < TOPK_BINS) T.hist[gt] = 0;                 // everybody has read it
+  if (c_in <= TOPK_LIST && c_hi < K && K <= c_hi + c_in) {
+    // ---- 3. ----
+    const float f_lo = lo > ninf ? lo : vmin, f_hi = hi < pinf ? hi : vmax;
+    const float f_scale = f_hi > f_lo ? static_cast<float>(TOPK_FINE) / (f_hi - f_lo) : 0.0f;
+    auto bin_of = [&](float v) { return min(static_cast<int>(fmaxf((v - f_lo) * f_scale, 0.0f)), TOPK_FINE - 1); };
+    for (int i = gt; i < c_in; i += GT) atomicAdd(&T.fine[bin_of(list[i])], 1);
+    gbar();
+    int bin, rank, pop;
+    {
+      constexpr int PER = TOPK_FINE / 32;
+      int h[PER];
+#pragma unroll
+      for (int q = 0; q < PER; q += 4) {
+        const int4 v = *reinterpret_cast<const int4*>(&T.fine[lane * PER + q]);
+        h[q] = v.x, h[q + 1] = v.y, h[q + 2] = v.z, h[q + 3] = v.w;
+      }
+      int mine = 0;
+#pragma unroll
+      for (int q = 0; q < PER; ++q) mine += h[q];
+      int incl = mine;                                 // suffix sum over the lanes
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int v = __shfl_down_sync(kFull, incl, o);
+        if (lane + o < 32) incl += v;
+      }
+      const int want = K - c_hi;                       // 1 <= want <= c_in
+      int above = incl - mine, b = 0, r = 0, p = 0;
+      const bool holds = above < want && want <= incl;   // exactly one lane
+#pragma unroll
+      for (int q = PER - 1; q >= 0; --q) {
+        if (holds && r == 0 && above + h[q] >= want) b = lane * PER + q, r = want - above, p = h[q];
+        above += h[q];
+      }
+      const int src = __ffs(__ballot_sync(kFull, holds)) - 1;
+      bin = __shfl_sync(kFull, b, src);
+      rank = __shfl_sync(kFull, r, src);               // rank inside that bin, from its top
+      pop = __shfl_sync(kFull, p, src);
     }
+    if (pop <= TOPK_TINY) {
+      for (int i = gt; i < c_in; i += GT) {
+        const float v = list[i];
+        if (bin_of(v) == bin) T.tiny[atomicAdd(&T.picked[now], 1)] = v;
+      }
+    } else if (gw == 0) {
+      const float t = topk_listed(list, c_in, K - c_hi, lane);
+      if (lane == 0) T.threshold = t;
+    }
+    gbar();
+    for (int q = gt; q < TOPK_FINE; q += GT) T.fine[q] = 0;
+    if (pop > TOPK_TINY) return T.threshold;
+    // lane l holds the bin's l-th value; the wanted one has fewer than `rank` values above it and at least `rank` not below
+    // it (equal values give the same answer)
+    const float v = lane < pop ? T.tiny[lane] : ninf;
+    int gtr = 0, geq = 0;
+    for (int j = 0; j < pop; ++j) {
+      const float o = __shfl_sync(kFull, v, j);
+      gtr += o > v;
+      geq += o >= v;
+    }
+    return __shfl_sync(kFull, v, __ffs(__ballot_sync(kFull, lane < pop && gtr < rank && rank <= geq)) - 1);
   }
-  gbar(grp);
-  T.hist[which][gt] = 0;                                  // nobody reads the histogram past this barrier
-  const int n_tiny = T.n_tiny[which];
-  if (n_tiny > TKG_TINY) {                                // a crowded bin (many equal values)
-    if (gt == 0) atomicAdd(slow_count, 1);
-    return tkg_exact_by_passes(zchunk, K, V, CH, T, grp, gt);
+  // ---- 4. bisection on bit patterns: count(>= L) >= K > count(>= H).  If fewer than K values lie above -inf the answer is
+  // -inf (nothing is cut). ----
+  if (gt == 0) atomicAdd(&P.counters->n_slow_topk, 1);
+  uint32_t L = TOPK_ORDER_NINF + 1u, H = 0xff800001u;   // just above -inf .. just above +inf
+  auto count = [&](uint32_t from) {
+    int n = 0;
+#pragma unroll 1
+    for (int c = 0; c < CH; ++c) {
+      if (here(c)) {
+        float z[8];
+        slow(c, z);
+#pragma unroll
+        for (int e = 0; e < 8; ++e) n += topk_order(z[e]) >= from;
+      }
+    }
+    return topk_group_sum<GW>(T, gw, lane, n, gbar);
+  };
+  const bool open = count(L) >= K;
+  for (int pass = 0; open && pass < 34 && H - L > 1u; ++pass) {
+    const uint32_t p = L + ((H - L) >> 1);
+    if (count(p) >= K) L = p;
+    else H = p;
   }
-  // lane l holds the bin's l-th value; the wanted one has fewer than `rank` values above it and at least
-  // `rank` values not below it (equal values give the same answer)
-  const float mine_v = lane < n_tiny ? T.tiny[which][lane] : __int_as_float(0xff800000);
-  int gtr = 0, geq = 0;
-  for (int j = 0; j < n_tiny; ++j) {                      // (a handful; the bound is the same for every thread)
-    const float o = __shfl_sync(kFull, mine_v, j);
-    gtr += o > mine_v ? 1 : 0;
-    geq += o >= mine_v ? 1 : 0;
-  }
-  const unsigned hit = __ballot_sync(kFull, lane < n_tiny && gtr < rank && rank <= geq);
-  if (hit == 0u) {                                        // cannot happen with a consistent histogram
-    if (gt == 0) atomicAdd(slow_count, 1);
-    return tkg_exact_by_passes(zchunk, K, V, CH, T, grp, gt);
-  }
-  return __shfl_sync(kFull, mine_v, __ffs(hit) - 1);
+  gbar();   // count[] is written again by the next search before its barriers
+  return open ? topk_from_order(L) : ninf;
 }
 
 }  // namespace lantern

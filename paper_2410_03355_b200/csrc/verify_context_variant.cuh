@@ -1,31 +1,13 @@
 // One compile-time variant (TONE, JSD, TOPK) of the fused context kernel for every row layout:
 // included by verify_context_v*.cu after defining LANTERN_VARIANT_{TONE,JSD,TOPK,NAME}.
 #include "verify_common.cuh"
-#if LANTERN_VARIANT_TOPK
-#include "verify_context_filtered.cuh"
-#else
 #include "verify_context.cuh"
-#endif
 
 namespace lantern {
 
-#if LANTERN_VARIANT_TOPK
-template <int CHC, bool BF16, bool UNC>
-static cudaError_t launch_one(const VerifyParams& P, long long items, int sms, cudaStream_t st) {
-  auto kc = lantern_context_topk_kernel<CHC, BF16, UNC, LANTERN_VARIANT_TONE, LANTERN_VARIANT_JSD, true>;
-  // one staging area of three row slots per consumer group; the numerators are kept over the rows they came from
-  const size_t smem_bytes = NGRP * ((static_cast<size_t>(3) * P.V * (BF16 ? 2 : 4) + 127) & ~static_cast<size_t>(127));
-  const long long ctas = (items + NGRP - 1) / NGRP;   // every CTA runs NGRP contexts at a time
-  const int grid = static_cast<int>(ctas < sms ? ctas : sms);
-  cudaError_t e = cudaFuncSetAttribute(kc, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem_bytes));
-  if (e != cudaSuccess) return e;
-  kc<<<grid, CTX_THREADS, smem_bytes, st>>>(P);
-  return cudaGetLastError();
-}
-#else
 template <class SHAPE, int CHC, bool BF16, bool UNC>
 static cudaError_t launch_shape(const VerifyParams& P, long long items, int sms, cudaStream_t st) {
-  auto kc = lantern_context_kernel<SHAPE, CHC, BF16, UNC, LANTERN_VARIANT_TONE, LANTERN_VARIANT_JSD>;
+  auto kc = lantern_context_kernel<SHAPE, CHC, BF16, UNC, LANTERN_VARIANT_TONE, LANTERN_VARIANT_JSD, LANTERN_VARIANT_TOPK>;
   const size_t groups = SHAPE::NGRP * SHAPE::AREAS;
   const int ctas = sms * SHAPE::CTAS;
   const int grid = static_cast<int>(items < ctas ? items : ctas);   // a few contexts get an SM each
@@ -43,8 +25,6 @@ static cudaError_t launch_one(const VerifyParams& P, long long items, int sms, c
   }
   return launch_shape<CtxNarrow, CHC, BF16, UNC>(P, items, sms, st);
 }
-#endif
-
 template <int CHC>
 static cudaError_t launch_layout(const VerifyParams& P, bool bf, bool un, long long items, int sms, cudaStream_t st) {
   return bf ? (un ? launch_one<CHC, true, true>(P, items, sms, st) : launch_one<CHC, true, false>(P, items, sms, st))

@@ -68,59 +68,6 @@ __device__ __forceinline__ int topk_count(const uint32_t (&key)[NE], uint32_t t,
   return tot;
 }
 
-// processed logits of one row as keys: base row (+ unconditional row at `branch` elements further on)
-template <bool BF16, bool UNC>
-__device__ __forceinline__ void topk_load_keys(const void* logits, size_t row_elem, size_t branch_elem, int V, float s,
-                                               float T, uint32_t (&key)[TK_CH * 8]) {
-  const int tid = threadIdx.x;
-#pragma unroll
-  for (int c = 0; c < TK_CH; ++c) {
-    const int g = c * TKT + tid;
-    float lc[8], lu[8];
-    if (g * 8 < V) {
-      if (BF16) {
-        const unsigned short* base = static_cast<const unsigned short*>(logits);
-        const uint4 x = __ldg(reinterpret_cast<const uint4*>(base + row_elem) + g);
-        const uint32_t xw[4] = {x.x, x.y, x.z, x.w};
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          lc[2 * i] = __uint_as_float(xw[i] << 16);
-          lc[2 * i + 1] = __uint_as_float(xw[i] & 0xffff0000u);
-        }
-        if (UNC) {
-          const uint4 y = __ldg(reinterpret_cast<const uint4*>(base + branch_elem + row_elem) + g);
-          const uint32_t yw[4] = {y.x, y.y, y.z, y.w};
-#pragma unroll
-          for (int i = 0; i < 4; ++i) {
-            lu[2 * i] = __uint_as_float(yw[i] << 16);
-            lu[2 * i + 1] = __uint_as_float(yw[i] & 0xffff0000u);
-          }
-        }
-      } else {
-        const float* base = static_cast<const float*>(logits);
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          const float4 x = __ldg(reinterpret_cast<const float4*>(base + row_elem) + 2 * g + h);
-          lc[4 * h] = x.x, lc[4 * h + 1] = x.y, lc[4 * h + 2] = x.z, lc[4 * h + 3] = x.w;
-          if (UNC) {
-            const float4 y = __ldg(reinterpret_cast<const float4*>(base + branch_elem + row_elem) + 2 * g + h);
-            lu[4 * h] = y.x, lu[4 * h + 1] = y.y, lu[4 * h + 2] = y.z, lu[4 * h + 3] = y.w;
-          }
-        }
-      }
-#pragma unroll
-      for (int e = 0; e < 8; ++e) {
-        float z = UNC ? __fmaf_rn(s, __fsub_rn(lc[e], lu[e]), lu[e]) : lc[e];
-        if (T != 1.0f) z = __fdiv_rn(z, T);
-        key[c * 8 + e] = topk_key(z);
-      }
-    } else {
-#pragma unroll
-      for (int e = 0; e < 8; ++e) key[c * 8 + e] = 0u;   // padding: below everything
-    }
-  }
-}
-
 // K-th largest of the block's keys, NE per thread (the key of -inf if fewer than K keys lie above -inf)
 template <int NE>
 __device__ __forceinline__ uint32_t topk_select_keys(const uint32_t (&key)[NE], int K, TopkShared& S) {
@@ -322,21 +269,16 @@ __device__ __forceinline__ float topk_select(const uint32_t (&key)[TK_CH * 8], i
 
 // raw row(s) of one job -> shared memory
 template <bool BF16, bool UNC>
-__device__ __forceinline__ void topk_issue(const VerifyParams& P, int item, bool drafter, unsigned char* stage,
+__device__ __forceinline__ void topk_issue(const VerifyParams& P, int item, unsigned char* stage,
                                            uint32_t rowbytes, unsigned long long* bar) {
   const size_t esize = BF16 ? 2 : 4;
   const size_t row = static_cast<size_t>(item) * P.V * esize;
   uint64_t* b = reinterpret_cast<uint64_t*>(bar);
-  if (drafter) {
-    mbar_expect_tx(b, rowbytes);
-    bulk_load(stage, static_cast<const unsigned char*>(P.draft) + row, rowbytes, b);
-  } else {
-    const unsigned char* base = static_cast<const unsigned char*>(P.target);
-    const size_t branch = static_cast<size_t>(P.B) * P.R * P.V * esize;
-    mbar_expect_tx(b, UNC ? 2 * rowbytes : rowbytes);
-    bulk_load(stage, base + row, rowbytes, b);
-    if (UNC) bulk_load(stage + rowbytes, base + branch + row, rowbytes, b);
-  }
+  const unsigned char* base = static_cast<const unsigned char*>(P.target);
+  const size_t branch = static_cast<size_t>(P.B) * P.R * P.V * esize;
+  mbar_expect_tx(b, UNC ? 2 * rowbytes : rowbytes);
+  bulk_load(stage, base + row, rowbytes, b);
+  if (UNC) bulk_load(stage + rowbytes, base + branch + row, rowbytes, b);
 }
 
 // staged raw row(s) -> keys of the processed logits
@@ -390,37 +332,30 @@ __device__ __forceinline__ void topk_keys_from_stage(const unsigned char* stage,
   }
 }
 
-// mode 0 (after the plan): per context with children, its target rows and -- in sampling -- its
-// drafter row, as separate jobs; mode 1 (after the walk): the target rows of the bonus draws.
+// Per context with children (after the plan), its target rows.
 template <bool BF16, bool UNC>
-__global__ void __launch_bounds__(TKT, 2) lantern_topk_kernel(VerifyParams P, int mode) {
+__global__ void __launch_bounds__(TKT, 2) lantern_topk_kernel(VerifyParams P) {
   extern __shared__ __align__(128) unsigned char tsm[];
   __shared__ TopkShared S;
   const int tid = threadIdx.x;
   const int V = P.V, R = P.R, K = P.top_k;
-  const float T = P.T == 0.0f ? 1.0f : P.T;   // greedy decoding works at temperature 1
+  const float T = 1.0f;   // greedy decoding works at temperature 1
   const uint32_t rowbytes = static_cast<uint32_t>(V) * (BF16 ? 2 : 4);
-  const bool sampling = P.T != 0.0f;
   const int n_heavy = P.counters->n_heavy;
   const int cap = P.B * P.N;
-  const int per = (mode == 0 && sampling) ? 2 : 1;
-  const long long njobs = mode == 0 ? static_cast<long long>(n_heavy + P.counters->n_light) * per : P.counters->n_bonus;
+  const long long njobs = static_cast<long long>(n_heavy) + P.counters->n_light;
   const long long G = gridDim.x;
   auto job_item = [&](long long j) -> int {
-    if (mode == 0) {
-      const int w = static_cast<int>(j / per);
-      return P.work[P.ctx_slots[w < n_heavy ? w : cap - 1 - (w - n_heavy)]].item;
-    }
-    return P.bonus_seq[j] * R + P.bonus_ctx[j];
+    const int w = static_cast<int>(j);
+    return P.work[P.ctx_slots[w < n_heavy ? w : cap - 1 - (w - n_heavy)]].item;
   };
-  auto job_is_drafter = [&](long long j) { return per == 2 && (j & 1); };
   uint64_t* bar = reinterpret_cast<uint64_t*>(&S.bar_full);
 
   long long j = blockIdx.x;
   if (tid == 0) {
     mbar_init(bar, 1);
     fence_mbar_init();
-    if (j < njobs) topk_issue<BF16, UNC>(P, job_item(j), job_is_drafter(j), tsm, rowbytes, &S.bar_full);
+    if (j < njobs) topk_issue<BF16, UNC>(P, job_item(j), tsm, rowbytes, &S.bar_full);
   }
   __syncthreads();
   if (j >= njobs) return;
@@ -429,22 +364,20 @@ __global__ void __launch_bounds__(TKT, 2) lantern_topk_kernel(VerifyParams P, in
   for (uint32_t it = 0; j < njobs; j += G, ++it) {
     const long long jn = j + G < njobs ? j + G : j;
     const int item_next = job_item(jn);   // consumed after the keys are out: no select on it before
-    const bool drafter = job_is_drafter(j);
     const bool landed = __syncthreads_and(mbar_wait(bar, it & 1, P.wait_tries) ? 1 : 0) != 0;
     if (!landed) {   // the copy did not complete within the wait limit: no filter for this row, reported
       if (tid == 0) {
-        (drafter ? P.thr_p : P.thr_q)[item] = __int_as_float(0xff800000);
-        if (mode == 0) atomicOr(&P.seq_status[item / R], LANTERN_ST_INTERNAL);
-        else if (P.out_status) atomicOr(&P.out_status[item / R], LANTERN_ST_INTERNAL);
+        P.thr_q[item] = __int_as_float(0xff800000);
+        atomicOr(&P.seq_status[item / R], LANTERN_ST_INTERNAL);
       }
       break;
     }
-    topk_keys_from_stage<BF16>(tsm, rowbytes, UNC && !drafter, V, P.cfg_scale, T, key);
+    topk_keys_from_stage<BF16>(tsm, rowbytes, UNC, V, P.cfg_scale, T, key);
     __syncthreads();   // the staging area is free
     if (tid == 0 && j + G < njobs)
-      topk_issue<BF16, UNC>(P, item_next, job_is_drafter(j + G), tsm, rowbytes, &S.bar_full);
+      topk_issue<BF16, UNC>(P, item_next, tsm, rowbytes, &S.bar_full);
     const float t = topk_select(key, K, V, S);
-    if (tid == 0) (drafter ? P.thr_p : P.thr_q)[item] = t;
+    if (tid == 0) P.thr_q[item] = t;
     item = item_next;
   }
 }
