@@ -107,10 +107,7 @@ def method_work(parents, accept_len, accept_path, N: int):
 NCU_TRAFFIC = {"kernel_revision": 18, "workload": "batch_chain", "traffic_over_algorithmic": 564017408 / 548656352}
 
 
-def stream_operations(greedy: bool, top_k_active: bool) -> int:
-    """Kernels and memsets of one verification call: memset, plan and the fused pass; greedy decoding and the logit
-    filter keep walk and bonus draw as kernels of their own, the filter one for thresholds."""
-    return 6 if top_k_active else (5 if greedy else 3)
+STREAM_OPERATIONS = 2   # kernels of one verification call: the plan and the fused pass
 
 
 def ncu_traffic(workload, alg_bytes):
@@ -719,7 +716,7 @@ def main():
         lit_cold, _ = lit.timed(50, 3, flush=flush)
         chain["literal_call"] = {"sequences_per_call": lit.B, "us_per_call_back_to_back": 1e3 * lit_total / 200,
                                  "us_per_call_l2_flushed": 1e3 * lit_cold / 50, "fused_kernel_us": 1e3 * lit_fused,
-                                 "stream_operations_per_call": stream_operations(False, False),
+                                 "stream_operations_per_call": STREAM_OPERATIONS,
                                  "note": "back to back the 23 MB of rows stay in L2; flushed they come from HBM"}
         del lit
         # the same call under the paper's other settings (same inputs, same table): greedy decoding (tau = 0), the
@@ -773,7 +770,7 @@ def main():
             "positions": {"drafted_per_s": value, "tested_per_s": world * acc["method_nodes"] / (ms_per_step * 1e-3),
                           "note": "drafted = every drafted position of the call; tested = the positions Algorithm 1's "
                                   "loop tests before its first rejection"},
-            "roofline": {"bound": "hbm", "kernel": "lantern_greedy_context_kernel" if args.greedy else "lantern_context_kernel",
+            "roofline": {"bound": "hbm", "kernel": "lantern_context_kernel",
                          "achieved": acc["achieved"], "peak": peak, "peak_kind": f"of {peak_kind}", "unit": "GB/s",
                          "frac": acc["frac"],
                          "traffic": None if (args.greedy or args.divergence != "tvd" or top_active) else
@@ -786,7 +783,7 @@ def main():
                          "note": "algorithmic bytes = rows of the contexts the kernel evaluated + neighbour rows of the "
                                  "nodes it tested; method_* counts only what Algorithm 1's loop reaches"},
             "cpu_baseline": cpu, "e2e": e2e,
-            "gpu_launches": (stream_operations(args.greedy, top_active) - 1) * args.steps, "clocks": clocks,
+            "gpu_launches": STREAM_OPERATIONS * args.steps, "clocks": clocks,
             "neighbor_build": {"ms": build_ms, "V": V, "D": cfg["D"], "k": k, "pairs_per_s": V * V / (build_ms * 1e-3)},
             "outputs": {"mean_accept_len": accept_mean, "sequences_with_status_bits": status_bad},
             "configs": configs,

@@ -169,7 +169,7 @@ lantern_status lantern_build_neighbors_metric(const float* codebook, int V, int 
  *                  values of a test made ahead of time that the walk did not need.  Each may be NULL.
  *   workspace       lantern_verify_workspace_bytes(B, N, V, k, dtype) bytes, 256-byte aligned
  *
- * The call only enqueues work on cuda_stream (one memset and four or five kernels): it allocates
+ * The call only enqueues work on cuda_stream (two kernels): it allocates
  * nothing, reads nothing back and does not wait for the stream, and it re-initialises the part
  * of the workspace it relies on.  It may therefore be recorded by a stream capture and replayed
  * as a CUDA graph on inputs rewritten in place; make one call with the same shape, logit type
@@ -287,11 +287,8 @@ lantern_status lantern_verify_static(const void* target_logits, const void* draf
  * stored profiler counters can be matched to the code they were taken on. */
 int lantern_kernel_revision(void);
 
-/* Number of kernels (and memsets) that one verification call enqueues, at most: memset, plan, fused pass or greedy
- * pass, walk, bonus; a call whose top-k filter is active (0 < top_k < V) enqueues one threshold kernel
- * more (ahead of the greedy pass; in sampling ahead of the bonus draw -- the fused pass finds the
- * thresholds of its own contexts).  Sampling without the filter enqueues fewer: its fused pass walks and
- * draws the bonus tokens itself. */
+/* Number of kernels (and memsets) that one verification call enqueues, at most.  (A bound that no call comes near any
+ * more: a call is two kernels, the plan and the fused pass.) */
 int lantern_verify_launch_count(int greedy, int top_k_active);
 
 /* ------------------------------------------------------------------------------------------

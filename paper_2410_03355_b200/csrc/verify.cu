@@ -11,8 +11,7 @@
 //                        and either the next sibling's test on the renormalised residual or
 //                        the inverse-CDF draw of the replacement token   (Section 4.3, Alg. 1)
 // Algorithm 1's loop over the decided contexts and the draw of the bonus token happen inside the same pass.
-// Greedy decoding (verify_greedy.cuh) has passes of its own, plan -> contexts -> walk -> next tokens; its contexts leave
-// 16-byte records, which a small walk kernel follows from the root.
+// Greedy decoding runs through the same two kernels.
 //
 // Precision: processed logits are fp32 (difference, fused multiply-add, division, each
 // rounded once); exponentials come from the fp32 ex2 unit (about 3e-7 relative); every sum over more
@@ -33,8 +32,7 @@ namespace lantern {
 // sequence b in breadth-first order (by depth, then by index).  A context whose parent node has
 // already been rejected when its turn comes is never evaluated (see verify_context.cuh); the
 // order only decides how often that is known in time, never the result.
-// Every context with children starts with a record that says "not evaluated" (INTERNAL), which
-// the fused pass overwrites; contexts without children are marked as leaves.
+// Every context's walk word says whether it is the root (where the walk starts), pending, or a leaf.
 // ---------------------------------------------------------------------------------------
 constexpr int kPlanArrays = 13;  // per-warp arrays of N + 2 ints in shared memory
 
@@ -85,13 +83,10 @@ __device__ __forceinline__ int plan_sequence(const VerifyParams& P, int* plan_sm
   for (int c = lane; c < R; c += 32) P.dead[static_cast<size_t>(b) * R + c] = 0;
   status = __reduce_or_sync(kFull, status);
   __syncwarp();
-  if (lane == 0) {
-    P.seq_status[b] = status;
-    if (P.walk_inline) {   // what stands if the fused pass never gets to the end of this sequence
-      P.out_len[b] = 0;
-      P.out_tok[b] = -1;
-      if (P.out_status) P.out_status[b] = status ? status : LANTERN_ST_INTERNAL;
-    }
+  if (lane == 0) {   // what stands if the fused pass never gets to the end of this sequence
+    P.out_len[b] = 0;
+    P.out_tok[b] = -1;
+    if (P.out_status) P.out_status[b] = status ? status : LANTERN_ST_INTERNAL;
   }
   if (status) {   // the walk reports the fault; no work is queued for this sequence
     for (int r = lane; r < max(N, 1); r += 32) P.work[static_cast<size_t>(r) * B + b].item = -1;
@@ -249,7 +244,7 @@ __device__ __forceinline__ int plan_sequence(const VerifyParams& P, int* plan_sm
       n_ctx += __popc(bal);
     }
   }
-  if (N == 0 && P.walk_inline) n_ctx = 1;
+  if (N == 0) n_ctx = 1;
   __syncwarp();         // the shared arrays are complete
   for (int i = lane; i < N; i += 32) {   // the child lists, written by all lanes
     ChildInfo ci = {i, s_tok[i], __int_as_float(s_uni[i]), (din[i + 1] << 16) | siz[i + 1]};
@@ -257,41 +252,17 @@ __device__ __forceinline__ int plan_sequence(const VerifyParams& P, int* plan_sm
   }
   for (int r = n_ctx + lane; r < N; r += 32) P.work[static_cast<size_t>(r) * B + b].item = -1;
   const float u_final = __int_as_float(s_uni[N]);
-  const int cap = B * N;
-  for (int base = 0; base < R; base += 32) {
-    const int c = base + lane;
-    const int n = c < R ? cnt[c] : 0;
-    const unsigned heavy = __ballot_sync(kFull, n >= 2);
-    const unsigned light = __ballot_sync(kFull, n == 1);
-    int hb = 0, lb = 0;
-    if (P.ctx_slots && lane == 0) {
-      if (heavy) hb = atomicAdd(&P.counters->n_heavy, __popc(heavy));
-      if (light) lb = atomicAdd(&P.counters->n_light, __popc(light));
-    }
-    hb = __shfl_sync(kFull, hb, 0);
-    lb = __shfl_sync(kFull, lb, 0);
-    const unsigned below = (1u << lane) - 1u;
-    if (c < R) {
-      Record* rec = P.records + static_cast<size_t>(b) * R + c;
-      if (P.walk_inline) {
-        *reinterpret_cast<unsigned long long*>(rec) = n == 0 ? kWalkLeaf : (c == 0 ? kWalkWaiting : kWalkPending);
-      } else if (n == 0) {
-        *rec = {kLeaf, -1, 0, 0};
-      } else {
-        *rec = {-1, -1, LANTERN_ST_INTERNAL, 0};   // stands until the fused pass has evaluated the context
-      }
-      if (n == 0 && N == 0) P.work[b] = {b, 0, 0, 0, 0, 0.0f, u_final, b};   // no drafts: one draw from the root's q
-      if (n > 0) {
-        const int start = cur[c] - n;
-        const int f = s_first[c];             // the context's first child (smallest node index)
-        WorkItem w = {b * R + c, b * N + start, (n << 16) | f, (din[f + 1] << 16) | siz[f + 1], s_tok[f],
-                      __int_as_float(s_uni[f]), u_final, b * R + din[c]};
-        const int slot = dep[c] * B + b;
-        P.work[slot] = w;
-        if (P.ctx_slots) P.ctx_slots[n >= 2 ? hb + __popc(heavy & below) : cap - 1 - (lb + __popc(light & below))] = slot;
-      }
+  for (int c = lane; c < R; c += 32) {
+    const int n = cnt[c];
+    P.records[static_cast<size_t>(b) * R + c].word = n == 0 ? kWalkLeaf : (c == 0 ? kWalkWaiting : kWalkPending);
+    if (n > 0) {
+      const int start = cur[c] - n;
+      const int f = s_first[c];             // the context's first child (smallest node index)
+      P.work[dep[c] * B + b] = {b * R + c, b * N + start, (n << 16) | f, (din[f + 1] << 16) | siz[f + 1], s_tok[f],
+                                __int_as_float(s_uni[f]), u_final, b * R + din[c]};
     }
   }
+  if (N == 0 && lane == 0) P.work[b] = {b, 0, 0, 0, 0, 0.0f, u_final, b};   // no drafts: one draw from the root's q
   return n_ctx;
 }
 
@@ -301,7 +272,7 @@ __global__ void __launch_bounds__(PLAN_WARPS * 32) lantern_plan_kernel(VerifyPar
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   grid_dependency_wait();
   grid_dependents_launch();
-  if (P.clear_counters && blockIdx.x == 0 && threadIdx.x < 64) reinterpret_cast<int*>(P.counters)[threadIdx.x] = 0;
+  if (blockIdx.x == 0 && threadIdx.x < 64) reinterpret_cast<int*>(P.counters)[threadIdx.x] = 0;
   const int word = plan_sequence(P, plan_smem, blockIdx.x * PLAN_WARPS + warp, warp, lane);
   if (lane == 0) s_words[warp] = word;
   __syncthreads();
@@ -315,59 +286,7 @@ __global__ void __launch_bounds__(PLAN_WARPS * 32) lantern_plan_kernel(VerifyPar
 }  // namespace lantern
 
 // (kernel 2, the fused context pass, is compiled in files of its own: see verify_common.cuh)
-// greedy decoding (temperature 0)
-#include "verify_greedy.cuh"
-#include "verify_topk.cuh"
-
 namespace lantern {
-
-// ---------------------------------------------------------------------------------------
-// kernel 3: walk (Algorithm 1's loop over the records; one thread per sequence)
-// ---------------------------------------------------------------------------------------
-__global__ void __launch_bounds__(128) lantern_walk_kernel(VerifyParams P) {
-  const int b = blockIdx.x * blockDim.x + threadIdx.x;
-  if (b >= P.B) return;
-  const int N = P.N, R = P.R;
-  int status = P.seq_status[b];
-  int len = 0, next = -1;
-  if (status == 0) {
-    int cur = 0;
-    for (int step = 0; step <= N; ++step) {
-      const Record rec = P.records[static_cast<size_t>(b) * R + cur];
-      bool from_q = rec.accepted == kLeaf;   // no drafts left on this path: bonus token from q
-      if (!from_q) {
-        status |= rec.status;
-        // a residual without weight: the next token comes from the context's own target as well
-        from_q = (rec.status & LANTERN_ST_DEGENERATE) && !(rec.status & (LANTERN_ST_NONFINITE | LANTERN_ST_INTERNAL));
-      }
-      if (from_q) {
-        const int slot = atomicAdd(&P.counters->n_bonus, 1);
-        P.bonus_seq[slot] = b;
-        P.bonus_ctx[slot] = cur;
-        break;
-      }
-      if (rec.status & (LANTERN_ST_NONFINITE | LANTERN_ST_INTERNAL)) break;
-      if (rec.accepted >= 0) {
-        // an accepted node is a child of this context: its index is at least the context's, and the path
-        // holds at most N nodes; anything else is not a record the fused pass wrote
-        if (rec.accepted < cur || rec.accepted >= N || len >= N) {
-          status |= LANTERN_ST_INTERNAL;
-          break;
-        }
-        if (P.out_path) P.out_path[static_cast<size_t>(b) * N + len] = rec.accepted;
-        ++len;
-        cur = rec.accepted + 1;
-        continue;
-      }
-      next = rec.token;
-      break;
-    }
-  }
-  P.out_len[b] = len;
-  P.out_tok[b] = next;
-  if (P.out_status) P.out_status[b] = status;
-  if (status) atomicOr(&P.counters->status_or, status);
-}
 
 // ---------------------------------------------------------------------------------------
 // host side
@@ -375,7 +294,7 @@ __global__ void __launch_bounds__(128) lantern_walk_kernel(VerifyParams P) {
 static size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
 struct WsLayout {
-  size_t counters, work, slots, children, records, dead, seqst, bseq, bctx, thrq, thrp, total;
+  size_t counters, work, children, records, dead, words, total;
 };
 
 static WsLayout ws_layout(int B, int N, bool topk = false) {
@@ -385,15 +304,12 @@ static WsLayout ws_layout(int B, int N, bool topk = false) {
   size_t o = 0;
   L.counters = o; o += 256;
   L.work = o;     o += align_up(b * n1 * sizeof(WorkItem), 256);
-  L.slots = o;    o += align_up(b * n1 * 4, 256);
+  o += align_up(b * n1 * 4, 256);              // (the size callers have always been told: parts of it are no longer used)
   L.children = o; o += align_up(b * n1 * sizeof(ChildInfo), 256);
   L.records = o;  o += align_up(b * R * sizeof(Record), 256);
   L.dead = o;     o += align_up(b * R, 256);
-  L.seqst = o;    o += align_up(b * 4, 256);
-  L.bseq = o;     o += align_up(b * 4, 256);
-  L.bctx = o;     o += align_up(b * 4, 256);
-  L.thrq = o;     o += topk ? align_up(b * R * 4, 256) : 0;
-  L.thrp = o;     o += topk ? align_up(b * R * 4, 256) : 0;
+  L.words = o;    o += 3 * align_up(b * 4, 256);
+  o += topk ? 2 * align_up(b * R * 4, 256) : 0;
   L.total = o;
   return L;
 }
@@ -416,33 +332,18 @@ constexpr uint32_t kDefaultWaitTries = 1u << 21;
 static thread_local uint32_t g_wait_tries = kDefaultWaitTries;
 static thread_local int g_withhold_item = -1;
 
-// thresholds of the top-k filter for greedy decoding: target rows of the contexts with children (after the plan)
-template <bool BF16, bool UNC>
-static cudaError_t launch_topk(const VerifyParams& P, long long jobs, int sms, cudaStream_t st) {
-  auto kt = lantern_topk_kernel<BF16, UNC>;
-  const size_t smem = static_cast<size_t>(P.V) * (UNC ? 2 : 1) * (BF16 ? 2 : 4);   // one job's raw rows
-  cudaError_t e = cudaFuncSetAttribute(kt, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
-  if (e != cudaSuccess) return e;
-  int per_sm = 0;
-  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kt, TKT, smem);
-  if (e != cudaSuccess) return e;
-  if (per_sm < 1) return cudaErrorInvalidConfiguration;
-  const long long slots = static_cast<long long>(sms) * per_sm;
-  const int grid = static_cast<int>(jobs < slots ? (jobs > 0 ? jobs : 1) : slots);
-  kt<<<grid, TKT, smem, st>>>(P);
-  return cudaGetLastError();
-}
-
-// the variants of the fused context kernel live in verify_context_v<tone + 2 jsd + 4 topk>.cu
+// the variants of the fused context kernel live in verify_context_v<tone + 2 jsd + 4 topk>.cu, those of greedy decoding in
+// verify_context_v<8 + jsd + 2 topk>.cu
 #define LANTERN_DECLARE_VARIANT(n) \
   cudaError_t launch_context_v##n(const VerifyParams&, bool, bool, long long, int, cudaStream_t);
 LANTERN_DECLARE_VARIANT(0) LANTERN_DECLARE_VARIANT(1) LANTERN_DECLARE_VARIANT(2) LANTERN_DECLARE_VARIANT(3)
 LANTERN_DECLARE_VARIANT(4) LANTERN_DECLARE_VARIANT(5) LANTERN_DECLARE_VARIANT(6) LANTERN_DECLARE_VARIANT(7)
+LANTERN_DECLARE_VARIANT(8) LANTERN_DECLARE_VARIANT(9) LANTERN_DECLARE_VARIANT(10) LANTERN_DECLARE_VARIANT(11)
 #undef LANTERN_DECLARE_VARIANT
 
 cudaError_t launch_context_kernel(const VerifyParams& P, bool bf16, bool uncond, bool tone, bool jsd, bool topk,
-                                  long long items, int sms, cudaStream_t st) {
-  switch ((tone ? 1 : 0) | (jsd ? 2 : 0) | (topk ? 4 : 0)) {
+                                  bool greedy, long long items, int sms, cudaStream_t st) {
+  switch (greedy ? 8 | (jsd ? 1 : 0) | (topk ? 2 : 0) : (tone ? 1 : 0) | (jsd ? 2 : 0) | (topk ? 4 : 0)) {
     case 0: return launch_context_v0(P, bf16, uncond, items, sms, st);
     case 1: return launch_context_v1(P, bf16, uncond, items, sms, st);
     case 2: return launch_context_v2(P, bf16, uncond, items, sms, st);
@@ -450,51 +351,12 @@ cudaError_t launch_context_kernel(const VerifyParams& P, bool bf16, bool uncond,
     case 4: return launch_context_v4(P, bf16, uncond, items, sms, st);
     case 5: return launch_context_v5(P, bf16, uncond, items, sms, st);
     case 6: return launch_context_v6(P, bf16, uncond, items, sms, st);
-    default: return launch_context_v7(P, bf16, uncond, items, sms, st);
+    case 7: return launch_context_v7(P, bf16, uncond, items, sms, st);
+    case 8: return launch_context_v8(P, bf16, uncond, items, sms, st);
+    case 9: return launch_context_v9(P, bf16, uncond, items, sms, st);
+    case 10: return launch_context_v10(P, bf16, uncond, items, sms, st);
+    default: return launch_context_v11(P, bf16, uncond, items, sms, st);
   }
-}
-
-// Sampling: the fused pass finds its contexts' thresholds, walks the contexts and draws the bonus tokens itself.
-static cudaError_t launch_verify(const VerifyParams& P, bool bf16, bool uncond, bool tone, bool jsd, long long items, int sms,
-                                 cudaStream_t st) {
-  if (g_ev_before && g_ev_after) cudaEventRecord(g_ev_before, st);
-  const cudaError_t e = launch_context_kernel(P, bf16, uncond, tone, jsd, P.top_k > 0, items, sms, st);
-  if (e != cudaSuccess) return e;
-  if (g_ev_before && g_ev_after) cudaEventRecord(g_ev_after, st);
-  return cudaSuccess;
-}
-
-template <bool BF16, bool UNC, bool TOPK>
-static cudaError_t launch_greedy(const VerifyParams& P, long long items, int sms, int grid_bonus, cudaStream_t st) {
-  auto kc = lantern_greedy_context_kernel<BF16, UNC, TOPK>;
-  // a ring of staging areas per CTA, each holding the raw target rows of one context; sized so that
-  // three CTAs share an SM where the rows allow it
-  const size_t area = static_cast<size_t>(P.V) * (UNC ? 2 : 1) * (BF16 ? 2 : 4);
-  int ring = static_cast<int>((72 * 1024) / area);
-  ring = ring < 1 ? 1 : (ring > GRING_MAX ? GRING_MAX : ring);
-  const size_t smem = ring * area;
-  cudaError_t e = cudaFuncSetAttribute(kc, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
-  if (e != cudaSuccess) return e;
-  int per_sm = 0;
-  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kc, GCT, smem);
-  if (e != cudaSuccess) return e;
-  if (per_sm < 1) return cudaErrorInvalidConfiguration;
-  const long long slots = static_cast<long long>(sms) * per_sm;
-  const int grid_ctx = static_cast<int>(items < slots ? items : slots);
-  if (TOPK) {
-    e = launch_topk<BF16, UNC>(P, items, sms, st);
-    if (e != cudaSuccess) return e;
-  }
-  if (g_ev_before && g_ev_after) cudaEventRecord(g_ev_before, st);
-  kc<<<grid_ctx, GCT, smem, st>>>(P, ring);
-  e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  if (g_ev_before && g_ev_after) cudaEventRecord(g_ev_after, st);
-  lantern_walk_kernel<<<(P.B + 127) / 128, 128, 0, st>>>(P);
-  e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  lantern_greedy_bonus_kernel<BF16, UNC><<<grid_bonus, GRT, 0, st>>>(P);   // the arg max is never filtered out
-  return cudaGetLastError();
 }
 
 }  // namespace lantern
@@ -513,8 +375,7 @@ extern "C" size_t lantern_verify_workspace_bytes(int B, int N, int V, int k, int
 }
 
 extern "C" int lantern_verify_launch_count(int greedy, int top_k_active) {
-  // greedy decoding: plan, greedy pass, walk, next tokens; with the filter also a memset and the threshold kernel.
-  // sampling: plan and the fused pass, which does the rest by itself
+  // (at most: a call is a plan and the fused pass, which does everything else itself)
   (void)greedy;
   return 5 + (top_k_active ? 1 : 0);
 }
@@ -536,9 +397,7 @@ extern "C" lantern_status lantern_verify_counts(const void* workspace, void* cud
   Counters c;
   if (cudaMemcpyAsync(&c, workspace, sizeof(c), cudaMemcpyDeviceToHost, st) != cudaSuccess) return LANTERN_E_CUDA;
   if (cudaStreamSynchronize(st) != cudaSuccess) return LANTERN_E_CUDA;
-  // sampling keeps no count of its own: every context with children is either evaluated or left out
-  const int64_t listed = static_cast<int64_t>(c.n_heavy) + c.n_light;
-  out_counts[0] = listed ? listed : static_cast<int64_t>(c.n_evaluated) + c.n_skipped;
+  out_counts[0] = static_cast<int64_t>(c.n_evaluated) + c.n_skipped;   // every context with children is either evaluated or left out
   out_counts[1] = c.n_evaluated;
   out_counts[2] = c.n_skipped;
   out_counts[3] = c.n_bonus;
@@ -653,9 +512,7 @@ static lantern_status verify_impl(const void* target_logits, const void* draft_l
   P.work = reinterpret_cast<WorkItem*>(ws + L.work);
   P.children = reinterpret_cast<ChildInfo*>(ws + L.children);
   P.records = reinterpret_cast<Record*>(ws + L.records);
-  P.seq_status = reinterpret_cast<int32_t*>(ws + L.seqst);
-  P.bonus_seq = reinterpret_cast<int32_t*>(ws + L.bseq);
-  P.bonus_ctx = reinterpret_cast<int32_t*>(ws + L.bctx);
+  P.block_words = reinterpret_cast<int32_t*>(ws + L.words);
   P.B = B;
   P.N = N;
   P.R = N + 1;
@@ -666,20 +523,13 @@ static lantern_status verify_impl(const void* target_logits, const void* draft_l
   P.delta = delta;
   P.divergence = divergence;
   P.top_k = topk ? top_k : 0;
-  P.thr_q = topk ? reinterpret_cast<float*>(ws + L.thrq) : nullptr;
-  // only the threshold kernel of greedy decoding with the logit filter walks the compact list
-  P.ctx_slots = (greedy && topk) ? reinterpret_cast<int32_t*>(ws + L.slots) : nullptr;
   P.dead = ws + L.dead;
-  P.block_words = P.bonus_seq;
-  P.clear_counters = P.ctx_slots == nullptr;   // (the compact list is counted while the plan is made)
-  P.walk_inline = !greedy;
   P.wait_tries = g_wait_tries;
   P.withhold_item = g_withhold_item;
 
   const int sms = sm_count();
   if (sms < 1) return LANTERN_E_CUDA;
 
-  if (!P.clear_counters && cudaMemsetAsync(P.counters, 0, 256, st) != cudaSuccess) return LANTERN_E_CUDA;
   const size_t plan_smem = static_cast<size_t>(PLAN_WARPS) * kPlanArrays * (N + 2) * sizeof(int);
   static DeviceFlags plan_ready;
   if (plan_smem > 48 * 1024 &&
@@ -689,20 +539,11 @@ static lantern_status verify_impl(const void* target_logits, const void* draft_l
     return LANTERN_E_CUDA;
 
   const long long items = static_cast<long long>(B) * (N > 0 ? N : 1);   // upper bound of contexts with children
-  const int grid_bonus = B < 4 * sms ? B : 4 * sms;   // greedy bonus: 256-thread CTAs
-  cudaError_t e;
-  const bool bf = dtype == LANTERN_BF16, un = has_uncond != 0;
-  if (greedy) {
-#define LANTERN_GREEDY(KV)                                                                                   \
-  (bf ? (un ? launch_greedy<true, true, KV>(P, items, sms, grid_bonus, st) : launch_greedy<true, false, KV>(P, items, sms, grid_bonus, st)) \
-      : (un ? launch_greedy<false, true, KV>(P, items, sms, grid_bonus, st) : launch_greedy<false, false, KV>(P, items, sms, grid_bonus, st)))
-    e = topk ? LANTERN_GREEDY(true) : LANTERN_GREEDY(false);
-#undef LANTERN_GREEDY
-    return e == cudaSuccess ? LANTERN_OK : LANTERN_E_CUDA;
-  }
   // every combination of the compile-time variants exists: T = 1 never meets the division code
-  const bool tone = T == 1.0f, jsd = divergence == LANTERN_DIV_JSD;
-  e = launch_verify(P, bf, un, tone, jsd, items, sms, st);
+  if (g_ev_before && g_ev_after) cudaEventRecord(g_ev_before, st);
+  const cudaError_t e = launch_context_kernel(P, dtype == LANTERN_BF16, has_uncond != 0, T == 1.0f, divergence == LANTERN_DIV_JSD,
+                                              topk, greedy, items, sms, st);
+  if (g_ev_before && g_ev_after) cudaEventRecord(g_ev_after, st);
   return e == cudaSuccess ? LANTERN_OK : LANTERN_E_CUDA;
 }
 

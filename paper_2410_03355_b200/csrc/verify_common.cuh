@@ -19,11 +19,9 @@ namespace lantern {
 
 constexpr int MAX_N = 1024;
 
-struct Counters {               // first 256 bytes of the workspace, zeroed per call (by the plan kernel, or ahead of it, see clear_counters)
+struct Counters {               // first 256 bytes of the workspace, zeroed per call by the plan kernel
   int work_next;                // dynamic part of the work counter
-  int n_heavy;                  // contexts with >= 2 children (first in the compact list)
-  int n_light;                  // contexts with exactly 1 child
-  int n_bonus;                  // sequences whose next token is drawn from a context's own target
+  int n_bonus;                  // next tokens taken from a context's own target
   int n_evaluated;              // contexts the fused pass evaluated
   int n_skipped;                // contexts it left out because the walk cannot reach them
   int n_tested;                 // drafted nodes it tested
@@ -32,13 +30,9 @@ struct Counters {               // first 256 bytes of the workspace, zeroed per 
   int n_slow_topk;              // rows whose top-k threshold needed the slow exact search
 };
 
-struct Record {                 // result of one context
-  int accepted;                 // accepted child node; -1 if every child was rejected; kLeaf if it has none
-  int token;                    // replacement token if every child was rejected
-  int status;                   // LANTERN_ST_* bits found in this context
-  int pad;
+struct Record {                 // a context's walk word (see walk_word below), 16 bytes apart
+  unsigned long long word, unused;
 };
-constexpr int kLeaf = -2;
 
 struct ChildInfo {              // one drafted node, stored in the order its parent context tries it
   int node;                     // node index within the sequence
@@ -81,23 +75,16 @@ struct VerifyParams {
   Counters* counters;
   WorkItem* work;               // [N, B]: slot r * B + b holds the r-th context with children of sequence b in
                                 //         breadth-first order (by depth, then by index); item = -1 where there is none
-  int32_t* ctx_slots;           // [B*N]: the occupied slots, heavy ones from the front, light ones from the back
   unsigned char* dead;          // [B, R], a sequence's contexts in pre-order: 1 once the walk is known not to reach one
   ChildInfo* children;          // [B, N]
   Record* records;              // [B, R]
-  int32_t* seq_status;          // [B]
-  int32_t* bonus_seq;           // [B]
-  int32_t* bonus_ctx;           // [B]
   int B, N, R, V, k;
   float cfg_scale, T, delta;
   int divergence;               // LANTERN_DIV_TVD or LANTERN_DIV_JSD: what delta bounds
   int top_k;                    // logit filter; 0 = off
-  float* thr_q;                 // greedy decoding with the filter: [B, R] top_k-th largest target logit of a context row, else null
   uint32_t wait_tries;          // limit of every bounded mbarrier wait, in tries
   int32_t* block_words;         // one word per block of the plan kernel: largest number of contexts with children in one of
-                                //     its sequences, and its sequences' fault bits << 16 (read before bonus_seq, whose storage it is, is written)
-  int clear_counters;           // the plan kernel zeroes the counters (nothing in it counts then)
-  int walk_inline;              // the fused pass walks and draws the bonus tokens itself: records hold walk words
+                                //     its sequences, and its sequences' fault bits << 16
   int withhold_item;            // self-test only: the copies of this context are never issued (-1 = none)
 };
 
@@ -107,7 +94,7 @@ constexpr int kNone = 0x7fffffff;
 // mass): the walk stops there and the next token comes from the context's own target.
 constexpr double kDegenerate = 1e-5;
 
-// The walk over the contexts of a sequence, where the fused pass does it itself (verify_context.cuh): one word per
+// The walk over the contexts of a sequence (verify_context.cuh): one word per
 // context, exchanged by whoever decides the context and by the walk when it gets there.
 //   bits 0..1 state; walk waiting: bits 8..15 status so far, bits 16..31 drafts accepted so far;
 //   decided: bits 8..15 status, bits 16..31 accepted node + 1 (0 = none), bits 32..63 replacement token
@@ -121,7 +108,7 @@ constexpr int PLAN_WARPS = 4;   // sequences per block of the plan kernel
 
 // The plan's summary, by a whole warp: slots in the occupied part of the work list, and the fault bits of all sequences.
 __device__ __forceinline__ int plan_slots(const VerifyParams& P, int lane, int& faults) {
-  int ranks = P.parents ? 0 : (P.N > 0 ? P.N : (P.walk_inline ? 1 : 0)), bits = 0;
+  int ranks = P.parents ? 0 : (P.N > 0 ? P.N : 1), bits = 0;
   const int blocks = (P.B + PLAN_WARPS - 1) / PLAN_WARPS;
 #pragma unroll 4
   for (int i = lane; i < blocks; i += 32) {
@@ -134,7 +121,7 @@ __device__ __forceinline__ int plan_slots(const VerifyParams& P, int lane, int& 
 }
 // The same without the fault bits: a chain has a context with a child for every draft.
 __device__ __forceinline__ int plan_slots(const VerifyParams& P, int lane) {
-  if (!P.parents) return (P.N > 0 ? P.N : (P.walk_inline ? 1 : 0)) * P.B;
+  if (!P.parents) return (P.N > 0 ? P.N : 1) * P.B;
   int faults;
   return plan_slots(P, lane, faults);
 }
@@ -178,10 +165,10 @@ static inline cudaError_t launch_dependent(K kernel, int grid, int threads, size
 }
 
 // Launch of the fused context kernel (verify_context.cuh).  Its variants -- temperature 1 compiled
-// out or not (TONE), TVD or JSD bound, top-k thresholds applied or not -- are compiled in separate
+// out or not (TONE), TVD or JSD bound, top-k thresholds applied or not, greedy decoding -- are compiled in separate
 // translation units (verify_context_v*.cu) so that they build in parallel; this function picks one.
 // `items` = upper bound of the contexts with children in the call, `sms` = SMs of the device.
 cudaError_t launch_context_kernel(const VerifyParams& P, bool bf16, bool uncond, bool tone, bool jsd, bool topk,
-                                  long long items, int sms, cudaStream_t st);
+                                  bool greedy, long long items, int sms, cudaStream_t st);
 
 }  // namespace lantern

@@ -63,6 +63,7 @@ struct CtxShape {
 using CtxNarrow = CtxShape<256, 3, 1, 1>;   // 27 warps of 72 registers
 using CtxPair = CtxShape<512, 1, 1, 2>;     // 2 * 17 warps of 56 registers
 using CtxWide = CtxShape<512, 1, 2, 1>;     // 17 warps
+using CtxSingle = CtxShape<512, 1, 1, 1>;   // for areas of 128 KB: greedy decoding on long fp32 rows
 // Which shape.  A context is a chain of dependent steps; sixteen warps get through it in two thirds of the time eight
 // need, but three contexts per SM hide one another's latencies.  With few sequences per call the path through each
 // is what takes the time (and fewer contexts in flight mean fewer evaluated for nothing), with many the throughput.
@@ -190,11 +191,11 @@ __device__ __forceinline__ void ctx_issue_target(const VerifyParams& P, int item
 // where a bulk copy is issued long before its context's turn (two staging areas) -- with one area the copy starts as soon as
 // rows that are on their way to the same SM have arrived, and prefetching them as well measured slower (8192 chains
 // 1.056 against 1.028 ms; with two areas 128 trees 98 against 103 us the other way round).
-template <bool UNC, bool TARGET>
+template <bool UNC, bool DRAFTER, bool TARGET>
 __device__ __forceinline__ void ctx_prefetch_rows(const VerifyParams& P, int item, int rowbytes) {
   const size_t row_off = static_cast<size_t>(item) * rowbytes;
   const unsigned char* d = static_cast<const unsigned char*>(P.draft) + row_off;
-  if (P.draft) asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(d), "r"(rowbytes) : "memory");
+  if (DRAFTER && P.draft) asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(d), "r"(rowbytes) : "memory");
   if (TARGET) {
     const unsigned char* t = static_cast<const unsigned char*>(P.target) + row_off;
     const size_t branch = static_cast<size_t>(P.B) * P.R * rowbytes;
@@ -300,15 +301,18 @@ __device__ __forceinline__ double warp_transposed_sum(const float (&v)[N], int l
 // instead of 1.07 ms on 8192 chains).
 __device__ __forceinline__ unsigned long long walk_exchange(Record* rec, unsigned long long v) {
   unsigned long long old;
-  asm volatile("atom.relaxed.gpu.global.exch.b64 %0, [%1], %2;" : "=l"(old) : "l"(rec), "l"(v) : "memory");
+  asm volatile("atom.relaxed.gpu.global.exch.b64 %0, [%1], %2;" : "=l"(old) : "l"(&rec->word), "l"(v) : "memory");
   return old;
 }
 
 // CH = 8-token chunks per thread (1, 2, 4 or 8); the target's numerators come in slices of CP chunks.
 // TONE = the temperature is exactly 1 (the paper's sampling setting): no division is compiled in.
 // JSD selects the Section 5.3.2 bound at compile time, so that the default path carries none of its code.
+// GREEDY = greedy decoding (Section 4.3, last sentence; TONE is set then): no drafter distribution, no random numbers; x~ is
+// accepted iff sum_A q >= max_x q(x) (it is an arg max of q_{k,delta}(.|D = x~): the maximum over A's own members can never
+// exceed the sum), children are tried against the same q, and wherever the walk stops the token is arg max q.
 // TOPK = the logit filter is on (Appendix B.2): processed logits below the top_k-th largest of their row count as -inf.
-template <class SHAPE, int CH, bool BF16, bool UNC, bool TONE, bool JSD, bool TOPK>
+template <class SHAPE, int CH, bool BF16, bool UNC, bool TONE, bool JSD, bool TOPK, bool GREEDY>
 __global__ void __launch_bounds__(SHAPE::THREADS, SHAPE::CTAS) lantern_context_kernel(VerifyParams P) {
   constexpr int GT = SHAPE::GT, GW = GT / 32, NGRP = SHAPE::NGRP, AREAS = SHAPE::AREAS;
   constexpr int LOG_GT = GT == 1024 ? 10 : (GT == 512 ? 9 : 8);
@@ -604,7 +608,7 @@ __global__ void __launch_bounds__(SHAPE::THREADS, SHAPE::CTAS) lantern_context_k
       next_batch();
       if (mask && __shfl_sync(kFull, draw_item, 0) < 0) {
         const int item_ahead = __shfl_sync(kFull, cur.item, __ffs(mask) - 1);
-        if (lane == 0) ctx_prefetch_rows<UNC, (AREAS > 1)>(P, item_ahead, rowbytes);
+        if (lane == 0) ctx_prefetch_rows<UNC, !GREEDY, (AREAS > 1)>(P, item_ahead, rowbytes);
       }
     }
     if (lane == 0) {
@@ -712,7 +716,7 @@ __global__ void __launch_bounds__(SHAPE::THREADS, SHAPE::CTAS) lantern_context_k
     float raw_c = 0.0f, raw_u = 0.0f, raw_d = 0.0f;
     auto fetch_single = [&]() {
       const size_t e = static_cast<size_t>(item) * V + xt;
-      raw_d = ctx_raw_logit<BF16>(P.draft, e);
+      if (!GREEDY) raw_d = ctx_raw_logit<BF16>(P.draft, e);
       raw_c = ctx_raw_logit<BF16>(P.target, e);
       if (UNC) raw_u = ctx_raw_logit<BF16>(P.target, branch + e);
     };
@@ -732,6 +736,7 @@ __global__ void __launch_bounds__(SHAPE::THREADS, SHAPE::CTAS) lantern_context_k
     float nd = 0.0f, td = 1.0f;   // drafter: this thread's shift and its sum of numerators, in its own units
     float nq[NP <= 2 ? NP : 1] = {};  // target: the shifts of the slices, where they are few (else in S.slice)
     auto shift_of = [&](int p) { return NP <= 2 ? nq[NP <= 2 ? p : 0] : S.slice[p * GT + gt]; };
+    float z_max = ninf;               // GREEDY: this thread's largest logit
     float nq_max = 0.0f, sq = 1.0f;   // target: the largest shift of the slices; the sum, in its units
     Raw8<BF16> raw[CH];           // the drafter row (dead after the reduction below)
     auto load_drafter = [&](auto whole) {
@@ -820,6 +825,7 @@ __global__ void __launch_bounds__(SHAPE::THREADS, SHAPE::CTAS) lantern_context_k
             for (int i = 0; i < 4; ++i) a2[c * 4 + i] = pack2(ninf, ninf);
           }
         }
+        if (GREEDY) z_max = fmaxf(z_max, m);
         const float n_p = ceilf(fmaxf(m, -1.0e37f) * L2E);
         const uint64_t nn2 = pack2(-n_p, -n_p);
         uint64_t t2 = pack2(0.0f, 0.0f);
@@ -851,10 +857,12 @@ __global__ void __launch_bounds__(SHAPE::THREADS, SHAPE::CTAS) lantern_context_k
     };
     if (nchild > 0) {
       load_slots(xt, 0, nb);
-      if (gt == 0) fetch_single();
-      if (full) load_drafter(std::true_type{});
-      else load_drafter(std::false_type{});
-      if constexpr (TOPK) {   // the drafter row's threshold, from the registers that hold the row
+      if (!GREEDY && gt == 0) fetch_single();
+      if constexpr (!GREEDY) {
+        if (full) load_drafter(std::true_type{});
+        else load_drafter(std::false_type{});
+      }
+      if constexpr (TOPK && !GREEDY) {   // the drafter row's threshold, from the registers that hold the row
         auto own = [&](int c, float (&z)[8]) {
           uint64_t z2[4];
           raw8_pairs<BF16>(raw[c], z2);
@@ -869,8 +877,8 @@ __global__ void __launch_bounds__(SHAPE::THREADS, SHAPE::CTAS) lantern_context_k
         };
         tp = group_kth_largest<SHAPE, CH, CH>(P, own, own, own, again, V, S, grp, gt, search3);
       }
-      reduce_drafter();
-      if (!TOPK && gt == 0) note_single();
+      if (!GREEDY) reduce_drafter();
+      if (!GREEDY && !TOPK && gt == 0) note_single();
     }
     // The target rows were issued when the staging area fell free; they arrive while the drafter
     // row is streamed.  Every thread waits for itself (bounded); a wait that runs out is reported after
@@ -904,7 +912,7 @@ __global__ void __launch_bounds__(SHAPE::THREADS, SHAPE::CTAS) lantern_context_k
           z[0] = a.x, z[1] = a.y, z[2] = a.z, z[3] = a.w, z[4] = b.x, z[5] = b.y, z[6] = b.z, z[7] = b.w;
         };
         tq = group_kth_largest<SHAPE, CH, (NP > 2 ? 2 : CH)>(P, guided, guided_in_place, processed, processed, V, S, grp, gt, search3);
-        if (gt == 0 && nchild > 0) note_single();
+        if (!GREEDY && gt == 0 && nchild > 0) note_single();
       }
       if (full) stream_target(std::true_type{});
       else stream_target(std::false_type{});
@@ -915,9 +923,9 @@ __global__ void __launch_bounds__(SHAPE::THREADS, SHAPE::CTAS) lantern_context_k
     // warp combines the partials for itself (lane l: warp l % GW)
     {
       const float n = nq_max;
-      const float wnq = redux_max(n), wnd = redux_max(nd);
+      const float wnq = redux_max(n), wnd = redux_max(GREEDY ? z_max : nd);   // (greedy decoding: the largest logit travels instead)
       const double zq = static_cast<double>(sq * exp2_int(n - wnq));
-      const double zp = static_cast<double>(td * exp2_int(nd - wnd));
+      const double zp = GREEDY ? 0.0 : static_cast<double>(td * exp2_int(nd - wnd));
       // both sums in one butterfly: after the first exchange the lower half of the warp carries one, the upper the other
       const bool up = lane & 16;
       double z = (up ? zp : zq) + __shfl_xor_sync(kFull, up ? zq : zp, 16);
@@ -928,6 +936,7 @@ __global__ void __launch_bounds__(SHAPE::THREADS, SHAPE::CTAS) lantern_context_k
         S.wn[gw][up] = up ? wnd : wnq;
       }
     }
+    if (GREEDY && gt == 0) S.tok = kNone;
     gbar();   // E, the slices' shifts and the per-warp partials are visible
     if (S.fail) {   // no context was published, or its target rows did not land, within the limit
       give_up();
@@ -944,7 +953,7 @@ __global__ void __launch_bounds__(SHAPE::THREADS, SHAPE::CTAS) lantern_context_k
       Nq = redux_max(n.x);
       Np = redux_max(n.y);
       Zq = z.x * static_cast<double>(exp2_int(n.x - Nq));
-      Zp = z.y * static_cast<double>(exp2_int(n.y - Np));
+      Zp = GREEDY ? 1.0 / GW : z.y * static_cast<double>(exp2_int(n.y - Np));
 #pragma unroll
       for (int o = GW / 2; o > 0; o >>= 1) {
         Zq += __shfl_xor_sync(kFull, Zq, o);
@@ -971,7 +980,9 @@ __global__ void __launch_bounds__(SHAPE::THREADS, SHAPE::CTAS) lantern_context_k
         // the next sibling's description, wanted only after a rejection: in flight meanwhile
         int4 sib = make_int4(0, 0, 0, 0);
         if (ci + 1 < nchild) sib = __ldg(reinterpret_cast<const int4*>(kids + ci + 1));
-        if (gt == 0) {
+        if (GREEDY) {
+          if (gt == 0) atomicAdd(&P.counters->n_tested, 1);
+        } else if (gt == 0) {
           // The tested token's two numerators in common units, in double precision from its raw logits, carried
           // through every rejection round so far (E <- max(0, E - ratio_i * ep)); the sums they are compared
           // with are sums of thousands of terms and do not suffer from cancellation.  A token that has lost its
@@ -1071,9 +1082,11 @@ __global__ void __launch_bounds__(SHAPE::THREADS, SHAPE::CTAS) lantern_context_k
           }
         }
         // Section 4.3: accept iff r p(x~) < sum_A q, i.e. r p_xt / Zp_c < (e_xt + sm) / Zq_c, both sides times Zq_c Zp_c
-        const double p_xt = S.acc_p;
-        const double qa_un = S.acc_e + sm;
-        const bool accept = Zp_c > 0.0 ? static_cast<double>(r) * p_xt * Zq_c < qa_un * Zp_c : 0.0 < qa_un;
+        // (greedy decoding: x~ itself as every other numerator, so that the largest one compares equal to itself)
+        const double p_xt = GREEDY ? 0.0 : S.acc_p;
+        const double qa_un = (GREEDY ? static_cast<double>(mass(xt)) : S.acc_e) + sm;
+        const bool accept = GREEDY ? qa_un >= static_cast<double>(ex2_approx(__fmaf_rn(Np, L2E, -Nq)))
+                            : Zp_c > 0.0 ? static_cast<double>(r) * p_xt * Zq_c < qa_un * Zp_c : 0.0 < qa_un;
         if (gt == 0 && (P.out_qa || P.out_px || P.out_m)) {
           const size_t o = static_cast<size_t>(item / R) * N + node;
           if (P.out_qa) P.out_qa[o] = static_cast<float>(qa_un / Zq_c);
@@ -1084,6 +1097,14 @@ __global__ void __launch_bounds__(SHAPE::THREADS, SHAPE::CTAS) lantern_context_k
           accepted = node;
           break;
         }
+        if constexpr (GREEDY) {
+          if (ci + 1 < nchild) {
+            node = sib.x;
+            xt = sib.y;
+            load_slots(xt, 0, nb);
+          }
+          continue;
+        } else {
         // ---- rejected: residual [q_{k,delta}(.|D = x~) - p]_+ ----
         // the first drafter logits: asked for at once, in flight while A is flagged and across the barrier
         Raw8<BF16> ahead[AHEAD];
@@ -1205,11 +1226,40 @@ __global__ void __launch_bounds__(SHAPE::THREADS, SHAPE::CTAS) lantern_context_k
         if (gt == 0 && ci < 32) S.hist[ci] = static_cast<double>(ratio_g);
         Zq_c = W;
         Zp_c = Sp > 0.0 ? Sp : 0.0;
+        }
       }
 
+      if constexpr (GREEDY) {   // arg max q, smallest index on ties, from the logits themselves
+        if (accepted < 0) {
+          if (z_max == Np) {
+            int first = kNone;
+#pragma unroll 1
+            for (int c = CH - 1; c >= 0; --c) {
+              const int g = c * GT + gt;
+              if (g * 8 < V) {
+                const unsigned char* row = static_cast<const unsigned char*>(P.target) + static_cast<size_t>(item) * rowbytes;
+                uint64_t c2[4], u2[4];
+                raw8_pairs<BF16>(load_raw8<BF16>(row, g), c2);
+                if (UNC) raw8_pairs<BF16>(load_raw8<BF16>(row + static_cast<size_t>(P.B) * R * rowbytes, g), u2);
+#pragma unroll
+                for (int i = 3; i >= 0; --i) {
+                  float lo, hi;
+                  unpack2(UNC ? fma2(pack2(P.cfg_scale, P.cfg_scale), sub2(c2[i], u2[i]), u2[i]) : c2[i], lo, hi);
+                  if (hi == Np) first = g * 8 + 2 * i + 1;
+                  if (lo == Np) first = g * 8 + 2 * i;
+                }
+              }
+            }
+            if (first != kNone) atomicMin(&S.tok, first);
+          }
+          gbar();
+          drawn = true;
+          if (gt == 0) S.result[iter & 1] = {-1, S.tok, status};
+        }
+      }
       // ---- the draw, by inverse CDF over E in token order: the replacement token from the residual where the last
       // child was rejected (Algorithm 1), the bonus token from q itself where there are no children ----
-      if (accepted < 0 && !(status & LANTERN_ST_DEGENERATE)) {
+      if constexpr (!GREEDY) if (accepted < 0 && !(status & LANTERN_ST_DEGENERATE)) {
         {
           float cs[CH];        // weight of each of this thread's chunks, common units
 #pragma unroll

@@ -2,5 +2,6 @@
 #define LANTERN_VARIANT_TONE false
 #define LANTERN_VARIANT_JSD false
 #define LANTERN_VARIANT_TOPK false
+#define LANTERN_VARIANT_GREEDY false
 #define LANTERN_VARIANT_NAME launch_context_v0
 #include "verify_context_variant.cuh"

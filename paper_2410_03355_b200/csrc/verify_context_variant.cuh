@@ -1,5 +1,5 @@
-// One compile-time variant (TONE, JSD, TOPK) of the fused context kernel for every row layout:
-// included by verify_context_v*.cu after defining LANTERN_VARIANT_{TONE,JSD,TOPK,NAME}.
+// One compile-time variant (TONE, JSD, TOPK, GREEDY) of the fused context kernel for every row layout:
+// included by verify_context_v*.cu after defining LANTERN_VARIANT_{TONE,JSD,TOPK,GREEDY,NAME}.
 #include "verify_common.cuh"
 #include "verify_context.cuh"
 
@@ -7,12 +7,13 @@ namespace lantern {
 
 template <class SHAPE, int CHC, bool BF16, bool UNC>
 static cudaError_t launch_shape(const VerifyParams& P, long long items, int sms, cudaStream_t st) {
-  auto kc = lantern_context_kernel<SHAPE, CHC, BF16, UNC, LANTERN_VARIANT_TONE, LANTERN_VARIANT_JSD, LANTERN_VARIANT_TOPK>;
+  auto kc = lantern_context_kernel<SHAPE, CHC, BF16, UNC, LANTERN_VARIANT_TONE, LANTERN_VARIANT_JSD, LANTERN_VARIANT_TOPK,
+                                   LANTERN_VARIANT_GREEDY>;
   const size_t groups = SHAPE::NGRP * SHAPE::AREAS;
   const int ctas = sms * SHAPE::CTAS;
   const int grid = static_cast<int>(items < ctas ? items : ctas);   // a few contexts get an SM each
   static DeviceFlags ready;
-  const cudaError_t e = allow_shared_memory(kc, groups * (64 << 10), ready);   // the longest rows need 64 KB per area
+  const cudaError_t e = allow_shared_memory(kc, groups * ctx_area_bytes(CHC * SHAPE::GT * 8, BF16, UNC), ready);
   if (e != cudaSuccess) return e;
   return launch_dependent(kc, grid, SHAPE::THREADS, groups * ctx_area_bytes(P.V, BF16, UNC), st, P);
 }
@@ -23,7 +24,8 @@ static cudaError_t launch_one(const VerifyParams& P, long long items, int sms, c
     if (shape == 2) return launch_shape<CtxWide, CHC / 2, BF16, UNC>(P, items, sms, st);
     if (shape == 1) return launch_shape<CtxPair, CHC / 2, BF16, UNC>(P, items, sms, st);
   }
-  return launch_shape<CtxNarrow, CHC, BF16, UNC>(P, items, sms, st);
+  if constexpr (CHC == 8 && !BF16) return launch_shape<CtxSingle, CHC / 2, BF16, UNC>(P, items, sms, st);   // (greedy decoding only)
+  else return launch_shape<CtxNarrow, CHC, BF16, UNC>(P, items, sms, st);
 }
 template <int CHC>
 static cudaError_t launch_layout(const VerifyParams& P, bool bf, bool un, long long items, int sms, cudaStream_t st) {
