@@ -33,7 +33,7 @@ constexpr int HB = 11;           // general path: radix-select digit, 2048 bins,
 constexpr int HBINS = 1 << HB;
 constexpr int SAMPLE = 1024;     // keys sampled per row
 constexpr int NBINS = 2048;      // bins of the counting sort, 16-bit counters, two to a word
-constexpr int CROWD = 255;       // largest bin that is ranked by pairwise comparison
+constexpr int CROWD = 1023;      // largest bin that is ranked by pairwise comparison
 constexpr int KEEP = 18;         // list entries per thread of a row's team, at most
 static_assert(SAMPLE <= NBINS / 2, "the sample is kept where the bins will be");
 
@@ -44,6 +44,8 @@ struct BuildParams {
   float* dist;
   int V, D, k;
   int row0, row_end;             // the rows of this launch
+  const int* map;                // the rows are the codes map[row0..], *count of them at most (null: the codes themselves)
+  const int* count;
   int cap;                       // entries of a row's keep list
   int want;                      // rank in the sample that bounds the k smallest keys; 0 = keep everything (cap = V)
 };
@@ -88,15 +90,12 @@ __device__ __forceinline__ float4 fetch_quad(const float* __restrict__ cb, int r
   return v;
 }
 
-__global__ void __launch_bounds__(256, 2) lantern_distance_tile_kernel(const float* __restrict__ cb, uint32_t* out, int V,
-                                                                       int D, int row0, int rows) {
-  __shared__ __align__(16) float As[DK][TM];
-  __shared__ __align__(16) float Bs[DK][TM];
+// The accumulators of one tile.  `row` and `col` are the codes this thread stages (element tid & 127 of either side); a code
+// of V and beyond reads as zero.
+__device__ __forceinline__ void distance_tile(const float* __restrict__ cb, int V, int D, int row, int col, float (&As)[DK][TM],
+                                              float (&Bs)[DK][TM], unsigned long long (&acc)[8][4]) {
   const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
-  const int rbase = row0 + blockIdx.y * TM, cbase = blockIdx.x * TM;
-  const int row_end = (row0 + rows < V) ? row0 + rows : V;
   const bool vec = (D & 3) == 0;
-  unsigned long long acc[8][4];
 #pragma unroll
   for (int r = 0; r < 8; ++r)
 #pragma unroll
@@ -106,8 +105,8 @@ __global__ void __launch_bounds__(256, 2) lantern_distance_tile_kernel(const flo
   float4 ra[2], rb[2];
 #pragma unroll
   for (int l = 0; l < 2; ++l) {
-    ra[l] = fetch_quad(cb, rbase + srow, row_end, D, 4 * (squad + 2 * l), vec);
-    rb[l] = fetch_quad(cb, cbase + srow, V, D, 4 * (squad + 2 * l), vec);
+    ra[l] = fetch_quad(cb, row, V, D, 4 * (squad + 2 * l), vec);
+    rb[l] = fetch_quad(cb, col, V, D, 4 * (squad + 2 * l), vec);
   }
   for (int d0 = 0; d0 < D; d0 += DK) {
 #pragma unroll
@@ -126,8 +125,8 @@ __global__ void __launch_bounds__(256, 2) lantern_distance_tile_kernel(const flo
     if (d0 + DK < D) {
 #pragma unroll
       for (int l = 0; l < 2; ++l) {
-        ra[l] = fetch_quad(cb, rbase + srow, row_end, D, d0 + DK + 4 * (squad + 2 * l), vec);
-        rb[l] = fetch_quad(cb, cbase + srow, V, D, d0 + DK + 4 * (squad + 2 * l), vec);
+        ra[l] = fetch_quad(cb, row, V, D, d0 + DK + 4 * (squad + 2 * l), vec);
+        rb[l] = fetch_quad(cb, col, V, D, d0 + DK + 4 * (squad + 2 * l), vec);
       }
     }
 #pragma unroll
@@ -150,27 +149,208 @@ __global__ void __launch_bounds__(256, 2) lantern_distance_tile_kernel(const flo
     }
     __syncthreads();
   }
-  const bool vec_out = (V & 3) == 0;
+}
+__device__ __forceinline__ uint32_t low_key(unsigned long long v) { return static_cast<uint32_t>(v); }
+__device__ __forceinline__ uint32_t high_key(unsigned long long v) { return static_cast<uint32_t>(v >> 32); }
+
+// code s of the sample, spread over the codebook by the golden ratio (so that no period of the code order is sampled in step)
+__device__ __forceinline__ int sampled_code(int s, int V) {
+  return static_cast<int>((static_cast<unsigned long long>(static_cast<uint32_t>(s) * 2654435769u) * static_cast<unsigned>(V)) >> 32);
+}
+
+// keys of rows x cols pairs -> out[local row, column], rows `pitch` apart
+struct DistParams {
+  const float* cb;
+  uint32_t* out;
+  int V, D;
+  int row0, row_end, cols, pitch;
+  const int* map;                // the rows are the codes map[row0..], *count of them at most (null: the codes themselves)
+  const int* count;
+  int sample;                    // the columns are the codes of the sample
+};
+
+__global__ void __launch_bounds__(256, 2) lantern_distance_tile_kernel(DistParams P) {
+  __shared__ __align__(16) float As[DK][TM];
+  __shared__ __align__(16) float Bs[DK][TM];
+  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
+  const int V = P.V, cols = P.cols;
+  const int row_end = P.count ? min(P.row_end, *P.count) : P.row_end;
+  const int rbase = P.row0 + blockIdx.y * TM, cbase = blockIdx.x * TM;
+  if (rbase >= row_end) return;
+  const int r_mine = rbase + (tid & 127), c_mine = cbase + (tid & 127);
+  const int row = r_mine < row_end ? (P.map ? P.map[r_mine] : r_mine) : V;
+  const int col = c_mine < cols ? (P.sample ? sampled_code(c_mine, V) : c_mine) : V;
+  unsigned long long acc[8][4];
+  distance_tile(P.cb, V, P.D, row, col, As, Bs, acc);
+  const bool vec_out = (P.pitch & 3) == 0;
 #pragma unroll
   for (int r = 0; r < 8; ++r) {
     const int gr = rbase + (r < 4 ? ty * 4 + r : 64 + ty * 4 + (r - 4));
     if (gr >= row_end) continue;
-    uint32_t* orow = out + static_cast<size_t>(gr - row0) * V;
+    uint32_t* orow = P.out + static_cast<size_t>(gr - P.row0) * P.pitch;
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
       const int gc = cbase + 64 * h + tx * 4;
-      const unsigned long long p0 = acc[r][2 * h], p1 = acc[r][2 * h + 1];
-      const uint32_t w[4] = {static_cast<uint32_t>(p0), static_cast<uint32_t>(p0 >> 32), static_cast<uint32_t>(p1),
-                             static_cast<uint32_t>(p1 >> 32)};
-      if (vec_out && gc + 3 < V) {
+      const uint32_t w[4] = {low_key(acc[r][2 * h]), high_key(acc[r][2 * h]), low_key(acc[r][2 * h + 1]), high_key(acc[r][2 * h + 1])};
+      if (vec_out && gc + 3 < cols) {
         *reinterpret_cast<uint4*>(orow + gc) = make_uint4(w[0], w[1], w[2], w[3]);
       } else {
 #pragma unroll
         for (int c = 0; c < 4; ++c)
-          if (gc + c < V) orow[gc + c] = w[c];
+          if (gc + c < cols) orow[gc + c] = w[c];
       }
     }
   }
+}
+
+// ---------------------------------------------------------------------------------------
+// Large D and a large codebook: every pair once.  (a - b)^2 and (b - a)^2 round alike, so key(j, i) = key(i, j) to the bit, and
+// half of the distance work -- which the fp32 pipes bound -- can go; but the keys of all pairs do not fit the scratch, and a row's
+// cannot be kept until the row is complete.  What fits are the rows' keep lists: with the bounds known beforehand (from 1024
+// sampled keys per row: one sixteenth of the work at V = 16384), a tile on or above the diagonal appends the keys
+// within the bounds to the lists of its rows and, mirrored, to those of its columns.
+//
+// A row's list: indices (16 bit) and as many keys as there is room for in its 1/V of the scratch, behind a counter; further keys in
+// the row's own part of the outputs, idx from entry 1 on (entry 0 holds the bound until the list is read), then dist.
+// ---------------------------------------------------------------------------------------
+struct ListParams {
+  unsigned char* scratch;
+  int32_t* idx;
+  float* dist;
+  int V, k, cap;
+  int region;                    // bytes of scratch per row
+  __device__ __forceinline__ int* counter(int i) const { return reinterpret_cast<int*>(scratch + static_cast<size_t>(i) * region); }
+  __device__ __forceinline__ unsigned short* index(int i) const {
+    return reinterpret_cast<unsigned short*>(scratch + static_cast<size_t>(i) * region + 16);
+  }
+  __device__ __forceinline__ uint32_t* key(int i, int e) const {
+    const int head = 16 + ((2 * cap + 3) & ~3), near = (region - head) >> 2;
+    if (e < near) return reinterpret_cast<uint32_t*>(scratch + static_cast<size_t>(i) * region + head) + e;
+    e -= near;
+    if (e < k - 1) return reinterpret_cast<uint32_t*>(idx) + static_cast<size_t>(i) * k + 1 + e;
+    return reinterpret_cast<uint32_t*>(dist) + static_cast<size_t>(i) * k + (e - (k - 1));
+  }
+  __device__ __forceinline__ float bound(int i) const { return __int_as_float(idx[static_cast<size_t>(i) * k]); }
+};
+// entries that a row's list has room for
+static int list_room(int region, int k, bool dist, int cap) {
+  const int head = 16 + ((2 * cap + 3) & ~3);
+  return head > region ? 0 : ((region - head) >> 2) + (k - 1) + (dist ? k : 0);
+}
+
+// Bound of every row from its sampled keys (scratch[i, 0..SAMPLE)), which its list's counter replaces; one warp per row.
+__global__ void __launch_bounds__(256) lantern_row_bound_kernel(ListParams L, int want) {
+  const int i = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+  if (i >= L.V) return;
+  const uint32_t* src = reinterpret_cast<const uint32_t*>(L.scratch) + static_cast<size_t>(i) * SAMPLE;
+  uint32_t key[SAMPLE / 32], most = 0u;
+#pragma unroll
+  for (int q = 0; q < SAMPLE / 32; ++q) {
+    key[q] = src[q * 32 + lane];
+    most = key[q] > most ? key[q] : most;
+  }
+  most = __reduce_max_sync(kFull, most);
+  const int room = want / 16 + 2;
+  uint32_t lo = 0u, hi = most;             // count(key <= hi) >= want > count(key <= lo); a few more than wanted will do
+  for (int pass = 0; pass < 48 && hi - lo > 1u; ++pass) {
+    uint32_t m = __float_as_uint(0.5f * __uint_as_float(lo) + 0.5f * __uint_as_float(hi));
+    if (!(m > lo && m < hi)) m = lo + ((hi - lo) >> 1);
+    int c0 = 0, c1 = 0;
+#pragma unroll
+    for (int q = 0; q < SAMPLE / 32; q += 2) {
+      c0 += key[q] <= m;
+      c1 += key[q + 1] <= m;
+    }
+    const int c = __reduce_add_sync(kFull, c0 + c1);
+    if (c >= want) hi = m;
+    else lo = m;
+    if (c >= want && c <= want + room) break;
+  }
+  if (lane == 0) {
+    L.idx[static_cast<size_t>(i) * L.k] = static_cast<int32_t>(hi);
+    *L.counter(i) = 0;                     // (all lanes have read the row: the reduction above)
+  }
+}
+
+__global__ void __launch_bounds__(256, 2) lantern_distance_lists_kernel(const float* __restrict__ cb, int D, ListParams L) {
+  __shared__ __align__(16) float As[DK][TM];
+  __shared__ __align__(16) float Bs[DK][TM];
+  __shared__ int s_n[2][TM], s_base[2][TM];
+  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
+  const int V = L.V;
+  // tile (tr, tc) with tr <= tc, numbered column by column: tc (tc + 1) / 2 + tr
+  int tc = static_cast<int>((sqrtf(8.0f * static_cast<float>(blockIdx.x) + 1.0f) - 1.0f) * 0.5f);
+  while (tc * (tc + 1) / 2 > static_cast<int>(blockIdx.x)) --tc;
+  while ((tc + 1) * (tc + 2) / 2 <= static_cast<int>(blockIdx.x)) ++tc;
+  const int tr = blockIdx.x - tc * (tc + 1) / 2;
+  const int rbase = tr * TM, cbase = tc * TM;
+  s_n[tid >> 7][tid & 127] = 0;
+  unsigned long long acc[8][4];
+  distance_tile(cb, V, D, rbase + (tid & 127), cbase + (tid & 127), As, Bs, acc);   // (its barriers publish s_n as well)
+  auto row_of = [&](int r) { return r < 4 ? ty * 4 + r : 64 + ty * 4 + (r - 4); };
+  auto col_of = [&](int c) { return c < 4 ? tx * 4 + c : 64 + tx * 4 + (c - 4); };
+  auto key_of = [&](int r, int c) { return c & 1 ? high_key(acc[r][c >> 1]) : low_key(acc[r][c >> 1]); };
+  const float never = __int_as_float(0xff800000);
+  float tb[8];                             // bounds, first of the rows, then of the columns
+  int at_r[8], at_c[8];                    // this thread's places in the lists' tile parts
+  const bool mirror = tr != tc;
+#pragma unroll
+  for (int r = 0; r < 8; ++r) {
+    const int i = rbase + row_of(r);
+    tb[r] = i < V ? L.bound(i) : never;
+    int n = 0;
+#pragma unroll
+    for (int c = 0; c < 8; ++c) n += cbase + col_of(c) < V && __uint_as_float(key_of(r, c)) <= tb[r];
+    at_r[r] = n ? atomicAdd(&s_n[0][row_of(r)], n) : 0;
+  }
+  float tcol[8];
+#pragma unroll
+  for (int c = 0; c < 8; ++c) {
+    const int j = cbase + col_of(c);
+    tcol[c] = mirror && j < V ? L.bound(j) : never;
+    int n = 0;
+#pragma unroll
+    for (int r = 0; r < 8; ++r) n += rbase + row_of(r) < V && __uint_as_float(key_of(r, c)) <= tcol[c];
+    at_c[c] = n ? atomicAdd(&s_n[1][col_of(c)], n) : 0;
+  }
+  __syncthreads();
+  {
+    const int side = tid >> 7, q = tid & 127, i = (side ? cbase : rbase) + q, n = s_n[side][q];
+    s_base[side][q] = n ? atomicAdd(L.counter(i), n) : 0;   // (n > 0: a code)
+  }
+  __syncthreads();
+  auto put = [&](int i, int e, int j, uint32_t key) {
+    if (e < L.cap) {
+      L.index(i)[e] = static_cast<unsigned short>(j);
+      *L.key(i, e) = key;
+    }
+  };
+#pragma unroll
+  for (int r = 0; r < 8; ++r) {
+    const int i = rbase + row_of(r);
+    int e = s_base[0][row_of(r)] + at_r[r];
+#pragma unroll
+    for (int c = 0; c < 8; ++c) {
+      const int j = cbase + col_of(c);
+      if (j < V && __uint_as_float(key_of(r, c)) <= tb[r]) put(i, e++, j, key_of(r, c));
+    }
+  }
+#pragma unroll
+  for (int c = 0; c < 8; ++c) {
+    const int j = cbase + col_of(c);
+    int e = s_base[1][col_of(c)] + at_c[c];
+#pragma unroll
+    for (int r = 0; r < 8; ++r) {
+      const int i = rbase + row_of(r);
+      if (i < V && __uint_as_float(key_of(r, c)) <= tcol[c]) put(j, e++, i, key_of(r, c));
+    }
+  }
+}
+
+// the rows whose lists failed (marked by idx[i, 0] = -1), in any order
+__global__ void lantern_failed_rows_kernel(const int32_t* idx, int V, int k, int* rows, int* count) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < V && idx[static_cast<size_t>(i) * k] < 0) rows[atomicAdd(count, 1)] = i;
 }
 
 // ---------------------------------------------------------------------------------------
@@ -241,7 +421,7 @@ struct GeneralShared {
 
 // The general path for row i, by the whole CTA: dsm = V keys, then the list of P2 composites.
 template <int KT>
-__device__ __noinline__ void knn_row_general(const BuildParams& P, int i, int P2, unsigned char* dsm, GeneralShared& S) {
+__device__ __noinline__ void knn_row_general(const BuildParams& P, int i, int local, int P2, unsigned char* dsm, GeneralShared& S) {
   uint32_t* keys = reinterpret_cast<uint32_t*>(dsm);                                  // [V]
   unsigned long long* list =
       reinterpret_cast<unsigned long long*>(dsm + ((static_cast<size_t>(P.V) * 4 + 15) & ~size_t(15)));  // [P2]
@@ -256,7 +436,7 @@ __device__ __noinline__ void knn_row_general(const BuildParams& P, int i, int P2
   if (!P.scratch && tid < D) S.ai[tid] = P.codebook[static_cast<size_t>(i) * D + tid];
   __syncthreads();
   for (int j = tid; j < V; j += KT) {
-    const uint32_t key = P.scratch ? P.scratch[static_cast<size_t>(i - P.row0) * V + j]
+    const uint32_t key = P.scratch ? P.scratch[static_cast<size_t>(local) * V + j]
                                    : __float_as_uint(key_of(S.ai, P.codebook + static_cast<size_t>(j) * D, D, (D & 3) == 0));
     keys[j] = key;
     if (j != i) {
@@ -411,13 +591,16 @@ static __host__ __device__ constexpr size_t row_bytes(int cap) {
   return ((static_cast<size_t>(cap + 2) * 8 + 15) & ~size_t(15)) + NBINS * 2;
 }
 
-// R rows per CTA of KT threads; KT / R threads rank a row.
+// R rows per CTA of KT threads; KT / R threads rank a row.  FROM: where the keys come from -- computed here (small D), read
+// from scratch rows, or already on lists.
 //
 // What bounds it (V = 16384, k = 1000, cycles of a CTA of eight rows, D = 8): the key pass 40 k, of which the fp32
 // pipes need 16 k and instruction issue 24 k; sample and bound 9 k; counting sort 13 k; ranking 11 k.
 // 0.55 ms per table; 1.20 ms when a CTA selected from all keys of one row (73 k warp instructions per row, now 26 k).
-template <int KT, int R, bool SCRATCH>
-__global__ void __launch_bounds__(KT, 1024 / KT) lantern_knn_rows_kernel(BuildParams P, int P2) {
+enum { FROM_CODES = 0, FROM_SCRATCH = 1, FROM_LISTS = 2 };
+template <int KT, int R, int FROM>
+__global__ void __launch_bounds__(KT, 1024 / KT) lantern_knn_rows_kernel(BuildParams P, ListParams L, int P2) {
+  constexpr bool SCRATCH = FROM == FROM_SCRATCH, LISTS = FROM == FROM_LISTS;
   constexpr int RT = KT / R;         // threads of a row's team
   constexpr int RW = RT / 32;
   constexpr int U = 2;               // codes per thread and step of the key pass
@@ -432,13 +615,14 @@ __global__ void __launch_bounds__(KT, 1024 / KT) lantern_knn_rows_kernel(BuildPa
   __shared__ uint32_t s_low[R][3 * RW], s_most[R][RW];
   const int tid = threadIdx.x, lane = tid & 31;
   const int V = P.V, D = P.D, k = P.k, cap = P.cap;
-  const int row0 = P.row0 + blockIdx.x * R, row_end = P.row_end;
+  const int row0 = P.row0 + blockIdx.x * R, row_end = P.count ? min(P.row_end, *P.count) : P.row_end;
+  if (row0 >= row_end) return;
   const bool vec = (D & 3) == 0;
   const size_t per_row = row_bytes(cap);
   auto list_of = [&](int r) { return reinterpret_cast<unsigned long long*>(dsm + r * per_row); };
   auto bins_of = [&](int r) { return reinterpret_cast<unsigned*>(dsm + (r + 1) * per_row - NBINS * 2); };
 
-  if (!SCRATCH) {
+  if (FROM == FROM_CODES) {
     for (int t = tid; t < SMALL_D * R; t += KT) {
       const int d = t / R, r = t % R;
       As[d][r] = (d < D && row0 + r < row_end) ? P.codebook[static_cast<size_t>(row0 + r) * D + d] : 0.0f;
@@ -448,22 +632,20 @@ __global__ void __launch_bounds__(KT, 1024 / KT) lantern_knn_rows_kernel(BuildPa
   __syncthreads();
 
   const int r = tid / RT, rt = tid % RT;   // this thread's team and its place in it
-  const int i = row0 + r;
+  const bool on = row0 + r < row_end;
+  const int local = row0 + r - P.row0;
+  const int i = on && P.map ? P.map[row0 + r] : row0 + r;
   auto team = [&]() { asm volatile("bar.sync %0, %1;" ::"r"(1 + r), "n"(RT) : "memory"); };
-  // ---- 1. the bound, from SAMPLE keys spread over the codebook by the golden ratio (so that no period of the
-  // code order is sampled in step) ----
-  {
-    auto sampled = [&](int s) {
-      return static_cast<int>((static_cast<unsigned long long>(static_cast<uint32_t>(s) * 2654435769u) * static_cast<unsigned>(V)) >> 32);
-    };
+  // ---- 1. the bound, from SAMPLE keys ----
+  if constexpr (!LISTS) {
     uint32_t key[SMP];
     if constexpr (SCRATCH) {
-      const uint32_t* src = P.scratch + static_cast<size_t>(i < row_end ? i - P.row0 : 0) * V;
+      const uint32_t* src = P.scratch + static_cast<size_t>(on ? local : 0) * V;
 #pragma unroll
-      for (int q = 0; q < SMP; ++q) key[q] = __ldg(src + sampled(q * RT + rt));
+      for (int q = 0; q < SMP; ++q) key[q] = __ldg(src + sampled_code(q * RT + rt, V));
     } else {   // every thread takes codes of the sample against all rows of the CTA
       for (int s = tid; s < SAMPLE; s += KT) {
-        const float* b = P.codebook + static_cast<size_t>(sampled(s)) * D;
+        const float* b = P.codebook + static_cast<size_t>(sampled_code(s, V)) * D;
         float acc[R];
 #pragma unroll
         for (int q = 0; q < R; ++q) acc[q] = 0.0f;
@@ -549,7 +731,7 @@ __global__ void __launch_bounds__(KT, 1024 / KT) lantern_knn_rows_kernel(BuildPa
   }
 
   // ---- 2. all keys; those within the bound go to their row's list ----
-  if constexpr (!SCRATCH) {
+  if constexpr (FROM == FROM_CODES) {
     float t_row[R];
 #pragma unroll
     for (int q = 0; q < R; ++q) t_row[q] = s_t[q];
@@ -649,9 +831,9 @@ __global__ void __launch_bounds__(KT, 1024 / KT) lantern_knn_rows_kernel(BuildPa
         }
       }
     }
-  } else if (i < row_end) {   // each team reads its own row of keys, W groups of four per thread at a time
+  } else if (SCRATCH && on) {   // each team reads its own row of keys, W groups of four per thread at a time
     constexpr int W = 4;
-    const uint32_t* src = P.scratch + static_cast<size_t>(i - P.row0) * V;
+    const uint32_t* src = P.scratch + static_cast<size_t>(local) * V;
     const float t = s_t[r];
     unsigned long long* list = list_of(r);
     const bool vec4 = (V & 3) == 0;
@@ -703,11 +885,13 @@ __global__ void __launch_bounds__(KT, 1024 / KT) lantern_knn_rows_kernel(BuildPa
   __syncthreads();
 
   // ---- 3. counting sort (in place, through registers) and ranking, a team per row ----
-  if (i < row_end) {
+  if (on) {
     unsigned long long* list = list_of(r);
     unsigned* bins = bins_of(r);
-    const int n = s_cnt[r];
-    const float lo = s_lo[r], scale = s_scale[r];
+    const int n = LISTS ? *L.counter(i) : s_cnt[r];
+    float lo = 0.0f, scale = 0.0f;
+    uint32_t key[KEEP], who[KEEP];    // this thread's entries: the key; index + 1 and place of arrival in its bin
+    if (!LISTS) lo = s_lo[r], scale = s_scale[r];
     auto bin_of = [&](uint32_t key) {   // monotone in the key
       // the square: near the bound the keys lie closer together (distances in D dimensions grow like the D/2-th root)
       const float x = fmaxf(__uint_as_float(key) - lo, 0.0f) * scale;
@@ -719,15 +903,44 @@ __global__ void __launch_bounds__(KT, 1024 / KT) lantern_knn_rows_kernel(BuildPa
     } else {
 #pragma unroll
       for (int q = 0; q < OWN; ++q) bins[q * RT + rt] = 0u;
+      if constexpr (LISTS) {            // read the list; its range (without the code itself) is where the bins go
+        uint32_t least = 0xffffffffu, most = 0u;
+#pragma unroll
+        for (int q = 0; q < KEEP; ++q) {
+          const int e = q * RT + rt;
+          if (e < n) {
+            key[q] = *L.key(i, e);
+            who[q] = L.index(i)[e] + 1u;
+            if (who[q] != static_cast<uint32_t>(i + 1)) {
+              least = key[q] < least ? key[q] : least;
+              most = key[q] > most ? key[q] : most;
+            }
+          }
+        }
+        least = __reduce_min_sync(kFull, least);
+        most = __reduce_max_sync(kFull, most);
+        if (lane == 0) s_low[r][rt >> 5] = least, s_most[r][rt >> 5] = most;
+      }
       team();
-      uint32_t key[KEEP], who[KEEP];    // this thread's entries: the key; index + 1 and place of arrival in its bin
+      if constexpr (LISTS) {
+        uint32_t least = 0xffffffffu, most = 0u;
+#pragma unroll
+        for (int w = 0; w < RW; ++w) {
+          least = s_low[r][w] < least ? s_low[r][w] : least;
+          most = s_most[r][w] > most ? s_most[r][w] : most;
+        }
+        lo = __uint_as_float(least);
+        scale = most > least ? 1.0f / (__uint_as_float(most) - lo) : 0.0f;
+      }
 #pragma unroll
       for (int q = 0; q < KEEP; ++q) {
         const int e = q * RT + rt;
         if (e < n) {
-          const unsigned long long c = list[e];
-          key[q] = static_cast<uint32_t>(c >> 32);
-          who[q] = static_cast<uint32_t>(c);
+          if (!LISTS) {
+            const unsigned long long c = list[e];
+            key[q] = static_cast<uint32_t>(c >> 32);
+            who[q] = static_cast<uint32_t>(c);
+          }
           if (who[q] == static_cast<uint32_t>(i + 1)) key[q] = who[q] = 0u;   // the code itself comes first
           const int b = bin_of(key[q]), sh = (b & 1) << 4;
           who[q] |= ((atomicAdd(&bins[b >> 1], 1u << sh) >> sh) & 0xffffu) << 16;
@@ -786,8 +999,15 @@ __global__ void __launch_bounds__(KT, 1024 / KT) lantern_knn_rows_kernel(BuildPa
     }
   }
   __syncthreads();
-  for (int q = 0; q < R; ++q)
-    if (s_slow[q]) knn_row_general<KT>(P, row0 + q, P2, dsm, S);
+  for (int q = 0; q < R; ++q) {
+    if (!s_slow[q]) continue;
+    const int l = row0 + q, code = P.map ? P.map[l] : l;
+    if constexpr (LISTS) {
+      if (tid == 0) P.idx[static_cast<size_t>(code) * k] = -1;   // done again from all keys
+    } else {
+      knn_row_general<KT>(P, code, l - P.row0, P2, dsm, S);
+    }
+  }
 }
 
 static int next_pow2(int x) {
@@ -805,12 +1025,12 @@ static int rows_per_block(int V) {
   return (r + TM - 1) / TM * TM;
 }
 
-template <int KT, int R, bool SCRATCH>
-static cudaError_t launch_rows(const BuildParams& P, int P2, size_t smem, cudaStream_t st) {
-  auto kk = lantern_knn_rows_kernel<KT, R, SCRATCH>;
+template <int KT, int R, int FROM>
+static cudaError_t launch_rows(const BuildParams& P, int P2, size_t smem, cudaStream_t st, const ListParams& L = {}) {
+  auto kk = lantern_knn_rows_kernel<KT, R, FROM>;
   const cudaError_t e = cudaFuncSetAttribute(kk, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
   if (e != cudaSuccess) return e;
-  kk<<<(P.row_end - P.row0 + R - 1) / R, KT, smem, st>>>(P, P2);
+  kk<<<(P.row_end - P.row0 + R - 1) / R, KT, smem, st>>>(P, L, P2);
   return cudaGetLastError();
 }
 
@@ -846,6 +1066,7 @@ extern "C" lantern_status lantern_build_neighbors(const float* codebook, int V, 
   P.V = V;
   P.D = D;
   P.k = k;
+  P.map = P.count = nullptr;
   // The k-th smallest of V keys has rank k SAMPLE / V in the sample, with a binomial spread; 3.5 standard deviations
   // above that the bound fails one row in some thousands, and the list is as long as the kept keys may be with the same
   // margin.  Few codes: the bound would keep most of them anyway.
@@ -869,23 +1090,80 @@ extern "C" lantern_status lantern_build_neighbors(const float* codebook, int V, 
   if (smem > kRowSmem || P.cap > KEEP * (1024 / R)) return LANTERN_E_SHAPE;
   auto select = [&]() {
     if (P.scratch)
-      return R == 8 ? launch_rows<512, 4, true>(P, P2, smem, st)
-                    : (R == 4 ? launch_rows<512, 2, true>(P, P2, smem, st) : launch_rows<512, 1, true>(P, P2, smem, st));
-    if (few) return launch_rows<256, 2, false>(P, P2, smem, st);
-    return R == 8 ? launch_rows<1024, 8, false>(P, P2, smem, st)
-                  : (R == 4 ? launch_rows<1024, 4, false>(P, P2, smem, st) : launch_rows<1024, 2, false>(P, P2, smem, st));
+      return R == 8 ? launch_rows<512, 4, FROM_SCRATCH>(P, P2, smem, st)
+                    : (R == 4 ? launch_rows<512, 2, FROM_SCRATCH>(P, P2, smem, st) : launch_rows<512, 1, FROM_SCRATCH>(P, P2, smem, st));
+    if (few) return launch_rows<256, 2, FROM_CODES>(P, P2, smem, st);
+    return R == 8 ? launch_rows<1024, 8, FROM_CODES>(P, P2, smem, st)
+                  : (R == 4 ? launch_rows<1024, 4, FROM_CODES>(P, P2, smem, st) : launch_rows<1024, 2, FROM_CODES>(P, P2, smem, st));
   };
-  const int rb = P.scratch ? rows_per_block(V) : V;
-  for (P.row0 = 0; P.row0 < V; P.row0 += rb) {
-    P.row_end = V - P.row0 < rb ? V : P.row0 + rb;
-    if (P.scratch) {
-      const int rows = P.row_end - P.row0;
-      const dim3 grid((V + TM - 1) / TM, (rows + TM - 1) / TM);
-      lantern_distance_tile_kernel<<<grid, 256, 0, st>>>(codebook, static_cast<uint32_t*>(workspace), V, D, P.row0, rows);
-      if (cudaGetLastError() != cudaSuccess) return LANTERN_E_CUDA;
+  DistParams T = {};
+  T.cb = codebook;
+  T.out = static_cast<uint32_t*>(workspace);
+  T.V = V;
+  T.D = D;
+  T.cols = T.pitch = V;
+  auto distances = [&](int row0, int row_end) {
+    T.row0 = row0;
+    T.row_end = row_end;
+    const dim3 grid((T.cols + TM - 1) / TM, (row_end - row0 + TM - 1) / TM);
+    lantern_distance_tile_kernel<<<grid, 256, 0, st>>>(T);
+    return cudaGetLastError();
+  };
+  // all rows, or the codes of P.map, a block of rows at a time
+  auto by_blocks = [&](int block) {
+    for (P.row0 = 0; P.row0 < V; P.row0 += block) {
+      P.row_end = V - P.row0 < block ? V : P.row0 + block;
+      cudaError_t e = P.scratch ? distances(P.row0, P.row_end) : cudaSuccess;
+      if (e == cudaSuccess) e = select();
+      if (e != cudaSuccess) return e;
     }
-    if (select() != cudaSuccess) return LANTERN_E_CUDA;
+    return cudaSuccess;
+  };
+  if (!P.scratch) return by_blocks(V) == cudaSuccess ? LANTERN_OK : LANTERN_E_CUDA;
+
+  // Every pair once, through lists, where the lists fit with 2.3 to 2.7 standard deviations of room: a row in some hundreds
+  // overflows its list and is done again from all its keys.
+  ListParams L;
+  L.scratch = static_cast<unsigned char*>(workspace);
+  L.idx = idx;
+  L.dist = dist;
+  L.V = V;
+  L.k = k;
+  L.region = rows_per_block(V) * 4;
+  L.cap = static_cast<int>((most + 2.7 * sqrt(static_cast<double>(most))) / f) & ~1;
+  const int least = static_cast<int>((most + 2.3 * sqrt(static_cast<double>(most))) / f);
+  while (L.cap > least && list_room(L.region, k, dist != nullptr, L.cap) < L.cap) L.cap -= 2;
+  if (V >= 4096 && P.want > 0 && R == 8 && L.cap > least && L.cap >= k && L.cap <= P.cap) {
+    T.sample = 1;
+    T.cols = T.pitch = SAMPLE;
+    cudaError_t e = distances(0, V);
+    if (e != cudaSuccess) return LANTERN_E_CUDA;
+    lantern_row_bound_kernel<<<(V + 7) / 8, 256, 0, st>>>(L, P.want);
+    if (cudaGetLastError() != cudaSuccess) return LANTERN_E_CUDA;
+    const int t = (V + TM - 1) / TM;
+    lantern_distance_lists_kernel<<<t * (t + 1) / 2, 256, 0, st>>>(codebook, D, L);
+    if (cudaGetLastError() != cudaSuccess) return LANTERN_E_CUDA;
+    const int cap = P.cap;
+    P.row0 = 0;
+    P.row_end = V;
+    P.cap = L.cap;
+    e = launch_rows<512, 4, FROM_LISTS>(P, P2, 4 * row_bytes(P.cap), st, L);
+    if (e != cudaSuccess) return LANTERN_E_CUDA;
+    // the rows whose lists failed, from all their keys: the list of them takes the last rows of the scratch
+    P.cap = cap;
+    const int block = rows_per_block(V) - TM;
+    int* rows = reinterpret_cast<int*>(static_cast<uint32_t*>(workspace) + static_cast<size_t>(block) * V);
+    int* count = rows + V;
+    if (cudaMemsetAsync(count, 0, sizeof(int), st) != cudaSuccess) return LANTERN_E_CUDA;
+    lantern_failed_rows_kernel<<<(V + 255) / 256, 256, 0, st>>>(idx, V, k, rows, count);
+    if (cudaGetLastError() != cudaSuccess) return LANTERN_E_CUDA;
+    P.map = T.map = rows;
+    P.count = T.count = count;
+    T.sample = 0;
+    T.cols = T.pitch = V;
+    return by_blocks(block) == cudaSuccess ? LANTERN_OK : LANTERN_E_CUDA;
   }
+  if (by_blocks(rows_per_block(V)) != cudaSuccess) return LANTERN_E_CUDA;
   return LANTERN_OK;
 }
 

@@ -119,3 +119,27 @@ def test_selection_paths_exact(V, D, k, kind):
     assert np.array_equal(gi[:, 0], np.arange(V))
     srt = np.sort(gi, axis=1)
     assert np.all(srt[:, 1:] != srt[:, :-1])
+
+
+@pytest.mark.parametrize("V,D,k,kind,with_dist", [
+    (4096, 40, 1000, "period", True), (4099, 33, 100, "gauss", True), (4100, 36, 30, "gauss", False),   # every pair once, through lists
+    (4096, 40, 300, "ties", True), (6144, 64, 700, "big clusters", True),                               # lists that fail
+    (4096, 40, 1000, "period", False), (4095, 40, 100, "gauss", True)])                                 # no room for lists; too few codes
+def test_lists_exact(V, D, k, kind, with_dist):
+    if kind == "ties":
+        cb = li.codebook_integer(V, D, lo=0, hi=2, seed=9)
+    elif kind == "gauss":
+        cb = li.codebook_gaussian(V, D, seed=11)
+    else:
+        cb = li.codebook_clustered(V, D, centres=512 if kind == "period" else 7, seed=10)
+    idx, dist = lt.build_neighbors(torch.from_numpy(cb).cuda(), k, with_dist=with_dist)
+    torch.cuda.synchronize()
+    gi = idx.cpu().numpy()
+    rows = np.unique(np.concatenate([np.arange(20), np.arange(V - 20, V), np.random.default_rng(1).integers(0, V, 24)])).astype(np.int32)
+    oi, od = oracle.build_neighbors(cb, k, rows=rows)
+    assert np.array_equal(gi[rows], oi)
+    if with_dist:
+        assert np.array_equal(dist.cpu().numpy()[rows].view(np.uint32), od.view(np.uint32))
+    assert np.array_equal(gi[:, 0], np.arange(V))
+    srt = np.sort(gi, axis=1)
+    assert np.all(srt[:, 1:] != srt[:, :-1])
