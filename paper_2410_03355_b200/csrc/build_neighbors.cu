@@ -272,11 +272,26 @@ __global__ void __launch_bounds__(256) lantern_row_bound_kernel(ListParams L, in
   }
 }
 
+// What a tile keeps (some 3000 entries at k = 1000) is first put in order of its lists in shared memory and then stored by
+// all threads alike: the address of an entry takes thirty instructions, too many to spend on every pair.
+constexpr int TILE_KEEP = 4096;
+struct TileLists {
+  uint32_t key[TILE_KEEP];
+  unsigned short code[TILE_KEEP];
+  unsigned char line[TILE_KEEP];
+};
+
 __global__ void __launch_bounds__(256, 2) lantern_distance_lists_kernel(const float* __restrict__ cb, int D, ListParams L) {
-  __shared__ __align__(16) float As[DK][TM];
-  __shared__ __align__(16) float Bs[DK][TM];
-  __shared__ int s_n[2][TM], s_base[2][TM];
-  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
+  __shared__ __align__(16) union {
+    struct {
+      float As[DK][TM], Bs[DK][TM];
+    } in;
+    TileLists out;
+  } S;
+  __shared__ float s_bound[2][TM];         // [0] the tile's rows, [1] its columns
+  __shared__ int s_n[2][TM], s_off[2][TM], s_base[2][TM], s_warp[8];
+  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4, lane = tid & 31;
+  const int side = tid >> 7, line = tid & 127;
   const int V = L.V;
   // tile (tr, tc) with tr <= tc, numbered column by column: tc (tc + 1) / 2 + tr
   int tc = static_cast<int>((sqrtf(8.0f * static_cast<float>(blockIdx.x) + 1.0f) - 1.0f) * 0.5f);
@@ -284,66 +299,99 @@ __global__ void __launch_bounds__(256, 2) lantern_distance_lists_kernel(const fl
   while ((tc + 1) * (tc + 2) / 2 <= static_cast<int>(blockIdx.x)) ++tc;
   const int tr = blockIdx.x - tc * (tc + 1) / 2;
   const int rbase = tr * TM, cbase = tc * TM;
-  s_n[tid >> 7][tid & 127] = 0;
+  const int mine = (side ? cbase : rbase) + line;   // the code whose list this thread looks after
+  s_n[side][line] = 0;
+  s_bound[side][line] = mine < V && (side == 0 || tr != tc) ? L.bound(mine) : __int_as_float(0xff800000);   // (-inf: keeps nothing)
   unsigned long long acc[8][4];
-  distance_tile(cb, V, D, rbase + (tid & 127), cbase + (tid & 127), As, Bs, acc);   // (its barriers publish s_n as well)
+  distance_tile(cb, V, D, rbase + line, cbase + line, S.in.As, S.in.Bs, acc);   // (its barriers publish the bounds as well)
   auto row_of = [&](int r) { return r < 4 ? ty * 4 + r : 64 + ty * 4 + (r - 4); };
   auto col_of = [&](int c) { return c < 4 ? tx * 4 + c : 64 + tx * 4 + (c - 4); };
+  // a pair with a code past the end is kept by nobody
+  if (cbase + TM > V) {
+#pragma unroll
+    for (int c = 0; c < 8; ++c)
+      if (cbase + col_of(c) >= V) {
+#pragma unroll
+        for (int r = 0; r < 8; ++r)
+          acc[r][c >> 1] |= c & 1 ? 0x7fffffff00000000ull : 0x7fffffffull;   // NaN
+      }
+  }
   auto key_of = [&](int r, int c) { return c & 1 ? high_key(acc[r][c >> 1]) : low_key(acc[r][c >> 1]); };
-  const float never = __int_as_float(0xff800000);
-  float tb[8];                             // bounds, first of the rows, then of the columns
-  int at_r[8], at_c[8];                    // this thread's places in the lists' tile parts
-  const bool mirror = tr != tc;
+  int at_r[8], at_c[8];                    // this thread's places in the tile's part of each list
 #pragma unroll
   for (int r = 0; r < 8; ++r) {
-    const int i = rbase + row_of(r);
-    tb[r] = i < V ? L.bound(i) : never;
+    const float t = s_bound[0][row_of(r)];
     int n = 0;
 #pragma unroll
-    for (int c = 0; c < 8; ++c) n += cbase + col_of(c) < V && __uint_as_float(key_of(r, c)) <= tb[r];
+    for (int c = 0; c < 8; ++c) n += __uint_as_float(key_of(r, c)) <= t;
     at_r[r] = n ? atomicAdd(&s_n[0][row_of(r)], n) : 0;
   }
-  float tcol[8];
 #pragma unroll
   for (int c = 0; c < 8; ++c) {
-    const int j = cbase + col_of(c);
-    tcol[c] = mirror && j < V ? L.bound(j) : never;
+    const float t = s_bound[1][col_of(c)];
     int n = 0;
 #pragma unroll
-    for (int r = 0; r < 8; ++r) n += rbase + row_of(r) < V && __uint_as_float(key_of(r, c)) <= tcol[c];
+    for (int r = 0; r < 8; ++r) n += __uint_as_float(key_of(r, c)) <= t;
     at_c[c] = n ? atomicAdd(&s_n[1][col_of(c)], n) : 0;
   }
   __syncthreads();
-  {
-    const int side = tid >> 7, q = tid & 127, i = (side ? cbase : rbase) + q, n = s_n[side][q];
-    s_base[side][q] = n ? atomicAdd(L.counter(i), n) : 0;   // (n > 0: a code)
+  const int n_mine = s_n[side][line];
+  s_base[side][line] = n_mine ? atomicAdd(L.counter(mine), n_mine) : 0;
+  int incl = n_mine;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int v = __shfl_up_sync(kFull, incl, o);
+    if (lane >= o) incl += v;
   }
+  if (lane == 31) s_warp[tid >> 5] = incl;
   __syncthreads();
-  auto put = [&](int i, int e, int j, uint32_t key) {
+  int before = 0, total = 0;
+#pragma unroll
+  for (int w = 0; w < 8; ++w) {
+    if (w < (tid >> 5)) before += s_warp[w];
+    total += s_warp[w];
+  }
+  s_off[side][line] = before + incl - n_mine;
+  __syncthreads();
+  auto put = [&](int code, int e, int other, uint32_t key) {
     if (e < L.cap) {
-      L.index(i)[e] = static_cast<unsigned short>(j);
-      *L.key(i, e) = key;
+      L.index(code)[e] = static_cast<unsigned short>(other);
+      *L.key(code, e) = key;
     }
   };
-#pragma unroll
-  for (int r = 0; r < 8; ++r) {
-    const int i = rbase + row_of(r);
-    int e = s_base[0][row_of(r)] + at_r[r];
-#pragma unroll
-    for (int c = 0; c < 8; ++c) {
-      const int j = cbase + col_of(c);
-      if (j < V && __uint_as_float(key_of(r, c)) <= tb[r]) put(i, e++, j, key_of(r, c));
-    }
-  }
-#pragma unroll
-  for (int c = 0; c < 8; ++c) {
-    const int j = cbase + col_of(c);
-    int e = s_base[1][col_of(c)] + at_c[c];
+  // every kept pair: list (0 = of its row, 1 = of its column) and line, place in the tile's part, the other code, the key
+  auto each = [&](auto take) {
 #pragma unroll
     for (int r = 0; r < 8; ++r) {
-      const int i = rbase + row_of(r);
-      if (i < V && __uint_as_float(key_of(r, c)) <= tcol[c]) put(j, e++, i, key_of(r, c));
+      const float t = s_bound[0][row_of(r)];
+      int e = at_r[r];
+#pragma unroll
+      for (int c = 0; c < 8; ++c)
+        if (__uint_as_float(key_of(r, c)) <= t) take(0, row_of(r), e++, cbase + col_of(c), key_of(r, c));
     }
+#pragma unroll
+    for (int c = 0; c < 8; ++c) {
+      const float t = s_bound[1][col_of(c)];
+      int e = at_c[c];
+#pragma unroll
+      for (int r = 0; r < 8; ++r)
+        if (__uint_as_float(key_of(r, c)) <= t) take(1, col_of(c), e++, rbase + row_of(r), key_of(r, c));
+    }
+  };
+  if (total <= TILE_KEEP) {
+    each([&](int sd, int ln, int e, int other, uint32_t key) {
+      const int p = s_off[sd][ln] + e;
+      S.out.key[p] = key;
+      S.out.code[p] = static_cast<unsigned short>(other);
+      S.out.line[p] = static_cast<unsigned char>(sd << 7 | ln);
+    });
+    __syncthreads();
+    for (int p = tid; p < total; p += 256) {
+      const int sd = S.out.line[p] >> 7, ln = S.out.line[p] & 127;
+      put((sd ? cbase : rbase) + ln, s_base[sd][ln] + p - s_off[sd][ln], S.out.code[p], S.out.key[p]);
+    }
+  } else {   // (codes of one cluster side by side)
+    each([&](int sd, int ln, int e, int other, uint32_t key) { put((sd ? cbase : rbase) + ln, s_base[sd][ln] + e, other, key); });
   }
 }
 
