@@ -36,7 +36,7 @@ namespace lantern {
 // ---------------------------------------------------------------------------------------
 constexpr int kPlanArrays = 13;  // per-warp arrays of N + 2 ints in shared memory
 
-// One sequence, by one warp; returns the number of its contexts with children, or its fault bits << 16.
+// One sequence of more than 64 drafts, by one warp; returns the number of its contexts with children, or its fault bits << 16.
 __device__ __forceinline__ int plan_sequence(const VerifyParams& P, int* plan_smem, int b, int warp, int lane) {
   const int N = P.N, R = P.R, B = P.B;
   if (b >= B) return 0;
@@ -89,7 +89,7 @@ __device__ __forceinline__ int plan_sequence(const VerifyParams& P, int* plan_sm
     if (P.out_status) P.out_status[b] = status ? status : LANTERN_ST_INTERNAL;
   }
   if (status) {   // the walk reports the fault; no work is queued for this sequence
-    for (int r = lane; r < max(N, 1); r += 32) P.work[static_cast<size_t>(r) * B + b].item = -1;
+    for (int r = lane; r < N; r += 32) P.work[static_cast<size_t>(r) * B + b].item = -1;
     return status << 16;
   }
 
@@ -244,7 +244,6 @@ __device__ __forceinline__ int plan_sequence(const VerifyParams& P, int* plan_sm
       n_ctx += __popc(bal);
     }
   }
-  if (N == 0) n_ctx = 1;
   __syncwarp();         // the shared arrays are complete
   for (int i = lane; i < N; i += 32) {   // the child lists, written by all lanes
     ChildInfo ci = {i, s_tok[i], __int_as_float(s_uni[i]), (din[i + 1] << 16) | siz[i + 1]};
@@ -262,18 +261,190 @@ __device__ __forceinline__ int plan_sequence(const VerifyParams& P, int* plan_sm
                                 __int_as_float(s_uni[f]), u_final, b * R + din[c]};
     }
   }
-  if (N == 0 && lane == 0) P.work[b] = {b, 0, 0, 0, 0, 0.0f, u_final, b};   // no drafts: one draw from the root's q
+  return n_ctx;
+}
+
+// The same for at most 64 drafts, two per lane: sets of nodes are 64-bit masks, so that a context's children, a node's
+// ancestors (by doubling) and the contexts of a level are one word each, and the rest are sums over the bits of a word.
+// A 60-node tree takes 2 us here; the general path above, with its level-by-level passes, 9 us.
+constexpr int PLAN_SMALL = 64;
+struct SmallPlan {
+  unsigned long long kids[PLAN_SMALL + 1];    // children of context c
+  unsigned long long level[PLAN_SMALL + 1];   // nodes of depth d that have children
+  unsigned long long anc[PLAN_SMALL];         // ancestors of node i
+  int jump[PLAN_SMALL];                       // doubling: the nearest ancestor not in anc yet, -1 = none
+  int size[PLAN_SMALL + 1];                   // contexts in the subtree of context c, itself included
+  int weight[PLAN_SMALL];                     // steps in pre-order from a node's parent to the node
+  int start[PLAN_SMALL + 1];                  // where the children of context c begin in the child lists
+  int rank[PLAN_SMALL + 1], span[PLAN_SMALL + 1], tok[PLAN_SMALL];
+  float uni[PLAN_SMALL];
+};
+
+__device__ __forceinline__ int plan_small(const VerifyParams& P, SmallPlan& S, int b, int lane) {
+  const int N = P.N, R = P.R, B = P.B;
+  if (b >= B) return 0;
+  int par[2], tok[2] = {0, 0};
+  float uni[2] = {0.0f, 0.0f}, u_final = 0.0f;
+  // all inputs at once
+#pragma unroll
+  for (int q = 0; q < 2; ++q) {
+    const int i = lane + 32 * q;
+    const size_t o = static_cast<size_t>(b) * N + i;
+    par[q] = i - 1;
+    if (i < N) {
+      tok[q] = P.tokens[o];
+      if (P.parents) par[q] = P.parents[o];
+      if (P.uniforms) uni[q] = P.uniforms[static_cast<size_t>(b) * R + i];
+    }
+  }
+  if (P.uniforms) u_final = P.uniforms[static_cast<size_t>(b) * R + N];
+  for (int c = lane; c <= PLAN_SMALL; c += 32) S.kids[c] = S.level[c] = 0ull, S.size[c] = 1;
+  for (int c = lane; c < R; c += 32) P.dead[static_cast<size_t>(b) * R + c] = 0;
+  const float qnan = __int_as_float(0x7fc00000);
+  int status = u_final >= 0.0f && u_final < 1.0f ? 0 : LANTERN_ST_BAD_UNIFORM;
+#pragma unroll
+  for (int q = 0; q < 2; ++q) {
+    const int i = lane + 32 * q;
+    const size_t o = static_cast<size_t>(b) * N + i;
+    if (i < N) {
+      if (static_cast<unsigned>(tok[q]) >= static_cast<unsigned>(P.V)) status |= LANTERN_ST_BAD_TOKEN;
+      if (par[q] < -1 || par[q] >= i) status |= LANTERN_ST_BAD_PARENT;
+      if (!(uni[q] >= 0.0f && uni[q] < 1.0f)) status |= LANTERN_ST_BAD_UNIFORM;
+      if (P.out_path) P.out_path[o] = -1;
+      if (P.out_qa) P.out_qa[o] = qnan;
+      if (P.out_px) P.out_px[o] = qnan;
+      if (P.out_m) P.out_m[o] = -1;
+    }
+  }
+  status = __reduce_or_sync(kFull, status);
+  if (lane == 0) {   // what stands if the fused pass never gets to the end of this sequence
+    P.out_len[b] = 0;
+    P.out_tok[b] = -1;
+    if (P.out_status) P.out_status[b] = status ? status : LANTERN_ST_INTERNAL;
+  }
+  if (status) {   // no work is queued for this sequence
+    for (int r = lane; r < max(N, 1); r += 32) P.work[static_cast<size_t>(r) * B + b].item = -1;
+    return status << 16;
+  }
+  if (N == 0) {   // no drafts: one draw from the root's q
+    if (lane == 0) {
+      P.records[b].word = kWalkLeaf;
+      P.work[b] = {b, 0, 0, 0, 0, 0.0f, u_final, b};
+    }
+    return 1;
+  }
+  __syncwarp();
+#pragma unroll
+  for (int q = 0; q < 2; ++q) {
+    const int i = lane + 32 * q;
+    if (i < N) {
+      atomicOr(&S.kids[par[q] + 1], 1ull << i);
+      S.anc[i] = par[q] >= 0 ? 1ull << par[q] : 0ull;
+      S.jump[i] = par[q];
+      S.tok[i] = tok[q];
+      S.uni[i] = uni[q];
+    }
+  }
+  __syncwarp();
+  for (;;) {
+    unsigned long long more_anc[2];
+    int to[2];
+    bool more = false;
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+      const int i = lane + 32 * q;
+      const int a = i < N ? S.jump[i] : -1;
+      to[q] = a >= 0 ? S.jump[a] : -1;
+      more_anc[q] = a >= 0 ? S.anc[a] : 0ull;
+      more |= to[q] >= 0;
+    }
+    __syncwarp();
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+      const int i = lane + 32 * q;
+      if (i < N) S.anc[i] |= more_anc[q], S.jump[i] = to[q];
+    }
+    __syncwarp();
+    if (!__any_sync(kFull, more)) break;
+  }
+  unsigned long long anc[2], below[2], with[2];   // ancestors, smaller nodes, earlier siblings
+  int depth[2], kids[2];
+#pragma unroll
+  for (int q = 0; q < 2; ++q) {
+    const int i = lane + 32 * q;
+    const bool on = i < N;
+    anc[q] = on ? S.anc[i] : 0ull;
+    below[q] = (1ull << i) - 1ull;
+    with[q] = on ? S.kids[par[q] + 1] & below[q] : 0ull;
+    depth[q] = __popcll(anc[q]) + 1;
+    kids[q] = on ? __popcll(S.kids[i + 1]) : 0;
+    if (kids[q]) atomicOr(&S.level[depth[q]], 1ull << i);
+    for (unsigned long long m = anc[q]; m; m &= m - 1ull) atomicAdd(&S.size[__ffsll(m)], 1);   // (context of node a: a + 1)
+  }
+  if (lane == 0) S.size[0] = R;
+  __syncwarp();
+#pragma unroll
+  for (int q = 0; q < 2; ++q) {
+    const int i = lane + 32 * q;
+    int w = 1;
+    for (unsigned long long m = with[q]; m; m &= m - 1ull) w += S.size[__ffsll(m)];
+    if (i < N) S.weight[i] = w;
+  }
+  // child lists in the order of the contexts
+  const int n_root = __popcll(S.kids[0]);
+  int carry = n_root, n_ctx = 1;
+#pragma unroll
+  for (int q = 0; q < 2; ++q) {
+    const int i = lane + 32 * q;
+    int incl = kids[q];
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int t = __shfl_up_sync(kFull, incl, o);
+      if (lane >= o) incl += t;
+    }
+    if (i < N) S.start[i + 1] = carry + incl - kids[q];
+    carry += __shfl_sync(kFull, incl, 31);
+    n_ctx += __popc(__ballot_sync(kFull, kids[q] > 0));
+  }
+  if (lane == 0) S.start[0] = 0, S.rank[0] = 0, S.span[0] = R;
+  __syncwarp();
+#pragma unroll
+  for (int q = 0; q < 2; ++q) {
+    const int i = lane + 32 * q;
+    if (i < N) {
+      int pos = S.weight[i], rank = 1;                   // pre-order position; breadth-first rank, where it has children
+      for (unsigned long long m = anc[q]; m; m &= m - 1ull) pos += S.weight[__ffsll(m) - 1];
+      for (int d = 1; d < depth[q]; ++d) rank += __popcll(S.level[d]);
+      S.rank[i + 1] = rank + __popcll(S.level[depth[q]] & below[q]);
+      S.span[i + 1] = pos << 16 | S.size[i + 1];
+      const ChildInfo info = {i, tok[q], uni[q], pos << 16 | S.size[i + 1]};
+      P.children[static_cast<size_t>(b) * N + S.start[par[q] + 1] + __popcll(with[q])] = info;
+    }
+  }
+  __syncwarp();
+  for (int r = n_ctx + lane; r < N; r += 32) P.work[static_cast<size_t>(r) * B + b].item = -1;
+  for (int c = lane; c < R; c += 32) {
+    const unsigned long long m = S.kids[c];
+    P.records[static_cast<size_t>(b) * R + c].word = m == 0ull ? kWalkLeaf : (c == 0 ? kWalkWaiting : kWalkPending);
+    if (m) {
+      const int f = __ffsll(m) - 1;                      // its first child
+      P.work[static_cast<size_t>(S.rank[c]) * B + b] = {b * R + c, b * N + S.start[c], __popcll(m) << 16 | f, S.span[f + 1], S.tok[f],
+                                                        S.uni[f], u_final, b * R + (S.span[c] >> 16)};
+    }
+  }
   return n_ctx;
 }
 
 __global__ void __launch_bounds__(PLAN_WARPS * 32) lantern_plan_kernel(VerifyParams P) {
   extern __shared__ int plan_smem[];
   __shared__ int s_words[PLAN_WARPS];
+  __shared__ SmallPlan s_small[PLAN_WARPS];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   grid_dependency_wait();
   grid_dependents_launch();
   if (blockIdx.x == 0 && threadIdx.x < 64) reinterpret_cast<int*>(P.counters)[threadIdx.x] = 0;
-  const int word = plan_sequence(P, plan_smem, blockIdx.x * PLAN_WARPS + warp, warp, lane);
+  const int b = blockIdx.x * PLAN_WARPS + warp;
+  const int word = P.N <= PLAN_SMALL ? plan_small(P, s_small[warp], b, lane) : plan_sequence(P, plan_smem, b, warp, lane);
   if (lane == 0) s_words[warp] = word;
   __syncthreads();
   if (threadIdx.x == 0) {
@@ -530,9 +701,9 @@ static lantern_status verify_impl(const void* target_logits, const void* draft_l
   const int sms = sm_count();
   if (sms < 1) return LANTERN_E_CUDA;
 
-  const size_t plan_smem = static_cast<size_t>(PLAN_WARPS) * kPlanArrays * (N + 2) * sizeof(int);
+  const size_t plan_smem = N <= PLAN_SMALL ? 0 : static_cast<size_t>(PLAN_WARPS) * kPlanArrays * (N + 2) * sizeof(int);
   static DeviceFlags plan_ready;
-  if (plan_smem > 48 * 1024 &&
+  if (plan_smem > 32 * 1024 &&   // (beside the kernel's static part)
       allow_shared_memory(lantern_plan_kernel, PLAN_WARPS * kPlanArrays * (MAX_N + 2) * sizeof(int), plan_ready) != cudaSuccess)
     return LANTERN_E_CUDA;
   if (launch_dependent(lantern_plan_kernel, (B + PLAN_WARPS - 1) / PLAN_WARPS, PLAN_WARPS * 32, plan_smem, st, P) != cudaSuccess)

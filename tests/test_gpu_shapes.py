@@ -47,3 +47,15 @@ def test_calls_without_drafts():
         edge = np.abs(cdf - u[:, None]).min(axis=1) / cdf[:, -1] < 1e-6
         assert np.array_equal(out.next_token.cpu().numpy()[~edge], want[~edge]) and edge.sum() <= max(1, B // 50)
         assert not out.status.any() and not out.accept_len.any()
+
+
+@pytest.mark.parametrize("N,depth", [(1, 1), (63, 9), (64, 30), (65, 30), (64, 2)])
+def test_plan_paths_against_oracle(N, depth):
+    """Up to 64 drafts the plan works on 64-bit sets of nodes, beyond that level by level."""
+    B, V = 9, 512
+    par = li.tree_parents(B, N, depth=depth, seed=N)
+    inp = li.verify_inputs(B, N, V, dtype=li.BF16, has_uncond=True, cfg_scale=2.0, rho=0.9, sigma_draft=0.5, parents=par, seed=N + depth)
+    host, dev = tables(li.codebook_gaussian(V, 8, seed=16), 40, inp.draft_tokens)
+    res = compare(inp, host, 0.3, run_gpu(inp, dev, 0.3))
+    assert_parity(res)
+    assert res["near"] <= near_ceiling(B)
