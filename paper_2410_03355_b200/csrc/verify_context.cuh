@@ -322,6 +322,9 @@ __global__ void __launch_bounds__(SHAPE::THREADS, SHAPE::CTAS) lantern_context_k
   constexpr int NP = CH / CP;                 // slices per thread
   constexpr int LOG_CP = CP == 2 ? 1 : 0;
   constexpr int AHEAD = BF16 ? (CH < 4 ? CH : 4) : (CH < 2 ? CH : 2);   // drafter groups in flight in a residual pass
+  // Few registers hold this thread's part of the drafter row, or there are registers enough: it is kept for the residual passes
+  // (which else read it again, a round trip to L2 per rejection).
+  constexpr bool HOLD = CH * (BF16 ? 4 : 8) <= 8 || (GT == 512 && SHAPE::CTAS == 1);
   static_assert(NP * GT <= 1024 && CH * GW <= 64, "tables of slices and blocks");
   extern __shared__ __align__(128) unsigned char smem[];
   __shared__ GroupShared<GW, TOPK> SG[NGRP];
@@ -738,7 +741,7 @@ __global__ void __launch_bounds__(SHAPE::THREADS, SHAPE::CTAS) lantern_context_k
     auto shift_of = [&](int p) { return NP <= 2 ? nq[NP <= 2 ? p : 0] : S.slice[p * GT + gt]; };
     float z_max = ninf;               // GREEDY: this thread's largest logit
     float nq_max = 0.0f, sq = 1.0f;   // target: the largest shift of the slices; the sum, in its units
-    Raw8<BF16> raw[CH];           // the drafter row (dead after the reduction below)
+    Raw8<BF16> raw[CH];           // the drafter row
     auto load_drafter = [&](auto whole) {
 #pragma unroll
       for (int c = 0; c < CH; ++c) {
@@ -1108,10 +1111,12 @@ __global__ void __launch_bounds__(SHAPE::THREADS, SHAPE::CTAS) lantern_context_k
         // ---- rejected: residual [q_{k,delta}(.|D = x~) - p]_+ ----
         // the first drafter logits: asked for at once, in flight while A is flagged and across the barrier
         Raw8<BF16> ahead[AHEAD];
+        if (!HOLD) {
 #pragma unroll
-        for (int c = 0; c < AHEAD; ++c) {
-          const int g = c * GT + gt;
-          ahead[c] = load_raw8<BF16>(drow, g * 8 < V ? g : 0);
+          for (int c = 0; c < AHEAD; ++c) {
+            const int g = c * GT + gt;
+            ahead[c] = load_raw8<BF16>(drow, g * 8 < V ? g : 0);
+          }
         }
         // members of A (x~ included) leave no residual mass: flag them with a negative sign
         for (int base = 0; base <= m; base += SLOTS * GT) {
@@ -1153,8 +1158,8 @@ __global__ void __launch_bounds__(SHAPE::THREADS, SHAPE::CTAS) lantern_context_k
           const uint64_t nr2 = pack2(-ratio, -ratio), nn2 = pack2(-nd, -nd);
 #pragma unroll
           for (int c = p * CP; c < (p + 1) * CP; ++c) {
-            const Raw8<BF16> raw = ahead[c % AHEAD];
-            if (c + AHEAD < CH) {   // the next groups travel during this one
+            const Raw8<BF16> drafted = HOLD ? raw[c] : ahead[c % AHEAD];
+            if (!HOLD && c + AHEAD < CH) {   // the next groups travel during this one
               const int g = (c + AHEAD) * GT + gt;
               ahead[c % AHEAD] = load_raw8<BF16>(drow, g * 8 < V ? g : 0);
             }
@@ -1163,7 +1168,7 @@ __global__ void __launch_bounds__(SHAPE::THREADS, SHAPE::CTAS) lantern_context_k
               float z[8];
               {
                 uint64_t z2[4];
-                raw8_pairs<BF16>(raw, z2);
+                raw8_pairs<BF16>(drafted, z2);
 #pragma unroll
                 for (int i = 0; i < 4; ++i) {
                   if (!TONE) z2[i] = divide_T(z2[i]);
