@@ -20,6 +20,7 @@
 #include <cuda_runtime.h>
 #include <math.h>
 #include <stdint.h>
+#include <type_traits>
 
 #include "lantern.h"
 #include "lantern_device.cuh"
@@ -174,6 +175,10 @@ __global__ void __launch_bounds__(256, 2) lantern_distance_tile_kernel(DistParam
   __shared__ __align__(16) float Bs[DK][TM];
   const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
   const int V = P.V, cols = P.cols;
+  grid_dependency_wait();
+  // Not where whole tables are made block by block: CTAs put in place early take the SMs that a short grid leaves free, and
+  // the grid after them is then crowded onto a few (V = 1500, D = 256: 117 -> 150 us).
+  if (P.sample || P.count) grid_dependents_launch();
   const int row_end = P.count ? min(P.row_end, *P.count) : P.row_end;
   const int rbase = P.row0 + blockIdx.y * TM, cbase = blockIdx.x * TM;
   if (rbase >= row_end) return;
@@ -240,6 +245,8 @@ static int list_room(int region, int k, bool dist, int cap) {
 
 // Bound of every row from its sampled keys (scratch[i, 0..SAMPLE)), which its list's counter replaces; one warp per row.
 __global__ void __launch_bounds__(256) lantern_row_bound_kernel(ListParams L, int want) {
+  grid_dependency_wait();
+  grid_dependents_launch();
   const int i = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
   if (i >= L.V) return;
   const uint32_t* src = reinterpret_cast<const uint32_t*>(L.scratch) + static_cast<size_t>(i) * SAMPLE;
@@ -292,6 +299,8 @@ __global__ void __launch_bounds__(256, 2) lantern_distance_lists_kernel(const fl
   __shared__ int s_n[2][TM], s_off[2][TM], s_base[2][TM], s_warp[8];
   const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4, lane = tid & 31;
   const int side = tid >> 7, line = tid & 127;
+  grid_dependency_wait();
+  grid_dependents_launch();
   const int V = L.V;
   // tile (tr, tc) with tr <= tc, numbered column by column: tc (tc + 1) / 2 + tr
   int tc = static_cast<int>((sqrtf(8.0f * static_cast<float>(blockIdx.x) + 1.0f) - 1.0f) * 0.5f);
@@ -395,10 +404,18 @@ __global__ void __launch_bounds__(256, 2) lantern_distance_lists_kernel(const fl
   }
 }
 
-// the rows whose lists failed (marked by idx[i, 0] = -1), in any order
-__global__ void lantern_failed_rows_kernel(const int32_t* idx, int V, int k, int* rows, int* count) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < V && idx[static_cast<size_t>(i) * k] < 0) rows[atomicAdd(count, 1)] = i;
+// the rows whose lists failed (marked by idx[i, 0] = -1), in any order; one CTA
+__global__ void __launch_bounds__(1024) lantern_failed_rows_kernel(const int32_t* idx, int V, int k, int* rows, int* count) {
+  __shared__ int s_n;
+  grid_dependency_wait();
+  grid_dependents_launch();
+  if (threadIdx.x == 0) s_n = 0;
+  __syncthreads();
+#pragma unroll 8
+  for (int i = threadIdx.x; i < V; i += 1024)
+    if (idx[static_cast<size_t>(i) * k] < 0) rows[atomicAdd(&s_n, 1)] = i;
+  __syncthreads();
+  if (threadIdx.x == 0) *count = s_n;
 }
 
 // ---------------------------------------------------------------------------------------
@@ -640,13 +657,14 @@ static __host__ __device__ constexpr size_t row_bytes(int cap) {
 }
 
 // R rows per CTA of KT threads; KT / R threads rank a row.  FROM: where the keys come from -- computed here (small D), read
-// from scratch rows, or already on lists.
+// from scratch rows, or already on lists.  ALL: every key is kept, so there is neither sample nor bound, and the
+// bins cover the range that the keys turn out to have.
 //
 // What bounds it (V = 16384, k = 1000, cycles of a CTA of eight rows, D = 8): the key pass 40 k, of which the fp32
 // pipes need 16 k and instruction issue 24 k; sample and bound 9 k; counting sort 13 k; ranking 11 k.
 // 0.55 ms per table; 1.20 ms when a CTA selected from all keys of one row (73 k warp instructions per row, now 26 k).
 enum { FROM_CODES = 0, FROM_SCRATCH = 1, FROM_LISTS = 2 };
-template <int KT, int R, int FROM>
+template <int KT, int R, int FROM, bool ALL>
 __global__ void __launch_bounds__(KT, 1024 / KT) lantern_knn_rows_kernel(BuildParams P, ListParams L, int P2) {
   constexpr bool SCRATCH = FROM == FROM_SCRATCH, LISTS = FROM == FROM_LISTS;
   constexpr int RT = KT / R;         // threads of a row's team
@@ -663,6 +681,8 @@ __global__ void __launch_bounds__(KT, 1024 / KT) lantern_knn_rows_kernel(BuildPa
   __shared__ uint32_t s_low[R][3 * RW], s_most[R][RW];
   const int tid = threadIdx.x, lane = tid & 31;
   const int V = P.V, D = P.D, k = P.k, cap = P.cap;
+  grid_dependency_wait();
+  if (LISTS || P.count) grid_dependents_launch();   // (see lantern_distance_tile_kernel)
   const int row0 = P.row0 + blockIdx.x * R, row_end = P.count ? min(P.row_end, *P.count) : P.row_end;
   if (row0 >= row_end) return;
   const bool vec = (D & 3) == 0;
@@ -685,7 +705,7 @@ __global__ void __launch_bounds__(KT, 1024 / KT) lantern_knn_rows_kernel(BuildPa
   const int i = on && P.map ? P.map[row0 + r] : row0 + r;
   auto team = [&]() { asm volatile("bar.sync %0, %1;" ::"r"(1 + r), "n"(RT) : "memory"); };
   // ---- 1. the bound, from SAMPLE keys ----
-  if constexpr (!LISTS) {
+  if constexpr (!LISTS && !ALL) {
     uint32_t key[SMP];
     if constexpr (SCRATCH) {
       const uint32_t* src = P.scratch + static_cast<size_t>(on ? local : 0) * V;
@@ -738,29 +758,26 @@ __global__ void __launch_bounds__(KT, 1024 / KT) lantern_knn_rows_kernel(BuildPa
     most = 0u;
 #pragma unroll
     for (int w = 0; w < RW; ++w) most = s_most[r][w] > most ? s_most[r][w] : most;
-    uint32_t t = 0x7f800000u;
-    if (P.want > 0) {
-      // bisection on the sampled values: count(key <= hi) >= want > count(key <= lo); a few more than wanted will do
-      const int room = P.want / 16 + 2;
-      uint32_t lo = 0u, hi = most;
-      for (int pass = 0; pass < 48 && hi - lo > 1u; ++pass) {
-        uint32_t m = __float_as_uint(0.5f * __uint_as_float(lo) + 0.5f * __uint_as_float(hi));
-        if (!(m > lo && m < hi)) m = lo + ((hi - lo) >> 1);
-        int c = 0;
+    // bisection on the sampled values: count(key <= hi) >= want > count(key <= lo); a few more than wanted will do
+    const int room = P.want / 16 + 2;
+    uint32_t lo = 0u, hi = most;
+    for (int pass = 0; pass < 48 && hi - lo > 1u; ++pass) {
+      uint32_t m = __float_as_uint(0.5f * __uint_as_float(lo) + 0.5f * __uint_as_float(hi));
+      if (!(m > lo && m < hi)) m = lo + ((hi - lo) >> 1);
+      int c = 0;
 #pragma unroll
-        for (int q = 0; q < SMP; ++q) c += key[q] <= m;
-        c = __reduce_add_sync(kFull, c);
-        if (lane == 0) s_vote[pass & 1][r][wv] = c;
-        team();
-        c = 0;
+      for (int q = 0; q < SMP; ++q) c += key[q] <= m;
+      c = __reduce_add_sync(kFull, c);
+      if (lane == 0) s_vote[pass & 1][r][wv] = c;
+      team();
+      c = 0;
 #pragma unroll
-        for (int w = 0; w < RW; ++w) c += s_vote[pass & 1][r][w];
-        if (c >= P.want) hi = m;
-        else lo = m;
-        if (c >= P.want && c <= P.want + room) break;
-      }
-      t = hi;
+      for (int w = 0; w < RW; ++w) c += s_vote[pass & 1][r][w];
+      if (c >= P.want) hi = m;
+      else lo = m;
+      if (c >= P.want && c <= P.want + room) break;
     }
+    const uint32_t t = hi;
     if (rt < 32) {
       uint32_t low = 0u, mine = lane < 3 * RW ? s_low[r][lane] : 0xffffffffu;
       for (int q = 0; q < 3; ++q) {
@@ -782,7 +799,7 @@ __global__ void __launch_bounds__(KT, 1024 / KT) lantern_knn_rows_kernel(BuildPa
   if constexpr (FROM == FROM_CODES) {
     float t_row[R];
 #pragma unroll
-    for (int q = 0; q < R; ++q) t_row[q] = s_t[q];
+    for (int q = 0; q < R; ++q) t_row[q] = ALL ? 0.0f : s_t[q];
     for (int base = 0; base < V; base += U * KT) {
       unsigned long long acc[U][R / 2];
       const float* b[U];
@@ -837,6 +854,19 @@ __global__ void __launch_bounds__(KT, 1024 / KT) lantern_knn_rows_kernel(BuildPa
             for (int q = 0; q < R / 2; ++q) acc[u][q] = 0x7fffffff7fffffffull;
           }
       }
+      if constexpr (ALL) {
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          const int j = base + u * KT + tid;
+          if (j < V) {
+#pragma unroll
+            for (int q = 0; q < R; ++q)
+              list_of(q)[j] = (static_cast<unsigned long long>(static_cast<uint32_t>(q & 1 ? acc[u][q / 2] >> 32 : acc[u][q / 2])) << 32) |
+                              static_cast<unsigned>(j + 1);
+          }
+        }
+        continue;
+      }
       // How many of this thread's keys each row keeps, four rows to a word (at most U each, 32 U per warp), and a
       // prefix over the warp; then one counter update per row and warp.  (Ballots and population counts in
       // their place kept the XU pipe busy for 24 of the pass's 51 thousand cycles.)
@@ -879,7 +909,7 @@ __global__ void __launch_bounds__(KT, 1024 / KT) lantern_knn_rows_kernel(BuildPa
         }
       }
     }
-  } else if (SCRATCH && on) {   // each team reads its own row of keys, W groups of four per thread at a time
+  } else if (SCRATCH && on && !ALL) {   // each team reads its own row of keys, W groups of four per thread at a time
     constexpr int W = 4;
     const uint32_t* src = P.scratch + static_cast<size_t>(local) * V;
     const float t = s_t[r];
@@ -936,10 +966,12 @@ __global__ void __launch_bounds__(KT, 1024 / KT) lantern_knn_rows_kernel(BuildPa
   if (on) {
     unsigned long long* list = list_of(r);
     unsigned* bins = bins_of(r);
-    const int n = LISTS ? *L.counter(i) : s_cnt[r];
+    const int n = LISTS ? *L.counter(i) : (ALL ? V : s_cnt[r]);
+    const uint32_t* row = SCRATCH ? P.scratch + static_cast<size_t>(local) * V : nullptr;
     float lo = 0.0f, scale = 0.0f;
     uint32_t key[KEEP], who[KEEP];    // this thread's entries: the key; index + 1 and place of arrival in its bin
-    if (!LISTS) lo = s_lo[r], scale = s_scale[r];
+    constexpr bool ranged = LISTS || ALL;   // the range of the bins comes from the entries themselves
+    if (!ranged) lo = s_lo[r], scale = s_scale[r];
     auto bin_of = [&](uint32_t key) {   // monotone in the key
       // the square: near the bound the keys lie closer together (distances in D dimensions grow like the D/2-th root)
       const float x = fmaxf(__uint_as_float(key) - lo, 0.0f) * scale;
@@ -951,14 +983,14 @@ __global__ void __launch_bounds__(KT, 1024 / KT) lantern_knn_rows_kernel(BuildPa
     } else {
 #pragma unroll
       for (int q = 0; q < OWN; ++q) bins[q * RT + rt] = 0u;
-      if constexpr (LISTS) {            // read the list; its range (without the code itself) is where the bins go
+      if (ranged) {                     // read the list; its range (without the code itself) is where the bins go
         uint32_t least = 0xffffffffu, most = 0u;
 #pragma unroll
         for (int q = 0; q < KEEP; ++q) {
           const int e = q * RT + rt;
           if (e < n) {
-            key[q] = *L.key(i, e);
-            who[q] = L.index(i)[e] + 1u;
+            key[q] = LISTS ? *L.key(i, e) : (SCRATCH ? __ldcs(row + e) : static_cast<uint32_t>(list[e] >> 32));
+            who[q] = LISTS ? L.index(i)[e] + 1u : static_cast<uint32_t>(e + 1);
             if (who[q] != static_cast<uint32_t>(i + 1)) {
               least = key[q] < least ? key[q] : least;
               most = key[q] > most ? key[q] : most;
@@ -970,7 +1002,7 @@ __global__ void __launch_bounds__(KT, 1024 / KT) lantern_knn_rows_kernel(BuildPa
         if (lane == 0) s_low[r][rt >> 5] = least, s_most[r][rt >> 5] = most;
       }
       team();
-      if constexpr (LISTS) {
+      if (ranged) {
         uint32_t least = 0xffffffffu, most = 0u;
 #pragma unroll
         for (int w = 0; w < RW; ++w) {
@@ -979,12 +1011,13 @@ __global__ void __launch_bounds__(KT, 1024 / KT) lantern_knn_rows_kernel(BuildPa
         }
         lo = __uint_as_float(least);
         scale = most > least ? 1.0f / (__uint_as_float(most) - lo) : 0.0f;
+        if (most > 0x7f800000u) s_slow[r] = 1;   // NaN
       }
 #pragma unroll
       for (int q = 0; q < KEEP; ++q) {
         const int e = q * RT + rt;
         if (e < n) {
-          if (!LISTS) {
+          if (!ranged) {
             const unsigned long long c = list[e];
             key[q] = static_cast<uint32_t>(c >> 32);
             who[q] = static_cast<uint32_t>(c);
@@ -1073,13 +1106,31 @@ static int rows_per_block(int V) {
   return (r + TM - 1) / TM * TM;
 }
 
-template <int KT, int R, int FROM>
+// A launch that may be put in place while the kernel before it on the stream drains.  A build is a chain of short launches --
+// two per block of rows, most of them without work where they only redo failed rows (38 at V = 16384) -- and every kernel
+// waits (grid_dependency_wait) before it reads.  D = 256, k = 1000: V = 16384 3174 -> 3088 us, with k = 25 V = 4096 377 -> 348.
+// First: nothing of the chain lies before it.
+template <class... Arg>
+static cudaError_t launch_chained(bool first, void (*kernel)(Arg...), dim3 grid, int threads, size_t smem, cudaStream_t st, Arg... arg) {
+  cudaLaunchAttribute attr = {};
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t c = {};
+  c.gridDim = grid;
+  c.blockDim = dim3(threads);
+  c.dynamicSmemBytes = smem;
+  c.stream = st;
+  c.attrs = &attr;
+  c.numAttrs = first ? 0 : 1;
+  return cudaLaunchKernelEx(&c, kernel, arg...);
+}
+
+template <int KT, int R, int FROM, bool ALL = false>
 static cudaError_t launch_rows(const BuildParams& P, int P2, size_t smem, cudaStream_t st, const ListParams& L = {}) {
-  auto kk = lantern_knn_rows_kernel<KT, R, FROM>;
+  auto kk = lantern_knn_rows_kernel<KT, R, FROM, ALL>;
   const cudaError_t e = cudaFuncSetAttribute(kk, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
   if (e != cudaSuccess) return e;
-  kk<<<(P.row_end - P.row0 + R - 1) / R, KT, smem, st>>>(P, L, P2);
-  return cudaGetLastError();
+  return launch_chained(FROM == FROM_CODES, kk, dim3((P.row_end - P.row0 + R - 1) / R), KT, smem, st, P, L, P2);
 }
 
 }  // namespace lantern
@@ -1117,11 +1168,13 @@ extern "C" lantern_status lantern_build_neighbors(const float* codebook, int V, 
   P.map = P.count = nullptr;
   // The k-th smallest of V keys has rank k SAMPLE / V in the sample, with a binomial spread; 3.5 standard deviations
   // above that the bound fails one row in some thousands, and the list is as long as the kept keys may be with the same
-  // margin.  Few codes: the bound would keep most of them anyway.
+  // margin.  Few codes: every key is kept and sorted.  The line: where keys are computed here a sample costs as
+  // much as the keys it stands for (V = 2048, D = 16, k = 25: 34 us per table without one, 38 with it), and a team's registers
+  // hold 2304 keys; where they are read the sample is cheap and sorting all is not (V = 2048, D = 40: 50 and 48 us).
   const double f = static_cast<double>(SAMPLE) / V, mean = k * f, sd = sqrt(mean * (1.0 - static_cast<double>(k) / V));
   const int want = static_cast<int>(mean + 3.5 * sd) + 3, most = want + want / 16 + 2;
   const double kept = (most + 3.5 * sqrt(static_cast<double>(most))) / f;
-  P.want = (V <= 2 * SAMPLE || kept >= V) ? 0 : want;
+  P.want = (V <= (D > SMALL_D ? SAMPLE : KEEP * 128) || kept >= V) ? 0 : want;
   P.cap = P.want ? (static_cast<int>(kept) + 7) & ~7 : V;
   // As many rows per CTA as their lists leave room for (and a team's registers hold): eight rows share every load of a
   // code.  The longest list, 7264 entries at V = 32768 and k = 4097, leaves room for two.  Rows read from
@@ -1130,20 +1183,28 @@ extern "C" lantern_status lantern_build_neighbors(const float* codebook, int V, 
   const int kt = P.scratch ? 512 : 1024;
   auto fits = [&](int R) { return R * per_row <= kRowSmem && P.cap <= KEEP * (1024 / R); };
   const int R = fits(8) ? 8 : (fits(4) ? 4 : 2);   // per 1024 threads
-  // Few codes: small CTAs of two rows, four to an SM, so that every SM has work in one wave (V = 1024: 25 us per table, host
-  // included, against 36 with eight rows per CTA).
-  const bool few = !P.scratch && V <= 2304 && fits(8);
+  // Few codes: small CTAs of two rows, four to an SM, so that the last wave is not mostly empty (V = 2400, D = 8, k = 25: 40 us
+  // per table, 50 with eight rows per CTA; from scratch V = 2693, D = 40: 107 and 110).  Two rows share a code's
+  // loads where eight could, which costs more the longer the codes are: D = 12 43 and 54 us, D = 16 68 and 65, D = 32 190 and 105;
+  // at D = 8 the two shapes meet at V = 3600 (73 and 69).
+  const bool few = (P.scratch ? V <= 4096 : D <= 12 && V <= 3072) && fits(8);
   const size_t rows_smem = few ? 2 * per_row : R * per_row * kt / 1024;
   const size_t smem = rows_smem > general ? rows_smem : general;
   if (smem > kRowSmem || P.cap > KEEP * (1024 / R)) return LANTERN_E_SHAPE;
-  auto select = [&]() {
+  auto with = [&](auto all) {
+    constexpr bool ALL = decltype(all)::value;
+    if (few) {
+      return P.scratch ? launch_rows<256, 2, FROM_SCRATCH, ALL>(P, P2, smem, st) : launch_rows<256, 2, FROM_CODES, ALL>(P, P2, smem, st);
+    }
     if (P.scratch)
-      return R == 8 ? launch_rows<512, 4, FROM_SCRATCH>(P, P2, smem, st)
-                    : (R == 4 ? launch_rows<512, 2, FROM_SCRATCH>(P, P2, smem, st) : launch_rows<512, 1, FROM_SCRATCH>(P, P2, smem, st));
-    if (few) return launch_rows<256, 2, FROM_CODES>(P, P2, smem, st);
-    return R == 8 ? launch_rows<1024, 8, FROM_CODES>(P, P2, smem, st)
-                  : (R == 4 ? launch_rows<1024, 4, FROM_CODES>(P, P2, smem, st) : launch_rows<1024, 2, FROM_CODES>(P, P2, smem, st));
+      return R == 8 ? launch_rows<512, 4, FROM_SCRATCH, ALL>(P, P2, smem, st)
+                    : (R == 4 ? launch_rows<512, 2, FROM_SCRATCH, ALL>(P, P2, smem, st)
+                              : launch_rows<512, 1, FROM_SCRATCH, ALL>(P, P2, smem, st));
+    return R == 8 ? launch_rows<1024, 8, FROM_CODES, ALL>(P, P2, smem, st)
+                  : (R == 4 ? launch_rows<1024, 4, FROM_CODES, ALL>(P, P2, smem, st)
+                            : launch_rows<1024, 2, FROM_CODES, ALL>(P, P2, smem, st));
   };
+  auto select = [&]() { return P.want > 0 ? with(std::false_type()) : with(std::true_type()); };
   DistParams T = {};
   T.cb = codebook;
   T.out = static_cast<uint32_t*>(workspace);
@@ -1154,8 +1215,7 @@ extern "C" lantern_status lantern_build_neighbors(const float* codebook, int V, 
     T.row0 = row0;
     T.row_end = row_end;
     const dim3 grid((T.cols + TM - 1) / TM, (row_end - row0 + TM - 1) / TM);
-    lantern_distance_tile_kernel<<<grid, 256, 0, st>>>(T);
-    return cudaGetLastError();
+    return launch_chained(row0 == 0 && !T.map, lantern_distance_tile_kernel, grid, 256, 0, st, T);
   };
   // all rows, or the codes of P.map, a block of rows at a time
   auto by_blocks = [&](int block) {
@@ -1170,7 +1230,10 @@ extern "C" lantern_status lantern_build_neighbors(const float* codebook, int V, 
   if (!P.scratch) return by_blocks(V) == cudaSuccess ? LANTERN_OK : LANTERN_E_CUDA;
 
   // Every pair once, through lists, where the lists fit with 2.3 to 2.7 standard deviations of room: a row in some hundreds
-  // overflows its list and is done again from all its keys.
+  // overflows its list and is done again from all its keys.  Half the distances (V^2 D) are saved, some 2 k entries per row go
+  // through memory instead (V k): with k = 500, D = 40, lists / blocks of rows take 115 / 108 us at V = 2693, 165 / 145 at 4096,
+  // 240 / 228 at 5000 and 253 / 279 at 6000; with D = 100, 156 / 159 at 2693 and 222 / 225 at 4096.  Below 2304 codes the
+  // sample is half of them (V = 2048, D = 40, k = 25: 68 / 48).
   ListParams L;
   L.scratch = static_cast<unsigned char*>(workspace);
   L.idx = idx;
@@ -1181,16 +1244,17 @@ extern "C" lantern_status lantern_build_neighbors(const float* codebook, int V, 
   L.cap = static_cast<int>((most + 2.7 * sqrt(static_cast<double>(most))) / f) & ~1;
   const int least = static_cast<int>((most + 2.3 * sqrt(static_cast<double>(most))) / f);
   while (L.cap > least && list_room(L.region, k, dist != nullptr, L.cap) < L.cap) L.cap -= 2;
-  if (V >= 4096 && P.want > 0 && R == 8 && L.cap > least && L.cap >= k && L.cap <= P.cap) {
+  const bool pays = V > 2304 && static_cast<long long>(V) * D >= 450ll * k;
+  if (pays && P.want > 0 && R == 8 && L.cap > least && L.cap >= k && L.cap <= P.cap) {
     T.sample = 1;
     T.cols = T.pitch = SAMPLE;
     cudaError_t e = distances(0, V);
     if (e != cudaSuccess) return LANTERN_E_CUDA;
-    lantern_row_bound_kernel<<<(V + 7) / 8, 256, 0, st>>>(L, P.want);
-    if (cudaGetLastError() != cudaSuccess) return LANTERN_E_CUDA;
+    e = launch_chained(false, lantern_row_bound_kernel, dim3((V + 7) / 8), 256, 0, st, L, P.want);
+    if (e != cudaSuccess) return LANTERN_E_CUDA;
     const int t = (V + TM - 1) / TM;
-    lantern_distance_lists_kernel<<<t * (t + 1) / 2, 256, 0, st>>>(codebook, D, L);
-    if (cudaGetLastError() != cudaSuccess) return LANTERN_E_CUDA;
+    e = launch_chained(false, lantern_distance_lists_kernel, dim3(t * (t + 1) / 2), 256, 0, st, codebook, D, L);
+    if (e != cudaSuccess) return LANTERN_E_CUDA;
     const int cap = P.cap;
     P.row0 = 0;
     P.row_end = V;
@@ -1202,9 +1266,8 @@ extern "C" lantern_status lantern_build_neighbors(const float* codebook, int V, 
     const int block = rows_per_block(V) - TM;
     int* rows = reinterpret_cast<int*>(static_cast<uint32_t*>(workspace) + static_cast<size_t>(block) * V);
     int* count = rows + V;
-    if (cudaMemsetAsync(count, 0, sizeof(int), st) != cudaSuccess) return LANTERN_E_CUDA;
-    lantern_failed_rows_kernel<<<(V + 255) / 256, 256, 0, st>>>(idx, V, k, rows, count);
-    if (cudaGetLastError() != cudaSuccess) return LANTERN_E_CUDA;
+    e = launch_chained(false, lantern_failed_rows_kernel, dim3(1), 1024, 0, st, static_cast<const int32_t*>(idx), V, k, rows, count);
+    if (e != cudaSuccess) return LANTERN_E_CUDA;
     P.map = T.map = rows;
     P.count = T.count = count;
     T.sample = 0;

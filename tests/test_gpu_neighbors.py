@@ -143,3 +143,30 @@ def test_lists_exact(V, D, k, kind, with_dist):
     assert np.array_equal(gi[:, 0], np.arange(V))
     srt = np.sort(gi, axis=1)
     assert np.all(srt[:, 1:] != srt[:, :-1])
+
+
+# few codes: every key kept or a sampled bound, CTAs of two rows or of eight, lists or blocks of rows -- each line from both sides
+@pytest.mark.parametrize("V,D,k", [
+    (1024, 40, 500), (1025, 40, 500), (2304, 12, 2304), (2305, 12, 40), (2304, 13, 700), (2305, 13, 700), (3072, 8, 500), (3073, 8, 500),
+    (2304, 64, 100), (2305, 64, 100), (2560, 45, 256), (2560, 45, 257), (4096, 33, 500), (4097, 33, 500)])
+@pytest.mark.parametrize("kind", ["sphere", "ties", "nan"])
+def test_few_codes_exact(V, D, k, kind):
+    cb = li.codebook_integer(V, D, lo=0, hi=2, seed=3) if kind == "ties" else li.codebook_gaussian(V, D, seed=4)
+    if kind == "nan":       # such a code is nobody's neighbour as long as there are others; which rows differ is not looked at
+        cb[V // 2, 0] = np.nan
+        if k == V:
+            pytest.skip("every code is asked for")
+    idx, dist = lt.build_neighbors(torch.from_numpy(cb).cuda(), k)
+    torch.cuda.synchronize()
+    rows = np.unique(np.concatenate([np.arange(9), np.arange(V - 9, V), np.random.default_rng(1).integers(0, V, 12)])).astype(np.int32)
+    rows = rows[rows != V // 2]
+    gi, gd = idx.cpu().numpy()[rows], dist.cpu().numpy()[rows]
+    if kind == "nan":
+        assert not np.any(gi == V // 2)
+        other = np.delete(cb, V // 2, axis=0)
+        oi, od = oracle.build_neighbors(other, k, rows=(rows - (rows > V // 2)).astype(np.int32))
+        oi = oi + (oi >= V // 2)
+    else:
+        oi, od = oracle.build_neighbors(cb, k, rows=rows)
+    assert np.array_equal(gi, oi)
+    assert np.array_equal(gd.view(np.uint32), od.view(np.uint32))
