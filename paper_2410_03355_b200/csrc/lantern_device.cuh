@@ -37,42 +37,14 @@ __device__ __forceinline__ double warp_incl_scan(double v, int lane) {
 //   f(S) = 1/2 [ S ln 2 + q0 ln(1 - x) + (q0 + S) ln(1 + x) ],   x = S / (2 q0 + S),
 // since (q0 + S) / mid = 1 + x and q0 / mid = 1 - x for mid = q0 + S/2.  f is increasing and
 // convex in S with f' = 1/2 [ln 2 + ln(1 + x)], so "f(S) < delta" is "S < S*" with f(S*) = delta,
-// and the prefix test stays a comparison of a running sum with one number per draft.  S* by
-// Newton's method from the upper bound 2 delta / ln 2 (f >= S ln2 / 2): four steps in single
-// precision, one in double precision (|f(S*) - delta| below 1e-8 over delta in [1e-7, 2],
-// q0 in [0, 1] on a CPU replica; the decision window is 1e-6).  Called by one thread per draft, which publishes the result: kept out of line
-// so that the callers' register budgets do not see it.
+// and the prefix test stays a comparison of a running sum with one number per draft.  It is found by a
+// whole warp (all 32 lanes call it and get the same value): S ln2 / 2 <= f(S) <= S ln 2, so the root lies
+// in [delta / ln 2, 2 delta / ln 2]; three rounds in which the 32 lanes evaluate f (single precision) at
+// 32 points of the current interval and a ballot picks the sub-interval narrow it by 33^3, and one Newton
+// step in double precision finishes (|f(S*) - delta| below 1e-8 over delta in [1e-7, 2], q0 in [0, 1] on a
+// CPU replica; the decision window is 1e-6).  A third of the latency of Newton's method by one thread,
+// and this sits on every context's critical path.
 // ---------------------------------------------------------------------------------------
-static __device__ __noinline__ double jsd_mass_bound(double delta, double q0) {
-  const double LN2 = 0.69314718055994530942;
-  if (!(delta > 0.0)) return 0.0;
-  if (!(q0 > 0.0)) return delta / LN2;   // f(S) = S ln 2 exactly
-  const float LN2F = 0.693147182464599609375f;
-  const float qf = static_cast<float>(q0), df = static_cast<float>(delta);
-  float Sf = 2.0f * df / LN2F;
-#pragma unroll 1
-  for (int it = 0; it < 4; ++it) {
-    const float x = Sf / (2.0f * qf + Sf);
-    const float lp = log1pf(x);
-    const float t = Sf * LN2F + (qf + Sf) * lp + qf * log1pf(-x);
-    Sf -= (0.5f * t - df) / (0.5f * (LN2F + lp));
-    Sf = Sf > 0.0f ? Sf : 0.0f;
-  }
-  double S = Sf > 0.0f ? static_cast<double>(Sf) : delta / LN2;
-  {
-    const double x = S / (2.0 * q0 + S);
-    const double lp = log1p(x);
-    const double t = S * LN2 + (q0 + S) * lp + q0 * log1p(-x);
-    S -= (0.5 * t - delta) / (0.5 * (LN2 + lp));
-  }
-  return S;
-}
-
-// The same bound found by a whole warp (all 32 lanes call it and get the same value): f is increasing and
-// S ln2 / 2 <= f(S) <= S ln 2, so the root lies in [delta / ln 2, 2 delta / ln 2]; three rounds in which the 32
-// lanes evaluate f (single precision) at 32 points of the current interval and a ballot picks the
-// sub-interval narrow it by 33^3, and one Newton step in double precision finishes.  A third of the
-// latency of the one-thread iteration above, which sits on every context's critical path.
 static __device__ __forceinline__ double jsd_mass_bound_warp(double delta, double q0, int lane) {
   const double LN2 = 0.69314718055994530942;
   if (!(delta > 0.0)) return 0.0;

@@ -315,8 +315,8 @@ __device__ __forceinline__ unsigned long long walk_exchange(Record* rec, unsigne
 template <class SHAPE, int CH, bool BF16, bool UNC, bool TONE, bool JSD, bool TOPK, bool GREEDY>
 __global__ void __launch_bounds__(SHAPE::THREADS, SHAPE::CTAS) lantern_context_kernel(VerifyParams P) {
   constexpr int GT = SHAPE::GT, GW = GT / 32, NGRP = SHAPE::NGRP, AREAS = SHAPE::AREAS;
-  constexpr int LOG_GT = GT == 1024 ? 10 : (GT == 512 ? 9 : 8);
-  static_assert((1 << LOG_GT) == GT, "256, 512 or 1024 threads per group");
+  constexpr int LOG_GT = GT == 512 ? 9 : 8;
+  static_assert((1 << LOG_GT) == GT, "256 or 512 threads per group");
   constexpr int SLOTS = 1024 / GT;            // neighbour slots per thread and scan round
   constexpr int CP = CH > 2 ? 2 : CH;         // chunks per slice
   constexpr int NP = CH / CP;                 // slices per thread
