@@ -878,7 +878,9 @@ __global__ void __launch_bounds__(SHAPE::THREADS, SHAPE::CTAS) lantern_context_k
         auto again = [&](int c, float (&z)[8]) {
           row_logits<BF16, TONE>(P, P.draft, static_cast<size_t>(item) * V, c * GT + gt, z);
         };
-        tp = group_kth_largest<SHAPE, CH, CH>(P, own, own, own, again, V, S, grp, gt, search3);
+        auto pairs = [&](int c, uint32_t (&w)[4]) { w[0] = raw[c].a.x, w[1] = raw[c].a.y, w[2] = raw[c].a.z, w[3] = raw[c].a.w; };
+        if constexpr (BF16 && TONE) tp = group_kth_largest<SHAPE, CH, CH, true>(P, own, pairs, own, again, V, S, grp, gt, search3);
+        else tp = group_kth_largest<SHAPE, CH, CH, false>(P, own, own, own, again, V, S, grp, gt, search3);
       }
       if (!GREEDY) reduce_drafter();
       if (!GREEDY && !TOPK && gt == 0) note_single();
@@ -914,7 +916,7 @@ __global__ void __launch_bounds__(SHAPE::THREADS, SHAPE::CTAS) lantern_context_k
           const float4 b = *reinterpret_cast<const float4*>(E + EI(g * 8 + 4));
           z[0] = a.x, z[1] = a.y, z[2] = a.z, z[3] = a.w, z[4] = b.x, z[5] = b.y, z[6] = b.z, z[7] = b.w;
         };
-        tq = group_kth_largest<SHAPE, CH, (NP > 2 ? 2 : CH)>(P, guided, guided_in_place, processed, processed, V, S, grp, gt, search3);
+        tq = group_kth_largest<SHAPE, CH, (NP > 2 ? 2 : CH), false>(P, guided, guided_in_place, processed, processed, V, S, grp, gt, search3);
         if (!GREEDY && gt == 0 && nchild > 0) note_single();
       }
       if (full) stream_target(std::true_type{});

@@ -17,6 +17,8 @@
 //      needed it.
 #pragma once
 
+#include <cuda_bf16.h>
+
 namespace lantern {
 
 // order-preserving bit pattern of a processed logit: NaN lowest, -0 as +0
@@ -52,6 +54,31 @@ __device__ __forceinline__ void row_logits(const VerifyParams& P, const void* ba
 #pragma unroll
     for (int e = 0; e < 8; ++e) z[e] = __fdiv_rn(z[e], P.T);
   }
+}
+
+// The two inner steps of the sweeps, predicated: only every twentieth value ends up on the list (1024 chains, K = 1000: 523 us
+// per call as C++ conditions, 506 like this).
+// n += z >= t
+__device__ __forceinline__ void topk_count(int& n, float z, float t) {
+  asm("{\n\t.reg .pred p;\n\tsetp.ge.f32 p, %1, %2;\n\t@p add.s32 %0, %0, 1;\n\t}" : "+r"(n) : "f"(z), "f"(t));
+}
+// *to++ = z if lo <= z < hi (to: an address in shared memory)
+__device__ __forceinline__ void topk_append(uint32_t& to, float z, float lo, float hi) {
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "setp.ge.f32 p, %1, %2;\n\t"
+      "setp.lt.and.f32 p, %1, %3, p;\n\t"
+      "@p st.shared.f32 [%0], %1;\n\t"
+      "@p add.u32 %0, %0, 4;\n\t}"
+      : "+r"(to)
+      : "f"(z), "f"(lo), "f"(hi)
+      : "memory");
+}
+
+// the smallest bf16 value >= x
+__device__ __forceinline__ float topk_bf16_up(float x) {
+  const uint32_t u = __float_as_uint(x);
+  return __uint_as_float((u & 0x80000000u ? u : u + 0xffffu) & 0xffff0000u);
 }
 
 // Step 3, by one warp: the rank-th largest of the n values in `list` (1 <= rank <= n, no NaN).
@@ -124,9 +151,10 @@ __device__ __forceinline__ int topk_group_sum(GroupTopk<GW, true>& T, int gw, in
 
 // The K-th largest processed logit of a row (0 < K < V); every thread of the group calls it and gets the same value.
 // The callables give the eight values of this thread's chunk c: for the sample, for the first and the second sweep (loops
-// unrolled UNROLL times), and for the slow path (in a rolled loop).  search3 = searches of this group so far, mod 3: its list
+// unrolled UNROLL times), and for the slow path (in a rolled loop).  PAIRS: the first sweep is given the values as pairs of
+// bf16, which they are then exactly, and counts two at a time.  search3 = searches of this group so far, mod 3: its list
 // counter is zero on entry, and the one after the next is cleared here.
-template <class SHAPE, int CH, int UNROLL, class Z0, class Z1, class Z2, class Z3, class SH>
+template <class SHAPE, int CH, int UNROLL, bool PAIRS, class Z0, class Z1, class Z2, class Z3, class SH>
 __device__ __forceinline__ float group_kth_largest(const VerifyParams& P, Z0& sampled, Z1& first, Z2& second, Z3& slow, int V, SH& S,
                                                    int grp, int gt, int& search3) {
   constexpr int GT = SHAPE::GT, GW = GT / 32;
@@ -190,15 +218,38 @@ __device__ __forceinline__ float group_kth_largest(const VerifyParams& P, Z0& sa
   }
   // ---- 2. ----
   int c_hi = 0, n_in = 0;
+  if constexpr (PAIRS) {
+    // against the next bf16 value from each edge on, which leaves the same values inside; at most 32 to a half word, so the
+    // counts are exact (1024 chains 506 -> 495 us per call)
+    lo = topk_bf16_up(lo), hi = topk_bf16_up(hi);
+    const __nv_bfloat162 lo2 = __float2bfloat162_rn(lo), hi2 = __float2bfloat162_rn(hi);
+    __nv_bfloat162 n_hi = __float2bfloat162_rn(0.0f), n_lo = n_hi;
 #pragma unroll UNROLL
-  for (int c = 0; c < CH; ++c) {
-    if (here(c)) {
-      float z[8];
-      first(c, z);
+    for (int c = 0; c < CH; ++c) {
+      if (here(c)) {
+        uint32_t w[4];
+        first(c, w);
 #pragma unroll
-      for (int e = 0; e < 8; ++e) {
-        c_hi += z[e] >= hi;
-        n_in += z[e] >= lo;
+        for (int e = 0; e < 4; ++e) {
+          const __nv_bfloat162 z = *reinterpret_cast<const __nv_bfloat162*>(&w[e]);
+          n_hi = __hadd2(n_hi, __hge2(z, hi2));
+          n_lo = __hadd2(n_lo, __hge2(z, lo2));
+        }
+      }
+    }
+    c_hi = static_cast<int>(__low2float(n_hi) + __high2float(n_hi));
+    n_in = static_cast<int>(__low2float(n_lo) + __high2float(n_lo));
+  } else {
+#pragma unroll UNROLL
+    for (int c = 0; c < CH; ++c) {
+      if (here(c)) {
+        float z[8];
+        first(c, z);
+#pragma unroll
+        for (int e = 0; e < 8; ++e) {
+          topk_count(c_hi, z[e], hi);
+          topk_count(n_in, z[e], lo);
+        }
       }
     }
   }
@@ -216,15 +267,14 @@ __device__ __forceinline__ float group_kth_largest(const VerifyParams& P, Z0& sa
     if (lane == 31) T.count[gw][1] = incl;
     const bool room = __all_sync(kFull, pos + n_in <= TOPK_LIST);
     if (room) {
-      float* to = list + pos;
+      uint32_t to = static_cast<uint32_t>(__cvta_generic_to_shared(list + pos));
 #pragma unroll UNROLL
       for (int c = 0; c < CH; ++c) {
         if (here(c)) {
           float z[8];
           second(c, z);
 #pragma unroll
-          for (int e = 0; e < 8; ++e)
-            if (z[e] >= lo && z[e] < hi) *to++ = z[e];
+          for (int e = 0; e < 8; ++e) topk_append(to, z[e], lo, hi);
         }
       }
     }
