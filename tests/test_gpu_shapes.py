@@ -59,3 +59,13 @@ def test_plan_paths_against_oracle(N, depth):
     res = compare(inp, host, 0.3, run_gpu(inp, dev, 0.3))
     assert_parity(res)
     assert res["near"] <= near_ceiling(B)
+
+
+@pytest.mark.parametrize("K", [100, 8192, 12000, 16000])
+def test_top_k_thresholds_of_bf16_rows(K):
+    """The drafter row of a call at temperature 1 is counted in pairs of bf16 values against bracket edges rounded up to
+    bf16: edges above, around and below zero."""
+    V, B, N = 16384, 24, 3
+    inp = li.verify_inputs(B, N, V, dtype=li.BF16, has_uncond=True, cfg_scale=4.0, rho=0.9, sigma_draft=0.8, seed=K)
+    host, dev = tables(li.codebook_gaussian(V, 8, seed=16), 50, inp.draft_tokens)
+    assert_parity(compare(inp, host, 0.2, run_gpu(inp, dev, 0.2, top_k=K), top_k=K))
