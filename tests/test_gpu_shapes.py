@@ -69,3 +69,15 @@ def test_top_k_thresholds_of_bf16_rows(K):
     inp = li.verify_inputs(B, N, V, dtype=li.BF16, has_uncond=True, cfg_scale=4.0, rho=0.9, sigma_draft=0.8, seed=K)
     host, dev = tables(li.codebook_gaussian(V, 8, seed=16), 50, inp.draft_tokens)
     assert_parity(compare(inp, host, 0.2, run_gpu(inp, dev, 0.2, top_k=K), top_k=K))
+
+
+@pytest.mark.parametrize("per_sm,extra,T", [(0, 30, 0.9), (2, 5, 0.9), (3, 5, 0.9), (3, 5, 1.3)])   # wide | pair | narrow
+def test_shapes_at_other_temperatures(per_sm, extra, T):
+    """Flat rows of 16384 tokens whose guidance branches agree: nearly every draft is accepted and nearly every token is drawn
+    from a context's own q."""
+    V, N, B = 16384, 2, per_sm * _sms() + extra
+    inp = li.verify_inputs(B, N, V, dtype=li.BF16, has_uncond=True, cfg_scale=7.5, T=T, rho=0.99, sigma_draft=0.7, seed=B)
+    host, dev = tables(li.codebook_gaussian(V, 8, seed=14), 100, inp.draft_tokens)
+    res = compare(inp, host, 0.2, run_gpu(inp, dev, 0.2))
+    assert_parity(res)
+    assert res["near"] <= near_ceiling(B)
