@@ -152,7 +152,7 @@ struct alignas(16) GroupShared {
   Exp2Split single[2];          // q(x~), p(x~) of the next child to test, not yet in common units (thread 0's own note)
   double acc_e, acc_p;          // double-precision numerators of the tested x~, common units
   double cut_sum;               // moved mass of A where the bound fell into a warp's slots
-  double jsd_mass;              // the JSD bound as a mass, common units
+  double jsd_mass[2];           // the JSD bound as a mass, common units, by scan round (mod 2)
   double hist[32];              // drafter/target scale ratio of each earlier rejection round of this context
   alignas(8) float wn[GW][2];   // the warps' units: their largest shifts
   float slice[TOPK ? TOPK_LIST : 1024];   // shift of every (slice, thread); before that the list of a threshold search
@@ -1013,10 +1013,11 @@ __global__ void __launch_bounds__(SHAPE::THREADS, SHAPE::CTAS) lantern_context_k
 
         // ---- A_{k,delta}(x~): gather + prefix scan with the strict bound ----
         double thr = delta * Zq_c;   // the bound in the units of the unnormalised sums
-        // Section 5.3.2: the mass whose JSD is delta; the group's last warp finds it together
+        // Section 5.3.2: the mass whose JSD is delta; the group's last warp finds it together.  (Two places: greedy decoding
+        // goes on to the next sibling without a barrier, while slower warps may not have read this one's yet.)
         if (JSD && gw == GW - 1) {
           const double mine = jsd_mass_bound_warp(delta, static_cast<double>(mass(xt)) / Zq_c, lane) * Zq_c;
-          if (lane == 0) S.jsd_mass = mine;
+          if (lane == 0) S.jsd_mass[round2] = mine;
         }
         double carry = 0.0, sm = 0.0;
         int m = k - 1;
@@ -1038,7 +1039,7 @@ __global__ void __launch_bounds__(SHAPE::THREADS, SHAPE::CTAS) lantern_context_k
           const double incl = warp_incl_scan(run, lane);
           if (lane == 31) S.wt[round2 * GW + gw] = incl;
           gbar();   // [scan 1]
-          if (JSD && base == 0) thr = S.jsd_mass;
+          if (JSD && base == 0) thr = S.jsd_mass[round2];
           // every warp: running totals of the warps (lane l: warp l % GW), the first one that reaches the bound
           double tot = S.wt[round2 * GW + (lane & (GW - 1))];
 #pragma unroll

@@ -86,6 +86,19 @@ def test_jsd_greedy(V, k, N, B, dtype, unc, delta):
     greedy_check(inp, host, dev, delta, divergence=oracle.DIV_JSD)
 
 
+@pytest.mark.parametrize("V,k,N,B,delta", [(1024, 200, 12, 300, 0.45), (16384, 1000, 9, 48, 0.45), (16384, 1000, 9, 48, 0.05)])
+def test_jsd_greedy_siblings(V, k, N, B, delta):
+    """Contexts with many children whose neighbour rows are shorter than one scan round: a bound that is hardly ever reached
+    leaves one group barrier per child, and every child has a bound of its own."""
+    par = np.full((B, N), -1, np.int32)                       # all but the last few nodes are children of the root
+    par[:, N - 3:] = np.arange(3, dtype=np.int32)
+    cb = li.codebook_gaussian(V, 8, seed=31)
+    inp = li.verify_inputs(B, N, V, dtype=li.BF16, has_uncond=True, cfg_scale=3.0, sigma_target=1.0, sigma_draft=3.0, rho=0.9,
+                           parents=par, seed=5 + V)
+    host, dev = tables(cb, k, inp.draft_tokens)
+    greedy_check(inp, host, dev, delta, divergence=oracle.DIV_JSD)
+
+
 def test_bad_variant_arguments():
     V, k = 512, 8
     dev = torch.zeros((V, k), dtype=torch.int32, device="cuda")
