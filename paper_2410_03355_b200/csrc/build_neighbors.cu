@@ -723,7 +723,7 @@ __global__ void __launch_bounds__(KT, 1024 / KT) lantern_knn_rows_kernel(BuildPa
     if constexpr (SCRATCH) {
       const uint32_t* src = P.scratch + static_cast<size_t>(on ? local : 0) * V;
 #pragma unroll
-      for (int q = 0; q < SMP; ++q) key[q] = __ldg(src + sampled_code(q * RT + rt, V));
+      for (int q = 0; q < SMP; ++q) key[q] = src[sampled_code(q * RT + rt, V)];   // (not a read-only load: this kernel may be in place while they are written)
     } else {   // every thread takes codes of the sample against all rows of the CTA
       for (int s = tid; s < SAMPLE; s += KT) {
         const float* b = P.codebook + static_cast<size_t>(sampled_code(s, V)) * D;

@@ -112,7 +112,7 @@ __device__ __forceinline__ int plan_slots(const VerifyParams& P, int lane, int& 
   const int blocks = (P.B + PLAN_WARPS - 1) / PLAN_WARPS;
 #pragma unroll 4
   for (int i = lane; i < blocks; i += 32) {
-    const int w = __ldg(P.block_words + i);
+    const int w = P.block_words[i];
     ranks = max(ranks, w & 0xffff);
     bits |= w >> 16;
   }

@@ -360,7 +360,10 @@ __global__ void __launch_bounds__(SHAPE::THREADS, SHAPE::CTAS) lantern_context_k
     for (int q = tid; q < NGRP * TOPK_BINS; q += SHAPE::THREADS) SG[q / TOPK_BINS].tk.hist[q % TOPK_BINS] = 0;
   }
   __syncthreads();
-  grid_dependency_wait();   // the plan, and whatever made the inputs
+  // The plan, and whatever made the inputs.  This kernel may be in place while the plan still writes: what the plan writes is read by
+  // ordinary loads, which stay behind this wait.  Logits and neighbour rows are read through the read-only path: they are
+  // complete before any CTA of this kernel starts, because every CTA of the plan lets it start only after a wait of its own.
+  grid_dependency_wait();
 
   // ======================= producer warps =======================
   // One warp per consumer group hands out work, keeps that group's copies going and walks.  Its 32 lanes look
@@ -397,8 +400,8 @@ __global__ void __launch_bounds__(SHAPE::THREADS, SHAPE::CTAS) lantern_context_k
     auto load_cand = [&](int start, int size) -> Cand {
       Cand c = {start + lane, -1, 0};
       if (lane < size && c.slot < total) {
-        c.item = __ldg(&P.work[c.slot].item);
-        c.mark = __ldg(&P.work[c.slot].mark);
+        c.item = P.work[c.slot].item;
+        c.mark = P.work[c.slot].mark;
       }
       return c;
     };
@@ -477,7 +480,7 @@ __global__ void __launch_bounds__(SHAPE::THREADS, SHAPE::CTAS) lantern_context_k
       for (int c = 0; c < nchild; ++c) {
         int node_c = nc0 & 0xffff, span_c = span0;
         if (c > 0) {
-          const int4 kid = __ldg(reinterpret_cast<const int4*>(P.children + cbase + c));
+          const int4 kid = *reinterpret_cast<const int4*>(P.children + cbase + c);
           node_c = kid.x, span_c = kid.w;
         }
         if (node_c != res.accepted)
@@ -545,8 +548,8 @@ __global__ void __launch_bounds__(SHAPE::THREADS, SHAPE::CTAS) lantern_context_k
         mask &= mask - 1;
         const int slot = __shfl_sync(kFull, cur.slot, l);
         if (lane == 0) {   // its description, in flight while the group is waited for
-          lo = __ldg(reinterpret_cast<const int4*>(P.work + slot));
-          hi = __ldg(reinterpret_cast<const int4*>(P.work + slot) + 1);
+          lo = *reinterpret_cast<const int4*>(P.work + slot);
+          hi = *(reinterpret_cast<const int4*>(P.work + slot) + 1);
         }
       }
       if (i >= 1 && !mbar_wait(&bar_next[grp], (i - 1) & 1, tries)) {
@@ -984,7 +987,7 @@ __global__ void __launch_bounds__(SHAPE::THREADS, SHAPE::CTAS) lantern_context_k
       for (int ci = 0; ci < nchild; ++ci) {
         // the next sibling's description, wanted only after a rejection: in flight meanwhile
         int4 sib = make_int4(0, 0, 0, 0);
-        if (ci + 1 < nchild) sib = __ldg(reinterpret_cast<const int4*>(kids + ci + 1));
+        if (ci + 1 < nchild) sib = *reinterpret_cast<const int4*>(kids + ci + 1);
         if (GREEDY) {
           if (gt == 0) atomicAdd(&P.counters->n_tested, 1);
         } else if (gt == 0) {
@@ -1004,7 +1007,7 @@ __global__ void __launch_bounds__(SHAPE::THREADS, SHAPE::CTAS) lantern_context_k
               e = static_cast<double>(bulk);
             }
             for (int j = 0; j < ci; ++j)
-              if (__ldg(&kids[j].token) == xt) pe = 0.0;
+              if (kids[j].token == xt) pe = 0.0;
           }
           S.acc_e = e;
           S.acc_p = pe;
@@ -1136,7 +1139,7 @@ __global__ void __launch_bounds__(SHAPE::THREADS, SHAPE::CTAS) lantern_context_k
         // thread's chunks hold one:
         uint32_t struck = 0;
         for (int j = 0; j <= ci; ++j) {
-          const int t = j == ci ? xt : __ldg(&kids[j].token);
+          const int t = j == ci ? xt : kids[j].token;
           if (((t >> 3) & (GT - 1)) == gt) struck |= 1u << (t >> (3 + LOG_GT));
         }
         const bool last = (ci + 1 == nchild);
@@ -1184,7 +1187,7 @@ __global__ void __launch_bounds__(SHAPE::THREADS, SHAPE::CTAS) lantern_context_k
               }
               if ((struck >> c) & 1u) {   // a token rejected in this context sits in this chunk
                 for (int j = 0; j <= ci; ++j) {
-                  const int t = __ldg(&kids[j].token);
+                  const int t = kids[j].token;
                   if ((t >> 3) == g) {
 #pragma unroll
                     for (int e = 0; e < 8; ++e) z[e] = (t & 7) == e ? ninf : z[e];

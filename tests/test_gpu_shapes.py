@@ -6,7 +6,7 @@ import torch
 
 import lantern_inputs as li
 import paper_2410_03355_b200 as lt
-from parity import assert_parity, compare, near_ceiling, run_gpu, tables
+from parity import assert_parity, compare, near_ceiling, run_gpu, tables, to_device
 
 pytestmark = pytest.mark.gpu
 
@@ -81,3 +81,29 @@ def test_shapes_at_other_temperatures(per_sm, extra, T):
     res = compare(inp, host, 0.2, run_gpu(inp, dev, 0.2))
     assert_parity(res)
     assert res["near"] <= near_ceiling(B)
+
+
+@pytest.mark.parametrize("V,B,N,tree", [(1024, 40, 6, False), (16384, 30, 20, True)])
+def test_calls_in_a_row_on_rewritten_inputs(V, B, N, tree):
+    """The fused pass is put in place while the plan still writes what it will read: calls that follow one another on the same
+    workspace, their inputs rewritten between them, answer as they do alone."""
+    state = []
+    for seed in (3, 4):
+        par = li.tree_parents(B, N, depth=5, seed=seed) if tree else None
+        inp = li.verify_inputs(B, N, V, dtype=li.BF16, has_uncond=True, cfg_scale=4.0, rho=0.9, sigma_draft=0.8, parents=par, seed=seed)
+        _, table = tables(li.codebook_gaussian(V, 8, seed=14), 100, inp.draft_tokens)
+        state.append((to_device(inp), run_gpu(inp, table, 0.2, trace=False)))
+    d = {n: t.clone() if t is not None else None for n, t in state[0][0].items()}
+    ws = torch.empty(lt.verify_workspace_bytes(B, N, V, 100, li.BF16), dtype=torch.uint8, device="cuda")
+    got = []
+    for i in range(60):
+        for n, t in state[i % 2][0].items():
+            if t is not None:
+                d[n].copy_(t)
+        got.append(lt.verify(d["target_logits"], d["draft_logits"], 4.0, 1.0, d["draft_tokens"], d["tree_parents"], table, 0.2,
+                             d["uniforms"], workspace=ws))
+    torch.cuda.synchronize()
+    for i, out in enumerate(got):
+        alone = state[i % 2][1]
+        for a in ("accept_len", "next_token", "accept_path", "status"):
+            assert torch.equal(getattr(out, a), getattr(alone, a)), (i, a)
