@@ -1136,7 +1136,8 @@ static cudaError_t launch_chained(bool first, void (*kernel)(Arg...), dim3 grid,
 template <int KT, int R, int FROM, bool ALL = false>
 static cudaError_t launch_rows(const BuildParams& P, int P2, size_t smem, cudaStream_t st, const ListParams& L = {}) {
   auto kk = lantern_knn_rows_kernel<KT, R, FROM, ALL>;
-  const cudaError_t e = cudaFuncSetAttribute(kk, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+  static DeviceFlags ready;
+  const cudaError_t e = allow_shared_memory(kk, kRowSmem, ready);
   if (e != cudaSuccess) return e;
   return launch_chained(FROM == FROM_CODES, kk, dim3((P.row_end - P.row0 + R - 1) / R), KT, smem, st, P, L, P2);
 }

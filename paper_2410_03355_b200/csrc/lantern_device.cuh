@@ -4,6 +4,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <atomic>
+
 namespace lantern {
 
 constexpr int kWarp = 32;
@@ -196,5 +198,22 @@ __device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
 // the kernel that depends on this one be put in place.
 __device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void grid_dependents_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+// Host side: which devices a kernel's shared-memory limit has been raised on (ordinals 0..63; beyond that it is raised every
+// time).  The limit belongs to the kernel and is shared by all host threads: always the largest value that any call needs.
+struct DeviceFlags {
+  std::atomic<unsigned long long> bits{0};
+};
+template <class K>
+static inline cudaError_t allow_shared_memory(K kernel, size_t bytes, DeviceFlags& ready) {
+  int dev = -1;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  const unsigned long long bit = dev >= 0 && dev < 64 ? 1ull << dev : 0ull;
+  if (ready.bits.load(std::memory_order_acquire) & bit) return cudaSuccess;
+  e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(bytes));
+  if (e == cudaSuccess) ready.bits.fetch_or(bit, std::memory_order_release);
+  return e;
+}
 
 }  // namespace lantern

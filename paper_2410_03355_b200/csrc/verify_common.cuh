@@ -7,7 +7,6 @@
 #include <math.h>
 #include <stdint.h>
 
-#include <atomic>
 #include <type_traits>
 
 #include "lantern.h"
@@ -132,21 +131,6 @@ __device__ __forceinline__ float sum8(const float* v) {
 
 
 // ---- host side ----
-// Which devices a kernel's shared-memory limit has been raised on (ordinals 0..63; beyond that it is raised every time).
-struct DeviceFlags {
-  std::atomic<unsigned long long> bits{0};
-};
-template <class K>
-static inline cudaError_t allow_shared_memory(K kernel, size_t bytes, DeviceFlags& ready) {
-  int dev = -1;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e != cudaSuccess) return e;
-  const unsigned long long bit = dev >= 0 && dev < 64 ? 1ull << dev : 0ull;
-  if (ready.bits.load(std::memory_order_acquire) & bit) return cudaSuccess;
-  e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(bytes));
-  if (e == cudaSuccess) ready.bits.fetch_or(bit, std::memory_order_release);
-  return e;
-}
 // Launch that lets the kernel be put in place while the one before it in the stream still runs (it waits for it by
 // grid_dependency_wait before it touches anything).
 template <class K>

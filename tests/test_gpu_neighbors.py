@@ -1,4 +1,6 @@
 """CUDA neighbour-table builder against the oracle: indices and distances bit-exact."""
+import threading
+
 import numpy as np
 import pytest
 import torch
@@ -170,3 +172,30 @@ def test_few_codes_exact(V, D, k, kind):
         oi, od = oracle.build_neighbors(cb, k, rows=rows)
     assert np.array_equal(gi, oi)
     assert np.array_equal(gd.view(np.uint32), od.view(np.uint32))
+
+
+def test_host_threads_with_tables_of_different_size():
+    """Tables whose rows need different amounts of shared memory, built by two host threads on streams of their own: the
+    kernel's limit is common to both."""
+    V, D, calls = 4000, 8, 3000
+    cb = torch.from_numpy(li.codebook_gaussian(V, D, seed=12)).cuda()
+    ks = (20, 700)
+    want = [lt.build_neighbors(cb, k, with_dist=False)[0] for k in ks]
+    got = [torch.empty_like(t) for t in want]
+    torch.cuda.synchronize()
+    lib = lt.load_library()
+    codes = [None, None]
+
+    def work(i, stream):
+        torch.cuda.set_device(0)
+        args = (cb.data_ptr(), V, D, ks[i], got[i].data_ptr(), None, None, 0, stream.cuda_stream)
+        codes[i] = {lib.lantern_build_neighbors(*args) for _ in range(calls)}
+
+    threads = [threading.Thread(target=work, args=(i, torch.cuda.Stream())) for i in range(2)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    torch.cuda.synchronize()
+    assert codes == [{0}, {0}]
+    assert all(torch.equal(a, b) for a, b in zip(got, want))
