@@ -14,8 +14,8 @@
 // Greedy decoding runs through the same two kernels.
 //
 // Precision: processed logits are fp32 (difference, fused multiply-add, division, each
-// rounded once); exponentials come from the fp32 ex2 unit (about 3e-7 relative); every sum over more
-// than eight terms and every threshold comparison is done in double precision.
+// rounded once); exponentials come from the fp32 ex2 unit (about 3e-7 relative); sums of up to 16 of them are formed in single
+// precision, longer sums and every threshold comparison in double precision.  Against 64 bits the normalisers are off by 3.3e-8 (flat rows) to 5e-8 rms.
 #include "verify_common.cuh"
 
 #include <stddef.h>

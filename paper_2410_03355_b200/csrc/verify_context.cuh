@@ -114,6 +114,8 @@ __device__ __forceinline__ Exp2Split exp2_split(float z) {
 __device__ __forceinline__ float exp2_int(float d) {
   return __int_as_float(__float_as_int(fmaxf(d, -127.0f) + 12583039.0f) << 23);   // 1.5 * 2^23 + 127
 }
+// a power of two as a double, without a conversion (of 0: 2^-127, which is as good where it scales a sum down)
+__device__ __forceinline__ double pow2_double(float f) { return __hiloint2double((__float_as_int(f) >> 3) + (896 << 20), 0); }
 // 2^d for an integer d held in a double, 0 far below the range of what it is compared with
 __device__ __forceinline__ double exp2_int_d(double d) {
   const int e = static_cast<int>(fmin(fmax(d, -1000.0), 1000.0));
@@ -155,7 +157,9 @@ struct alignas(16) GroupShared {
   double jsd_mass[2];           // the JSD bound as a mass, common units, by scan round (mod 2)
   double hist[32];              // drafter/target scale ratio of each earlier rejection round of this context
   alignas(8) float wn[GW][2];   // the warps' units: their largest shifts
-  float slice[TOPK ? TOPK_LIST : 1024];   // shift of every (slice, thread); before that the list of a threshold search
+  // shift of every (slice, thread), and from entry 1024 on, with four slices per thread, their sums; before that the list of a
+  // threshold search
+  float slice[TOPK ? TOPK_LIST : (GW == 8 ? 2048 : 1024)];
   int cut_m;                    // |A| - 1 that goes with cut_sum
   int badslot[3];               // first neighbour slot with an entry outside [0, V), by scan round (mod 3)
   int tok;
@@ -263,6 +267,15 @@ __device__ __forceinline__ uint32_t raw8_max(const Raw8<BF16>& d, uint32_t m) {
   return __float_as_uint(v);
 }
 
+// totals over the warp of two per-thread values: lanes 0..15 end with the first, lanes 16..31 with the second
+__device__ __forceinline__ double warp_pair_sum(double a, double b, int lane) {
+  const bool up = lane & 16;
+  double z = (up ? b : a) + __shfl_xor_sync(kFull, up ? a : b, 16);
+#pragma unroll
+  for (int o = 8; o > 0; o >>= 1) z += __shfl_xor_sync(kFull, z, o);
+  return z;
+}
+
 // Totals over the warp of N per-thread values at once: every exchange halves the values a lane still carries, so
 // N values cost N - 1 exchanges plus the rest of the butterfly instead of 5 N.  Lane l ends with the total of
 // value l / (32 / N).
@@ -325,7 +338,7 @@ __global__ void __launch_bounds__(SHAPE::THREADS, SHAPE::CTAS) lantern_context_k
   // Few registers hold this thread's part of the drafter row, or there are registers enough: it is kept for the residual passes
   // (which else read it again, a round trip to L2 per rejection).
   constexpr bool HOLD = CH * (BF16 ? 4 : 8) <= 8 || (GT == 512 && SHAPE::CTAS == 1);
-  static_assert(NP * GT <= 1024 && CH * GW <= 64, "tables of slices and blocks");
+  static_assert(NP * GT <= 1024 && CH * GW <= 64 && TOPK_LIST >= 2048, "tables of slices and blocks");
   extern __shared__ __align__(128) unsigned char smem[];
   __shared__ GroupShared<GW, TOPK> SG[NGRP];
   // Per group: next context published / the next context may be chosen / context i finished (by i mod 2: the producer may
@@ -739,11 +752,15 @@ __global__ void __launch_bounds__(SHAPE::THREADS, SHAPE::CTAS) lantern_context_k
     // ---------------- streaming part, thread-local ----------------
     // values travel as packed pairs (tokens 2i, 2i+1 of a chunk)
     const uint64_t L2 = pack2(L2E, L2E);
-    float nd = 0.0f, td = 1.0f;   // drafter: this thread's shift and its sum of numerators, in its own units
+    float nd = 0.0f;              // drafter: this thread's shift and its sum of numerators, in its own units
+    // (sums of up to 16 numerators are formed in single precision, from there on in double: in single precision all the way a
+    // normaliser of 16384 numerators was off by up to 1.9e-7 where one of a thread's 64 outweighs the others)
+    double td = 1.0;
     float nq[NP <= 2 ? NP : 1] = {};  // target: the shifts of the slices, where they are few (else in S.slice)
+    float tq_sum[NP <= 2 ? NP : 1] = {};   // ... and their sums, likewise
     auto shift_of = [&](int p) { return NP <= 2 ? nq[NP <= 2 ? p : 0] : S.slice[p * GT + gt]; };
+    auto sum_of = [&](int p) { return NP <= 2 ? tq_sum[NP <= 2 ? p : 0] : S.slice[1024 + p * GT + gt]; };
     float z_max = ninf;               // GREEDY: this thread's largest logit
-    float nq_max = 0.0f, sq = 1.0f;   // target: the largest shift of the slices; the sum, in its units
     Raw8<BF16> raw[CH];           // the drafter row
     auto load_drafter = [&](auto whole) {
 #pragma unroll
@@ -766,7 +783,8 @@ __global__ void __launch_bounds__(SHAPE::THREADS, SHAPE::CTAS) lantern_context_k
       // a slice without any finite logit (padding, masked tokens) still needs a finite shift
       nd = ceilf(fmaxf(m, -1.0e37f) * L2E);
       const uint64_t nn2 = pack2(-nd, -nd);
-      uint64_t t2 = pack2(0.0f, 0.0f);
+      uint64_t t2 = 0;
+      td = 0.0;
 #pragma unroll
       for (int c = 0; c < CH; ++c) {
         uint64_t z2[4];
@@ -782,19 +800,20 @@ __global__ void __launch_bounds__(SHAPE::THREADS, SHAPE::CTAS) lantern_context_k
           unpack2(fma2(z2[i], L2, nn2), lo, hi);
           z2[i] = pack2(ex2_approx(lo), ex2_approx(hi));
         }
-        t2 = add2(t2, add2(add2(z2[0], z2[1]), add2(z2[2], z2[3])));
+        const uint64_t s2 = add2(add2(z2[0], z2[1]), add2(z2[2], z2[3]));
+        t2 = c % CP ? add2(t2, s2) : s2;
+        if (c % CP == CP - 1) {
+          float lo, hi;
+          unpack2(t2, lo, hi);
+          td += static_cast<double>(lo + hi);
+        }
       }
-      float lo, hi;
-      unpack2(t2, lo, hi);
-      td = lo + hi;
     };
     // target: guidance combine, slice maximum, numerators, partial sum; E replaces the raw rows
     auto stream_target = [&](auto whole) {
       const unsigned char* rc = stage;
       const unsigned char* ru = stage + rowbytes;
       const uint64_t s2 = pack2(P.cfg_scale, P.cfg_scale);
-      float n_run = -3.0e37f;
-      sq = 0.0f;
 #pragma unroll (NP > 2 ? 1 : NP)
       for (int p = 0; p < NP; ++p) {   // (rolled where there are many: three groups in different phases fill the instruction cache)
         uint64_t a2[CP * 4];
@@ -854,12 +873,9 @@ __global__ void __launch_bounds__(SHAPE::THREADS, SHAPE::CTAS) lantern_context_k
         float lo, hi;
         unpack2(t2, lo, hi);
         S.slice[p * GT + gt] = n_p;
-        if (NP <= 2) nq[NP <= 2 ? p : 0] = n_p;
-        const float n_new = fmaxf(n_run, n_p);
-        sq = __fmaf_rn(sq, exp2_int(n_run - n_new), (lo + hi) * exp2_int(n_p - n_new));
-        n_run = n_new;
+        if (NP <= 2) nq[NP <= 2 ? p : 0] = n_p, tq_sum[NP <= 2 ? p : 0] = lo + hi;
+        else S.slice[1024 + p * GT + gt] = lo + hi;
       }
-      nq_max = n_run;
     };
     if (nchild > 0) {
       load_slots(xt, 0, nb);
@@ -930,15 +946,15 @@ __global__ void __launch_bounds__(SHAPE::THREADS, SHAPE::CTAS) lantern_context_k
     // per warp: the largest shift and the sum in its units, for target and drafter; then one barrier, and every
     // warp combines the partials for itself (lane l: warp l % GW)
     {
-      const float n = nq_max;
-      const float wnq = redux_max(n), wnd = redux_max(GREEDY ? z_max : nd);   // (greedy decoding: the largest logit travels instead)
-      const double zq = static_cast<double>(sq * exp2_int(n - wnq));
-      const double zp = GREEDY ? 0.0 : static_cast<double>(td * exp2_int(nd - wnd));
-      // both sums in one butterfly: after the first exchange the lower half of the warp carries one, the upper the other
-      const bool up = lane & 16;
-      double z = (up ? zp : zq) + __shfl_xor_sync(kFull, up ? zq : zp, 16);
+      float n = shift_of(0);      // (without a context: what the last one left; nobody looks at it)
 #pragma unroll
-      for (int o = 8; o > 0; o >>= 1) z += __shfl_xor_sync(kFull, z, o);
+      for (int p = 1; p < NP; ++p) n = fmaxf(n, shift_of(p));
+      const float wnq = redux_max(n), wnd = redux_max(GREEDY ? z_max : nd);   // (greedy decoding: the largest logit travels instead)
+      const bool up = lane & 16;
+      double sq = 0.0;            // (sums of up to 16 numerators are in single precision)
+#pragma unroll
+      for (int p = 0; p < NP; ++p) sq += static_cast<double>(sum_of(p) * exp2_int(shift_of(p) - wnq));
+      const double z = warp_pair_sum(sq, GREEDY ? 0.0 : td * pow2_double(exp2_int(nd - wnd)), lane);
       if ((lane & 15) == 0) {
         S.wz[gw][up] = z;
         S.wn[gw][up] = up ? wnd : wnq;
@@ -1155,13 +1171,14 @@ __global__ void __launch_bounds__(SHAPE::THREADS, SHAPE::CTAS) lantern_context_k
         // of E; the residual replaces E (it is the next sibling's target, or what the draw reads)
         const float ratio_g = Zp_c > 0.0 ? static_cast<float>(Zq_c / Zp_c) : 0.0f;
         const float fd = exp2_int(nd - Np);   // this thread's drafter units -> common units
-        float wsum = 0.0f, psum = 0.0f;       // common units; the thread's own units
+        double wsum = 0.0, psum = 0.0;        // common units; the thread's own units
 #pragma unroll
         for (int p = 0; p < NP; ++p) {
           // (a slice whose numerators are all negligible has factor 0; nothing of it survives anyway)
           const float fq = exp2_int(shift_of(p) - Nq);
           const float ratio = fq > 0.0f ? ratio_g * (fd / fq) : 0.0f;
           const uint64_t nr2 = pack2(-ratio, -ratio), nn2 = pack2(-nd, -nd);
+          float w_p = 0.0f, p_p = 0.0f;       // the slice's part of either sum
 #pragma unroll
           for (int c = p * CP; c < (p + 1) * CP; ++c) {
             const Raw8<BF16> drafted = HOLD ? raw[c] : ahead[c % AHEAD];
@@ -1211,15 +1228,15 @@ __global__ void __launch_bounds__(SHAPE::THREADS, SHAPE::CTAS) lantern_context_k
               *reinterpret_cast<ulonglong2*>(E + EI(g * 8 + 4)) = make_ulonglong2(w2[2], w2[3]);
               float lo, hi;
               unpack2(ps2, lo, hi);
-              psum += lo + hi;
+              p_p += lo + hi;
               unpack2(add2(add2(w2[0], w2[1]), add2(w2[2], w2[3])), lo, hi);
-              wsum = __fmaf_rn(lo + hi, fq, wsum);
+              w_p += lo + hi;
             }
           }
+          if (!last) wsum += static_cast<double>(w_p * fq), psum += static_cast<double>(p_p);
         }
         if (last) break;   // the draw below takes it from here
-        const float both[2] = {wsum, psum * fd};
-        const double z = warp_transposed_sum<2>(both, lane);
+        const double z = warp_pair_sum(wsum, psum * pow2_double(fd), lane);
         if ((lane & 15) == 0) S.wz[gw][lane >> 4] = z;
         if (gt == 0) note_single();
         gbar();   // [totals] also publishes the written-back residual

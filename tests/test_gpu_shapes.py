@@ -107,3 +107,28 @@ def test_calls_in_a_row_on_rewritten_inputs(V, B, N, tree):
         alone = state[i % 2][1]
         for a in ("accept_len", "next_token", "accept_path", "status"):
             assert torch.equal(getattr(out, a), getattr(alone, a)), (i, a)
+
+
+@pytest.mark.parametrize("V,per_sm,extra", [(16384, 0, 40), (16384, 3, 5), (8192, 0, 40)])   # 32, 64 and 32 tokens per thread
+def test_long_sums_keep_small_terms(V, per_sm, extra):
+    """Normalisers to which 256 tokens add 1 each and all others 3 to 5e-9: a thread that has one of the 256 loses in single
+    precision what it adds after that.  Numerators are exact here (2^0, and small ones whose own error does not count), so
+    p(x~) and q(x~) of a token of weight 1 show the sums alone.  At most the 15 small terms of one 16-term sum may go per thread
+    (7.4e-8), and the stored fp32 value is rounded (3e-8)."""
+    B = per_sm * _sms() + extra
+    lone_p, lone_q = -19.125, -19.5
+    target = torch.full((1, B, 3, V), lone_q, dtype=torch.bfloat16, device="cuda")
+    draft = torch.full((B, 3, V), lone_p, dtype=torch.bfloat16, device="cuda")
+    draft[:, :, 0:2048:8] = 0.0
+    target[:, :, :, 1:2048:8] = 0.0
+    tokens = torch.tensor([[8, 16], [1, 16]], dtype=torch.int32, device="cuda").repeat((B + 1) // 2, 1)[:B].contiguous()
+    uniforms = torch.tensor([[0.99, 0.99, 0.5], [0.0, 0.5, 0.5]], device="cuda").repeat((B + 1) // 2, 1)[:B].contiguous()
+    parents = torch.full((B, 2), -1, dtype=torch.int32, device="cuda")
+    table = torch.arange(V, dtype=torch.int32, device="cuda")[:, None].contiguous()
+    out = lt.verify(target, draft, 0.0, 1.0, tokens, parents, table, 0.0, uniforms, trace=True)
+    torch.cuda.synchronize()
+    zp = 256 + (V - 256) * np.exp(lone_p)
+    zq = 256 + (V - 256) * np.exp(lone_q)
+    qa, px = out.node_qa.cpu().double().numpy(), out.node_px.cpu().double().numpy()
+    for got, want in ((px[0::2, 0], 1 / zp), (px[0::2, 1], 1 / (zp - 1)), (qa[1::2, 0], 1 / zq)):   # the first child, a sibling after it
+        assert np.abs(got / want - 1).max() < 1.2e-7
