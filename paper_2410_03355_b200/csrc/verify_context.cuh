@@ -630,6 +630,9 @@ __global__ void __launch_bounds__(SHAPE::THREADS, SHAPE::CTAS) lantern_context_k
         if (lane == 0) ctx_prefetch_rows<UNC, !GREEDY, (AREAS > 1)>(P, item_ahead, rowbytes);
       }
     }
+    // (a call that was given up elsewhere: the group's last context has to be finished by all its warps before the terminator is
+    // published, because the first to see that overwrite what the others may still read)
+    if (clean && open) clean = mbar_wait(&bar_done[grp][(i - 1) & 1], ((i - 1) >> 1) & 1, tries);
     if (lane == 0) {
       if (clean) {   // the group is waiting for its next context: hand it the terminator
         if (i == 0 || mbar_wait(&bar_next[grp], (i - 1) & 1, tries)) {
