@@ -63,7 +63,7 @@ struct CtxShape {
 using CtxNarrow = CtxShape<256, 3, 1, 1>;   // 27 warps of 72 registers
 using CtxPair = CtxShape<512, 1, 1, 2>;     // 2 * 17 warps of 56 registers
 using CtxWide = CtxShape<512, 1, 2, 1>;     // 17 warps
-using CtxSingle = CtxShape<512, 1, 1, 1>;   // for areas of 128 KB: greedy decoding on long fp32 rows
+using CtxSingle = CtxShape<512, 1, 1, 1>;   // for areas of 128 KB: greedy decoding on long fp32 rows with guidance
 // Which shape.  A context is a chain of dependent steps; sixteen warps get through it in two thirds of the time eight
 // need, but three contexts per SM hide one another's latencies.  With few sequences per call the path through each
 // is what takes the time (and fewer contexts in flight mean fewer evaluated for nothing), with many the throughput.
@@ -73,7 +73,7 @@ using CtxSingle = CtxShape<512, 1, 1, 1>;   // for areas of 128 KB: greedy decod
 // (128 trees of 8192 tokens 78 / 78 / 88).
 static inline int ctx_shape(const VerifyParams& P, int sms) {   // 0 = narrow, 1 = pair, 2 = wide
   if (P.V <= 8192) return 0;
-  if (P.B <= 2 * sms) return 2;
+  if (P.B <= (P.parents ? 2 : 1) * sms) return 2;
   return P.B <= (P.parents ? 10 : 3) * sms ? 1 : 0;
 }
 
@@ -318,6 +318,16 @@ __device__ __forceinline__ unsigned long long walk_exchange(Record* rec, unsigne
   return old;
 }
 
+// A walk that has fallen behind the deciding of its contexts pays a round trip to L2 per step.  After this many steps in one go it
+// reads the words of 32 contexts at once, from the next one on, and follows those that lead on to the next: a chain's contexts do.
+// (29 chains of 443 drafts, 200 us instead of 980 per call.  Paths of a few contexts never get there.)
+constexpr int kWalkAlone = 6;
+__device__ __forceinline__ unsigned long long walk_look(const Record* rec) {
+  unsigned long long w;
+  asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(w) : "l"(&rec->word) : "memory");
+  return w;
+}
+
 // CH = 8-token chunks per thread (1, 2, 4 or 8); the target's numerators come in slices of CP chunks.
 // TONE = the temperature is exactly 1 (the paper's sampling setting): no division is compiled in.
 // JSD selects the Section 5.3.2 bound at compile time, so that the default path carries none of its code.
@@ -499,42 +509,62 @@ __global__ void __launch_bounds__(SHAPE::THREADS, SHAPE::CTAS) lantern_context_k
         if (node_c != res.accepted)
           for (int o = lane; o < (span_c & 0xffff); o += 32) marks[(span_c >> 16) + o] = 1;
       }
-      if (lane == 0) {
-        Record* recs = P.records + static_cast<size_t>(b) * R;
-        int at = item - b * R, accepted = res.accepted, token = res.token, status = res.status;
-        unsigned long long w = walk_exchange(recs + at, walk_word(kWalkDecided, status, accepted + 1, token));
-        if ((w & 3u) == kWalkWaiting) {   // the walk stands here already: go on with it
-          int st = static_cast<int>(w >> 8) & 0xff, len = static_cast<int>(w >> 16) & 0xffff;
-          for (;;) {
-            st |= status;
-            if (status & (LANTERN_ST_NONFINITE | LANTERN_ST_INTERNAL)) {
-              finish(b, -1, st);
-              break;
-            }
-            bool from_q = (status & LANTERN_ST_DEGENERATE) != 0;   // a residual without weight: draw from the context's own target
-            if (!from_q) {
-              if (accepted < 0) {
-                finish(b, token, st);
-                break;
-              }
-              if (P.out_path) P.out_path[static_cast<size_t>(b) * N + len] = accepted;
-              atomicMax(&P.out_len[b], ++len);   // (pieces of the path may be stored out of order)
-              at = accepted + 1;
-              w = walk_exchange(recs + at, walk_word(kWalkWaiting, st, len));
-              from_q = (w & 3u) == kWalkLeaf;                      // no drafts left on this path: bonus token from q
-            }
-            if (from_q) {
-              draw_item = b * R + at;
-              draw_status = st;
-              draw_u = p_u;
-              break;
-            }
-            if ((w & 3u) != kWalkDecided) break;                   // whoever decides that context goes on
-            status = static_cast<int>(w >> 8) & 0xff;
-            accepted = static_cast<int>(w >> 16 & 0xffff) - 1;
-            token = static_cast<int>(w >> 32);
+      // (all lanes follow the walk; lane 0 exchanges and stores)
+      Record* recs = P.records + static_cast<size_t>(b) * R;
+      int at = item - b * R, accepted = res.accepted, token = res.token, status = res.status;
+      auto exchange = [&](unsigned long long v) {
+        unsigned long long w = 0;
+        if (lane == 0) w = walk_exchange(recs + at, v);
+        return __shfl_sync(kFull, w, 0);
+      };
+      unsigned long long w = exchange(walk_word(kWalkDecided, status, accepted + 1, token));
+      if ((w & 3u) == kWalkWaiting) {   // the walk stands here already: go on with it
+        int st = static_cast<int>(w >> 8) & 0xff, len = static_cast<int>(w >> 16) & 0xffff;
+        const int len_before = len;
+        int32_t* path = P.out_path ? P.out_path + static_cast<size_t>(b) * N : nullptr;
+        for (int steps = 0;;) {
+          st |= status;
+          if (status & (LANTERN_ST_NONFINITE | LANTERN_ST_INTERNAL)) {
+            if (lane == 0) finish(b, -1, st);
+            break;
           }
+          bool from_q = (status & LANTERN_ST_DEGENERATE) != 0;   // a residual without weight: draw from the context's own target
+          if (!from_q) {
+            if (accepted < 0) {
+              if (lane == 0) finish(b, token, st);
+              break;
+            }
+            if (lane == 0 && path) path[len] = accepted;
+            ++len;
+            at = accepted + 1;
+            w = 0;
+            if (++steps > kWalkAlone) {
+              // the contexts that were decided in favour of the node numbered as they are, from this one on, are followed at once
+              for (int run = 32; run == 32;) {
+                const unsigned long long seen = at + lane < R ? walk_look(recs + at + lane) : 0;
+                const bool on = (seen & 0xffffffffull) == (walk_word(kWalkDecided, 0, at + lane + 1) & 0xffffffffull);
+                const unsigned off = ~__ballot_sync(kFull, on);
+                run = off ? __ffs(off) - 1 : 32;
+                if (lane < run && path) path[len + lane] = at + lane;
+                len += run, at += run;
+                if (run < 32) w = __shfl_sync(kFull, seen, run);
+              }
+            }
+            if ((w & 3u) != kWalkDecided) w = exchange(walk_word(kWalkWaiting, st, len));   // (a decided word stays as it is)
+            from_q = (w & 3u) == kWalkLeaf;                      // no drafts left on this path: bonus token from q
+          }
+          if (from_q) {
+            draw_item = b * R + at;
+            draw_status = st;
+            draw_u = p_u;
+            break;
+          }
+          if ((w & 3u) != kWalkDecided) break;                   // whoever decides that context goes on
+          status = static_cast<int>(w >> 8) & 0xff;
+          accepted = static_cast<int>(w >> 16 & 0xffff) - 1;
+          token = static_cast<int>(w >> 32);
         }
+        if (lane == 0 && len > len_before) atomicMax(&P.out_len[b], len);   // (pieces of the path may be stored out of order)
       }
       __syncwarp();
       return true;

@@ -19,13 +19,17 @@ static cudaError_t launch_shape(const VerifyParams& P, long long items, int sms,
 }
 template <int CHC, bool BF16, bool UNC>
 static cudaError_t launch_one(const VerifyParams& P, long long items, int sms, cudaStream_t st) {
-  if constexpr (CHC == 8 && BF16) {   // rows beyond 8192 tokens
+  constexpr bool LONG_F32 = CHC == 8 && !BF16;   // fp32 rows beyond 8192 tokens: greedy decoding only
+  if constexpr (LONG_F32 && !LANTERN_VARIANT_GREEDY) return cudaErrorInvalidValue;
+  else if constexpr (LONG_F32 && UNC) return launch_shape<CtxSingle, CHC / 2, BF16, UNC>(P, items, sms, st);
+  else if constexpr (CHC == 8) {                 // rows beyond 8192 tokens whose area takes 64 KB
     const int shape = ctx_shape(P, sms);
     if (shape == 2) return launch_shape<CtxWide, CHC / 2, BF16, UNC>(P, items, sms, st);
     if (shape == 1) return launch_shape<CtxPair, CHC / 2, BF16, UNC>(P, items, sms, st);
+    return launch_shape<CtxNarrow, CHC, BF16, UNC>(P, items, sms, st);
+  } else {
+    return launch_shape<CtxNarrow, CHC, BF16, UNC>(P, items, sms, st);
   }
-  if constexpr (CHC == 8 && !BF16) return launch_shape<CtxSingle, CHC / 2, BF16, UNC>(P, items, sms, st);   // (greedy decoding only)
-  else return launch_shape<CtxNarrow, CHC, BF16, UNC>(P, items, sms, st);
 }
 template <int CHC>
 static cudaError_t launch_layout(const VerifyParams& P, bool bf, bool un, long long items, int sms, cudaStream_t st) {
