@@ -132,3 +132,20 @@ def test_long_sums_keep_small_terms(V, per_sm, extra):
     qa, px = out.node_qa.cpu().double().numpy(), out.node_px.cpu().double().numpy()
     for got, want in ((px[0::2, 0], 1 / zp), (px[0::2, 1], 1 / (zp - 1)), (qa[1::2, 0], 1 / zq)):   # the first child, a sibling after it
         assert np.abs(got / want - 1).max() < 1.2e-7
+
+
+@pytest.mark.parametrize("N", [6, 7, 8, 38, 39, 40, 71, 200])
+@pytest.mark.parametrize("tree", [False, True])
+def test_long_walks_against_oracle(N, tree):
+    """After six steps a walk looks 32 contexts ahead: paths that end before, at and behind those lines, in chains and along
+    paths of a tree whose nodes are numbered in steps of two."""
+    B, V = 24, 512
+    par = None
+    if tree:     # a spine of the even nodes; every odd one is a second child of its spine node's parent
+        par = np.tile(np.maximum(np.arange(N) // 2 * 2 - 2, -1).astype(np.int32), (B, 1))
+    inp = li.verify_inputs(B, N, V, dtype=li.BF16, has_uncond=True, cfg_scale=2.0, rho=0.99, sigma_draft=0.25, parents=par, seed=N)
+    host, dev = tables(li.codebook_gaussian(V, 8, seed=16), 64, inp.draft_tokens)
+    gpu = run_gpu(inp, dev, 0.2)
+    res = compare(inp, host, 0.2, gpu)
+    assert_parity(res)
+    assert res["near"] <= near_ceiling(B) and (N < 38 or tree or gpu.accept_len.max() > 7)
