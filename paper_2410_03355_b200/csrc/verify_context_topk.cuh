@@ -12,9 +12,10 @@
 //      bins over the bracket, every warp finds the bin that holds the wanted rank by a suffix scan of its own, and ranks
 //      the handful of values of that bin; a crowded bin (ties) is left to one warp, which searches the
 //      list by two pivots per pass, set where the rank should lie if the values were spread evenly;
-//   4. otherwise (a sample that misleads, a list too long) by plain bisection on the order-preserving bit patterns,
-//      one pass over the row per step: slow, exact, and bounded by 34 passes.  lantern_verify_counts reports how many rows
-//      needed it.
+//   4. otherwise (a sample that misleads, a list too long: ties, or a mask value that stretches the sample's range) by a radix
+//      search on the order-preserving bit patterns: the patterns' range, a histogram of 256 bins over it, on with the bin that holds
+//      the wanted rank.  Two passes over the row a round; a round takes eight bits off the range, which is exact after four.
+//      lantern_verify_counts reports how many rows needed it.
 #pragma once
 
 #include <cuda_bf16.h>
@@ -139,14 +140,38 @@ __device__ __forceinline__ float topk_listed(const float* list, int n, int rank,
   return topk_from_order(cL == rank ? up : (cH == rank - 1 ? down : L));
 }
 
-// sum of a per-thread count over the group (every thread gets it); two group barriers
-template <int GW, class BAR>
-__device__ __forceinline__ int topk_group_sum(GroupTopk<GW, true>& T, int gw, int lane, int a, BAR& gbar) {
-  a = __reduce_add_sync(kFull, a);
-  gbar();               // the previous readers of count[] are done
-  if (lane == 0) T.count[gw][0] = a;
-  gbar();
-  return __reduce_add_sync(kFull, lane < GW ? T.count[lane][0] : 0);
+// The bin of a histogram of TOPK_FINE bins that holds the want-th largest value, its rank inside that bin (from the top) and the
+// bin's population; every warp for itself.  False if there are fewer values.
+__device__ __forceinline__ bool topk_find_bin(const int (&fine)[TOPK_FINE], int want, int lane, int& bin, int& rank, int& pop) {
+  constexpr int PER = TOPK_FINE / 32;
+  int h[PER];
+#pragma unroll
+  for (int q = 0; q < PER; q += 4) {
+    const int4 v = *reinterpret_cast<const int4*>(&fine[lane * PER + q]);
+    h[q] = v.x, h[q + 1] = v.y, h[q + 2] = v.z, h[q + 3] = v.w;
+  }
+  int mine = 0;
+#pragma unroll
+  for (int q = 0; q < PER; ++q) mine += h[q];
+  int incl = mine;                                     // suffix sum over the lanes
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int v = __shfl_down_sync(kFull, incl, o);
+    if (lane + o < 32) incl += v;
+  }
+  int above = incl - mine, b = 0, r = 0, p = 0;
+  const bool holds = above < want && want <= incl;     // one lane at most
+#pragma unroll
+  for (int q = PER - 1; q >= 0; --q) {
+    if (holds && r == 0 && above + h[q] >= want) b = lane * PER + q, r = want - above, p = h[q];
+    above += h[q];
+  }
+  const unsigned who = __ballot_sync(kFull, holds);
+  const int src = who ? __ffs(who) - 1 : 0;
+  bin = __shfl_sync(kFull, b, src);
+  rank = __shfl_sync(kFull, r, src);
+  pop = __shfl_sync(kFull, p, src);
+  return who != 0;
 }
 
 // The K-th largest processed logit of a row (0 < K < V); every thread of the group calls it and gets the same value.
@@ -296,36 +321,7 @@ __device__ __forceinline__ float group_kth_largest(const VerifyParams& P, Z0& sa
     for (int i = gt; i < c_in; i += GT) atomicAdd(&T.fine[bin_of(list[i])], 1);
     gbar();
     int bin, rank, pop;
-    {
-      constexpr int PER = TOPK_FINE / 32;
-      int h[PER];
-#pragma unroll
-      for (int q = 0; q < PER; q += 4) {
-        const int4 v = *reinterpret_cast<const int4*>(&T.fine[lane * PER + q]);
-        h[q] = v.x, h[q + 1] = v.y, h[q + 2] = v.z, h[q + 3] = v.w;
-      }
-      int mine = 0;
-#pragma unroll
-      for (int q = 0; q < PER; ++q) mine += h[q];
-      int incl = mine;                                 // suffix sum over the lanes
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const int v = __shfl_down_sync(kFull, incl, o);
-        if (lane + o < 32) incl += v;
-      }
-      const int want = K - c_hi;                       // 1 <= want <= c_in
-      int above = incl - mine, b = 0, r = 0, p = 0;
-      const bool holds = above < want && want <= incl;   // exactly one lane
-#pragma unroll
-      for (int q = PER - 1; q >= 0; --q) {
-        if (holds && r == 0 && above + h[q] >= want) b = lane * PER + q, r = want - above, p = h[q];
-        above += h[q];
-      }
-      const int src = __ffs(__ballot_sync(kFull, holds)) - 1;
-      bin = __shfl_sync(kFull, b, src);
-      rank = __shfl_sync(kFull, r, src);               // rank inside that bin, from its top
-      pop = __shfl_sync(kFull, p, src);
-    }
+    topk_find_bin(T.fine, K - c_hi, lane, bin, rank, pop);   // 1 <= K - c_hi <= c_in
     if (pop <= TOPK_TINY) {
       for (int i = gt; i < c_in; i += GT) {
         const float v = list[i];
@@ -349,31 +345,57 @@ __device__ __forceinline__ float group_kth_largest(const VerifyParams& P, Z0& sa
     }
     return __shfl_sync(kFull, v, __ffs(__ballot_sync(kFull, lane < pop && gtr < rank && rank <= geq)) - 1);
   }
-  // ---- 4. bisection on bit patterns: count(>= L) >= K > count(>= H).  If fewer than K values lie above -inf the answer is
-  // -inf (nothing is cut). ----
+  // ---- 4.  (If fewer than K values lie above -inf the answer is -inf: nothing is cut.) ----
   if (gt == 0) atomicAdd(&P.counters->n_slow_topk, 1);
-  uint32_t L = TOPK_ORDER_NINF + 1u, H = 0xff800001u;   // just above -inf .. just above +inf
-  auto count = [&](uint32_t from) {
-    int n = 0;
+  uint32_t L = TOPK_ORDER_NINF + 1u, H = 0xff800000u;   // the wanted pattern lies in [L, H]: just above -inf .. +inf
+  auto each_key = [&](auto take) {
 #pragma unroll 1
     for (int c = 0; c < CH; ++c) {
       if (here(c)) {
         float z[8];
         slow(c, z);
 #pragma unroll
-        for (int e = 0; e < 8; ++e) n += topk_order(z[e]) >= from;
+        for (int e = 0; e < 8; ++e) {
+          const uint32_t key = topk_order(z[e]);
+          if (key >= L && key <= H) take(key);
+        }
       }
     }
-    return topk_group_sum<GW>(T, gw, lane, n, gbar);
   };
-  const bool open = count(L) >= K;
-  for (int pass = 0; open && pass < 34 && H - L > 1u; ++pass) {
-    const uint32_t p = L + ((H - L) >> 1);
-    if (count(p) >= K) L = p;
-    else H = p;
+  int want = K;
+#pragma unroll 1
+  for (int round = 0; round < 5; ++round) {
+    uint32_t least = 0xffffffffu, most = 0u;
+    each_key([&](uint32_t key) {
+      least = key < least ? key : least;
+      most = key > most ? key : most;
+    });
+    least = __reduce_min_sync(kFull, least);
+    most = __reduce_max_sync(kFull, most);
+    gbar();                                             // the previous readers of count[] and of fine[] are done
+    if (lane == 0) T.count[gw][0] = static_cast<int>(least), T.count[gw][1] = static_cast<int>(most);
+    if (round > 0)
+      for (int q = gt; q < TOPK_FINE; q += GT) T.fine[q] = 0;
+    gbar();
+    L = __reduce_min_sync(kFull, lane < GW ? static_cast<uint32_t>(T.count[lane][0]) : 0xffffffffu);
+    H = __reduce_max_sync(kFull, lane < GW ? static_cast<uint32_t>(T.count[lane][1]) : 0u);
+    if (L > H) break;                                   // no value above -inf
+    const int shift = max(0, 24 - __clz(H - L));
+    each_key([&](uint32_t key) { atomicAdd(&T.fine[(key - L) >> shift], 1); });
+    gbar();
+    int bin, rank, pop;
+    const bool found = topk_find_bin(T.fine, want, lane, bin, rank, pop);
+    L = found ? L + (static_cast<uint32_t>(bin) << shift) : TOPK_ORDER_NINF;
+    if (!found || shift == 0) {
+      H = L;
+      break;
+    }
+    H = min(H, L + ((1u << shift) - 1u));
+    want = rank;
   }
-  gbar();   // count[] is written again by the next search before its barriers
-  return open ? topk_from_order(L) : ninf;
+  gbar();                                               // fine[] and count[] are free again
+  for (int q = gt; q < TOPK_FINE; q += GT) T.fine[q] = 0;
+  return L == H ? topk_from_order(L) : ninf;
 }
 
 }  // namespace lantern

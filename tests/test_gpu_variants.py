@@ -187,3 +187,35 @@ def test_top_k_nan_rows_are_still_reported():
     assert np.array_equal(g.status.cpu().numpy(), ora.status) and ora.status[3] and ora.status[6]
     ok = ora.status == 0
     assert np.array_equal(g.accept_len.cpu().numpy()[ok], ora.accept_len[ok])
+
+
+@pytest.mark.parametrize("V,B,dtype,unc,T", [(16384, 20, li.BF16, True, 1.0), (16384, 20, li.BF16, True, 0.0), (2000, 30, li.F32, False, 0.9),
+                                             (8192, 12, li.F32, True, 0.0)])
+@pytest.mark.parametrize("rows", ["lowest", "-1e9", "flat", "coarse", "few"])
+def test_top_k_of_masked_and_tied_rows(V, B, dtype, unc, T, rows):
+    """Rows whose sample says little about the threshold: half of the tokens masked by the type's lowest value or by -1e9, all logits
+    equal, a few dozen different ones, and fewer logits above -inf than are to be kept."""
+    N, K = 4, 700
+    inp = li.verify_inputs(B, N, V, dtype=dtype, has_uncond=unc, cfg_scale=2.0 if unc else 1.0, T=T or 1.0, rho=0.9, sigma_draft=0.5, seed=V)
+    bf16 = dtype == li.BF16
+    low = {"lowest": np.uint16(0xff7f) if bf16 else np.finfo(np.float32).min, "-1e9": np.uint16(0xce6e) if bf16 else np.float32(-1e9)}
+    for a in (inp.target_logits, inp.draft_logits):
+        if rows in low:
+            a[..., V // 2:] = low[rows]
+        elif rows == "flat":
+            a[...] = 0
+        elif rows == "coarse":
+            f = torch.from_numpy(a).view(torch.int16).view(torch.bfloat16).float().numpy() if bf16 else a
+            f = np.round(f * 2) / 2
+            a[...] = torch.from_numpy(f).bfloat16().view(torch.int16).numpy().view(np.uint16) if bf16 else f
+        elif not unc:      # (guidance of -inf by -inf is no number)
+            a[..., 300:] = -np.inf
+    if rows in low:
+        inp.draft_tokens[...] %= V // 2
+    if rows == "few" and not unc:
+        inp.draft_tokens[...] %= 300
+    host, dev = _table(V, 60, inp.draft_tokens)
+    if T == 0.0:
+        greedy_check(inp, host, dev, 0.2, top_k=K)
+    else:
+        assert_parity(compare(inp, host, 0.2, run_gpu(inp, dev, 0.2, top_k=K), top_k=K))
