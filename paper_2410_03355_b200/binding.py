@@ -264,7 +264,7 @@ def aggregate_all(logits: torch.Tensor, cfg_scale: float, T: float, neighbor_idx
 
 
 def verify_launch_count(greedy: bool = False, top_k_active: bool = False) -> int:
-    """Stream operations (kernels + 1 memset) enqueued by one verify() call."""
+    """lantern_verify_launch_count: an upper bound of the kernels that one verify() call enqueues (it is two)."""
     return int(load_library().lantern_verify_launch_count(int(greedy), int(top_k_active)))
 
 

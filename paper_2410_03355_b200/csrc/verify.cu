@@ -272,7 +272,7 @@ struct SmallPlan {
   unsigned long long kids[PLAN_SMALL + 1];    // children of context c
   unsigned long long level[PLAN_SMALL + 1];   // nodes of depth d that have children
   unsigned long long anc[PLAN_SMALL];         // ancestors of node i
-  int jump[PLAN_SMALL];                       // doubling: the nearest ancestor not in anc yet, -1 = none
+  int jump[PLAN_SMALL];                       // doubling: the farthest ancestor in anc so far, -1 = none beyond it
   int size[PLAN_SMALL + 1];                   // contexts in the subtree of context c, itself included
   int weight[PLAN_SMALL];                     // steps in pre-order from a node's parent to the node
   int start[PLAN_SMALL + 1];                  // where the children of context c begin in the child lists
@@ -755,8 +755,8 @@ extern "C" lantern_status lantern_verify_static(const void* target_logits, const
   void* ws = nullptr;
   const lantern_status rc = static_workspace_address(&ws);
   if (rc != LANTERN_OK) return rc;
-  // lantern_verify zeroes the counters at the head of the scratch on the stream before its first
-  // kernel, so whatever the previous call left in the array does not matter.
+  // The plan kernel resets what the call relies on (counters, marks, words), so whatever the previous call left in the array
+  // does not matter.
   return lantern_verify(target_logits, draft_logits, dtype, cfg_scale, has_uncond, T, draft_tokens, tree_parents,
                         neighbor_idx, k, delta, uniforms, B, N, V, out_accept_len, out_next_token, out_accept_path,
                         out_status, out_node_qa, out_node_px, out_node_m, ws, LANTERN_STATIC_WORKSPACE_BYTES,

@@ -14,7 +14,7 @@
 
 namespace lantern {
 
-#define LANTERN_CONTEXT_KERNEL_REVISION 19   // bump on every change to the fused context kernel
+#define LANTERN_CONTEXT_KERNEL_REVISION 20   // bump on every change to the fused context kernel
 
 constexpr int MAX_N = 1024;
 
@@ -24,7 +24,7 @@ struct Counters {               // first 256 bytes of the workspace, zeroed per 
   int n_evaluated;              // contexts the fused pass evaluated
   int n_skipped;                // contexts it left out because the walk cannot reach them
   int n_tested;                 // drafted nodes it tested
-  int status_or;                // OR of every sequence's status bits (written by the walk and later kernels)
+  int status_or;                // OR of every sequence's status bits
   int abort;                    // a bounded wait ran out somewhere: no further work is handed out
   int n_slow_topk;              // rows whose top-k threshold needed the slow exact search
 };
