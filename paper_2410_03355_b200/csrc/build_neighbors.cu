@@ -14,7 +14,9 @@
 //   2. one pass over all keys keeps those <= t (composites key << 32 | index + 1; the code itself: 0);
 //   3. the keep list -- some 1.5 k entries -- is counting-sorted into 2048 bins, in place through registers, every
 //      entry ranked inside its bin and stored at its final position, so that ties are taken by smaller index.
-// A row whose sample misled (fewer than k kept, or more than fit) or whose keys crowd a bin (massive ties)
+// Where many keys equal the bound (codes that are the same: dead ones, say), the bound is one on (key, index): of the keys equal to t
+// those of codes up to an index are kept, found in the sample like t itself, and their bins go by index.
+// A row whose sample misled (fewer than k kept, or more than fit) or whose keys crowd a bin all the same
 // takes the general path: radix select down to the exact threshold key over all V keys, compaction, bitonic
 // sort of the composites.
 #include <cuda_runtime.h>
@@ -159,6 +161,9 @@ __device__ __forceinline__ int sampled_code(int s, int V) {
   return static_cast<int>((static_cast<unsigned long long>(static_cast<uint32_t>(s) * 2654435769u) * static_cast<unsigned>(V)) >> 32);
 }
 
+// the largest float below t >= 0 (below 0: anything negative)
+__device__ __forceinline__ float key_below(float t) { return t > 0.0f ? __uint_as_float(__float_as_uint(t) - 1u) : -1.0f; }
+
 // keys of rows x cols pairs -> out[local row, column], rows `pitch` apart
 struct DistParams {
   const float* cb;
@@ -236,6 +241,7 @@ struct ListParams {
     return reinterpret_cast<uint32_t*>(dist) + static_cast<size_t>(i) * k + (e - (k - 1));
   }
   __device__ __forceinline__ float bound(int i) const { return __int_as_float(idx[static_cast<size_t>(i) * k]); }
+  __device__ __forceinline__ int* last(int i) const { return counter(i) + 1; }   // of keys equal to the bound: codes up to this one (V: all)
 };
 // entries that a row's list has room for
 static int list_room(int region, int k, bool dist, int cap) {
@@ -259,6 +265,7 @@ __global__ void __launch_bounds__(256) lantern_row_bound_kernel(ListParams L, in
   most = __reduce_max_sync(kFull, most);
   const int room = want / 16 + 2;
   uint32_t lo = 0u, hi = most;             // count(key <= hi) >= want > count(key <= lo); a few more than wanted will do
+  int c_hi = SAMPLE;
   for (int pass = 0; pass < 48 && hi - lo > 1u; ++pass) {
     uint32_t m = __float_as_uint(0.5f * __uint_as_float(lo) + 0.5f * __uint_as_float(hi));
     if (!(m > lo && m < hi)) m = lo + ((hi - lo) >> 1);
@@ -269,13 +276,29 @@ __global__ void __launch_bounds__(256) lantern_row_bound_kernel(ListParams L, in
       c1 += key[q + 1] <= m;
     }
     const int c = __reduce_add_sync(kFull, c0 + c1);
-    if (c >= want) hi = m;
+    if (c >= want) hi = m, c_hi = c;
     else lo = m;
     if (c >= want && c <= want + room) break;
+  }
+  int last = L.V;
+  if (c_hi > want + room) {                // ties: the same bisection on the index of the codes that lie at the bound
+    int from = -1;
+    last = L.V - 1;
+    while (last - from > 1) {
+      const int m = (from + last) >> 1;
+      int c = 0;
+#pragma unroll
+      for (int q = 0; q < SAMPLE / 32; ++q) c += key[q] < hi || (key[q] == hi && sampled_code(q * 32 + lane, L.V) <= m);
+      c = __reduce_add_sync(kFull, c);
+      if (c >= want) last = m;
+      else from = m;
+      if (c >= want && c <= want + room) break;
+    }
   }
   if (lane == 0) {
     L.idx[static_cast<size_t>(i) * L.k] = static_cast<int32_t>(hi);
     *L.counter(i) = 0;                     // (all lanes have read the row: the reduction above)
+    *L.last(i) = last;
   }
 }
 
@@ -296,6 +319,8 @@ __global__ void __launch_bounds__(256, 2) lantern_distance_lists_kernel(const fl
     TileLists out;
   } S;
   __shared__ float s_bound[2][TM];         // [0] the tile's rows, [1] its columns
+  __shared__ float s_tie[2][TM];           // where only some of the other side's codes count if their keys equal the bound: the bound
+  __shared__ int s_last[2][TM], s_mixed;
   __shared__ int s_n[2][TM], s_off[2][TM], s_base[2][TM], s_warp[8];
   const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4, lane = tid & 31;
   const int side = tid >> 7, line = tid & 127;
@@ -310,7 +335,21 @@ __global__ void __launch_bounds__(256, 2) lantern_distance_lists_kernel(const fl
   const int rbase = tr * TM, cbase = tc * TM;
   const int mine = (side ? cbase : rbase) + line;   // the code whose list this thread looks after
   s_n[side][line] = 0;
-  s_bound[side][line] = mine < V && (side == 0 || tr != tc) ? L.bound(mine) : __int_as_float(0xff800000);   // (-inf: keeps nothing)
+  if (tid == 0) s_mixed = 0;
+  __syncthreads();
+  {
+    float t = __int_as_float(0xff800000), tie = __int_as_float(0x7fffffff);   // (-inf: keeps nothing; NaN: equals nothing)
+    if (mine < V && (side == 0 || tr != tc)) {
+      const int first = side ? rbase : cbase, last = *L.last(mine);
+      t = L.bound(mine);
+      if (last < min(first + TM, V) - 1) {   // keys equal to the bound count only for codes up to `last`: some here, or none
+        if (last >= first) tie = t, s_last[side][line] = last, s_mixed = 1;
+        t = key_below(t);
+      }
+    }
+    s_bound[side][line] = t;
+    s_tie[side][line] = tie;
+  }
   unsigned long long acc[8][4];
   distance_tile(cb, V, D, rbase + line, cbase + line, S.in.As, S.in.Bs, acc);   // (its barriers publish the bounds as well)
   auto row_of = [&](int r) { return r < 4 ? ty * 4 + r : 64 + ty * 4 + (r - 4); };
@@ -326,6 +365,24 @@ __global__ void __launch_bounds__(256, 2) lantern_distance_lists_kernel(const fl
       }
   }
   auto key_of = [&](int r, int c) { return c & 1 ? high_key(acc[r][c >> 1]) : low_key(acc[r][c >> 1]); };
+  auto put = [&](int code, int e, int other, uint32_t key) {
+    if (e < L.cap) {
+      L.index(code)[e] = static_cast<unsigned short>(other);
+      *L.key(code, e) = key;
+    }
+  };
+  if (s_mixed) {                           // one tile per tied list: entry by entry
+#pragma unroll
+    for (int r = 0; r < 8; ++r) {
+#pragma unroll
+      for (int c = 0; c < 8; ++c) {
+        const int lr = row_of(r), lc = col_of(c);
+        const uint32_t key = key_of(r, c);
+        if (__uint_as_float(key) == s_tie[0][lr] && cbase + lc <= s_last[0][lr]) put(rbase + lr, atomicAdd(L.counter(rbase + lr), 1), cbase + lc, key);
+        if (__uint_as_float(key) == s_tie[1][lc] && rbase + lr <= s_last[1][lc]) put(cbase + lc, atomicAdd(L.counter(cbase + lc), 1), rbase + lr, key);
+      }
+    }
+  }
   int at_r[8], at_c[8];                    // this thread's places in the tile's part of each list
 #pragma unroll
   for (int r = 0; r < 8; ++r) {
@@ -362,12 +419,6 @@ __global__ void __launch_bounds__(256, 2) lantern_distance_lists_kernel(const fl
   }
   s_off[side][line] = before + incl - n_mine;
   __syncthreads();
-  auto put = [&](int code, int e, int other, uint32_t key) {
-    if (e < L.cap) {
-      L.index(code)[e] = static_cast<unsigned short>(other);
-      *L.key(code, e) = key;
-    }
-  };
   // every kept pair: list (0 = of its row, 1 = of its column) and line, place in the tile's part, the other code, the key
   auto each = [&](auto take) {
 #pragma unroll
@@ -690,6 +741,7 @@ __global__ void __launch_bounds__(KT, 1024 / KT) lantern_knn_rows_kernel(BuildPa
   __shared__ GeneralShared S;
   __shared__ int s_cnt[R], s_wsum[R][RW], s_slow[R];
   __shared__ float s_t[R], s_lo[R], s_scale[R];
+  __shared__ int s_last[R];          // of keys equal to the bound: codes up to this one (V: all)
   __shared__ int s_vote[2][R][RW];
   __shared__ uint32_t s_low[R][3 * RW], s_most[R][RW];
   const int tid = threadIdx.x, lane = tid & 31;
@@ -709,7 +761,7 @@ __global__ void __launch_bounds__(KT, 1024 / KT) lantern_knn_rows_kernel(BuildPa
       As[d][r] = (d < D && row0 + r < row_end) ? P.codebook[static_cast<size_t>(row0 + r) * D + d] : 0.0f;
     }
   }
-  if (tid < R) s_cnt[tid] = 0, s_slow[tid] = 0;
+  if (tid < R) s_cnt[tid] = 0, s_slow[tid] = 0, s_last[tid] = V;
   __syncthreads();
 
   const int r = tid / RT, rt = tid % RT;   // this thread's team and its place in it
@@ -774,23 +826,43 @@ __global__ void __launch_bounds__(KT, 1024 / KT) lantern_knn_rows_kernel(BuildPa
     // bisection on the sampled values: count(key <= hi) >= want > count(key <= lo); a few more than wanted will do
     const int room = P.want / 16 + 2;
     uint32_t lo = 0u, hi = most;
-    for (int pass = 0; pass < 48 && hi - lo > 1u; ++pass) {
-      uint32_t m = __float_as_uint(0.5f * __uint_as_float(lo) + 0.5f * __uint_as_float(hi));
-      if (!(m > lo && m < hi)) m = lo + ((hi - lo) >> 1);
-      int c = 0;
-#pragma unroll
-      for (int q = 0; q < SMP; ++q) c += key[q] <= m;
+    int pass = 0, c_hi = SAMPLE;
+    auto vote = [&](int c) {                // the team's sum
       c = __reduce_add_sync(kFull, c);
       if (lane == 0) s_vote[pass & 1][r][wv] = c;
       team();
       c = 0;
 #pragma unroll
       for (int w = 0; w < RW; ++w) c += s_vote[pass & 1][r][w];
-      if (c >= P.want) hi = m;
+      ++pass;
+      return c;
+    };
+    while (pass < 48 && hi - lo > 1u) {
+      uint32_t m = __float_as_uint(0.5f * __uint_as_float(lo) + 0.5f * __uint_as_float(hi));
+      if (!(m > lo && m < hi)) m = lo + ((hi - lo) >> 1);
+      int c = 0;
+#pragma unroll
+      for (int q = 0; q < SMP; ++q) c += key[q] <= m;
+      c = vote(c);
+      if (c >= P.want) hi = m, c_hi = c;
       else lo = m;
       if (c >= P.want && c <= P.want + room) break;
     }
     const uint32_t t = hi;
+    if (c_hi > P.want + room) {             // ties: the same bisection on the index of the codes that lie at the bound
+      int from = -1, last = V - 1;
+      while (last - from > 1) {
+        const int m = (from + last) >> 1;
+        int c = 0;
+#pragma unroll
+        for (int q = 0; q < SMP; ++q) c += key[q] < t || (key[q] == t && sampled_code(q * RT + rt, V) <= m);
+        c = vote(c);
+        if (c >= P.want) last = m;
+        else from = m;
+        if (c >= P.want && c <= P.want + room) break;
+      }
+      if (rt == 0) s_last[r] = last;
+    }
     if (rt < 32) {
       uint32_t low = 0u, mine = lane < 3 * RW ? s_low[r][lane] : 0xffffffffu;
       for (int q = 0; q < 3; ++q) {
@@ -814,6 +886,11 @@ __global__ void __launch_bounds__(KT, 1024 / KT) lantern_knn_rows_kernel(BuildPa
 #pragma unroll
     for (int q = 0; q < R; ++q) t_row[q] = ALL ? 0.0f : s_t[q];
     const uint32_t lists = static_cast<uint32_t>(__cvta_generic_to_shared(dsm));
+    int tied_to = V;                         // the smallest index up to which a row takes keys equal to its bound
+    if constexpr (!ALL) {
+#pragma unroll
+      for (int q = 0; q < R; ++q) tied_to = min(tied_to, s_last[q]);
+    }
     for (int base = 0; base < V; base += U * KT) {
       unsigned long long acc[U][R / 2];
       const float* b[U];
@@ -868,6 +945,23 @@ __global__ void __launch_bounds__(KT, 1024 / KT) lantern_knn_rows_kernel(BuildPa
             for (int q = 0; q < R / 2; ++q) acc[u][q] = 0x7fffffff7fffffffull;
           }
       }
+      if (!ALL && base + U * KT > tied_to) {   // (uniform, and never where no row has ties)
+#pragma unroll
+        for (int q = 0; q < R; ++q) {
+          const int last = s_last[q];
+          if (last >= base + U * KT || last >= V) continue;
+          const float t = s_t[q];
+          if (last < base) {
+            t_row[q] = key_below(t);
+          } else {
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+              const float key = __uint_as_float(static_cast<uint32_t>(q & 1 ? acc[u][q / 2] >> 32 : acc[u][q / 2]));
+              if (base + u * KT + tid > last && key == t) acc[u][q / 2] |= q & 1 ? 0x7fffffff00000000ull : 0x7fffffffull;   // NaN
+            }
+          }
+        }
+      }
       if constexpr (ALL) {
 #pragma unroll
         for (int u = 0; u < U; ++u) {
@@ -921,6 +1015,7 @@ __global__ void __launch_bounds__(KT, 1024 / KT) lantern_knn_rows_kernel(BuildPa
     constexpr int W = 4;
     const uint32_t* src = P.scratch + static_cast<size_t>(local) * V;
     const float t = s_t[r];
+    const int last = s_last[r];
     unsigned long long* list = list_of(r);
     const bool vec4 = (V & 3) == 0;
     for (int base = 0; base < V; base += W * 4 * RT) {
@@ -936,6 +1031,16 @@ __global__ void __launch_bounds__(KT, 1024 / KT) lantern_knn_rows_kernel(BuildPa
           if (j0 + 1 < V) key[w].y = __ldcs(src + j0 + 1);
           if (j0 + 2 < V) key[w].z = __ldcs(src + j0 + 2);
           if (j0 + 3 < V) key[w].w = __ldcs(src + j0 + 3);
+        }
+      }
+      if (base + W * 4 * RT > last) {   // ties beyond the last code that counts (uniform over the team)
+#pragma unroll
+        for (int w = 0; w < W; ++w) {
+          const int j0 = base + w * 4 * RT + 4 * rt;
+          if (j0 > last && __uint_as_float(key[w].x) == t) key[w].x = 0x7fffffffu;
+          if (j0 + 1 > last && __uint_as_float(key[w].y) == t) key[w].y = 0x7fffffffu;
+          if (j0 + 2 > last && __uint_as_float(key[w].z) == t) key[w].z = 0x7fffffffu;
+          if (j0 + 3 > last && __uint_as_float(key[w].w) == t) key[w].w = 0x7fffffffu;
         }
       }
       // thread by thread: how many of the sixteen are kept, where they go, then the entries
@@ -968,22 +1073,34 @@ __global__ void __launch_bounds__(KT, 1024 / KT) lantern_knn_rows_kernel(BuildPa
       }
     }
   }
+  if (!LISTS && !ALL && on && rt == 0 && s_last[r] < i && s_t[r] == 0.0f) {   // the code itself lies behind the last tie that counts
+    const int at = atomicAdd(&s_cnt[r], 1);
+    if (at < cap) list_of(r)[at] = static_cast<unsigned>(i + 1);
+  }
   __syncthreads();
 
   // ---- 3. counting sort (in place, through registers) and ranking, a team per row ----
   if (on) {
     unsigned long long* list = list_of(r);
     unsigned* bins = bins_of(r);
-    const int n = LISTS ? *L.counter(i) : (ALL ? V : s_cnt[r]);
+    const int last = LISTS ? *L.last(i) : (ALL ? V : s_last[r]);
+    const bool tied = last < V;
+    const uint32_t tie = tied ? __float_as_uint(LISTS ? L.bound(i) : s_t[r]) : 0u;
+    const bool self_left = LISTS && tied && tie == 0u && last < i;   // (as above)
+    const int n = LISTS ? *L.counter(i) + (self_left ? 1 : 0) : (ALL ? V : s_cnt[r]);
     const uint32_t* row = SCRATCH ? P.scratch + static_cast<size_t>(local) * V : nullptr;
     float lo = 0.0f, scale = 0.0f;
     uint32_t key[KEEP], who[KEEP];    // this thread's entries: the key; index + 1 and place of arrival in its bin
     constexpr bool ranged = LISTS || ALL;   // the range of the bins comes from the entries themselves
     if (!ranged) lo = s_lo[r], scale = s_scale[r];
-    auto bin_of = [&](uint32_t key) {   // monotone in the key
+    // with ties the upper half of the bins is for keys equal to the bound, by index
+    const float per_bin = tied ? static_cast<float>(NBINS / 2) : static_cast<float>(NBINS);
+    const float per_index = static_cast<float>(NBINS / 2) / static_cast<float>(last + 2);
+    auto bin_of = [&](uint32_t key, uint32_t id) {   // monotone in (key, index + 1)
+      if (tied && key == tie) return NBINS / 2 + min(static_cast<int>(static_cast<float>(id & 0xffffu) * per_index), NBINS / 2 - 1);
       // the square: near the bound the keys lie closer together (distances in D dimensions grow like the D/2-th root)
       const float x = fmaxf(__uint_as_float(key) - lo, 0.0f) * scale;
-      return min(static_cast<int>(x * x * static_cast<float>(NBINS)), NBINS - 1);
+      return min(static_cast<int>(x * x * per_bin), (tied ? NBINS / 2 : NBINS) - 1);
     };
     auto bin_at = [&](int b) { return static_cast<int>((bins[b >> 1] >> ((b & 1) << 4)) & 0xffffu); };
     if (n < k || n > cap) {
@@ -997,8 +1114,12 @@ __global__ void __launch_bounds__(KT, 1024 / KT) lantern_knn_rows_kernel(BuildPa
         for (int q = 0; q < KEEP; ++q) {
           const int e = q * RT + rt;
           if (e < n) {
-            key[q] = LISTS ? *L.key(i, e) : (SCRATCH ? __ldcs(row + e) : static_cast<uint32_t>(list[e] >> 32));
-            who[q] = LISTS ? L.index(i)[e] + 1u : static_cast<uint32_t>(e + 1);
+            if (LISTS && self_left && e == n - 1) {
+              key[q] = 0u, who[q] = static_cast<uint32_t>(i + 1);
+            } else {
+              key[q] = LISTS ? *L.key(i, e) : (SCRATCH ? __ldcs(row + e) : static_cast<uint32_t>(list[e] >> 32));
+              who[q] = LISTS ? L.index(i)[e] + 1u : static_cast<uint32_t>(e + 1);
+            }
             if (who[q] != static_cast<uint32_t>(i + 1)) {
               least = key[q] < least ? key[q] : least;
               most = key[q] > most ? key[q] : most;
@@ -1031,7 +1152,7 @@ __global__ void __launch_bounds__(KT, 1024 / KT) lantern_knn_rows_kernel(BuildPa
             who[q] = static_cast<uint32_t>(c);
           }
           if (who[q] == static_cast<uint32_t>(i + 1)) key[q] = who[q] = 0u;   // the code itself comes first
-          const int b = bin_of(key[q]), sh = (b & 1) << 4;
+          const int b = bin_of(key[q], who[q]), sh = (b & 1) << 4;
           who[q] |= ((atomicAdd(&bins[b >> 1], 1u << sh) >> sh) & 0xffffu) << 16;
         }
       }
@@ -1067,14 +1188,14 @@ __global__ void __launch_bounds__(KT, 1024 / KT) lantern_knn_rows_kernel(BuildPa
 #pragma unroll
         for (int q = 0; q < KEEP; ++q) {
           if (q * RT + rt < n)
-            list[bin_at(bin_of(key[q])) + (who[q] >> 16)] = (static_cast<unsigned long long>(key[q]) << 32) | (who[q] & 0xffffu);
+            list[bin_at(bin_of(key[q], who[q])) + (who[q] >> 16)] = (static_cast<unsigned long long>(key[q]) << 32) | (who[q] & 0xffffu);
         }
         team();
         int32_t* irow = P.idx + static_cast<size_t>(i) * k;
         float* drow = P.dist ? P.dist + static_cast<size_t>(i) * k : nullptr;
         for (int p = rt; p < n; p += RT) {
           const unsigned long long c = list[p];
-          const int b = bin_of(static_cast<uint32_t>(c >> 32));
+          const int b = bin_of(static_cast<uint32_t>(c >> 32), static_cast<uint32_t>(c));
           const int start = bin_at(b), end = b + 1 < NBINS ? bin_at(b + 1) : n;
           if (start >= k) break;
           int rank = start;

@@ -199,3 +199,31 @@ def test_host_threads_with_tables_of_different_size():
     torch.cuda.synchronize()
     assert codes == [{0}, {0}]
     assert all(torch.equal(a, b) for a, b in zip(got, want))
+
+
+@pytest.mark.parametrize("V,D,k,with_dist", [
+    (2400, 8, 200, True), (9000, 8, 1000, True), (4500, 16, 2500, False),      # keys computed: CTAs of two rows, of eight, of four
+    (2600, 40, 300, False), (6000, 33, 1500, False),                          # read from scratch
+    (4096, 40, 500, True), (4400, 36, 30, True)])                             # every pair once, through lists
+@pytest.mark.parametrize("dead", ["first", "last", "mixed", "all", "few values"])
+def test_many_equal_codes_exact(V, D, k, with_dist, dead):
+    """Codes that are the same (dead ones): more keys equal a row's bound than it takes, and those of the smallest index count."""
+    rng = np.random.default_rng(V + k)
+    cb = rng.standard_normal((V, D)).astype(np.float32)
+    if dead == "few values":
+        cb = cb[rng.integers(0, 5, V)]
+    else:
+        at = {"first": np.arange(V // 2), "last": np.arange(V // 2, V), "mixed": rng.permutation(V)[:V // 2], "all": np.arange(V)}[dead]
+        cb[at] = cb[0]
+    cb = np.ascontiguousarray(cb)
+    idx, dist = lt.build_neighbors(torch.from_numpy(cb).cuda(), k, with_dist=with_dist)
+    torch.cuda.synchronize()
+    gi = idx.cpu().numpy()
+    rows = np.unique(np.concatenate([np.arange(12), np.arange(V // 2 - 6, V // 2 + 6), np.arange(V - 12, V), rng.integers(0, V, 24)])).astype(np.int32)
+    oi, od = oracle.build_neighbors(cb, k, rows=rows)
+    assert np.array_equal(gi[rows], oi)
+    if with_dist:
+        assert np.array_equal(dist.cpu().numpy()[rows].view(np.uint32), od.view(np.uint32))
+    assert np.array_equal(gi[:, 0], np.arange(V))
+    srt = np.sort(gi, axis=1)
+    assert np.all(srt[:, 1:] != srt[:, :-1])
