@@ -1087,126 +1087,131 @@ __global__ void __launch_bounds__(KT, 1024 / KT) lantern_knn_rows_kernel(BuildPa
     const bool tied = last < V;
     const uint32_t tie = tied ? __float_as_uint(LISTS ? L.bound(i) : s_t[r]) : 0u;
     const bool self_left = LISTS && tied && tie == 0u && last < i;   // (as above)
-    const int n = LISTS ? *L.counter(i) + (self_left ? 1 : 0) : (ALL ? V : s_cnt[r]);
-    const uint32_t* row = SCRATCH ? P.scratch + static_cast<size_t>(local) * V : nullptr;
-    float lo = 0.0f, scale = 0.0f;
-    uint32_t key[KEEP], who[KEEP];    // this thread's entries: the key; index + 1 and place of arrival in its bin
-    constexpr bool ranged = LISTS || ALL;   // the range of the bins comes from the entries themselves
-    if (!ranged) lo = s_lo[r], scale = s_scale[r];
-    // with ties the upper half of the bins is for keys equal to the bound, by index
-    const float per_bin = tied ? static_cast<float>(NBINS / 2) : static_cast<float>(NBINS);
-    const float per_index = static_cast<float>(NBINS / 2) / static_cast<float>(last + 2);
-    auto bin_of = [&](uint32_t key, uint32_t id) {   // monotone in (key, index + 1)
-      if (tied && key == tie) return NBINS / 2 + min(static_cast<int>(static_cast<float>(id & 0xffffu) * per_index), NBINS / 2 - 1);
-      // the square: near the bound the keys lie closer together (distances in D dimensions grow like the D/2-th root)
-      const float x = fmaxf(__uint_as_float(key) - lo, 0.0f) * scale;
-      return min(static_cast<int>(x * x * per_bin), (tied ? NBINS / 2 : NBINS) - 1);
-    };
-    auto bin_at = [&](int b) { return static_cast<int>((bins[b >> 1] >> ((b & 1) << 4)) & 0xffffu); };
-    if (n < k || n > cap) {
-      if (rt == 0) s_slow[r] = 1;
-    } else {
+    auto rank_row = [&](auto with_ties) {   // (rows without ties in code of their own: 542 us per table of D = 8, 570 in common code)
+      constexpr bool TIED = decltype(with_ties)::value;
+      const int n = LISTS ? *L.counter(i) + (TIED && self_left ? 1 : 0) : (ALL ? V : s_cnt[r]);
+      const uint32_t* row = SCRATCH ? P.scratch + static_cast<size_t>(local) * V : nullptr;
+      float lo = 0.0f, scale = 0.0f;
+      uint32_t key[KEEP], who[KEEP];    // this thread's entries: the key; index + 1 and place of arrival in its bin
+      constexpr bool ranged = LISTS || ALL;   // the range of the bins comes from the entries themselves
+      if (!ranged) lo = s_lo[r], scale = s_scale[r];
+      // with ties the upper half of the bins is for keys equal to the bound, by index
+      constexpr int KEY_BINS = TIED ? NBINS / 2 : NBINS;
+      const float per_index = TIED ? static_cast<float>(NBINS / 2) / static_cast<float>(last + 2) : 0.0f;
+      auto bin_of = [&](uint32_t key, uint32_t id) {   // monotone in (key, index + 1)
+        if (TIED && key == tie) return NBINS / 2 + min(static_cast<int>(static_cast<float>(id & 0xffffu) * per_index), NBINS / 2 - 1);
+        // the square: near the bound the keys lie closer together (distances in D dimensions grow like the D/2-th root)
+        const float x = fmaxf(__uint_as_float(key) - lo, 0.0f) * scale;
+        return min(static_cast<int>(x * x * static_cast<float>(KEY_BINS)), KEY_BINS - 1);
+      };
+      auto bin_at = [&](int b) { return static_cast<int>((bins[b >> 1] >> ((b & 1) << 4)) & 0xffffu); };
+      if (n < k || n > cap) {
+        if (rt == 0) s_slow[r] = 1;
+      } else {
 #pragma unroll
-      for (int q = 0; q < OWN; ++q) bins[q * RT + rt] = 0u;
-      if (ranged) {                     // read the list; its range (without the code itself) is where the bins go
-        uint32_t least = 0xffffffffu, most = 0u;
+        for (int q = 0; q < OWN; ++q) bins[q * RT + rt] = 0u;
+        if (ranged) {                     // read the list; its range (without the code itself) is where the bins go
+          uint32_t least = 0xffffffffu, most = 0u;
+#pragma unroll
+          for (int q = 0; q < KEEP; ++q) {
+            const int e = q * RT + rt;
+            if (e < n) {
+              if (LISTS && TIED && self_left && e == n - 1) {
+                key[q] = 0u, who[q] = static_cast<uint32_t>(i + 1);
+              } else {
+                key[q] = LISTS ? *L.key(i, e) : (SCRATCH ? __ldcs(row + e) : static_cast<uint32_t>(list[e] >> 32));
+                who[q] = LISTS ? L.index(i)[e] + 1u : static_cast<uint32_t>(e + 1);
+              }
+              if (who[q] != static_cast<uint32_t>(i + 1)) {
+                least = key[q] < least ? key[q] : least;
+                most = key[q] > most ? key[q] : most;
+              }
+            }
+          }
+          least = __reduce_min_sync(kFull, least);
+          most = __reduce_max_sync(kFull, most);
+          if (lane == 0) s_low[r][rt >> 5] = least, s_most[r][rt >> 5] = most;
+        }
+        team();
+        if (ranged) {
+          uint32_t least = 0xffffffffu, most = 0u;
+#pragma unroll
+          for (int w = 0; w < RW; ++w) {
+            least = s_low[r][w] < least ? s_low[r][w] : least;
+            most = s_most[r][w] > most ? s_most[r][w] : most;
+          }
+          lo = __uint_as_float(least);
+          scale = most > least ? 1.0f / (__uint_as_float(most) - lo) : 0.0f;
+          if (most > 0x7f800000u) s_slow[r] = 1;   // NaN
+        }
 #pragma unroll
         for (int q = 0; q < KEEP; ++q) {
           const int e = q * RT + rt;
           if (e < n) {
-            if (LISTS && self_left && e == n - 1) {
-              key[q] = 0u, who[q] = static_cast<uint32_t>(i + 1);
-            } else {
-              key[q] = LISTS ? *L.key(i, e) : (SCRATCH ? __ldcs(row + e) : static_cast<uint32_t>(list[e] >> 32));
-              who[q] = LISTS ? L.index(i)[e] + 1u : static_cast<uint32_t>(e + 1);
+            if (!ranged) {
+              const unsigned long long c = list[e];
+              key[q] = static_cast<uint32_t>(c >> 32);
+              who[q] = static_cast<uint32_t>(c);
             }
-            if (who[q] != static_cast<uint32_t>(i + 1)) {
-              least = key[q] < least ? key[q] : least;
-              most = key[q] > most ? key[q] : most;
-            }
+            if (who[q] == static_cast<uint32_t>(i + 1)) key[q] = who[q] = 0u;   // the code itself comes first
+            const int b = bin_of(key[q], who[q]), sh = (b & 1) << 4;
+            who[q] |= ((atomicAdd(&bins[b >> 1], 1u << sh) >> sh) & 0xffffu) << 16;
           }
-        }
-        least = __reduce_min_sync(kFull, least);
-        most = __reduce_max_sync(kFull, most);
-        if (lane == 0) s_low[r][rt >> 5] = least, s_most[r][rt >> 5] = most;
-      }
-      team();
-      if (ranged) {
-        uint32_t least = 0xffffffffu, most = 0u;
-#pragma unroll
-        for (int w = 0; w < RW; ++w) {
-          least = s_low[r][w] < least ? s_low[r][w] : least;
-          most = s_most[r][w] > most ? s_most[r][w] : most;
-        }
-        lo = __uint_as_float(least);
-        scale = most > least ? 1.0f / (__uint_as_float(most) - lo) : 0.0f;
-        if (most > 0x7f800000u) s_slow[r] = 1;   // NaN
-      }
-#pragma unroll
-      for (int q = 0; q < KEEP; ++q) {
-        const int e = q * RT + rt;
-        if (e < n) {
-          if (!ranged) {
-            const unsigned long long c = list[e];
-            key[q] = static_cast<uint32_t>(c >> 32);
-            who[q] = static_cast<uint32_t>(c);
-          }
-          if (who[q] == static_cast<uint32_t>(i + 1)) key[q] = who[q] = 0u;   // the code itself comes first
-          const int b = bin_of(key[q], who[q]), sh = (b & 1) << 4;
-          who[q] |= ((atomicAdd(&bins[b >> 1], 1u << sh) >> sh) & 0xffffu) << 16;
-        }
-      }
-      team();
-      unsigned loc[OWN];
-      int s = 0;
-#pragma unroll
-      for (int q = 0; q < OWN; ++q) {
-        loc[q] = bins[rt * OWN + q];
-        s += static_cast<int>((loc[q] & 0xffffu) + (loc[q] >> 16));
-      }
-      int incl = s;
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const int t = __shfl_up_sync(kFull, incl, o);
-        if (lane >= o) incl += t;
-      }
-      if (lane == 31) s_wsum[r][rt >> 5] = incl;
-      team();
-      unsigned at = static_cast<unsigned>(incl - s);
-#pragma unroll
-      for (int w = 0; w < RW; ++w)
-        if (w < (rt >> 5)) at += static_cast<unsigned>(s_wsum[r][w]);
-#pragma unroll
-      for (int q = 0; q < OWN; ++q) {   // every count becomes the place where its bin starts
-        const unsigned c0 = loc[q] & 0xffffu, c1 = loc[q] >> 16;
-        bins[rt * OWN + q] = at | ((at + c0) << 16);
-        if ((c0 > CROWD && at < static_cast<unsigned>(k)) || (c1 > CROWD && at + c0 < static_cast<unsigned>(k))) s_slow[r] = 1;
-        at += c0 + c1;
-      }
-      team();
-      if (!s_slow[r]) {
-#pragma unroll
-        for (int q = 0; q < KEEP; ++q) {
-          if (q * RT + rt < n)
-            list[bin_at(bin_of(key[q], who[q])) + (who[q] >> 16)] = (static_cast<unsigned long long>(key[q]) << 32) | (who[q] & 0xffffu);
         }
         team();
-        int32_t* irow = P.idx + static_cast<size_t>(i) * k;
-        float* drow = P.dist ? P.dist + static_cast<size_t>(i) * k : nullptr;
-        for (int p = rt; p < n; p += RT) {
-          const unsigned long long c = list[p];
-          const int b = bin_of(static_cast<uint32_t>(c >> 32), static_cast<uint32_t>(c));
-          const int start = bin_at(b), end = b + 1 < NBINS ? bin_at(b + 1) : n;
-          if (start >= k) break;
-          int rank = start;
-          for (int u = start; u < end; ++u) rank += list[u] < c;
-          if (rank < k) {
-            irow[rank] = c ? static_cast<int32_t>(static_cast<uint32_t>(c)) - 1 : i;
-            if (drow) drow[rank] = __uint_as_float(static_cast<uint32_t>(c >> 32));
+        unsigned loc[OWN];
+        int s = 0;
+#pragma unroll
+        for (int q = 0; q < OWN; ++q) {
+          loc[q] = bins[rt * OWN + q];
+          s += static_cast<int>((loc[q] & 0xffffu) + (loc[q] >> 16));
+        }
+        int incl = s;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+          const int t = __shfl_up_sync(kFull, incl, o);
+          if (lane >= o) incl += t;
+        }
+        if (lane == 31) s_wsum[r][rt >> 5] = incl;
+        team();
+        unsigned at = static_cast<unsigned>(incl - s);
+#pragma unroll
+        for (int w = 0; w < RW; ++w)
+          if (w < (rt >> 5)) at += static_cast<unsigned>(s_wsum[r][w]);
+#pragma unroll
+        for (int q = 0; q < OWN; ++q) {   // every count becomes the place where its bin starts
+          const unsigned c0 = loc[q] & 0xffffu, c1 = loc[q] >> 16;
+          bins[rt * OWN + q] = at | ((at + c0) << 16);
+          if ((c0 > CROWD && at < static_cast<unsigned>(k)) || (c1 > CROWD && at + c0 < static_cast<unsigned>(k))) s_slow[r] = 1;
+          at += c0 + c1;
+        }
+        team();
+        if (!s_slow[r]) {
+#pragma unroll
+          for (int q = 0; q < KEEP; ++q) {
+            if (q * RT + rt < n)
+              list[bin_at(bin_of(key[q], who[q])) + (who[q] >> 16)] = (static_cast<unsigned long long>(key[q]) << 32) | (who[q] & 0xffffu);
+          }
+          team();
+          int32_t* irow = P.idx + static_cast<size_t>(i) * k;
+          float* drow = P.dist ? P.dist + static_cast<size_t>(i) * k : nullptr;
+          for (int p = rt; p < n; p += RT) {
+            const unsigned long long c = list[p];
+            const int b = bin_of(static_cast<uint32_t>(c >> 32), static_cast<uint32_t>(c));
+            const int start = bin_at(b), end = b + 1 < NBINS ? bin_at(b + 1) : n;
+            if (start >= k) break;
+            int rank = start;
+            for (int u = start; u < end; ++u) rank += list[u] < c;
+            if (rank < k) {
+              irow[rank] = c ? static_cast<int32_t>(static_cast<uint32_t>(c)) - 1 : i;
+              if (drow) drow[rank] = __uint_as_float(static_cast<uint32_t>(c >> 32));
+            }
           }
         }
       }
-    }
+    };
+    if (!ALL && tied) rank_row(std::true_type{});
+    else rank_row(std::false_type{});
   }
   __syncthreads();
   for (int q = 0; q < R; ++q) {
