@@ -295,9 +295,6 @@ __global__ void __launch_bounds__(256) lantern_row_bound_kernel(ListParams L, in
       if (c >= want && c <= want + room) break;
     }
   }
-  // whole tiles, so that none has to tell one tie from another: 64 keys more or fewer, where the bound leaves more than that to spare
-  if (last < L.V) last = max((last + 1 + TM / 2) / TM, 1) * TM - 1;
-  if (last >= L.V - 1) last = L.V;
   if (lane == 0) {
     L.idx[static_cast<size_t>(i) * L.k] = static_cast<int32_t>(hi);
     *L.counter(i) = 0;                     // (all lanes have read the row: the reduction above)
@@ -322,6 +319,8 @@ __global__ void __launch_bounds__(256, 2) lantern_distance_lists_kernel(const fl
     TileLists out;
   } S;
   __shared__ float s_bound[2][TM];         // [0] the tile's rows, [1] its columns
+  __shared__ float s_tie[2][TM];           // where only some of the other side's codes count if their keys equal the bound: the bound
+  __shared__ int s_last[2][TM], s_mixed;
   __shared__ int s_n[2][TM], s_off[2][TM], s_base[2][TM], s_warp[8];
   const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4, lane = tid & 31;
   const int side = tid >> 7, line = tid & 127;
@@ -336,13 +335,20 @@ __global__ void __launch_bounds__(256, 2) lantern_distance_lists_kernel(const fl
   const int rbase = tr * TM, cbase = tc * TM;
   const int mine = (side ? cbase : rbase) + line;   // the code whose list this thread looks after
   s_n[side][line] = 0;
+  if (tid == 0) s_mixed = 0;
+  __syncthreads();
   {
-    float t = __int_as_float(0xff800000);  // (-inf: keeps nothing)
+    float t = __int_as_float(0xff800000), tie = __int_as_float(0x7fffffff);   // (-inf: keeps nothing; NaN: equals nothing)
     if (mine < V && (side == 0 || tr != tc)) {
+      const int first = side ? rbase : cbase, last = *L.last(mine);
       t = L.bound(mine);
-      if (*L.last(mine) < (side ? rbase : cbase)) t = key_below(t);   // of keys equal to the bound none here counts, else all
+      if (last < min(first + TM, V) - 1) {   // keys equal to the bound count only for codes up to `last`: some here, or none
+        if (last >= first) tie = t, s_last[side][line] = last, s_mixed = 1;
+        t = key_below(t);
+      }
     }
     s_bound[side][line] = t;
+    s_tie[side][line] = tie;
   }
   unsigned long long acc[8][4];
   distance_tile(cb, V, D, rbase + line, cbase + line, S.in.As, S.in.Bs, acc);   // (its barriers publish the bounds as well)
@@ -359,6 +365,24 @@ __global__ void __launch_bounds__(256, 2) lantern_distance_lists_kernel(const fl
       }
   }
   auto key_of = [&](int r, int c) { return c & 1 ? high_key(acc[r][c >> 1]) : low_key(acc[r][c >> 1]); };
+  auto put = [&](int code, int e, int other, uint32_t key) {
+    if (e < L.cap) {
+      L.index(code)[e] = static_cast<unsigned short>(other);
+      *L.key(code, e) = key;
+    }
+  };
+  if (s_mixed) {                           // one tile per tied list: entry by entry
+#pragma unroll
+    for (int r = 0; r < 8; ++r) {
+#pragma unroll
+      for (int c = 0; c < 8; ++c) {
+        const int lr = row_of(r), lc = col_of(c);
+        const uint32_t key = key_of(r, c);
+        if (__uint_as_float(key) == s_tie[0][lr] && cbase + lc <= s_last[0][lr]) put(rbase + lr, atomicAdd(L.counter(rbase + lr), 1), cbase + lc, key);
+        if (__uint_as_float(key) == s_tie[1][lc] && rbase + lr <= s_last[1][lc]) put(cbase + lc, atomicAdd(L.counter(cbase + lc), 1), rbase + lr, key);
+      }
+    }
+  }
   int at_r[8], at_c[8];                    // this thread's places in the tile's part of each list
 #pragma unroll
   for (int r = 0; r < 8; ++r) {
@@ -395,12 +419,6 @@ __global__ void __launch_bounds__(256, 2) lantern_distance_lists_kernel(const fl
   }
   s_off[side][line] = before + incl - n_mine;
   __syncthreads();
-  auto put = [&](int code, int e, int other, uint32_t key) {
-    if (e < L.cap) {
-      L.index(code)[e] = static_cast<unsigned short>(other);
-      *L.key(code, e) = key;
-    }
-  };
   // every kept pair: list (0 = of its row, 1 = of its column) and line, place in the tile's part, the other code, the key
   auto each = [&](auto take) {
 #pragma unroll
@@ -873,130 +891,126 @@ __global__ void __launch_bounds__(KT, 1024 / KT) lantern_knn_rows_kernel(BuildPa
 #pragma unroll
       for (int q = 0; q < R; ++q) tied_to = min(tied_to, s_last[q]);
     }
-    auto key_pass = [&](auto with_ties) {
-      for (int base = 0; base < V; base += U * KT) {
-        unsigned long long acc[U][R / 2];
-        const float* b[U];
+    for (int base = 0; base < V; base += U * KT) {
+      unsigned long long acc[U][R / 2];
+      const float* b[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const int j = base + u * KT + tid;
+        b[u] = P.codebook + static_cast<size_t>(j < V ? j : 0) * D;
+#pragma unroll
+        for (int q = 0; q < R / 2; ++q) acc[u][q] = 0ull;
+      }
+      for (int d0 = 0; d0 < D; d0 += 4) {
+        float4 v[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          if (vec) {
+            v[u] = __ldg(reinterpret_cast<const float4*>(b[u] + d0));
+          } else {   // zero padding (As is zero there too) adds fma(0, 0, acc) = acc exactly
+            v[u].x = __ldg(b[u] + d0);
+            v[u].y = d0 + 1 < D ? __ldg(b[u] + d0 + 1) : 0.0f;
+            v[u].z = d0 + 2 < D ? __ldg(b[u] + d0 + 2) : 0.0f;
+            v[u].w = d0 + 3 < D ? __ldg(b[u] + d0 + 3) : 0.0f;
+          }
+        }
+#pragma unroll
+        for (int dd = 0; dd < 4; ++dd) {
+          unsigned long long a2[R / 2];
+          if (R >= 4) {
+#pragma unroll
+            for (int q = 0; q < R / 2; q += 2) {
+              const ulonglong2 a = *reinterpret_cast<const ulonglong2*>(&As[d0 + dd][2 * q]);
+              a2[q] = a.x, a2[(q + 1) % (R / 2)] = a.y;
+            }
+          } else {
+            a2[0] = *reinterpret_cast<const unsigned long long*>(&As[d0 + dd][0]);
+          }
+#pragma unroll
+          for (int u = 0; u < U; ++u) {
+            const unsigned long long bb = dup2(dd == 0 ? v[u].x : (dd == 1 ? v[u].y : (dd == 2 ? v[u].z : v[u].w)));
+#pragma unroll
+            for (int q = 0; q < R / 2; ++q) {
+              const unsigned long long t = sub2(a2[q], bb);
+              acc[u][q] = fma2(t, t, acc[u][q]);
+            }
+          }
+        }
+      }
+      if (base + U * KT > V) {   // codes past the end: NaN, never kept
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+          if (base + u * KT + tid >= V) {
+#pragma unroll
+            for (int q = 0; q < R / 2; ++q) acc[u][q] = 0x7fffffff7fffffffull;
+          }
+      }
+      if (!ALL && base + U * KT > tied_to) {   // (uniform, and never where no row has ties)
+#pragma unroll
+        for (int q = 0; q < R; ++q) {
+          const int last = s_last[q];
+          if (last >= base + U * KT || last >= V) continue;
+          const float t = s_t[q];
+          if (last < base) {
+            t_row[q] = key_below(t);
+          } else {
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+              const float key = __uint_as_float(static_cast<uint32_t>(q & 1 ? acc[u][q / 2] >> 32 : acc[u][q / 2]));
+              if (base + u * KT + tid > last && key == t) acc[u][q / 2] |= q & 1 ? 0x7fffffff00000000ull : 0x7fffffffull;   // NaN
+            }
+          }
+        }
+      }
+      if constexpr (ALL) {
 #pragma unroll
         for (int u = 0; u < U; ++u) {
           const int j = base + u * KT + tid;
-          b[u] = P.codebook + static_cast<size_t>(j < V ? j : 0) * D;
+          if (j < V) {
 #pragma unroll
-          for (int q = 0; q < R / 2; ++q) acc[u][q] = 0ull;
-        }
-        for (int d0 = 0; d0 < D; d0 += 4) {
-          float4 v[U];
-#pragma unroll
-          for (int u = 0; u < U; ++u) {
-            if (vec) {
-              v[u] = __ldg(reinterpret_cast<const float4*>(b[u] + d0));
-            } else {   // zero padding (As is zero there too) adds fma(0, 0, acc) = acc exactly
-              v[u].x = __ldg(b[u] + d0);
-              v[u].y = d0 + 1 < D ? __ldg(b[u] + d0 + 1) : 0.0f;
-              v[u].z = d0 + 2 < D ? __ldg(b[u] + d0 + 2) : 0.0f;
-              v[u].w = d0 + 3 < D ? __ldg(b[u] + d0 + 3) : 0.0f;
-            }
-          }
-#pragma unroll
-          for (int dd = 0; dd < 4; ++dd) {
-            unsigned long long a2[R / 2];
-            if (R >= 4) {
-#pragma unroll
-              for (int q = 0; q < R / 2; q += 2) {
-                const ulonglong2 a = *reinterpret_cast<const ulonglong2*>(&As[d0 + dd][2 * q]);
-                a2[q] = a.x, a2[(q + 1) % (R / 2)] = a.y;
-              }
-            } else {
-              a2[0] = *reinterpret_cast<const unsigned long long*>(&As[d0 + dd][0]);
-            }
-#pragma unroll
-            for (int u = 0; u < U; ++u) {
-              const unsigned long long bb = dup2(dd == 0 ? v[u].x : (dd == 1 ? v[u].y : (dd == 2 ? v[u].z : v[u].w)));
-#pragma unroll
-              for (int q = 0; q < R / 2; ++q) {
-                const unsigned long long t = sub2(a2[q], bb);
-                acc[u][q] = fma2(t, t, acc[u][q]);
-              }
-            }
+            for (int q = 0; q < R; ++q)
+              list_of(q)[j] = (static_cast<unsigned long long>(static_cast<uint32_t>(q & 1 ? acc[u][q / 2] >> 32 : acc[u][q / 2])) << 32) |
+                              static_cast<unsigned>(j + 1);
           }
         }
-        if (base + U * KT > V) {   // codes past the end: NaN, never kept
-#pragma unroll
-          for (int u = 0; u < U; ++u)
-            if (base + u * KT + tid >= V) {
-#pragma unroll
-              for (int q = 0; q < R / 2; ++q) acc[u][q] = 0x7fffffff7fffffffull;
-            }
-        }
-        if (decltype(with_ties)::value && base + U * KT > tied_to) {
-#pragma unroll
-          for (int q = 0; q < R; ++q) {
-            const int last = s_last[q];
-            if (last >= base + U * KT || last >= V) continue;
-            const float t = s_t[q];
-            if (last < base) {
-              t_row[q] = key_below(t);
-            } else {
-#pragma unroll
-              for (int u = 0; u < U; ++u) {
-                const float key = __uint_as_float(static_cast<uint32_t>(q & 1 ? acc[u][q / 2] >> 32 : acc[u][q / 2]));
-                if (base + u * KT + tid > last && key == t) acc[u][q / 2] |= q & 1 ? 0x7fffffff00000000ull : 0x7fffffffull;   // NaN
-              }
-            }
-          }
-        }
-        if constexpr (ALL) {
-#pragma unroll
-          for (int u = 0; u < U; ++u) {
-            const int j = base + u * KT + tid;
-            if (j < V) {
-#pragma unroll
-              for (int q = 0; q < R; ++q)
-                list_of(q)[j] = (static_cast<unsigned long long>(static_cast<uint32_t>(q & 1 ? acc[u][q / 2] >> 32 : acc[u][q / 2])) << 32) |
-                                static_cast<unsigned>(j + 1);
-            }
-          }
-          continue;
-        }
-        // How many of this thread's keys each row keeps, four rows to a word (at most U each, 32 U per warp), and a
-        // prefix over the warp; then one counter update per row and warp.  (Ballots and population counts in
-        // their place kept the XU pipe busy for 24 of the pass's 51 thousand cycles.)
-        constexpr int NW = (R + 3) / 4;
-        auto key_of_row = [&](int u, int q) {
-          return __uint_as_float(static_cast<uint32_t>(q & 1 ? acc[u][q / 2] >> 32 : acc[u][q / 2]));
-        };
-        uint32_t cnt[NW] = {}, incl[NW], tot[NW];
-#pragma unroll
-        for (int q = 0; q < R; ++q)
-#pragma unroll
-          for (int u = 0; u < U; ++u)
-            if (key_of_row(u, q) <= t_row[q]) cnt[q / 4] += 1u << (8 * (q % 4));
-#pragma unroll
-        for (int w = 0; w < NW; ++w) {
-          incl[w] = cnt[w];
-#pragma unroll
-          for (int o = 1; o < 32; o <<= 1) {
-            const uint32_t v = __shfl_up_sync(kFull, incl[w], o);
-            if (lane >= o) incl[w] += v;
-          }
-          tot[w] = __shfl_sync(kFull, incl[w], 31);
-          incl[w] -= cnt[w];
-        }
-        const int mine = ((NW > 1 && (lane & 4) ? tot[NW - 1] : tot[0]) >> (8 * (lane & 3))) & 0xffu;
-        int start = 0;
-        if (lane < R && mine) start = atomicAdd(&s_cnt[lane], mine);
-#pragma unroll
-        for (int q = 0; q < R; ++q) {
-          int at = __shfl_sync(kFull, start, q) + static_cast<int>((incl[q / 4] >> (8 * (q % 4))) & 0xffu);
-          at = at < cap ? at : cap;                        // (the list has room for U more)
-          uint32_t to = lists + static_cast<uint32_t>(q * static_cast<int>(per_row) + at * 8);
-#pragma unroll
-          for (int u = 0; u < U; ++u) append_key(to, key_of_row(u, q), t_row[q], static_cast<uint32_t>(base + u * KT + tid + 1));
-        }
+        continue;
       }
-    };
-    if (!ALL && tied_to < V) key_pass(std::true_type{});
-    else key_pass(std::false_type{});
+      // How many of this thread's keys each row keeps, four rows to a word (at most U each, 32 U per warp), and a
+      // prefix over the warp; then one counter update per row and warp.  (Ballots and population counts in
+      // their place kept the XU pipe busy for 24 of the pass's 51 thousand cycles.)
+      constexpr int NW = (R + 3) / 4;
+      auto key_of_row = [&](int u, int q) {
+        return __uint_as_float(static_cast<uint32_t>(q & 1 ? acc[u][q / 2] >> 32 : acc[u][q / 2]));
+      };
+      uint32_t cnt[NW] = {}, incl[NW], tot[NW];
+#pragma unroll
+      for (int q = 0; q < R; ++q)
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+          if (key_of_row(u, q) <= t_row[q]) cnt[q / 4] += 1u << (8 * (q % 4));
+#pragma unroll
+      for (int w = 0; w < NW; ++w) {
+        incl[w] = cnt[w];
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+          const uint32_t v = __shfl_up_sync(kFull, incl[w], o);
+          if (lane >= o) incl[w] += v;
+        }
+        tot[w] = __shfl_sync(kFull, incl[w], 31);
+        incl[w] -= cnt[w];
+      }
+      const int mine = ((NW > 1 && (lane & 4) ? tot[NW - 1] : tot[0]) >> (8 * (lane & 3))) & 0xffu;
+      int start = 0;
+      if (lane < R && mine) start = atomicAdd(&s_cnt[lane], mine);
+#pragma unroll
+      for (int q = 0; q < R; ++q) {
+        int at = __shfl_sync(kFull, start, q) + static_cast<int>((incl[q / 4] >> (8 * (q % 4))) & 0xffu);
+        at = at < cap ? at : cap;                        // (the list has room for U more)
+        uint32_t to = lists + static_cast<uint32_t>(q * static_cast<int>(per_row) + at * 8);
+#pragma unroll
+        for (int u = 0; u < U; ++u) append_key(to, key_of_row(u, q), t_row[q], static_cast<uint32_t>(base + u * KT + tid + 1));
+      }
+    }
   } else if (SCRATCH && on && !ALL) {   // each team reads its own row of keys, W groups of four per thread at a time
     constexpr int W = 4;
     const uint32_t* src = P.scratch + static_cast<size_t>(local) * V;
