@@ -116,9 +116,9 @@ __device__ __forceinline__ float exp2_int(float d) {
 }
 // a power of two as a double, without a conversion (of 0: 2^-127, which is as good where it scales a sum down)
 __device__ __forceinline__ double pow2_double(float f) { return __hiloint2double((__float_as_int(f) >> 3) + (896 << 20), 0); }
-// 2^d for an integer d held in a double, 0 far below the range of what it is compared with
+// 2^d for an integer d held in a double, 0 far below the range of what it is compared with (the conversion saturates)
 __device__ __forceinline__ double exp2_int_d(double d) {
-  const int e = static_cast<int>(fmin(fmax(d, -1000.0), 1000.0));
+  const int e = min(__double2int_rn(d), 1000);
   return e <= -1000 ? 0.0 : __hiloint2double((1023 + e) << 20, 0);
 }
 
@@ -151,8 +151,9 @@ template <int GW, bool TOPK>
 struct alignas(16) GroupShared {
   alignas(16) double wz[GW][2]; // per-warp sums of numerators (target, drafter), in the warp's units
   double wt[64];                // per-(chunk, warp) totals for scans and block sums
-  Exp2Split single[2];          // q(x~), p(x~) of the next child to test, not yet in common units (thread 0's own note)
-  double acc_e, acc_p;          // double-precision numerators of the tested x~, common units
+  // q(x~), p(x~) of the next child to test, not yet in common units, of context i in single[i & 1]: the first threads may note the next
+  // context's before the last ones have read the current one's
+  Exp2Split single[2][2];
   double cut_sum;               // moved mass of A where the bound fell into a warp's slots
   double jsd_mass[2];           // the JSD bound as a mass, common units, by scan round (mod 2)
   double hist[32];              // drafter/target scale ratio of each earlier rejection round of this context
@@ -208,12 +209,17 @@ __device__ __forceinline__ void ctx_prefetch_rows(const VerifyParams& P, int ite
   }
 }
 
-// one logit of a row in global memory, widened to fp32
+// One logit of a row in global memory, as it lies there, and the same widened to fp32.  The load is issued early and used late, by
+// a few threads under a condition: widened there and then, those threads would wait for it inside the condition.
 template <bool BF16>
-__device__ __forceinline__ float ctx_raw_logit(const void* base, size_t elem) {
-  if (BF16) return __uint_as_float(static_cast<uint32_t>(__ldg(static_cast<const unsigned short*>(base) + elem)) << 16);
-  return __ldg(static_cast<const float*>(base) + elem);
+__device__ __forceinline__ uint32_t ctx_raw_logit(const void* base, size_t elem) {
+  uint32_t w;
+  if (BF16) asm volatile("ld.global.nc.u16 %0, [%1];" : "=r"(w) : "l"(static_cast<const unsigned short*>(base) + elem));
+  else asm volatile("ld.global.nc.u32 %0, [%1];" : "=r"(w) : "l"(static_cast<const float*>(base) + elem));
+  return w;
 }
+template <bool BF16>
+__device__ __forceinline__ float ctx_widen(uint32_t w) { return __uint_as_float(BF16 ? w << 16 : w); }
 
 // eight raw logits of one 16-byte group (bf16) or 32 bytes (fp32) of a row in global memory
 template <bool BF16>
@@ -308,6 +314,10 @@ __device__ __forceinline__ double warp_transposed_sum(const float (&v)[N], int l
   for (; o > 0; o >>= 1) d[0] += __shfl_xor_sync(kFull, d[0], o);
   return d[0];
 }
+
+// one bit per token of a thread
+template <int CH>
+using StruckMask = typename std::conditional<(CH > 4), uint64_t, uint32_t>::type;
 
 // Exchange of a walk word.  The word carries everything its receiver needs and what the two sides store besides does
 // not depend on order, so no fence is paid for (with acquire and release the producers became the bottleneck: 1.12
@@ -762,25 +772,27 @@ __global__ void __launch_bounds__(SHAPE::THREADS, SHAPE::CTAS) lantern_context_k
     const int nchild = item < 0 ? 0 : cur.nchild;                      // 0: nothing but a draw from q
     const unsigned char* drow = static_cast<const unsigned char*>(P.draft) + static_cast<size_t>(item) * rowbytes;
 
-    // first child: its neighbour row and, for thread 0, its raw logits; issued now, used after the streaming part
+    // first child: its neighbour row and its raw logits (target: thread 0, drafter: thread 1); issued now, used after the
+    // streaming part
     int node = cur.node0;
     int xt = cur.tok0;
     int nb[SLOTS];
-    float raw_c = 0.0f, raw_u = 0.0f, raw_d = 0.0f;
-    auto fetch_single = [&]() {
+    uint32_t raw_z = 0u, raw_u = 0u;
+    auto fetch_single = [&]() {   // (threads 0 and 1)
       const size_t e = static_cast<size_t>(item) * V + xt;
-      if (!GREEDY) raw_d = ctx_raw_logit<BF16>(P.draft, e);
-      raw_c = ctx_raw_logit<BF16>(P.target, e);
+      raw_z = ctx_raw_logit<BF16>(gt == 0 ? P.target : P.draft, e);
       if (UNC) raw_u = ctx_raw_logit<BF16>(P.target, branch + e);
     };
     float tq = ninf, tp = ninf;   // top-k thresholds of the target and the drafter row
     auto note_single = [&]() {
-      float zq = raw_c, zp = raw_d;
-      if (UNC) zq = __fmaf_rn(P.cfg_scale, __fsub_rn(raw_c, raw_u), raw_u);
-      if (!TONE) zq = __fdiv_rn(zq, P.T), zp = __fdiv_rn(zp, P.T);
-      if (TOPK) zq = zq < tq ? ninf : zq, zp = zp < tp ? ninf : zp;
-      S.single[0] = exp2_split(zq);
-      S.single[1] = exp2_split(zp);
+      float z = ctx_widen<BF16>(raw_z);
+      if (UNC) {
+        const float u = ctx_widen<BF16>(raw_u), l = __fmaf_rn(P.cfg_scale, __fsub_rn(z, u), u);
+        z = gt == 0 ? l : z;
+      }
+      if (!TONE) z = __fdiv_rn(z, P.T);
+      if (TOPK) z = z < (gt == 0 ? tq : tp) ? ninf : z;
+      S.single[iter & 1][gt] = exp2_split(z);
     };
 
     // ---------------- streaming part, thread-local ----------------
@@ -913,7 +925,7 @@ __global__ void __launch_bounds__(SHAPE::THREADS, SHAPE::CTAS) lantern_context_k
     };
     if (nchild > 0) {
       load_slots(xt, 0, nb);
-      if (!GREEDY && gt == 0) fetch_single();
+      if (!GREEDY && gt < 2) fetch_single();
       if constexpr (!GREEDY) {
         if (full) load_drafter(std::true_type{});
         else load_drafter(std::false_type{});
@@ -936,7 +948,7 @@ __global__ void __launch_bounds__(SHAPE::THREADS, SHAPE::CTAS) lantern_context_k
         else tp = group_kth_largest<SHAPE, CH, CH, false>(P, own, own, own, again, V, S, grp, gt, search3);
       }
       if (!GREEDY) reduce_drafter();
-      if (!GREEDY && !TOPK && gt == 0) note_single();
+      if (!GREEDY && !TOPK && gt < 2) note_single();
     }
     // The target rows were issued when the staging area fell free; they arrive while the drafter
     // row is streamed.  Every thread waits for itself (bounded); a wait that runs out is reported after
@@ -970,7 +982,7 @@ __global__ void __launch_bounds__(SHAPE::THREADS, SHAPE::CTAS) lantern_context_k
           z[0] = a.x, z[1] = a.y, z[2] = a.z, z[3] = a.w, z[4] = b.x, z[5] = b.y, z[6] = b.z, z[7] = b.w;
         };
         tq = group_kth_largest<SHAPE, CH, (NP > 2 ? 2 : CH), false>(P, guided, guided_in_place, processed, processed, V, S, grp, gt, search3);
-        if (!GREEDY && gt == 0 && nchild > 0) note_single();
+        if (!GREEDY && gt < 2 && nchild > 0) note_single();
       }
       if (full) stream_target(std::true_type{});
       else stream_target(std::false_type{});
@@ -1032,37 +1044,14 @@ __global__ void __launch_bounds__(SHAPE::THREADS, SHAPE::CTAS) lantern_context_k
       const double delta = static_cast<double>(P.delta);
       const ChildInfo* kids = P.children + cur.cbase;
       float r = cur.r0;
+      StruckMask<CH> struck = 0;   // this thread's tokens that were rejected in this context: bit 8 c + e for token e of chunk c
       auto mass = [&](int n) { return E[EI(n)] * exp2_int(S.slice[owner_slice(n)] - Nq); };   // common units
 
       for (int ci = 0; ci < nchild; ++ci) {
         // the next sibling's description, wanted only after a rejection: in flight meanwhile
         int4 sib = make_int4(0, 0, 0, 0);
         if (ci + 1 < nchild) sib = *reinterpret_cast<const int4*>(kids + ci + 1);
-        if (GREEDY) {
-          if (gt == 0) atomicAdd(&P.counters->n_tested, 1);
-        } else if (gt == 0) {
-          // The tested token's two numerators in common units, in double precision from its raw logits, carried
-          // through every rejection round so far (E <- max(0, E - ratio_i * ep)); the sums they are compared
-          // with are sums of thousands of terms and do not suffer from cancellation.  A token that has lost its
-          // mass (it lay in an earlier A, or was itself rejected before) has none.
-          const Exp2Split q = S.single[0], p = S.single[1];
-          double e = q.y * exp2_int_d(q.n - static_cast<double>(Nq));
-          double pe = p.y * exp2_int_d(p.n - static_cast<double>(Np));
-          if (ci > 0) {
-            const float bulk = mass(xt);
-            if (ci <= 32) {
-              for (int i = 0; i < ci; ++i) e = fmax(0.0, e - S.hist[i] * pe);
-              if (bulk == 0.0f) e = 0.0;
-            } else {
-              e = static_cast<double>(bulk);
-            }
-            for (int j = 0; j < ci; ++j)
-              if (kids[j].token == xt) pe = 0.0;
-          }
-          S.acc_e = e;
-          S.acc_p = pe;
-          atomicAdd(&P.counters->n_tested, 1);   // work accounting (a fire-and-forget reduction)
-        }
+        if (gt == 0) atomicAdd(&P.counters->n_tested, 1);   // work accounting (a fire-and-forget reduction)
 
         // ---- A_{k,delta}(x~): gather + prefix scan with the strict bound ----
         double thr = delta * Zq_c;   // the bound in the units of the unnormalised sums
@@ -1140,10 +1129,32 @@ __global__ void __launch_bounds__(SHAPE::THREADS, SHAPE::CTAS) lantern_context_k
             if (bad <= m) status |= LANTERN_ST_BAD_TABLE;
           }
         }
+        // The tested token's two numerators in common units, in double precision from its raw logits, carried
+        // through every rejection round so far (E <- max(0, E - ratio_i * ep)); the sums they are compared
+        // with are sums of thousands of terms and do not suffer from cancellation.  A token that has lost its
+        // mass (it lay in an earlier A, or was itself rejected before) has none.  Every thread for itself: by one thread, which
+        // the others then waited for, it took 0.5 us of a context's 5.8 (wide shape), and 0.9 for a second sibling.
+        double e_xt = 0.0, p_xt = 0.0;
+        if constexpr (!GREEDY) {
+          const Exp2Split q = S.single[iter & 1][0], p = S.single[iter & 1][1];
+          e_xt = q.y * exp2_int_d(q.n - static_cast<double>(Nq));
+          p_xt = p.y * exp2_int_d(p.n - static_cast<double>(Np));
+          if (ci > 0) {
+            const float bulk = mass(xt);
+            if (ci <= 32) {
+              for (int i = 0; i < ci; ++i) e_xt = fmax(0.0, e_xt - S.hist[i] * p_xt);
+              if (bulk == 0.0f) e_xt = 0.0;
+            } else {
+              e_xt = static_cast<double>(bulk);
+            }
+            bool again = false;
+            for (int j = lane; j < ci; j += 32) again |= kids[j].token == xt;
+            if (__any_sync(kFull, again)) p_xt = 0.0;
+          }
+        }
         // Section 4.3: accept iff r p(x~) < sum_A q, i.e. r p_xt / Zp_c < (e_xt + sm) / Zq_c, both sides times Zq_c Zp_c
         // (greedy decoding: x~ itself as every other numerator, so that the largest one compares equal to itself)
-        const double p_xt = GREEDY ? 0.0 : S.acc_p;
-        const double qa_un = (GREEDY ? static_cast<double>(mass(xt)) : S.acc_e) + sm;
+        const double qa_un = (GREEDY ? static_cast<double>(mass(xt)) : e_xt) + sm;
         const bool accept = GREEDY ? qa_un >= static_cast<double>(ex2_approx(__fmaf_rn(Np, L2E, -Nq)))
                             : Zp_c > 0.0 ? static_cast<double>(r) * p_xt * Zq_c < qa_un * Zp_c : 0.0 < qa_un;
         if (gt == 0 && (P.out_qa || P.out_px || P.out_m)) {
@@ -1185,20 +1196,15 @@ __global__ void __launch_bounds__(SHAPE::THREADS, SHAPE::CTAS) lantern_context_k
         }
         if (gt == 0) E[EI(xt)] = -fabsf(E[EI(xt)]);
         // x~ leaves the drafter distribution for the following siblings: the residual pass below strikes
-        // every token rejected so far (children 0..ci) from the drafter logits it fetches.  Which of this
-        // thread's chunks hold one:
-        uint32_t struck = 0;
-        for (int j = 0; j <= ci; ++j) {
-          const int t = j == ci ? xt : kids[j].token;
-          if (((t >> 3) & (GT - 1)) == gt) struck |= 1u << (t >> (3 + LOG_GT));
-        }
+        // every token rejected so far (children 0..ci) from the drafter logits
+        if (((xt >> 3) & (GT - 1)) == gt) struck |= StruckMask<CH>(1) << ((xt >> (3 + LOG_GT)) * 8 + (xt & 7));
         const bool last = (ci + 1 == nchild);
         if (!last) {   // next sibling's neighbour row and raw logits, in flight during the residual pass
           node = sib.x;
           xt = sib.y;
           r = __int_as_float(sib.z);
           load_slots(xt, 0, nb);
-          if (gt == 0) fetch_single();
+          if (gt < 2) fetch_single();
         }
         gbar();   // [flags]
         // w = E - (p'/q' scale ratio) * ep in common units, i.e. E - ratio * ep in the slice's own units
@@ -1236,14 +1242,9 @@ __global__ void __launch_bounds__(SHAPE::THREADS, SHAPE::CTAS) lantern_context_k
                   }
                 }
               }
-              if ((struck >> c) & 1u) {   // a token rejected in this context sits in this chunk
-                for (int j = 0; j <= ci; ++j) {
-                  const int t = kids[j].token;
-                  if ((t >> 3) == g) {
+              if (const uint32_t gone = static_cast<uint32_t>(struck >> (8 * c)) & 0xffu) {   // tokens rejected in this context
 #pragma unroll
-                    for (int e = 0; e < 8; ++e) z[e] = (t & 7) == e ? ninf : z[e];
-                  }
-                }
+                for (int e = 0; e < 8; ++e) z[e] = (gone >> e) & 1u ? ninf : z[e];
               }
               const ulonglong2 ea = *reinterpret_cast<const ulonglong2*>(E + EI(g * 8));
               const ulonglong2 eb = *reinterpret_cast<const ulonglong2*>(E + EI(g * 8 + 4));
@@ -1272,7 +1273,8 @@ __global__ void __launch_bounds__(SHAPE::THREADS, SHAPE::CTAS) lantern_context_k
         if (last) break;   // the draw below takes it from here
         const double z = warp_pair_sum(wsum, psum * pow2_double(fd), lane);
         if ((lane & 15) == 0) S.wz[gw][lane >> 4] = z;
-        if (gt == 0) note_single();
+        if (gt < 2) note_single();
+        if (gt == 0 && ci < 32) S.hist[ci] = static_cast<double>(ratio_g);
         gbar();   // [totals] also publishes the written-back residual
         const double2 z2 = *reinterpret_cast<const double2*>(S.wz[lane & (GW - 1)]);
         double W = z2.x, Sp = z2.y;
@@ -1285,7 +1287,6 @@ __global__ void __launch_bounds__(SHAPE::THREADS, SHAPE::CTAS) lantern_context_k
           status |= LANTERN_ST_DEGENERATE;
           break;
         }
-        if (gt == 0 && ci < 32) S.hist[ci] = static_cast<double>(ratio_g);
         Zq_c = W;
         Zp_c = Sp > 0.0 ? Sp : 0.0;
         }
