@@ -23,7 +23,7 @@
 namespace lantern {
 
 // ---------------------------------------------------------------------------------------
-// kernel 1: plan.  One warp per sequence: validate tokens / parents / uniforms, bucket the
+// kernel 1: plan.  One warp per sequence, two for a tree of at most 64 drafts: validate tokens / parents / uniforms, bucket the
 // nodes by parent context (children in node order), initialise the per-node outputs, and write
 // one self-contained work item per context with children.
 //
@@ -36,7 +36,7 @@ namespace lantern {
 // ---------------------------------------------------------------------------------------
 constexpr int kPlanArrays = 13;  // per-warp arrays of N + 2 ints in shared memory
 
-// One sequence of more than 64 drafts, by one warp; returns the number of its contexts with children, or its fault bits << 16.
+// A tree of more than 64 drafts, by one warp; returns its plan_word.
 __device__ __forceinline__ int plan_sequence(const VerifyParams& P, int* plan_smem, int b, int warp, int lane) {
   const int N = P.N, R = P.R, B = P.B;
   if (b >= B) return 0;
@@ -61,7 +61,7 @@ __device__ __forceinline__ int plan_sequence(const VerifyParams& P, int* plan_sm
     const size_t o = static_cast<size_t>(b) * N + i;
     const int tok = P.tokens[o];
     if (static_cast<unsigned>(tok) >= static_cast<unsigned>(P.V)) status |= LANTERN_ST_BAD_TOKEN;
-    const int par = P.parents ? P.parents[o] : i - 1;
+    const int par = P.parents[o];
     if (par < -1 || par >= i) status |= LANTERN_ST_BAD_PARENT;
     else atomicAdd(&cnt[par + 1], 1);
     s_par[i] = par;
@@ -89,8 +89,11 @@ __device__ __forceinline__ int plan_sequence(const VerifyParams& P, int* plan_sm
     if (P.out_status) P.out_status[b] = status ? status : LANTERN_ST_INTERNAL;
   }
   if (status) {   // the walk reports the fault; no work is queued for this sequence
-    for (int r = lane; r < N; r += 32) P.work[static_cast<size_t>(r) * B + b].item = -1;
-    return status << 16;
+    for (int r = lane; r < N; r += 32) {
+      P.work[static_cast<size_t>(r) * B + b].item = -1;
+      if (P.leaves) P.leaves[static_cast<size_t>(r) * B + b] = -1;
+    }
+    return plan_word(0, 0, status);
   }
 
   ChildInfo* kids = P.children + static_cast<size_t>(b) * N;
@@ -100,17 +103,7 @@ __device__ __forceinline__ int plan_sequence(const VerifyParams& P, int* plan_sm
   // context with children (dep).  All of it by the whole warp, 32 nodes at a time.
   int n_ctx = 0;
   const unsigned below = (1u << lane) - 1u;
-  if (!P.parents) {
-    // a chain: context c has the one child c, lies c deep, and has the R - c contexts from itself on behind it
-    for (int c = lane; c < R; c += 32) {
-      cur[c] = c < N ? c + 1 : N;
-      siz[c] = R - c;
-      din[c] = c;
-      dep[c] = c;
-      if (c < N) s_pos[c] = c, s_first[c] = c;
-    }
-    n_ctx = N;
-  } else {
+  {
     // -- child-list offsets: cur[c] = end of the children of context c
     int carry = 0;
     for (int base = 0; base < R; base += 32) {
@@ -261,196 +254,211 @@ __device__ __forceinline__ int plan_sequence(const VerifyParams& P, int* plan_sm
                                 __int_as_float(s_uni[f]), u_final, b * R + din[c]};
     }
   }
-  return n_ctx;
+  if (P.leaves) {   // the contexts without children, by number
+    int n = 0;
+    for (int base = 0; base < R; base += 32) {
+      const int c = base + lane;
+      const bool leaf = c < R && cnt[c] == 0;
+      const unsigned bal = __ballot_sync(kFull, leaf);
+      if (leaf) P.leaves[static_cast<size_t>(n + __popc(bal & below)) * B + b] = din[c] << 16 | c;
+      n += __popc(bal);
+    }
+    for (int r = n + lane; r < N; r += 32) P.leaves[static_cast<size_t>(r) * B + b] = -1;
+  }
+  return plan_word(n_ctx, R - n_ctx, 0);
 }
 
-// The same for at most 64 drafts, two per lane: sets of nodes are 64-bit masks, so that a context's children, a node's
-// ancestors (by doubling) and the contexts of a level are one word each, and the rest are sums over the bits of a word.
-// A 60-node tree takes 2 us here; the general path above, with its level-by-level passes, 9 us.
-constexpr int PLAN_SMALL = 64;
-struct SmallPlan {
-  unsigned long long kids[PLAN_SMALL + 1];    // children of context c
-  unsigned long long level[PLAN_SMALL + 1];   // nodes of depth d that have children
-  unsigned long long anc[PLAN_SMALL];         // ancestors of node i
-  int jump[PLAN_SMALL];                       // doubling: the farthest ancestor in anc so far, -1 = none beyond it
-  int size[PLAN_SMALL + 1];                   // contexts in the subtree of context c, itself included
-  int weight[PLAN_SMALL];                     // steps in pre-order from a node's parent to the node
-  int start[PLAN_SMALL + 1];                  // where the children of context c begin in the child lists
-  int rank[PLAN_SMALL + 1], span[PLAN_SMALL + 1], tok[PLAN_SMALL];
-  float uni[PLAN_SMALL];
-};
+// The faults of one draft's inputs, and what stands in its outputs until the fused pass has tested it.
+__device__ __forceinline__ int plan_node(const VerifyParams& P, int b, int i, int& tok, float& uni) {
+  const size_t o = static_cast<size_t>(b) * P.N + i;
+  tok = P.tokens[o];
+  uni = P.uniforms ? P.uniforms[static_cast<size_t>(b) * P.R + i] : 0.0f;   // (greedy decoding draws nothing and passes no uniforms)
+  const float qnan = __int_as_float(0x7fc00000);
+  if (P.out_path) P.out_path[o] = -1;
+  if (P.out_qa) P.out_qa[o] = qnan;
+  if (P.out_px) P.out_px[o] = qnan;
+  if (P.out_m) P.out_m[o] = -1;
+  return (static_cast<unsigned>(tok) < static_cast<unsigned>(P.V) ? 0 : LANTERN_ST_BAD_TOKEN) | (uni >= 0.0f && uni < 1.0f ? 0 : LANTERN_ST_BAD_UNIFORM);
+}
+__device__ __forceinline__ float plan_final(const VerifyParams& P, int b, int& status) {
+  const float u = P.uniforms ? P.uniforms[static_cast<size_t>(b) * P.R + P.N] : 0.0f;
+  if (!(u >= 0.0f && u < 1.0f)) status |= LANTERN_ST_BAD_UNIFORM;
+  return u;
+}
+// what stands for the sequence if the fused pass never gets to its end
+__device__ __forceinline__ void plan_outcome(const VerifyParams& P, int b, int status) {
+  P.out_len[b] = 0;
+  P.out_tok[b] = -1;
+  if (P.out_status) P.out_status[b] = status ? status : LANTERN_ST_INTERNAL;
+}
+// no work is queued for a sequence with a fault
+__device__ __forceinline__ int plan_fault(const VerifyParams& P, int b, int from, int stride, int status) {
+  for (int r = from; r < max(P.N, 1); r += stride) {
+    P.work[static_cast<size_t>(r) * P.B + b].item = -1;
+    if (P.leaves) P.leaves[static_cast<size_t>(r) * P.B + b] = -1;
+  }
+  return plan_word(0, 0, status);
+}
 
-__device__ __forceinline__ int plan_small(const VerifyParams& P, SmallPlan& S, int b, int lane) {
+// A chain, by one warp: context c has the one child c, lies c deep, and has the R - c contexts from itself on behind it.  Nothing has to be
+// worked out, so that the time is that of the loads and the stores (8192 chains of 7: 4.8 us through the code for trees).
+__device__ __forceinline__ int plan_chain(const VerifyParams& P, int b, int lane) {
   const int N = P.N, R = P.R, B = P.B;
   if (b >= B) return 0;
-  int par[2], tok[2] = {0, 0};
-  float uni[2] = {0.0f, 0.0f}, u_final = 0.0f;
-  // all inputs at once
-#pragma unroll
-  for (int q = 0; q < 2; ++q) {
-    const int i = lane + 32 * q;
-    const size_t o = static_cast<size_t>(b) * N + i;
-    par[q] = i - 1;
-    if (i < N) {
-      tok[q] = P.tokens[o];
-      if (P.parents) par[q] = P.parents[o];
-      if (P.uniforms) uni[q] = P.uniforms[static_cast<size_t>(b) * R + i];
-    }
-  }
-  if (P.uniforms) u_final = P.uniforms[static_cast<size_t>(b) * R + N];
-  for (int c = lane; c <= PLAN_SMALL; c += 32) S.kids[c] = S.level[c] = 0ull, S.size[c] = 1;
-  for (int c = lane; c < R; c += 32) P.dead[static_cast<size_t>(b) * R + c] = 0;
-  const float qnan = __int_as_float(0x7fc00000);
-  int status = u_final >= 0.0f && u_final < 1.0f ? 0 : LANTERN_ST_BAD_UNIFORM;
-#pragma unroll
-  for (int q = 0; q < 2; ++q) {
-    const int i = lane + 32 * q;
-    const size_t o = static_cast<size_t>(b) * N + i;
-    if (i < N) {
-      if (static_cast<unsigned>(tok[q]) >= static_cast<unsigned>(P.V)) status |= LANTERN_ST_BAD_TOKEN;
-      if (par[q] < -1 || par[q] >= i) status |= LANTERN_ST_BAD_PARENT;
-      if (!(uni[q] >= 0.0f && uni[q] < 1.0f)) status |= LANTERN_ST_BAD_UNIFORM;
-      if (P.out_path) P.out_path[o] = -1;
-      if (P.out_qa) P.out_qa[o] = qnan;
-      if (P.out_px) P.out_px[o] = qnan;
-      if (P.out_m) P.out_m[o] = -1;
-    }
+  int status = 0, tok = 0, first_tok = 0;
+  float uni = 0.0f, first_uni = 0.0f;
+  const float u_final = plan_final(P, b, status);
+  for (int c = lane; c < R; c += 32) {
+    if (c < N) status |= plan_node(P, b, c, tok, uni);
+    if (c == lane) first_tok = tok, first_uni = uni;
+    P.dead[static_cast<size_t>(b) * R + c] = 0;
   }
   status = __reduce_or_sync(kFull, status);
-  if (lane == 0) {   // what stands if the fused pass never gets to the end of this sequence
-    P.out_len[b] = 0;
-    P.out_tok[b] = -1;
-    if (P.out_status) P.out_status[b] = status ? status : LANTERN_ST_INTERNAL;
-  }
-  if (status) {   // no work is queued for this sequence
-    for (int r = lane; r < max(N, 1); r += 32) P.work[static_cast<size_t>(r) * B + b].item = -1;
-    return status << 16;
-  }
-  if (N == 0) {   // no drafts: one draw from the root's q
-    if (lane == 0) {
-      P.records[b].word = kWalkLeaf;
-      P.work[b] = {b, 0, 0, 0, 0, 0.0f, u_final, b};
-    }
-    return 1;
-  }
-  __syncwarp();
-#pragma unroll
-  for (int q = 0; q < 2; ++q) {
-    const int i = lane + 32 * q;
-    if (i < N) {
-      atomicOr(&S.kids[par[q] + 1], 1ull << i);
-      S.anc[i] = par[q] >= 0 ? 1ull << par[q] : 0ull;
-      S.jump[i] = par[q];
-      S.tok[i] = tok[q];
-      S.uni[i] = uni[q];
-    }
-  }
-  __syncwarp();
-  for (;;) {
-    unsigned long long more_anc[2];
-    int to[2];
-    bool more = false;
-#pragma unroll
-    for (int q = 0; q < 2; ++q) {
-      const int i = lane + 32 * q;
-      const int a = i < N ? S.jump[i] : -1;
-      to[q] = a >= 0 ? S.jump[a] : -1;
-      more_anc[q] = a >= 0 ? S.anc[a] : 0ull;
-      more |= to[q] >= 0;
-    }
-    __syncwarp();
-#pragma unroll
-    for (int q = 0; q < 2; ++q) {
-      const int i = lane + 32 * q;
-      if (i < N) S.anc[i] |= more_anc[q], S.jump[i] = to[q];
-    }
-    __syncwarp();
-    if (!__any_sync(kFull, more)) break;
-  }
-  unsigned long long anc[2], below[2], with[2];   // ancestors, smaller nodes, earlier siblings
-  int depth[2], kids[2];
-#pragma unroll
-  for (int q = 0; q < 2; ++q) {
-    const int i = lane + 32 * q;
-    const bool on = i < N;
-    anc[q] = on ? S.anc[i] : 0ull;
-    below[q] = (1ull << i) - 1ull;
-    with[q] = on ? S.kids[par[q] + 1] & below[q] : 0ull;
-    depth[q] = __popcll(anc[q]) + 1;
-    kids[q] = on ? __popcll(S.kids[i + 1]) : 0;
-    if (kids[q]) atomicOr(&S.level[depth[q]], 1ull << i);
-    for (unsigned long long m = anc[q]; m; m &= m - 1ull) atomicAdd(&S.size[__ffsll(m)], 1);   // (context of node a: a + 1)
-  }
-  if (lane == 0) S.size[0] = R;
-  __syncwarp();
-#pragma unroll
-  for (int q = 0; q < 2; ++q) {
-    const int i = lane + 32 * q;
-    int w = 1;
-    for (unsigned long long m = with[q]; m; m &= m - 1ull) w += S.size[__ffsll(m)];
-    if (i < N) S.weight[i] = w;
-  }
-  // child lists in the order of the contexts
-  const int n_root = __popcll(S.kids[0]);
-  int carry = n_root, n_ctx = 1;
-#pragma unroll
-  for (int q = 0; q < 2; ++q) {
-    const int i = lane + 32 * q;
-    int incl = kids[q];
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const int t = __shfl_up_sync(kFull, incl, o);
-      if (lane >= o) incl += t;
-    }
-    if (i < N) S.start[i + 1] = carry + incl - kids[q];
-    carry += __shfl_sync(kFull, incl, 31);
-    n_ctx += __popc(__ballot_sync(kFull, kids[q] > 0));
-  }
-  if (lane == 0) S.start[0] = 0, S.rank[0] = 0, S.span[0] = R;
-  __syncwarp();
-#pragma unroll
-  for (int q = 0; q < 2; ++q) {
-    const int i = lane + 32 * q;
-    if (i < N) {
-      int pos = S.weight[i], rank = 1;                   // pre-order position; breadth-first rank, where it has children
-      for (unsigned long long m = anc[q]; m; m &= m - 1ull) pos += S.weight[__ffsll(m) - 1];
-      for (int d = 1; d < depth[q]; ++d) rank += __popcll(S.level[d]);
-      S.rank[i + 1] = rank + __popcll(S.level[depth[q]] & below[q]);
-      S.span[i + 1] = pos << 16 | S.size[i + 1];
-      const ChildInfo info = {i, tok[q], uni[q], pos << 16 | S.size[i + 1]};
-      P.children[static_cast<size_t>(b) * N + S.start[par[q] + 1] + __popcll(with[q])] = info;
-    }
-  }
-  __syncwarp();
-  for (int r = n_ctx + lane; r < N; r += 32) P.work[static_cast<size_t>(r) * B + b].item = -1;
+  if (lane == 0) plan_outcome(P, b, status);
+  if (status) return plan_fault(P, b, lane, 32, status);
   for (int c = lane; c < R; c += 32) {
-    const unsigned long long m = S.kids[c];
-    P.records[static_cast<size_t>(b) * R + c].word = m == 0ull ? kWalkLeaf : (c == 0 ? kWalkWaiting : kWalkPending);
-    if (m) {
-      const int f = __ffsll(m) - 1;                      // its first child
-      P.work[static_cast<size_t>(S.rank[c]) * B + b] = {b * R + c, b * N + S.start[c], __popcll(m) << 16 | f, S.span[f + 1], S.tok[f],
-                                                        S.uni[f], u_final, b * R + (S.span[c] >> 16)};
+    tok = first_tok, uni = first_uni;
+    if (c != lane && c < N) {   // (from the second 32 on: read again)
+      tok = P.tokens[static_cast<size_t>(b) * N + c];
+      uni = P.uniforms ? P.uniforms[static_cast<size_t>(b) * R + c] : 0.0f;
     }
+    const int span = (c + 1) << 16 | (N - c);
+    P.records[static_cast<size_t>(b) * R + c].word = c == N ? kWalkLeaf : (c == 0 ? kWalkWaiting : kWalkPending);
+    if (c < N) {
+      P.children[static_cast<size_t>(b) * N + c] = {c, tok, uni, span};
+      P.work[static_cast<size_t>(c) * B + b] = {b * R + c, b * N + c, 1 << 16 | c, span, tok, uni, u_final, b * R + c};
+    } else if (N == 0) {        // no drafts: one draw from the root's q
+      P.work[b] = {b * R, 0, 0, 0, 0, 0.0f, u_final, b * R};
+    }
+    if (P.leaves && c < N) P.leaves[static_cast<size_t>(c) * B + b] = c == 0 ? N << 16 | N : -1;
   }
-  return n_ctx;
+  return N > 0 ? plan_word(N, 1, 0) : plan_word(1, 0, 0);
 }
 
-__global__ void __launch_bounds__(PLAN_WARPS * 32) lantern_plan_kernel(VerifyParams P) {
+// A tree of at most 64 drafts, by two warps, a draft per thread: sets of nodes are 64-bit masks, and what else is needed is summed up on
+// the way from a node to the root (paths are short where a tree is wide).  By one warp with two drafts per lane, and the ancestors by
+// doubling, a 60-node tree took 6.4 us here, of which 1 us is the inputs' way.
+constexpr int PLAN_SMALL = 64;
+struct alignas(8) SmallPlan {
+  unsigned kids[PLAN_SMALL + 1][2];    // children of context c
+  unsigned level[PLAN_SMALL + 1][2];   // nodes of depth d that have children
+  unsigned parents[2];                 // nodes that have children
+  int size[PLAN_SMALL + 1];            // contexts behind context c
+  int par[PLAN_SMALL], weight[PLAN_SMALL];   // parent; steps in pre-order from the parent to the node
+  int start[PLAN_SMALL + 1];           // where the children of context c begin in the child lists
+  int rank[PLAN_SMALL + 1], span[PLAN_SMALL + 1], tok[PLAN_SMALL];
+  float uni[PLAN_SMALL];
+  int status, placed;
+};
+
+__device__ __forceinline__ int plan_small(const VerifyParams& P, SmallPlan& S, int b, int seq, int t) {
+  const int N = P.N, R = P.R, B = P.B;
+  if (b >= B) return 0;
+  auto sync = [&]() { asm volatile("bar.sync %0, 64;" ::"r"(1 + seq) : "memory"); };
+  auto kids_of = [&](int c) { return *reinterpret_cast<const unsigned long long*>(S.kids[c]); };
+  auto level_at = [&](int d) { return *reinterpret_cast<const unsigned long long*>(S.level[d]); };
+  const bool on = t < N;
+  int status = 0, par = -1, tok = 0;
+  float uni = 0.0f;
+  if (on) {
+    par = P.parents[static_cast<size_t>(b) * N + t];
+    status = plan_node(P, b, t, tok, uni);
+    if (par < -1 || par >= t) status |= LANTERN_ST_BAD_PARENT;
+  }
+  const float u_final = plan_final(P, b, status);
+  for (int c = t; c < R; c += 64) {
+    P.dead[static_cast<size_t>(b) * R + c] = 0;
+    S.kids[c][0] = S.kids[c][1] = S.level[c][0] = S.level[c][1] = 0u, S.size[c] = 0;
+  }
+  if (t == 0) S.status = 0;
+  if (on) S.par[t] = par, S.tok[t] = tok, S.uni[t] = uni;
+  sync();
+  if (status) atomicOr(&S.status, status);
+  sync();
+  status = S.status;
+  if (t == 0) plan_outcome(P, b, status);
+  if (status) return plan_fault(P, b, t, 64, status);
+  // up to the root: depth, and every ancestor counts the node
+  int depth = 1;
+  if (on) {
+    atomicOr(&S.kids[par + 1][t >> 5], 1u << (t & 31));
+    for (int a = par; a >= 0; a = S.par[a]) {
+      atomicAdd(&S.size[a + 1], 1);
+      ++depth;
+    }
+  }
+  if (t == 0) S.size[0] = N;
+  sync();
+  const unsigned long long below = (1ull << t) - 1ull, with = on ? kids_of(par + 1) & below : 0ull;   // earlier siblings
+  if (t == 0) S.placed = __popcll(kids_of(0));
+  int weight = 1, n_kids = 0;
+  if (on) {
+    for (unsigned long long m = with; m; m &= m - 1ull) weight += S.size[__ffsll(m)] + 1;   // (context of node a: a + 1)
+    S.weight[t] = weight;
+    n_kids = __popcll(kids_of(t + 1));
+    if (n_kids) atomicOr(&S.level[depth][t >> 5], 1u << (t & 31));
+  }
+  {
+    const unsigned some = __ballot_sync(kFull, n_kids > 0);
+    if ((t & 31) == 0) S.parents[t >> 5] = some;
+  }
+  sync();
+  if (t == 0) S.start[0] = 0, S.rank[0] = 0, S.span[0] = R;
+  if (on) {
+    if (n_kids) S.start[t + 1] = atomicAdd(&S.placed, n_kids);
+    // pre-order position; breadth-first rank, where it has children
+    int pos = weight, rank = 1 + __popcll(level_at(depth) & below), d = depth;
+    for (int a = par; a >= 0; a = S.par[a]) pos += S.weight[a], rank += __popcll(level_at(--d));
+    S.rank[t + 1] = rank;
+    S.span[t + 1] = pos << 16 | (S.size[t + 1] + 1);
+  }
+  sync();
+  if (on) P.children[static_cast<size_t>(b) * N + S.start[par + 1] + __popcll(with)] = {t, tok, uni, S.span[t + 1]};
+  // contexts with children (by rank) and without (by number)
+  const unsigned long long has_kids = *reinterpret_cast<const unsigned long long*>(S.parents);
+  const int n_ctx = 1 + __popcll(has_kids), n_leaf = R - n_ctx;
+  for (int c = t; c < R; c += 64) {
+    const unsigned long long m = kids_of(c);
+    P.records[static_cast<size_t>(b) * R + c].word = m == 0ull ? kWalkLeaf : (c == 0 ? kWalkWaiting : kWalkPending);
+    if (m) {
+      const int f = __ffsll(m) - 1;       // its first child
+      P.work[static_cast<size_t>(S.rank[c]) * B + b] = {b * R + c, b * N + S.start[c], __popcll(m) << 16 | f, S.span[f + 1], S.tok[f],
+                                                        S.uni[f], u_final, b * R + (S.span[c] >> 16)};
+    } else if (P.leaves) {
+      const int r = (c - 1) - __popcll(has_kids & ((1ull << (c - 1)) - 1ull));
+      P.leaves[static_cast<size_t>(r) * B + b] = S.span[c] >> 16 << 16 | c;
+    }
+  }
+  for (int r = n_ctx + t; r < N; r += 64) P.work[static_cast<size_t>(r) * B + b].item = -1;
+  if (P.leaves)
+    for (int r = n_leaf + t; r < N; r += 64) P.leaves[static_cast<size_t>(r) * B + b] = -1;
+  return plan_word(n_ctx, n_leaf, 0);
+}
+
+// threads of the plan kernel per sequence
+static inline __host__ __device__ int plan_threads(const VerifyParams& P) { return P.parents && P.N > 0 && P.N <= PLAN_SMALL ? 64 : 32; }
+
+__global__ void __launch_bounds__(PLAN_SEQS * 64) lantern_plan_kernel(VerifyParams P) {
   extern __shared__ int plan_smem[];
-  __shared__ int s_words[PLAN_WARPS];
-  __shared__ SmallPlan s_small[PLAN_WARPS];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  __shared__ int s_words[PLAN_SEQS];
+  __shared__ SmallPlan s_small[PLAN_SEQS];
+  const int per = plan_threads(P), seq = threadIdx.x / per, t = threadIdx.x % per;
   grid_dependency_wait();
   grid_dependents_launch();
   if (blockIdx.x == 0 && threadIdx.x < 64) reinterpret_cast<int*>(P.counters)[threadIdx.x] = 0;
-  const int b = blockIdx.x * PLAN_WARPS + warp;
-  const int word = P.N <= PLAN_SMALL ? plan_small(P, s_small[warp], b, lane) : plan_sequence(P, plan_smem, b, warp, lane);
-  if (lane == 0) s_words[warp] = word;
+  const int b = blockIdx.x * PLAN_SEQS + seq;
+  const int word = !P.parents || P.N == 0 ? plan_chain(P, b, t)
+                                          : (per == 64 ? plan_small(P, s_small[seq], b, seq, t) : plan_sequence(P, plan_smem, b, seq, t));
+  if (t == 0) s_words[seq] = word;
   __syncthreads();
   if (threadIdx.x == 0) {
-    int ranks = 0, bits = 0;
-    for (int w = 0; w < PLAN_WARPS; ++w) ranks = max(ranks, s_words[w] & 0xffff), bits |= s_words[w] >> 16;
-    P.block_words[blockIdx.x] = bits << 16 | ranks;
+    int ranks = 0, leaves = 0, bits = 0;
+    for (int w = 0; w < PLAN_SEQS; ++w) {
+      ranks = max(ranks, s_words[w] & 0x7ff);
+      leaves = max(leaves, s_words[w] >> 11 & 0x7ff);
+      bits |= s_words[w] >> 22;
+    }
+    P.block_words[blockIdx.x] = plan_word(ranks, leaves, bits);
   }
 }
 
@@ -465,7 +473,7 @@ namespace lantern {
 static size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
 struct WsLayout {
-  size_t counters, work, children, records, dead, words, total;
+  size_t counters, work, leaves, children, records, dead, words, total;
 };
 
 static WsLayout ws_layout(int B, int N, bool topk = false) {
@@ -475,11 +483,11 @@ static WsLayout ws_layout(int B, int N, bool topk = false) {
   size_t o = 0;
   L.counters = o; o += 256;
   L.work = o;     o += align_up(b * n1 * sizeof(WorkItem), 256);
-  o += align_up(b * n1 * 4, 256);              // (the size callers have always been told: parts of it are no longer used)
+  L.leaves = o;   o += align_up(b * n1 * 4, 256);
   L.children = o; o += align_up(b * n1 * sizeof(ChildInfo), 256);
   L.records = o;  o += align_up(b * R * sizeof(Record), 256);
   L.dead = o;     o += align_up(b * R, 256);
-  L.words = o;    o += 3 * align_up(b * 4, 256);
+  L.words = o;    o += 3 * align_up(b * 4, 256);   // (the size callers have always been told: parts of it are no longer used)
   o += topk ? 2 * align_up(b * R * 4, 256) : 0;
   L.total = o;
   return L;
@@ -601,6 +609,9 @@ static lantern_status verify_impl(const void* target_logits, const void* draft_l
                                   float* out_node_qa, float* out_node_px, int32_t* out_node_m, void* workspace,
                                   size_t workspace_bytes, void* cuda_stream);
 
+// Few contexts: the SMs have room for bonus draws ahead of time, and the call is short enough for the draw at its end to count.
+static bool leaves_pay(int B, int N, int sms) { return N > 0 && static_cast<long long>(B) * (N + 1) <= 4ll * sms; }
+
 extern "C" lantern_status lantern_verify(const void* target_logits, const void* draft_logits, int dtype,
                                          float cfg_scale, int has_uncond, float T, const int32_t* draft_tokens,
                                          const int32_t* tree_parents, const int32_t* neighbor_idx, int k,
@@ -663,6 +674,8 @@ static lantern_status verify_impl(const void* target_logits, const void* draft_l
   if (!workspace || workspace_bytes < L.total || (reinterpret_cast<uintptr_t>(workspace) & 255))
     return LANTERN_E_WORKSPACE;
 
+  const int sms = sm_count();
+  if (sms < 1) return LANTERN_E_CUDA;
   cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
   unsigned char* ws = static_cast<unsigned char*>(workspace);
   VerifyParams P;
@@ -695,18 +708,17 @@ static lantern_status verify_impl(const void* target_logits, const void* draft_l
   P.divergence = divergence;
   P.top_k = topk ? top_k : 0;
   P.dead = ws + L.dead;
+  P.leaves = leaves_pay(B, N, sms) ? reinterpret_cast<int32_t*>(ws + L.leaves) : nullptr;
   P.wait_tries = g_wait_tries;
   P.withhold_item = g_withhold_item;
 
-  const int sms = sm_count();
-  if (sms < 1) return LANTERN_E_CUDA;
 
-  const size_t plan_smem = N <= PLAN_SMALL ? 0 : static_cast<size_t>(PLAN_WARPS) * kPlanArrays * (N + 2) * sizeof(int);
+  const size_t plan_smem = !tree_parents || N <= PLAN_SMALL ? 0 : static_cast<size_t>(PLAN_SEQS) * kPlanArrays * (N + 2) * sizeof(int);
   static DeviceFlags plan_ready;
   if (plan_smem > 32 * 1024 &&   // (beside the kernel's static part)
-      allow_shared_memory(lantern_plan_kernel, PLAN_WARPS * kPlanArrays * (MAX_N + 2) * sizeof(int), plan_ready) != cudaSuccess)
+      allow_shared_memory(lantern_plan_kernel, PLAN_SEQS * kPlanArrays * (MAX_N + 2) * sizeof(int), plan_ready) != cudaSuccess)
     return LANTERN_E_CUDA;
-  if (launch_dependent(lantern_plan_kernel, (B + PLAN_WARPS - 1) / PLAN_WARPS, PLAN_WARPS * 32, plan_smem, st, P) != cudaSuccess)
+  if (launch_dependent(lantern_plan_kernel, (B + PLAN_SEQS - 1) / PLAN_SEQS, PLAN_SEQS * plan_threads(P), plan_smem, st, P) != cudaSuccess)
     return LANTERN_E_CUDA;
 
   const long long items = static_cast<long long>(B) * (N > 0 ? N : 1);   // upper bound of contexts with children

@@ -14,7 +14,7 @@
 
 namespace lantern {
 
-#define LANTERN_CONTEXT_KERNEL_REVISION 21   // bump on every change to the fused context kernel
+#define LANTERN_CONTEXT_KERNEL_REVISION 22   // bump on every change to the fused context kernel
 
 constexpr int MAX_N = 1024;
 
@@ -74,6 +74,8 @@ struct VerifyParams {
   Counters* counters;
   WorkItem* work;               // [N, B]: slot r * B + b holds the r-th context with children of sequence b in
                                 //         breadth-first order (by depth, then by index); item = -1 where there is none
+  int32_t* leaves;              // [N, B]: slot r * B + b holds the r-th context without children of sequence b, (its place in
+                                //         pre-order << 16) | its number, -1 where there is none; null: not listed (see verify.cu)
   unsigned char* dead;          // [B, R], a sequence's contexts in pre-order: 1 once the walk is known not to reach one
   ChildInfo* children;          // [B, N]
   Record* records;              // [B, R]
@@ -82,8 +84,7 @@ struct VerifyParams {
   int divergence;               // LANTERN_DIV_TVD or LANTERN_DIV_JSD: what delta bounds
   int top_k;                    // logit filter; 0 = off
   uint32_t wait_tries;          // limit of every bounded mbarrier wait, in tries
-  int32_t* block_words;         // one word per block of the plan kernel: largest number of contexts with children in one of
-                                //     its sequences, and its sequences' fault bits << 16
+  int32_t* block_words;         // one word per block of the plan kernel: see plan_word
   int withhold_item;            // self-test only: the copies of this context are never issued (-1 = none)
 };
 
@@ -97,32 +98,40 @@ constexpr double kDegenerate = 1e-5;
 // context, exchanged by whoever decides the context and by the walk when it gets there.
 //   bits 0..1 state; walk waiting: bits 8..15 status so far, bits 16..31 drafts accepted so far;
 //   decided: bits 8..15 status, bits 16..31 accepted node + 1 (0 = none), bits 32..63 replacement token
-enum : unsigned { kWalkPending = 0, kWalkWaiting = 1, kWalkDecided = 2, kWalkLeaf = 3 };
+// A context without children starts as kWalkLeaf: the bonus draw is made by the walk when it gets there, or ahead of time by a
+// producer that has exchanged kWalkLeaf for kWalkPending first; its decided word carries kWalkDrawn.
+enum : unsigned { kWalkPending = 0, kWalkWaiting = 1, kWalkDecided = 2, kWalkLeaf = 3, kWalkDrawn = 4 };
 __device__ __forceinline__ unsigned long long walk_word(unsigned state, unsigned status, unsigned count, int token = 0) {
   return state | (status << 8) | (static_cast<unsigned long long>(count) << 16) |
          (static_cast<unsigned long long>(static_cast<unsigned>(token)) << 32);
 }
 
-constexpr int PLAN_WARPS = 4;   // sequences per block of the plan kernel
+constexpr int PLAN_SEQS = 4;    // sequences per block of the plan kernel
 
-// The plan's summary, by a whole warp: slots in the occupied part of the work list, and the fault bits of all sequences.
-__device__ __forceinline__ int plan_slots(const VerifyParams& P, int lane, int& faults) {
-  int ranks = P.parents ? 0 : (P.N > 0 ? P.N : 1), bits = 0;
-  const int blocks = (P.B + PLAN_WARPS - 1) / PLAN_WARPS;
+// A block of the plan kernel sums up its sequences in one word: the largest number of contexts with children in one of them, the
+// largest number of contexts without, and all fault bits.
+__device__ __forceinline__ int plan_word(int ranks, int leaves, int faults) { return faults << 22 | leaves << 11 | ranks; }
+// The plan's summary, by a whole warp: slots in the occupied parts of the work list and of the list of leaves, and the fault bits
+// of all sequences.
+struct PlanSummary {
+  int slots, leaf_slots, faults;
+};
+__device__ __forceinline__ PlanSummary plan_summary(const VerifyParams& P, int lane) {
+  int ranks = P.N > 0 ? 0 : 1, leaves = 0, bits = 0;
+  const int blocks = (P.B + PLAN_SEQS - 1) / PLAN_SEQS;
 #pragma unroll 4
   for (int i = lane; i < blocks; i += 32) {
     const int w = P.block_words[i];
-    ranks = max(ranks, w & 0xffff);
-    bits |= w >> 16;
+    ranks = max(ranks, w & 0x7ff);
+    leaves = max(leaves, w >> 11 & 0x7ff);
+    bits |= w >> 22;
   }
-  faults = __reduce_or_sync(kFull, bits);
-  return __reduce_max_sync(kFull, ranks) * P.B;
+  return {__reduce_max_sync(kFull, ranks) * P.B, P.leaves ? __reduce_max_sync(kFull, leaves) * P.B : 0, static_cast<int>(__reduce_or_sync(kFull, bits))};
 }
-// The same without the fault bits: a chain has a context with a child for every draft.
-__device__ __forceinline__ int plan_slots(const VerifyParams& P, int lane) {
-  if (!P.parents) return (P.N > 0 ? P.N : 1) * P.B;
-  int faults;
-  return plan_slots(P, lane, faults);
+// The same without the fault bits: a chain has a context with a child for every draft, and one leaf.
+__device__ __forceinline__ PlanSummary plan_extent(const VerifyParams& P, int lane) {
+  if (!P.parents) return {(P.N > 0 ? P.N : 1) * P.B, P.leaves ? P.B : 0, 0};
+  return plan_summary(P, lane);
 }
 
 __device__ __forceinline__ float sum8(const float* v) {

@@ -397,6 +397,16 @@ __global__ void __launch_bounds__(SHAPE::THREADS, SHAPE::CTAS) lantern_context_k
   // The plan, and whatever made the inputs.  This kernel may be in place while the plan still writes: what the plan writes is read by
   // ordinary loads, which stay behind this wait.  Logits and neighbour rows are read through the read-only path: they are
   // complete before any CTA of this kernel starts, because every CTA of the plan lets it start only after a wait of its own.
+  // Before that: rows that are going to be read whatever the plan says are asked into L2 while it runs -- the root of the sequence that this
+  // group begins with, or every row of a call so small that no group gets more than a few.
+  if (lane == 0 && tid >= NGRP * GT) {
+    const int G = gridDim.x * NGRP, me = ((tid - NGRP * GT) >> 5) * gridDim.x + blockIdx.x;
+    if (P.leaves) {
+      for (int c = me; c < P.B * R; c += G) ctx_prefetch_rows<UNC, !GREEDY, true>(P, c, rowbytes);
+    } else if (me < P.B) {
+      ctx_prefetch_rows<UNC, !GREEDY, true>(P, me * R, rowbytes);
+    }
+  }
   grid_dependency_wait();
 
   // ======================= producer warps =======================
@@ -411,7 +421,6 @@ __global__ void __launch_bounds__(SHAPE::THREADS, SHAPE::CTAS) lantern_context_k
   if (tid >= NGRP * GT) {
     const int grp = (tid - NGRP * GT) >> 5;
     GroupShared<GW, TOPK>& S = SG[grp];
-    const int total = plan_slots(P, lane);       // occupied part of the slot array
     const int G = gridDim.x * NGRP;              // producers in the grid
     const int me = grp * gridDim.x + blockIdx.x; // few contexts: one to an SM before any SM gets a second one
     const uint32_t tries = P.wait_tries;
@@ -421,33 +430,57 @@ __global__ void __launch_bounds__(SHAPE::THREADS, SHAPE::CTAS) lantern_context_k
     // far to find that many live ones: tree workloads leave most slots empty or dead, and every batch costs a
     // round trip to the work list.
     int slots_seen = 0, live_seen = 0;
+    // slots of the work list that are in use, and those of the list of leaves behind them
+    PlanSummary extent = {P.B * (N > 0 ? N : 1), P.leaves ? P.B * N : 0, 0};   // (at most, until the plan's summary has been read)
     auto batch_size = [&](int at) {
-      const int share = (total - at) / (4 * G);
+      const int share = (extent.slots + extent.leaf_slots - at) / (4 * G);
       const int live = share < 1 ? 1 : (share > 2 ? 2 : share);
       const int s = live * ((slots_seen + 1) / (live_seen + 1));
       return s < 1 ? 1 : (s > 32 ? 32 : s);
     };
-    // what a lane keeps of a candidate: its slot, its context and its dead mark (the rest is read when it is taken)
+    // What a lane keeps of a candidate: its slot, its context and its dead mark (the rest is read when it is taken).  Slots beyond those
+    // of the contexts with children are those of the leaves.
     struct Cand {
       int slot, item, mark;
     };
     auto load_cand = [&](int start, int size) -> Cand {
       Cand c = {start + lane, -1, 0};
-      if (lane < size && c.slot < total) {
-        c.item = P.work[c.slot].item;
-        c.mark = P.work[c.slot].mark;
+      const int leaf = c.slot - extent.slots;
+      if (lane < size) {
+        if (leaf < 0) {
+          c.item = P.work[c.slot].item;
+          c.mark = P.work[c.slot].mark;
+        } else if (leaf < extent.leaf_slots) {
+          const int w = P.leaves[leaf], b = leaf % P.B;
+          if (w >= 0) c.item = b * R + (w & 0xffff), c.mark = b * R + (w >> 16);
+        }
       }
       return c;
+    };
+    // the rest, by the candidate's lane
+    auto load_item = [&](const Cand& c, int4& lo, int4& hi) {
+      if (c.slot < extent.slots) {
+        lo = *reinterpret_cast<const int4*>(P.work + c.slot);
+        hi = *(reinterpret_cast<const int4*>(P.work + c.slot) + 1);
+      } else {                 // nothing but a draw
+        lo = make_int4(c.item, 0, 0, 0), hi = make_int4(0, 0, 0, 0);
+        if (P.uniforms) hi.z = __float_as_int(P.uniforms[static_cast<size_t>(c.item / R) * R + N]);
+      }
     };
     auto is_dead = [&](int mark) -> bool {
       return *reinterpret_cast<const volatile unsigned char*>(P.dead + mark) != 0;
     };
+    // A bonus draw ahead of time: the leaf is taken if the walk has not got there yet.
+    auto claim_leaf = [&](int item) -> bool {
+      return atomicCAS(&P.records[item].word, static_cast<unsigned long long>(kWalkLeaf), static_cast<unsigned long long>(kWalkPending)) ==
+             static_cast<unsigned long long>(kWalkLeaf);
+    };
     int n_eval = 0, n_skip = 0, n_draw = 0;
     // live candidates of a batch, as a lane mask
-    auto filter = [&](const Cand& c) -> unsigned {
+    auto filter = [&](const Cand& c, bool first) -> unsigned {
       const bool has = c.item >= 0;
-      const bool dead = has && is_dead(c.mark);
-      n_skip += __popc(__ballot_sync(kFull, dead));
+      const bool dead = has && !first && is_dead(c.mark);
+      n_skip += __popc(__ballot_sync(kFull, dead && c.slot < extent.slots));
       const unsigned live = __ballot_sync(kFull, has && !dead);
       live_seen += __popc(live);
       return live;
@@ -455,8 +488,17 @@ __global__ void __launch_bounds__(SHAPE::THREADS, SHAPE::CTAS) lantern_context_k
     // Tickets for the dynamic batches are asked for two batches ahead and the candidates of a batch are read one batch
     // ahead, so that a producer waits for neither.
     const int b0 = batch_size(0);
-    Cand cur = load_cand(me * b0, b0), nxt;
-    bool cur_end = me * b0 >= total, nxt_end = false, primed = false;
+    Cand cur = {me * b0 + lane, -1, 0}, nxt;
+    int4 lo = make_int4(-1, 0, 0, 0), hi = make_int4(0, 0, 0, 0);      // the description of this lane's candidate
+    if (lane < b0 && cur.slot < extent.slots) load_item(cur, lo, hi);   // (the first batch at once, beside the summary)
+    cur.item = lo.x, cur.mark = hi.w;
+    extent = plan_extent(P, lane);
+    const int total = extent.slots + extent.leaf_slots;
+    bool cur_end = me * b0 >= total, nxt_end = false, primed = false, described = true;   // (lo and hi: only of the first batch, and until used)
+    if (me * b0 + b0 > extent.slots) {   // (the leaves begin earlier than was assumed)
+      cur = load_cand(me * b0, b0);
+      if (cur.item >= 0) load_item(cur, lo, hi);
+    }
     int ticket = 0, ticket_size = 0, seen = G * b0;
     auto ask = [&]() {       // (lane 0 holds the answer)
       ticket_size = batch_size(seen < total ? seen : total);
@@ -470,7 +512,7 @@ __global__ void __launch_bounds__(SHAPE::THREADS, SHAPE::CTAS) lantern_context_k
       ask();
     };
     ask();
-    unsigned mask = filter(cur);
+    unsigned mask = filter(cur, true);
     auto next_batch = [&]() {   // make `mask` non-empty if any live context is left
       if (!primed) {
         primed = true;
@@ -479,8 +521,9 @@ __global__ void __launch_bounds__(SHAPE::THREADS, SHAPE::CTAS) lantern_context_k
       while (mask == 0 && !cur_end) {
         cur = nxt;
         cur_end = nxt_end;
+        described = false;
         if (!cur_end) load_next();
-        mask = filter(cur);
+        mask = filter(cur, false);
       }
     };
     // A sequence's final outcome.  (Its status stood at INTERNAL until now, see the plan kernel.)
@@ -489,8 +532,10 @@ __global__ void __launch_bounds__(SHAPE::THREADS, SHAPE::CTAS) lantern_context_k
       if (P.out_status) P.out_status[b] = status;
       if (status) atomicOr(&P.counters->status_or, status);
     };
-    // Lane 0: a pending draw from a context's own q, and the context handed out last (everything its result needs;
-    // nc0 = nchild << 16 | node0, 0 for a draw).  `open`: that context's result has not been taken yet.
+    // A pending draw from a context's own q, and the context handed out last (everything its result needs;
+    // nc0 = nchild << 16 | node0, kDrawForWalk for a draw the walk has asked for, kDrawAhead for one made ahead of it).
+    // `open`: that context's result has not been taken yet.
+    constexpr int kDrawForWalk = 0, kDrawAhead = 1;
     int draw_item = -1, draw_status = 0;
     float draw_u = 0.0f;
     int p_item = 0, p_cbase = 0, p_nc0 = 0, p_span0 = 0, p_status = 0;
@@ -501,17 +546,28 @@ __global__ void __launch_bounds__(SHAPE::THREADS, SHAPE::CTAS) lantern_context_k
       if (!mbar_wait(&bar_done[grp][j & 1], (j >> 1) & 1, tries)) return false;
       open = false;
       const CtxResult res = S.result[j & 1];
-      const int item = __shfl_sync(kFull, p_item, 0), nc0 = __shfl_sync(kFull, p_nc0, 0);
+      const int item = p_item, nc0 = p_nc0;
       const int b = item / R;
-      if (nc0 == 0) {
+      if (nc0 == kDrawForWalk) {
+        ++n_draw;
         if (lane == 0) finish(b, res.token, p_status | res.status);
         return true;
       }
+      Record* recs = P.records + static_cast<size_t>(b) * R;
+      // Few sequences: most of a path has been decided by the time the walk comes along.  The words of all its contexts (two to a
+      // lane) travel together with the first exchange, and what was decided is followed without further round trips.
+      unsigned long long seen0 = 0, seen1 = 0;
+      bool looked = P.leaves && R <= 64;
+      auto look = [&]() {
+        if (lane < R) seen0 = walk_look(recs + lane);
+        if (lane + 32 < R) seen1 = walk_look(recs + lane + 32);
+      };
+      if (looked) look();
       // Algorithm 1 goes on from the accepted child only: every context behind another child is dead.  In
       // pre-order those are one contiguous range per child.
-      const int cbase = __shfl_sync(kFull, p_cbase, 0), span0 = __shfl_sync(kFull, p_span0, 0), nchild = nc0 >> 16;
+      const int cbase = p_cbase, span0 = p_span0, nchild = nc0 >> 16;
       unsigned char* marks = P.dead + static_cast<size_t>(b) * R;
-      for (int c = 0; c < nchild; ++c) {
+      for (int c = 0; c < nchild; ++c) {   // (none behind a leaf)
         int node_c = nc0 & 0xffff, span_c = span0;
         if (c > 0) {
           const int4 kid = *reinterpret_cast<const int4*>(P.children + cbase + c);
@@ -521,14 +577,14 @@ __global__ void __launch_bounds__(SHAPE::THREADS, SHAPE::CTAS) lantern_context_k
           for (int o = lane; o < (span_c & 0xffff); o += 32) marks[(span_c >> 16) + o] = 1;
       }
       // (all lanes follow the walk; lane 0 exchanges and stores)
-      Record* recs = P.records + static_cast<size_t>(b) * R;
       int at = item - b * R, accepted = res.accepted, token = res.token, status = res.status;
       auto exchange = [&](unsigned long long v) {
         unsigned long long w = 0;
         if (lane == 0) w = walk_exchange(recs + at, v);
         return __shfl_sync(kFull, w, 0);
       };
-      unsigned long long w = exchange(walk_word(kWalkDecided, status, accepted + 1, token));
+      bool drawn = nc0 == kDrawAhead;
+      unsigned long long w = exchange(walk_word(kWalkDecided | (drawn ? kWalkDrawn : 0u), status, accepted + 1, token));
       if ((w & 3u) == kWalkWaiting) {   // the walk stands here already: go on with it
         int st = static_cast<int>(w >> 8) & 0xff, len = static_cast<int>(w >> 16) & 0xffff;
         const int len_before = len;
@@ -542,6 +598,7 @@ __global__ void __launch_bounds__(SHAPE::THREADS, SHAPE::CTAS) lantern_context_k
           bool from_q = (status & LANTERN_ST_DEGENERATE) != 0;   // a residual without weight: draw from the context's own target
           if (!from_q) {
             if (accepted < 0) {
+              n_draw += drawn;
               if (lane == 0) finish(b, token, st);
               break;
             }
@@ -549,7 +606,15 @@ __global__ void __launch_bounds__(SHAPE::THREADS, SHAPE::CTAS) lantern_context_k
             ++len;
             at = accepted + 1;
             w = 0;
-            if (++steps > kWalkAlone) {
+            if (R <= 64) {
+              if (looked || steps > 2) {
+                if (!looked) look();
+                looked = true;
+                const unsigned long long w0 = __shfl_sync(kFull, seen0, at & 31), w1 = __shfl_sync(kFull, seen1, at & 31);
+                w = at < 32 ? w0 : w1;
+              }
+              ++steps;
+            } else if (++steps > kWalkAlone) {
               // the contexts that were decided in favour of the node numbered as they are, from this one on, are followed at once
               for (int run = 32; run == 32;) {
                 const unsigned long long seen = at + lane < R ? walk_look(recs + at + lane) : 0;
@@ -574,6 +639,7 @@ __global__ void __launch_bounds__(SHAPE::THREADS, SHAPE::CTAS) lantern_context_k
           status = static_cast<int>(w >> 8) & 0xff;
           accepted = static_cast<int>(w >> 16 & 0xffff) - 1;
           token = static_cast<int>(w >> 32);
+          drawn = (w & kWalkDrawn) != 0;
         }
         if (lane == 0 && len > len_before) atomicMax(&P.out_len[b], len);   // (pieces of the path may be stored out of order)
       }
@@ -581,6 +647,7 @@ __global__ void __launch_bounds__(SHAPE::THREADS, SHAPE::CTAS) lantern_context_k
       return true;
     };
     int i = 0;        // contexts handed to the group so far
+    int stop = 0;     // the abort flag, as it stood when the last context was handed out
     bool clean = true;
     for (;;) {
       const bool drawing = __shfl_sync(kFull, draw_item, 0) >= 0;
@@ -595,48 +662,43 @@ __global__ void __launch_bounds__(SHAPE::THREADS, SHAPE::CTAS) lantern_context_k
           continue;
         }
       }
-      int l = 0;
-      int4 lo = make_int4(0, 0, 0, 0), hi = make_int4(0, 0, 0, 0);
-      if (!drawing) {
+      int l = 0;               // the lane that hands it out
+      bool leaf = false;
+      int it_status = 0;
+      if (drawing) {
+        lo = make_int4(draw_item, 0, 0, 0), hi = make_int4(0, 0, __float_as_int(draw_u), 0);
+        it_status = draw_status;
+        draw_item = -1;
+      } else {                 // (a work slot without children is a draw from the outset: a call without drafts)
         l = __ffs(mask) - 1;
         mask &= mask - 1;
-        const int slot = __shfl_sync(kFull, cur.slot, l);
-        if (lane == 0) {   // its description, in flight while the group is waited for
-          lo = *reinterpret_cast<const int4*>(P.work + slot);
-          hi = *(reinterpret_cast<const int4*>(P.work + slot) + 1);
-        }
+        leaf = __shfl_sync(kFull, cur.slot, l) >= extent.slots;
+        if (!described && lane == l) load_item(cur, lo, hi);   // in flight while the group is waited for
+        described = false;
       }
       if (i >= 1 && !mbar_wait(&bar_next[grp], (i - 1) & 1, tries)) {
         clean = false;   // the group never came this far: it has given up, and so does its producer
         break;
       }
-      // as late as possible: has the context died meanwhile, has the call been given up?
-      const int gone = (!drawing && lane == l && is_dead(cur.mark)) ? 1 : 0;
-      const int stop = *reinterpret_cast<const volatile int*>(&P.counters->abort);
-      if (__any_sync(kFull, stop != 0)) break;
-      if (__any_sync(kFull, gone)) {
-        ++n_skip;
-        continue;
+      if (__any_sync(kFull, stop != 0)) break;   // the call has been given up
+      // as late as possible: has the context died meanwhile?  (Not the first one: nothing has been decided.)
+      if (!drawing && (i > 0 || leaf)) {
+        int gone = 0;
+        if (lane == l) gone = (is_dead(cur.mark) ? 1 : 0) | (leaf && !claim_leaf(cur.item) ? 1 : 0);
+        if (__any_sync(kFull, gone)) {
+          n_skip += leaf ? 0 : 1;
+          continue;
+        }
       }
-      GroupItem it;
-      int it_status = 0;
-      if (drawing) {
-        it.item = draw_item, it.cbase = 0, it.nchild = 0, it.node0 = 0, it.span0 = 0, it.tok0 = 0, it.r0 = 0.0f, it.u_final = draw_u;
-        it_status = draw_status;
-        draw_item = -1;
-      } else {   // (a work slot without children is a draw from the outset: a call without drafts)
-        it.item = lo.x, it.cbase = lo.y, it.nchild = lo.z >> 16, it.node0 = lo.z & 0xffff, it.span0 = lo.w;
-        it.tok0 = hi.x, it.r0 = __int_as_float(hi.y), it.u_final = __int_as_float(hi.z);
-      }
-      if (lane == 0) {
-        S.work[i & 1] = it;
+      if (lane == l) {
+        S.work[i & 1] = {lo.x, lo.y, lo.z >> 16, lo.z & 0xffff, hi.x, lo.w, __int_as_float(hi.y), __int_as_float(hi.z)};
         mbar_arrive(&bar_item[grp]);
       }
       const int area = i % AREAS;
       auto issue = [&]() {
-        if (lane == 0 && it.item != P.withhold_item) {   // (self-test of the bounded waits: nothing is copied)
+        if (lane == l && lo.x != P.withhold_item) {   // (self-test of the bounded waits: nothing is copied)
           fence_proxy_async();
-          ctx_issue_target<UNC>(P, it.item, smem + (grp * AREAS + area) * area_bytes, rowbytes, &bar_rows[grp][area]);
+          ctx_issue_target<UNC>(P, lo.x, smem + (grp * AREAS + area) * area_bytes, rowbytes, &bar_rows[grp][area]);
         }
       };
       bool ok = true;
@@ -651,11 +713,11 @@ __global__ void __launch_bounds__(SHAPE::THREADS, SHAPE::CTAS) lantern_context_k
           if (open) take_result(i - 1);
         }
       }
-      const bool draw_now = __shfl_sync(kFull, it.nchild, 0) == 0;
-      n_draw += draw_now ? 1 : 0;
-      n_eval += draw_now ? 0 : 1;
-      p_item = it.item, p_cbase = it.cbase, p_nc0 = draw_now ? 0 : (it.nchild << 16 | it.node0), p_span0 = it.span0;
-      p_status = it_status, p_u = it.u_final;
+      p_item = __shfl_sync(kFull, lo.x, l), p_cbase = __shfl_sync(kFull, lo.y, l), p_span0 = __shfl_sync(kFull, lo.w, l);
+      p_nc0 = __shfl_sync(kFull, lo.z, l), p_u = __int_as_float(__shfl_sync(kFull, hi.z, l));
+      p_status = it_status;
+      if (p_nc0 == 0) p_nc0 = leaf ? kDrawAhead : kDrawForWalk;
+      else ++n_eval;
       open = true;
       ++i;
       if (!ok) {
@@ -665,6 +727,7 @@ __global__ void __launch_bounds__(SHAPE::THREADS, SHAPE::CTAS) lantern_context_k
       // Look ahead: the next live context (a batch swap, if the current batch is used up, happens here, where
       // nothing waits for it) and an L2 prefetch of its rows -- of a context that has passed the dead check,
       // so that hardly any prefetched row goes unused.
+      stop = *reinterpret_cast<const volatile int*>(&P.counters->abort);
       next_batch();
       if (mask && __shfl_sync(kFull, draw_item, 0) < 0) {
         const int item_ahead = __shfl_sync(kFull, cur.item, __ffs(mask) - 1);
@@ -686,8 +749,7 @@ __global__ void __launch_bounds__(SHAPE::THREADS, SHAPE::CTAS) lantern_context_k
       if (n_draw) atomicAdd(&P.counters->n_bonus, n_draw);
     }
     if (me == 0) {   // sequences that the plan found at fault
-      int faults;
-      plan_slots(P, lane, faults);
+      const int faults = plan_summary(P, lane).faults;
       if (faults && lane == 0) atomicOr(&P.counters->status_or, faults);
     }
     return;

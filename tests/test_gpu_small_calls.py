@@ -1,0 +1,60 @@
+"""Calls of few contexts: bonus draws are made ahead of the walk, which follows what has been decided in one go; the plan has
+code of its own for chains and for trees of at most 64 drafts."""
+import numpy as np
+import pytest
+import torch
+
+import lantern_inputs as li
+import paper_2410_03355_b200 as lt
+import test_gpu_greedy as greedy
+from parity import assert_parity, compare, near_ceiling, run_gpu, tables, to_device
+
+pytestmark = pytest.mark.gpu
+
+
+def _sms():
+    return torch.cuda.get_device_properties(0).multi_processor_count
+
+
+def _inputs(B, N, tree, seed, V=512, **kw):
+    par = li.tree_parents(B, N, depth=min(N, 7), seed=seed) if tree else None
+    return li.verify_inputs(B, N, V, dtype=li.BF16, has_uncond=True, cfg_scale=2.0, rho=0.9, sigma_draft=0.4, parents=par, seed=seed, **kw)
+
+
+@pytest.mark.parametrize("tree", [False, True])
+@pytest.mark.parametrize("N", [1, 2, 31, 32, 33, 63, 64, 70])
+@pytest.mark.parametrize("many", [0, 1, 2])   # one sequence; as many as have their bonus draws made ahead; one more
+def test_small_calls_against_oracle(N, tree, many):
+    B = 1 if many == 0 else 4 * _sms() // (N + 1) + many - 1
+    B = min(B, 40) if N < 31 and many == 1 else B
+    inp = _inputs(B, N, tree, seed=7 * N + many)
+    host, dev = tables(li.codebook_gaussian(512, 8, seed=18), 40, inp.draft_tokens)
+    res = compare(inp, host, 0.4, run_gpu(inp, dev, 0.4))
+    assert_parity(res)
+    assert res["near"] <= near_ceiling(B)
+
+
+@pytest.mark.parametrize("N,tree", [(5, False), (20, True)])
+def test_draws_ahead_are_counted_once_and_repeat(N, tree):
+    """Who makes a draw depends on timing; the outputs do not, and every sequence that ends on a leaf has one."""
+    B = 12
+    inp = _inputs(B, N, tree, seed=N)
+    host, dev = tables(li.codebook_gaussian(512, 8, seed=18), 40, inp.draft_tokens)
+    d = to_device(inp)
+    ws = torch.empty(lt.verify_workspace_bytes(B, N, inp.V, 40), dtype=torch.uint8, device="cuda")
+    want = None
+    for _ in range(200):
+        out = lt.verify(d["target_logits"], d["draft_logits"], 2.0, 1.0, d["draft_tokens"], d["tree_parents"], dev, 0.4, d["uniforms"], workspace=ws)
+        got = [t.cpu().numpy() for t in (out.accept_len, out.next_token, out.accept_path, out.status)]
+        want = got if want is None else want
+        assert all(np.array_equal(a, b) for a, b in zip(got, want))
+        par = inp.tree_parents if tree else np.broadcast_to(np.arange(-1, N - 1), (B, N))
+        last = [got[2][b, got[0][b] - 1] if got[0][b] else -1 for b in range(B)]
+        assert lt.verify_counts(ws)["from_q"] == sum(not (par[b] == last[b]).any() for b in range(B))
+
+
+@pytest.mark.parametrize("N,tree", [(6, False), (33, True)])
+def test_greedy_small_calls(N, tree):
+    inp = _inputs(3, N, tree, seed=50 + N)
+    host, dev = tables(li.codebook_gaussian(512, 8, seed=18), 40, inp.draft_tokens)
+    greedy.check(inp, host, dev, 0.4)
