@@ -1,4 +1,4 @@
-"""ctypes binding of liblantern.so: argument marshalling only.
+"""Binding of liblantern.so: argument marshalling only, through ctypes and, for the usual form of verify(), natively (csrc/call.cpp).
 
 Functions mirror the C entry points of include/lantern.h.  Tensors must live on a CUDA device;
 there is no CPU path: a missing library or a CPU tensor raises.
@@ -19,6 +19,7 @@ ST_BAD_TOKEN, ST_BAD_PARENT, ST_BAD_UNIFORM, ST_NONFINITE, ST_DEGENERATE, ST_BAD
 _HERE = os.path.dirname(os.path.abspath(__file__))
 _LIB_PATH = os.path.join(_HERE, "liblantern.so")
 _lib = None
+_call = None
 
 
 class LanternError(RuntimeError):
@@ -33,7 +34,7 @@ def library_path() -> str:
 
 def load_library():
     """Load liblantern.so (built in-tree by paper_2410_03355_b200.build). Fails loudly if absent."""
-    global _lib
+    global _lib, _call
     if _lib is not None:
         return _lib
     if not os.path.exists(_LIB_PATH):
@@ -79,7 +80,9 @@ def load_library():
     lib.lantern_verify.restype = i32
     lib.lantern_verify.argtypes = [vp, vp, i32, f32, i32, f32, vp, vp, vp, i32, f32, vp, i32, i32, i32,
                                    vp, vp, vp, vp, vp, vp, vp, vp, sz, vp]
-    _lib = lib
+    from . import _call as call      # the native part of verify(), built beside the library
+    call.bind(ctypes.cast(lib.lantern_verify_ex, ctypes.c_void_p).value)
+    _lib, _call = lib, call
     return lib
 
 
@@ -194,9 +197,17 @@ def verify(target_logits: torch.Tensor, draft_logits: Optional[torch.Tensor], cf
     T == 0 selects greedy decoding: draft_logits and uniforms are not read and may be None.
     divergence "tvd" | "jsd": what delta bounds (Section 5.3.2); top_k: logit filter, 0 = off (Appendix B.2).
     """
+    lib = load_library()
+    if out is not None and workspace is not None and stream is None:
+        # nothing to allocate: the arguments go to the library natively, unless one of them is not what it has to be
+        rc = _call.verify(target_logits, draft_logits, cfg_scale, T, draft_tokens, tree_parents, neighbor_idx, delta, uniforms, out,
+                          workspace, DIVERGENCES.get(divergence), top_k)
+        if rc is not None:
+            if rc != 0:
+                raise LanternError(rc, "lantern_verify_ex")
+            return out
     if divergence not in DIVERGENCES:
         raise ValueError(f"divergence must be one of {sorted(DIVERGENCES)}")
-    lib = load_library()
     if T != 0 and (uniforms is None or (draft_logits is None and target_logits.shape[2] > 1)):
         raise ValueError("sampling (T > 0) needs draft_logits and uniforms")
     C, B, R, V = target_logits.shape

@@ -1,4 +1,5 @@
-"""Builds the CUDA library in-tree: csrc/*.cu -> paper_2410_03355_b200/liblantern.so (sm_100a)."""
+"""Builds the CUDA library in-tree: csrc/*.cu -> paper_2410_03355_b200/liblantern.so (sm_100a), and the native part of the
+binding: csrc/call.cpp -> paper_2410_03355_b200/_call.so."""
 from __future__ import annotations
 
 import os
@@ -9,6 +10,7 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "liblantern.so")
+CALL = os.path.join(HERE, "_call.so")
 
 OBJ = os.path.join(HERE, "_build")
 
@@ -21,11 +23,11 @@ def sources():
 
 
 def _stale() -> bool:
-    if not os.path.exists(LIB):
+    if not os.path.exists(LIB) or not os.path.exists(CALL):
         return True
-    t = os.path.getmtime(LIB)
+    t = min(os.path.getmtime(LIB), os.path.getmtime(CALL))
     deps = sources() + [os.path.join(CSRC, f) for f in os.listdir(CSRC) if f.endswith(".cuh")]
-    deps.append(os.path.join(ROOT, "include", "lantern.h"))
+    deps += [os.path.join(CSRC, "call.cpp"), os.path.join(ROOT, "include", "lantern.h")]
     return any(os.path.getmtime(d) > t for d in deps)
 
 
@@ -45,8 +47,24 @@ def build(force: bool = False, verbose: bool = False) -> str:
         subprocess.check_call(common + ["-c", src, "-o", obj])
         return obj
 
+    def compile_call():    # (the libraries are torch's, which is imported before it)
+        import sysconfig
+
+        import torch
+        at = os.path.dirname(torch.__file__)
+        inc = os.path.join(at, "include")
+        subprocess.check_call([nvcc, "-gencode", "arch=compute_100a,code=sm_100a", "-cudart", "none", "-O2", "-std=c++17",
+                               "-Xcompiler", "-fPIC", "-shared",
+                               f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}",
+                               "-I", os.path.join(ROOT, "include"), "-I", sysconfig.get_paths()["include"], "-I", inc,
+                               "-I", os.path.join(inc, "torch", "csrc", "api", "include"),
+                               os.path.join(CSRC, "call.cpp"), "-o", CALL, "-L", os.path.join(at, "lib"),
+                               "-ltorch_python", "-ltorch_cpu", "-lc10_cuda", "-lc10"])
+
     with ThreadPoolExecutor(max_workers=min(8, os.cpu_count() or 1)) as pool:
+        call = pool.submit(compile_call)
         objs = list(pool.map(compile_one, sources()))
+        call.result()
     subprocess.check_call([nvcc, "-gencode", "arch=compute_100a,code=sm_100a", "-shared", "-o", LIB] + objs)
     return LIB
 

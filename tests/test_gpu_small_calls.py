@@ -1,5 +1,7 @@
 """Calls of few contexts: bonus draws are made ahead of the walk, which follows what has been decided in one go; the plan has
-code of its own for chains and for trees of at most 64 drafts."""
+code of its own for chains and for trees of at most 64 drafts.  And the forms a call's arguments can take."""
+import dataclasses
+
 import numpy as np
 import pytest
 import torch
@@ -58,3 +60,48 @@ def test_greedy_small_calls(N, tree):
     inp = _inputs(3, N, tree, seed=50 + N)
     host, dev = tables(li.codebook_gaussian(512, 8, seed=18), 40, inp.draft_tokens)
     greedy.check(inp, host, dev, 0.4)
+
+
+def test_forms_of_a_call():
+    """Outputs and workspace given or not, integer scalars, a stream, tensor subclasses: the same results; what was refused
+    is refused."""
+    B, N = 5, 6
+    inp = _inputs(B, N, True, seed=3)
+    host, dev = tables(li.codebook_gaussian(512, 8, seed=18), 40, inp.draft_tokens)
+    d = to_device(inp)
+    ws = torch.empty(lt.verify_workspace_bytes(B, N, inp.V, 40), dtype=torch.uint8, device="cuda")
+
+    def call(**kw):
+        a = dict(target=d["target_logits"], draft=d["draft_logits"], cfg=2.0, T=1.0, tokens=d["draft_tokens"], parents=d["tree_parents"], nbr=dev,
+                 delta=0.4, uniforms=d["uniforms"])
+        rest = {k: v for k, v in kw.items() if k not in a}
+        a.update({k: v for k, v in kw.items() if k in a})
+        out = lt.verify(*a.values(), **rest)
+        torch.cuda.synchronize()
+        return out
+
+    def same(x, y):
+        for f in ("accept_len", "next_token", "accept_path", "status"):
+            assert torch.equal(getattr(x, f), getattr(y, f)), f
+
+    want = call()
+    out = dataclasses.replace(call(), node_qa=torch.empty((B, N), device="cuda"))
+    assert call(out=out, workspace=ws) is out
+    same(out, want)
+    for kw in (dict(cfg=2, T=1), dict(target=torch.nn.Parameter(d["target_logits"], requires_grad=False)), dict(stream=torch.cuda.Stream()),
+               dict(cfg=np.float32(2.0))):
+        torch.cuda.synchronize()
+        same(call(out=out, workspace=ws, **kw), want)
+    part = lt.VerifyOutputs(out.accept_len, out.next_token, None, None, None, None, None)
+    call(out=part, workspace=ws)
+    assert torch.equal(part.next_token, want.next_token)
+    refused = [dict(target=d["target_logits"].half()), dict(draft=d["draft_logits"].float()), dict(tokens=d["draft_tokens"].long()),
+               dict(uniforms=d["uniforms"].cpu()), dict(nbr=dev[:100]), dict(uniforms=None), dict(divergence="kl"),
+               dict(tokens=d["draft_tokens"].t().contiguous().t()), dict(target=d["target_logits"][:, :, :, :256]),
+               dict(out=dataclasses.replace(out, accept_len=out.accept_len.long()))]
+    for kw in refused:
+        with pytest.raises(ValueError):
+            call(**{**dict(out=out, workspace=ws), **kw})
+    for kw in (dict(workspace=ws[:256]), dict(T=-1.0), dict(delta=float("nan")), dict(top_k=-1)):
+        with pytest.raises(lt.binding.LanternError):
+            call(**{**dict(out=out, workspace=ws), **kw})
