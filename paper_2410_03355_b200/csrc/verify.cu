@@ -19,6 +19,7 @@
 #include "verify_common.cuh"
 
 #include <stddef.h>
+#include <string.h>
 
 namespace lantern {
 
@@ -609,6 +610,24 @@ static lantern_status verify_impl(const void* target_logits, const void* draft_l
                                   float* out_node_qa, float* out_node_px, int32_t* out_node_m, void* workspace,
                                   size_t workspace_bytes, void* cuda_stream);
 
+// what divide_by_T (verify_context.cuh) goes by
+static void set_divisor(VerifyParams& P, float T) {
+  const double inv = 1.0 / static_cast<double>(T);
+  auto pair = [](float f) {
+    uint32_t w;
+    memcpy(&w, &f, 4);
+    return static_cast<uint64_t>(w) << 32 | w;
+  };
+  P.T_plain = T >= 0x1p-100f && T <= 0x1p100f;
+  P.T_neg = pair(-T);
+  const float y = P.T_plain ? static_cast<float>(inv) : 1.0f;
+  const float hi = static_cast<double>(y) > inv ? nextafterf(y, 0.0f) : y;
+  const float lo = P.T_plain ? static_cast<float>(inv - static_cast<double>(hi)) : 0.0f;
+  P.T_inv = pair(y);
+  P.T_inv_hi = pair(hi);
+  P.T_inv_lo = pair(lo > 0.0f ? lo : 0x1p-126f);   // (a power of two leaves nothing; the product with -inf has to be -inf)
+}
+
 // Few contexts: the SMs have room for bonus draws ahead of time, and the call is short enough for the draw at its end to count.
 static bool leaves_pay(int B, int N, int sms) { return N > 0 && static_cast<long long>(B) * (N + 1) <= 4ll * sms; }
 
@@ -705,6 +724,7 @@ static lantern_status verify_impl(const void* target_logits, const void* draft_l
   P.cfg_scale = cfg_scale;
   P.T = T;
   P.delta = delta;
+  set_divisor(P, T);
   P.divergence = divergence;
   P.top_k = topk ? top_k : 0;
   P.dead = ws + L.dead;

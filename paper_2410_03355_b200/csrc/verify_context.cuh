@@ -315,6 +315,33 @@ __device__ __forceinline__ double warp_transposed_sum(const float (&v)[N], int l
   return d[0];
 }
 
+// Four pairs of logits divided by the temperature, each quotient rounded once (IEEE division).  With y_hi + y_lo = 1 / T to 47 bits,
+// q = fl(l y_hi + fl(l y_lo)) is off by hardly more than half a unit in the last place, so that the remainder r = l - q T is exact, and
+// fl(q + r y) with y = fl(1 / T) is the correctly rounded quotient (Markstein, IBM J. Res. Dev. 34(1), 1990): four packed operations a
+// pair where a division takes some ten instructions a value.  Where q is -inf (a masked token: l = -inf, or so low that the quotient
+// overflows) the remainder is no number or +inf; its bound keeps the quotient -inf, as it should be (y_lo > 0), and a NaN a NaN.  (Where
+// q is +inf the row is reported, be it as +inf or as a NaN.)  Exact for 2^-100 <= T <= 2^100 and |l| of 2^-100 and above, or
+// zero; below, z is off by a unit in the last place of a number that is nothing beside any other logit.
+static __device__ __noinline__ uint64_t divide_pair(uint64_t v, float T) {
+  float lo, hi;
+  unpack2(v, lo, hi);
+  return pack2(__fdiv_rn(lo, T), __fdiv_rn(hi, T));
+}
+__device__ __forceinline__ void divide_by_T(const VerifyParams& P, uint64_t (&z)[4]) {
+  if (P.T_plain) {
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const uint64_t q = fma2(z[i], P.T_inv_hi, mul2(z[i], P.T_inv_lo));
+      float lo, hi;
+      unpack2(fma2(P.T_neg, q, z[i]), lo, hi);
+      z[i] = fma2(pack2(fminf(lo, 3.402823466e38f), fminf(hi, 3.402823466e38f)), P.T_inv, q);
+    }
+  } else {
+#pragma unroll
+    for (int i = 0; i < 4; ++i) z[i] = divide_pair(z[i], P.T);
+  }
+}
+
 // one bit per token of a thread
 template <int CH>
 using StruckMask = typename std::conditional<(CH > 4), uint64_t, uint32_t>::type;
@@ -772,11 +799,6 @@ __global__ void __launch_bounds__(SHAPE::THREADS, SHAPE::CTAS) lantern_context_k
   const size_t branch = static_cast<size_t>(P.B) * R * V;   // elements from a conditional row to its unconditional one
   const uint32_t tries = P.wait_tries;
   auto gbar = [&]() { asm volatile("bar.sync %0, %1;" ::"r"(1 + grp), "n"(GT) : "memory"); };   // the group's threads
-  auto divide_T = [&](uint64_t v) {
-    float lo, hi;
-    unpack2(v, lo, hi);
-    return pack2(__fdiv_rn(lo, P.T), __fdiv_rn(hi, P.T));
-  };
   // this thread's slots SLOTS gt .. of a neighbour row, from slot `base` on (slot 0 is the token itself,
   // entries past the row are not looked at)
   auto load_slots = [&](int token, int base, int (&n)[SLOTS]) {
@@ -897,9 +919,9 @@ __global__ void __launch_bounds__(SHAPE::THREADS, SHAPE::CTAS) lantern_context_k
       for (int c = 0; c < CH; ++c) {
         uint64_t z2[4];
         raw8_pairs<BF16>(raw[c], z2);
+        if (!TONE) divide_by_T(P, z2);
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
-          if (!TONE) z2[i] = divide_T(z2[i]);
           float lo, hi;
           if (TOPK) {
             unpack2(z2[i], lo, hi);
@@ -939,11 +961,14 @@ __global__ void __launch_bounds__(SHAPE::THREADS, SHAPE::CTAS) lantern_context_k
               staged_pairs<BF16>(rc, g, c2);
               if (UNC) staged_pairs<BF16>(ru, g, u2);
             }
+            if (UNC && !TOPK) {
+#pragma unroll
+              for (int i = 0; i < 4; ++i) c2[i] = fma2(s2, sub2(c2[i], u2[i]), u2[i]);   // l_u + s (l_c - l_u)
+            }
+            if (!TONE && !TOPK) divide_by_T(P, c2);
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
               uint64_t l2 = c2[i];
-              if (UNC && !TOPK) l2 = fma2(s2, sub2(c2[i], u2[i]), u2[i]);   // l_u + s (l_c - l_u)
-              if (!TONE && !TOPK) l2 = divide_T(l2);
               float lo, hi;
               unpack2(l2, lo, hi);
               if (TOPK) {   // (a NaN stays, to be reported)
@@ -996,11 +1021,9 @@ __global__ void __launch_bounds__(SHAPE::THREADS, SHAPE::CTAS) lantern_context_k
         auto own = [&](int c, float (&z)[8]) {
           uint64_t z2[4];
           raw8_pairs<BF16>(raw[c], z2);
+          if (!TONE) divide_by_T(P, z2);
 #pragma unroll
-          for (int i = 0; i < 4; ++i) {
-            if (!TONE) z2[i] = divide_T(z2[i]);
-            unpack2(z2[i], z[2 * i], z[2 * i + 1]);
-          }
+          for (int i = 0; i < 4; ++i) unpack2(z2[i], z[2 * i], z[2 * i + 1]);
         };
         auto again = [&](int c, float (&z)[8]) {
           row_logits<BF16, TONE>(P, P.draft, static_cast<size_t>(item) * V, c * GT + gt, z);
@@ -1023,13 +1046,13 @@ __global__ void __launch_bounds__(SHAPE::THREADS, SHAPE::CTAS) lantern_context_k
           uint64_t c2[4], u2[4];
           staged_pairs<BF16>(stage, g, c2);
           if (UNC) staged_pairs<BF16>(stage + rowbytes, g, u2);
+          if (UNC) {
 #pragma unroll
-          for (int i = 0; i < 4; ++i) {
-            uint64_t l2 = c2[i];
-            if (UNC) l2 = fma2(pack2(P.cfg_scale, P.cfg_scale), sub2(c2[i], u2[i]), u2[i]);
-            if (!TONE) l2 = divide_T(l2);
-            unpack2(l2, z[2 * i], z[2 * i + 1]);
+            for (int i = 0; i < 4; ++i) c2[i] = fma2(pack2(P.cfg_scale, P.cfg_scale), sub2(c2[i], u2[i]), u2[i]);
           }
+          if (!TONE) divide_by_T(P, c2);
+#pragma unroll
+          for (int i = 0; i < 4; ++i) unpack2(c2[i], z[2 * i], z[2 * i + 1]);
         };
         auto guided_in_place = [&](int c, float (&z)[8]) {
           const int g = c * GT + gt;
@@ -1294,9 +1317,9 @@ __global__ void __launch_bounds__(SHAPE::THREADS, SHAPE::CTAS) lantern_context_k
               {
                 uint64_t z2[4];
                 raw8_pairs<BF16>(drafted, z2);
+                if (!TONE) divide_by_T(P, z2);
 #pragma unroll
                 for (int i = 0; i < 4; ++i) {
-                  if (!TONE) z2[i] = divide_T(z2[i]);
                   unpack2(z2[i], z[2 * i], z[2 * i + 1]);
                   if (TOPK) {
                     z[2 * i] = z[2 * i] < tp ? ninf : z[2 * i];

@@ -105,3 +105,24 @@ def test_forms_of_a_call():
     for kw in (dict(workspace=ws[:256]), dict(T=-1.0), dict(delta=float("nan")), dict(top_k=-1)):
         with pytest.raises(lt.binding.LanternError):
             call(**{**dict(out=out, workspace=ws), **kw})
+
+
+@pytest.mark.parametrize("top_k", [0, 100])
+@pytest.mark.parametrize("T", [0.7, 0.9, 1.2, 0.5, 3.0, 1e-31, 1e31])
+def test_temperatures_with_masked_tokens(T, top_k):
+    """Quotients by the temperature: powers of two, others, and such as go the long way; tokens masked by -inf and by the lowest
+    bf16 value, whose quotient overflows."""
+    V, B, N = 512, 24, 3
+    far = not 0.1 < T < 10                   # logits of a like size then
+    inp = li.verify_inputs(B, N, V, dtype=li.BF16, has_uncond=False, cfg_scale=1.0, T=1.0 if far else T, sigma_draft=0.5, seed=5)
+    if far:
+        inp = dataclasses.replace(inp, T=T, **{f: li.f32_to_bf16_bits(li.bf16_bits_to_f32(getattr(inp, f)) * np.float32(T))
+                                               for f in ("target_logits", "draft_logits")})
+    rng = np.random.default_rng(4)
+    keep = np.zeros((B, V), bool)
+    keep[np.arange(B)[:, None], inp.draft_tokens] = True
+    for arr in (inp.target_logits[0], inp.draft_logits):
+        for value in (0xff80, 0xff7f):       # -inf, the lowest finite value
+            arr[np.broadcast_to(((rng.random((B, V)) < 0.2) & ~keep)[:, None, :], arr.shape)] = value
+    host, dev = tables(li.codebook_gaussian(V, 8, seed=19), 40, inp.draft_tokens)
+    assert_parity(compare(inp, host, 0.3, run_gpu(inp, dev, 0.3, top_k=top_k), top_k=top_k))
