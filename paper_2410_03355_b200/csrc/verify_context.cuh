@@ -435,6 +435,8 @@ __global__ void __launch_bounds__(SHAPE::THREADS, SHAPE::CTAS) lantern_context_k
     }
   }
   grid_dependency_wait();
+  // (Small calls: the next call's plan may be in place, waiting, when this kernel ends.  One tree 19.0 -> 18.3 us per call.)
+  if (P.leaves) grid_dependents_launch();
 
   // ======================= producer warps =======================
   // One warp per consumer group hands out work, keeps that group's copies going and walks.  Its 32 lanes look
@@ -676,7 +678,14 @@ __global__ void __launch_bounds__(SHAPE::THREADS, SHAPE::CTAS) lantern_context_k
     int i = 0;        // contexts handed to the group so far
     int stop = 0;     // the abort flag, as it stood when the last context was handed out
     bool clean = true;
+    // A context handed to a group that has siblings to try yet waits for all of them: in a small call of trees the next one is chosen
+    // when the group's result is known (8 trees 38.0 -> 36.5 us per call; chains have no siblings, and lose by it).
+    const bool late = P.leaves && P.parents;
     for (;;) {
+      if (late && open && !take_result(i - 1)) {
+        clean = false;
+        break;
+      }
       const bool drawing = __shfl_sync(kFull, draw_item, 0) >= 0;
       if (!drawing) {
         if (mask == 0) next_batch();
