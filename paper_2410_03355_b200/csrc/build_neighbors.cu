@@ -702,9 +702,9 @@ __device__ __noinline__ void knn_row_general(const BuildParams& P, int i, int lo
   __syncthreads();
 }
 
-// bytes of shared memory per row: keep list (and two entries that take what does not fit), bins
+// bytes of shared memory per row: keep list (and four entries that take what does not fit), bins
 static __host__ __device__ constexpr size_t row_bytes(int cap) {
-  return ((static_cast<size_t>(cap + 2) * 8 + 15) & ~size_t(15)) + NBINS * 2;
+  return ((static_cast<size_t>(cap + 4) * 8 + 15) & ~size_t(15)) + NBINS * 2;
 }
 
 // *to++ = {who, key} if key <= t (to: an address in shared memory), predicated: one key in eleven is kept at
@@ -720,7 +720,7 @@ __device__ __forceinline__ void append_key(uint32_t& to, float key, float t, uin
       : "memory");
 }
 
-// R rows per CTA of KT threads; KT / R threads rank a row.  FROM: where the keys come from -- computed here (small D), read
+// R rows per CTA of KT threads; KT / R threads rank a row; U codes per thread and step of the key pass.  FROM: where the keys come from -- computed here (small D), read
 // from scratch rows, or already on lists.  ALL: every key is kept, so there is neither sample nor bound, and the
 // bins cover the range that the keys turn out to have.
 //
@@ -728,12 +728,11 @@ __device__ __forceinline__ void append_key(uint32_t& to, float key, float t, uin
 // pipes need 16 k and instruction issue 24 k; sample and bound 9 k; counting sort 13 k; ranking 11 k.
 // 0.54 ms per table; 1.20 ms when a CTA selected from all keys of one row (73 k warp instructions per row, now 26 k).
 enum { FROM_CODES = 0, FROM_SCRATCH = 1, FROM_LISTS = 2 };
-template <int KT, int R, int FROM, bool ALL>
+template <int KT, int R, int FROM, bool ALL, int U>
 __global__ void __launch_bounds__(KT, 1024 / KT) lantern_knn_rows_kernel(BuildParams P, ListParams L, int P2) {
   constexpr bool SCRATCH = FROM == FROM_SCRATCH, LISTS = FROM == FROM_LISTS;
   constexpr int RT = KT / R;         // threads of a row's team
   constexpr int RW = RT / 32;
-  constexpr int U = 2;               // codes per thread and step of the key pass
   constexpr int OWN = NBINS / 2 / RT;   // words of bins per thread of a team
   constexpr int SMP = SAMPLE / RT;   // sampled keys per thread of a team
   extern __shared__ __align__(16) unsigned char dsm[];
@@ -1259,9 +1258,9 @@ static cudaError_t launch_chained(bool first, void (*kernel)(Arg...), dim3 grid,
   return cudaLaunchKernelEx(&c, kernel, arg...);
 }
 
-template <int KT, int R, int FROM, bool ALL = false>
+template <int KT, int R, int FROM, bool ALL = false, int U = 2>
 static cudaError_t launch_rows(const BuildParams& P, int P2, size_t smem, cudaStream_t st, const ListParams& L = {}) {
-  auto kk = lantern_knn_rows_kernel<KT, R, FROM, ALL>;
+  auto kk = lantern_knn_rows_kernel<KT, R, FROM, ALL, U>;
   static DeviceFlags ready;
   const cudaError_t e = allow_shared_memory(kk, kRowSmem, ready);
   if (e != cudaSuccess) return e;
@@ -1335,6 +1334,12 @@ extern "C" lantern_status lantern_build_neighbors(const float* codebook, int V, 
       return R == 8 ? launch_rows<512, 4, FROM_SCRATCH, ALL>(P, P2, smem, st)
                     : (R == 4 ? launch_rows<512, 2, FROM_SCRATCH, ALL>(P, P2, smem, st)
                               : launch_rows<512, 1, FROM_SCRATCH, ALL>(P, P2, smem, st));
+    // Four codes a step instead of two halve what a step costs besides the keys (a prefix over the warp, a counter update), where the
+    // codes fill such steps (V = 16384: D = 8 555 -> 544 us per table, D = 16 787 -> 763, D = 32 1580 -> 1472; V = 6000, whose second
+    // step would be half empty, D = 24 215 and 261).
+    if constexpr (!ALL) {
+      if (R == 8 && (V + 2047) / 2048 % 2 == 0) return launch_rows<1024, 8, FROM_CODES, ALL, 4>(P, P2, smem, st);
+    }
     return R == 8 ? launch_rows<1024, 8, FROM_CODES, ALL>(P, P2, smem, st)
                   : (R == 4 ? launch_rows<1024, 4, FROM_CODES, ALL>(P, P2, smem, st)
                             : launch_rows<1024, 2, FROM_CODES, ALL>(P, P2, smem, st));

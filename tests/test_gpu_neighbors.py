@@ -227,3 +227,21 @@ def test_many_equal_codes_exact(V, D, k, with_dist, dead):
     assert np.array_equal(gi[:, 0], np.arange(V))
     srt = np.sort(gi, axis=1)
     assert np.all(srt[:, 1:] != srt[:, :-1])
+
+
+@pytest.mark.parametrize("V,D,k,kind", [
+    (8192, 8, 300, "gauss"), (8191, 16, 300, "period"), (6145, 13, 64, "gauss"), (6144, 16, 64, "gauss"), (8193, 32, 200, "gauss"),
+    (16384, 4, 30, "ties"), (12289, 20, 1000, "period")])
+def test_steps_of_the_key_pass_exact(V, D, k, kind):
+    """Four codes per thread and step where the number of steps of two is even, two elsewhere: on either side, full and ragged."""
+    if kind == "ties":
+        cb = li.codebook_integer(V, D, lo=-2, hi=3, seed=9)
+    elif kind == "period":
+        cb = li.codebook_clustered(V, D, centres=512, seed=10)
+    else:
+        cb = li.codebook_gaussian(V, D, seed=11)
+    gi, gd = _gpu(cb, k)
+    rows = np.unique(np.concatenate([np.arange(12), np.arange(V - 12, V), np.random.default_rng(1).integers(0, V, 24)])).astype(np.int32)
+    oi, od = oracle.build_neighbors(cb, k, rows=rows)
+    assert np.array_equal(gi[rows], oi)
+    assert np.array_equal(gd[rows].view(np.uint32), od.view(np.uint32))
