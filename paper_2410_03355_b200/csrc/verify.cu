@@ -618,11 +618,15 @@ static void set_divisor(VerifyParams& P, float T) {
     memcpy(&w, &f, 4);
     return static_cast<uint64_t>(w) << 32 | w;
   };
-  P.T_plain = T >= 0x1p-100f && T <= 0x1p100f;
+  P.T_fast = T >= 0x1p-100f && T <= 0x1p100f;
+  const float least = fmaxf(0x1p-100f, T * 0x1p-125f);
+  uint32_t bits;
+  memcpy(&bits, &least, 4);
+  P.T_least = 2u * bits - 1u;
   P.T_neg = pair(-T);
-  const float y = P.T_plain ? static_cast<float>(inv) : 1.0f;
+  const float y = P.T_fast ? static_cast<float>(inv) : 1.0f;
   const float hi = static_cast<double>(y) > inv ? nextafterf(y, 0.0f) : y;
-  const float lo = P.T_plain ? static_cast<float>(inv - static_cast<double>(hi)) : 0.0f;
+  const float lo = P.T_fast ? static_cast<float>(inv - static_cast<double>(hi)) : 0.0f;
   P.T_inv = pair(y);
   P.T_inv_hi = pair(hi);
   P.T_inv_lo = pair(lo > 0.0f ? lo : 0x1p-126f);   // (a power of two leaves nothing; the product with -inf has to be -inf)

@@ -14,7 +14,7 @@
 
 namespace lantern {
 
-#define LANTERN_CONTEXT_KERNEL_REVISION 24   // bump on every change to the fused context kernel
+#define LANTERN_CONTEXT_KERNEL_REVISION 25   // bump on every change to the fused context kernel
 
 constexpr int MAX_N = 1024;
 
@@ -85,7 +85,8 @@ struct VerifyParams {
   int top_k;                    // logit filter; 0 = off
   // l / T without a division (divide_by_T): each as a pair of equal fp32 values
   uint64_t T_neg, T_inv, T_inv_hi, T_inv_lo;   // -T, the reciprocal rounded to nearest; rounded towards zero, and what that leaves
-  int T_plain;                  // 0: T is so large or so small that a division is done after all
+  int T_fast;                   // 0: T is so large or so small that a division is done after all
+  uint32_t T_least;             // 2 bits(|l|) - 1 of the smallest |l| whose quotient is always a division's
   uint32_t wait_tries;          // limit of every bounded mbarrier wait, in tries
   int32_t* block_words;         // one word per block of the plan kernel: see plan_word
   int withhold_item;            // self-test only: the copies of this context are never issued (-1 = none)

@@ -1,6 +1,8 @@
 """CUDA variants against the oracle: cosine neighbour metric (Section 5.3.1), JSD bound
 (Section 5.3.2) and top-k logit filter (Appendix B.2) in sampling and in greedy decoding.  Comparison rules are those of
 tests/parity.py and tests/test_gpu_greedy.py (the cut's window is in JSD units here)."""
+import dataclasses
+
 import numpy as np
 import pytest
 import torch
@@ -219,3 +221,28 @@ def test_top_k_of_masked_and_tied_rows(V, B, dtype, unc, T, rows):
         greedy_check(inp, host, dev, 0.2, top_k=K)
     else:
         assert_parity(compare(inp, host, 0.2, run_gpu(inp, dev, 0.2, top_k=K), top_k=K))
+
+
+@pytest.mark.parametrize("dtype", [li.F32, li.BF16])
+@pytest.mark.parametrize("T", [0.9, 3.0, 1.2e30, 1.2e-30])
+def test_topk_thresholds_among_tiny_quotients(T, dtype):
+    """Logits and quotients around and below the smallest normal number, where the quotient's remainder is lost: a threshold is the
+    value of the tokens it is compared with all the same, be they part of a row or the drafted one, which is the K-th largest here."""
+    V, B, N, K = 512, 48, 3, 100
+    rng = np.random.default_rng(6)
+    inp = li.verify_inputs(B, N, V, dtype=dtype, has_uncond=False, cfg_scale=1.0, seed=5)
+
+    def tiny(shape):
+        e = rng.integers(-146, -112, shape)
+        z = rng.choice([-1.0, 1.0], shape) * rng.uniform(1.0, 2.0, shape) * 2.0 ** e
+        x = (z * (T if T > 1e10 else 1.0)).astype(np.float32)
+        return x if dtype == li.F32 else li.f32_to_bf16_bits(x)
+
+    inp = dataclasses.replace(inp, T=T, target_logits=tiny(inp.target_logits.shape), draft_logits=tiny(inp.draft_logits.shape))
+    rows = [a if dtype == li.F32 else li.bf16_bits_to_f32(a) for a in (inp.draft_logits, inp.target_logits[0])]
+    for i in range(N):
+        inp.draft_tokens[:, i] = np.argsort(-rows[i % 2][:, i], axis=1, kind="stable")[:, K - 1]
+    host, dev = tables(li.codebook_gaussian(V, 8, seed=19), 16, inp.draft_tokens)
+    res = compare(inp, host, 0.3, run_gpu(inp, dev, 0.3, top_k=K), top_k=K)
+    assert_parity(res)
+    assert res["nodes_tested"] >= B
