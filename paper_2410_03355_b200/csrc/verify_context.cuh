@@ -636,6 +636,7 @@ __global__ void __launch_bounds__(SHAPE::THREADS, SHAPE::CTAS) lantern_context_k
         for (int steps = 0;;) {
           st |= status;
           if (status & (LANTERN_ST_NONFINITE | LANTERN_ST_INTERNAL)) {
+            n_draw += drawn;                                     // (a draw from a row that is not finite is one all the same)
             if (lane == 0) finish(b, -1, st);
             break;
           }

@@ -55,6 +55,35 @@ def test_draws_ahead_are_counted_once_and_repeat(N, tree):
         assert lt.verify_counts(ws)["from_q"] == sum(not (par[b] == last[b]).any() for b in range(B))
 
 
+def _outputs(B, N):
+    i32 = dict(dtype=torch.int32, device="cuda")
+    return lt.VerifyOutputs(torch.empty(B, **i32), torch.empty(B, **i32), torch.empty((B, N), **i32), torch.empty(B, **i32), None, None, None)
+
+
+def _run(d, dev, out, ws):
+    lt.verify(d["target_logits"], d["draft_logits"], 2.0, 1.0, d["draft_tokens"], d["tree_parents"], dev, 0.4, d["uniforms"], out=out, workspace=ws)
+
+
+@pytest.mark.parametrize("V,B", [(512, 6), (512, 400), (16384, 6)])
+def test_draws_from_rows_that_are_not_finite_are_counted(V, B):
+    """Every sequence comes to its leaf, every other leaf's row holds a NaN: a draw all the same, whoever makes it (in calls of few
+    contexts a group ahead of the walk)."""
+    N = 3
+    inp = _inputs(B, N, False, seed=6, V=V)
+    inp.draft_logits[:, :N] = inp.target_logits[0, :, :N]
+    inp.target_logits[1, :, :N] = inp.target_logits[0, :, :N]      # target and drafter are the same: accepted
+    inp.target_logits[0, ::2, N, 5] = 0x7fc0
+    host, dev = tables(li.codebook_gaussian(V, 8, seed=18), 40, inp.draft_tokens)
+    d = to_device(inp)
+    ws = torch.empty(lt.verify_workspace_bytes(B, N, V, 40), dtype=torch.uint8, device="cuda")
+    for _ in range(20):
+        out = _outputs(B, N)
+        _run(d, dev, out, ws)
+        assert lt.verify_counts(ws)["from_q"] == B
+        assert (out.accept_len == N).all() and (out.status[::2] == lt.ST_NONFINITE).all() and not out.status[1::2].any()
+    assert_parity(compare(inp, host, 0.4, out))
+
+
 @pytest.mark.parametrize("N,tree", [(6, False), (33, True)])
 def test_greedy_small_calls(N, tree):
     inp = _inputs(3, N, tree, seed=50 + N)
