@@ -1165,6 +1165,10 @@ __global__ void __launch_bounds__(SHAPE::THREADS, SHAPE::CTAS) lantern_context_k
         int4 sib = make_int4(0, 0, 0, 0);
         if (ci + 1 < nchild) sib = *reinterpret_cast<const int4*>(kids + ci + 1);
         if (gt == 0) atomicAdd(&P.counters->n_tested, 1);   // work accounting (a fire-and-forget reduction)
+        // What the rejections so far have left of x~.  Read here, between the barrier that publishes the residual and the scan's: behind
+        // the scan a warp that is ahead may have flagged it already.
+        [[maybe_unused]] float bulk = 0.0f;
+        if (!GREEDY && ci > 0) bulk = mass(xt);
 
         // ---- A_{k,delta}(x~): gather + prefix scan with the strict bound ----
         double thr = delta * Zq_c;   // the bound in the units of the unnormalised sums
@@ -1253,7 +1257,6 @@ __global__ void __launch_bounds__(SHAPE::THREADS, SHAPE::CTAS) lantern_context_k
           e_xt = q.y * exp2_int_d(q.n - static_cast<double>(Nq));
           p_xt = p.y * exp2_int_d(p.n - static_cast<double>(Np));
           if (ci > 0) {
-            const float bulk = mass(xt);
             if (ci <= 32) {
               for (int i = 0; i < ci; ++i) e_xt = fmax(0.0, e_xt - S.hist[i] * p_xt);
               if (bulk == 0.0f) e_xt = 0.0;

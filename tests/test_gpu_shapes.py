@@ -5,6 +5,7 @@ import pytest
 import torch
 
 import lantern_inputs as li
+import oracle
 import paper_2410_03355_b200 as lt
 from parity import assert_parity, compare, near_ceiling, run_gpu, tables, to_device
 
@@ -149,3 +150,24 @@ def test_long_walks_against_oracle(N, tree):
     res = compare(inp, host, 0.2, gpu)
     assert_parity(res)
     assert res["near"] <= near_ceiling(B) and (N < 38 or tree or gpu.accept_len.max() > 7)
+
+
+@pytest.mark.parametrize("V,B,N", [(512, 40, 60), (512, 300, 34), (1000, 12, 33), (16384, 4, 60), (16384, 160, 36)])
+def test_contexts_of_more_than_33_siblings(V, B, N):
+    """All drafts are children of the root and nearly all of them are rejected: from the 34th on a token's own numerator is that of the
+    residual.  (Narrow, wide and, for trees, again the wide shape with a second context per group.)"""
+    par = np.full((B, N), -1, np.int32)
+    inp = li.verify_inputs(B, N, V, dtype=li.BF16, has_uncond=True, cfg_scale=2.0, rho=0.9, sigma_draft=0.6, parents=par, seed=N)
+    rng = np.random.default_rng(V + N)
+    for b in range(B):            # the drafter thinks much of tokens of which the target thinks little
+        at = rng.choice(V, size=N, replace=False)
+        inp.draft_tokens[b] = at
+        inp.draft_logits[b, 0, at] = li.f32_to_bf16_bits(rng.uniform(6.0, 8.0, N))
+        inp.target_logits[:, b, 0, at] = li.f32_to_bf16_bits(rng.uniform(-9.0, -3.0, N))
+    host, dev = tables(li.codebook_gaussian(V, 8, seed=18), 24, inp.draft_tokens)
+    gpu = run_gpu(inp, dev, 1.0 / V)
+    ora = oracle.verify_inputs(inp, host, 1.0 / V)
+    res = compare(inp, host, 1.0 / V, gpu, ora=ora)
+    assert_parity(res)
+    assert res["near"] <= near_ceiling(B)
+    assert (ora.tested.sum(1) >= min(N, 34)).mean() > 0.2
