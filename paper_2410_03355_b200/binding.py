@@ -7,7 +7,10 @@ from __future__ import annotations
 
 import ctypes
 import dataclasses
+import importlib.util
 import os
+import sysconfig
+import warnings
 from typing import Optional
 
 import torch
@@ -30,6 +33,27 @@ class LanternError(RuntimeError):
 
 def library_path() -> str:
     return _LIB_PATH
+
+
+def call_path() -> str:
+    """The native part of verify(), for the torch and the Python that run: it reads their objects, so that each pair has a file of its own."""
+    abi = int(torch._C._GLIBCXX_USE_CXX11_ABI)
+    return os.path.join(_HERE, f"_call.torch-{torch.__version__}-abi{abi}{sysconfig.get_config_var('EXT_SUFFIX')}")
+
+
+def _load_call():
+    """The native part of verify(), or None where it has not been built: verify() goes through ctypes then."""
+    path = call_path()
+    if not os.path.exists(path):
+        return None
+    spec = importlib.util.spec_from_file_location(f"{__package__}._call", path)
+    try:
+        module = importlib.util.module_from_spec(spec)
+        spec.loader.exec_module(module)
+    except ImportError as e:
+        warnings.warn(f"{path} does not load ({e}): verify() goes through ctypes")
+        return None
+    return module
 
 
 def load_library():
@@ -80,9 +104,11 @@ def load_library():
     lib.lantern_verify.restype = i32
     lib.lantern_verify.argtypes = [vp, vp, i32, f32, i32, f32, vp, vp, vp, i32, f32, vp, i32, i32, i32,
                                    vp, vp, vp, vp, vp, vp, vp, vp, sz, vp]
-    from . import _call as call      # the native part of verify(), built beside the library
-    call.bind(ctypes.cast(lib.lantern_verify_ex, ctypes.c_void_p).value)
-    _lib, _call = lib, call
+    call = _load_call()
+    if call is not None:
+        call.bind(ctypes.cast(lib.lantern_verify_ex, ctypes.c_void_p).value)
+    _call = call
+    _lib = lib      # (last: what another thread finds loaded is loaded whole)
     return lib
 
 
@@ -198,7 +224,7 @@ def verify(target_logits: torch.Tensor, draft_logits: Optional[torch.Tensor], cf
     divergence "tvd" | "jsd": what delta bounds (Section 5.3.2); top_k: logit filter, 0 = off (Appendix B.2).
     """
     lib = load_library()
-    if out is not None and workspace is not None and stream is None:
+    if _call is not None and out is not None and workspace is not None and stream is None:
         # nothing to allocate: the arguments go to the library natively, unless one of them is not what it has to be
         rc = _call.verify(target_logits, draft_logits, cfg_scale, T, draft_tokens, tree_parents, neighbor_idx, delta, uniforms, out,
                           workspace, DIVERGENCES.get(divergence), top_k)

@@ -91,7 +91,7 @@ def test_greedy_small_calls(N, tree):
     greedy.check(inp, host, dev, 0.4)
 
 
-def test_forms_of_a_call():
+def test_forms_of_a_call(monkeypatch):
     """Outputs and workspace given or not, integer scalars, a stream, tensor subclasses: the same results; what was refused
     is refused."""
     B, N = 5, 6
@@ -121,6 +121,11 @@ def test_forms_of_a_call():
                dict(cfg=np.float32(2.0))):
         torch.cuda.synchronize()
         same(call(out=out, workspace=ws, **kw), want)
+    assert lt.binding._call is not None          # the native part of the binding is there, and the answers are the same without it
+    with monkeypatch.context() as m:
+        m.setattr(lt.binding, "_call", None)
+        assert call(out=out, workspace=ws) is out
+        same(out, want)
     part = lt.VerifyOutputs(out.accept_len, out.next_token, None, None, None, None, None)
     call(out=part, workspace=ws)
     assert torch.equal(part.next_token, want.next_token)

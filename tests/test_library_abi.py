@@ -62,3 +62,20 @@ def test_cpu_tensors_are_refused():
     import paper_2410_03355_b200 as lt
     with pytest.raises(ValueError):
         lt.build_neighbors(torch.zeros(16, 8), 4)
+
+
+def test_native_part_of_the_binding_belongs_to_one_torch_and_python(monkeypatch):
+    """It reads torch's and Python's objects: another torch or Python has a file of its own, and without one the library loads and
+    the binding goes through ctypes."""
+    import torch
+    from paper_2410_03355_b200 import binding, build
+    build.build()
+    path = binding.call_path()
+    assert os.path.exists(path) and not build._call_stale()
+    monkeypatch.setattr(binding, "_lib", None)
+    monkeypatch.setattr(binding, "_call", None)
+    assert binding.load_library() and binding._call is not None
+    monkeypatch.setattr(torch, "__version__", "0.0.1")
+    assert binding.call_path() != path and build._call_stale()
+    monkeypatch.setattr(binding, "_lib", None)
+    assert binding.load_library().lantern_status_string(0) == b"ok" and binding._call is None
