@@ -84,6 +84,49 @@ def test_draws_from_rows_that_are_not_finite_are_counted(V, B):
     assert_parity(compare(inp, host, 0.4, out))
 
 
+def _equal(x, y):
+    return all(torch.equal(getattr(x, f), getattr(y, f)) for f in ("accept_len", "next_token", "accept_path", "status"))
+
+
+@pytest.mark.parametrize("V,B,N,tree", [(512, 40, 7, False), (512, 9, 60, True), (16384, 32, 7, False), (16384, 2, 60, True)])
+def test_calls_in_a_row(V, B, N, tree):
+    """Calls of different inputs with one workspace, without a wait in between, among them a large call and one whose plan finds a
+    fault; and two of them in one captured graph."""
+    inps = [_inputs(B, N, tree, seed=s, V=V) for s in (1, 2, 3)]
+    inps[2].draft_tokens[B // 2, N - 1] = V     # out of range
+    big = _inputs(4 * _sms() // (N + 1) + 40, N, tree, seed=4, V=V)
+    host, dev = tables(li.codebook_gaussian(V, 8, seed=18), 40, np.concatenate([i.draft_tokens.ravel() for i in inps + [big]]))
+    every = inps + [big]
+    ds = [to_device(i) for i in every]
+    ws = torch.empty(lt.verify_workspace_bytes(big.B, N, V, 40), dtype=torch.uint8, device="cuda")
+    want = [_outputs(i.B, N) for i in every]
+    for d, out in zip(ds, want):                # one at a time, each held against the oracle
+        _run(d, dev, out, ws)
+        torch.cuda.synchronize()
+    for i, out in zip(inps[:2] + [big], want[:2] + want[3:]):
+        assert_parity(compare(i, host, 0.4, out))
+    assert want[2].status.cpu().numpy()[B // 2] == lt.ST_BAD_TOKEN
+    order = [0, 1, 0, 2, 1, 3, 0, 0, 2, 3, 3, 1] * 8
+    got = [_outputs(every[q].B, N) for q in order]
+    torch.cuda.synchronize()
+    for q, out in zip(order, got):
+        _run(ds[q], dev, out, ws)
+    torch.cuda.synchronize()
+    assert all(_equal(out, want[q]) for q, out in zip(order, got))
+    graph, pair = torch.cuda.CUDAGraph(), [_outputs(B, N), _outputs(B, N)]
+    with torch.cuda.graph(graph):
+        for q in (0, 1):
+            _run(ds[q], dev, pair[q], ws)
+    for _ in range(20):
+        for out in pair:
+            out.accept_len.fill_(-9)
+            out.next_token.fill_(-9)
+        graph.replay()
+        graph.replay()
+        torch.cuda.synchronize()
+        assert _equal(pair[0], want[0]) and _equal(pair[1], want[1])
+
+
 @pytest.mark.parametrize("N,tree", [(6, False), (33, True)])
 def test_greedy_small_calls(N, tree):
     inp = _inputs(3, N, tree, seed=50 + N)
