@@ -439,15 +439,12 @@ __global__ void __launch_bounds__(SHAPE::THREADS, SHAPE::CTAS) lantern_context_k
   // The plan, and whatever made the inputs.  This kernel may be in place while the plan still writes: what the plan writes is read by
   // ordinary loads, which stay behind this wait.  Logits and neighbour rows are read through the read-only path: they are
   // complete before any CTA of this kernel starts, because every CTA of the plan lets it start only after a wait of its own.
-  // Before that: rows that are going to be read whatever the plan says are asked into L2 while it runs -- the root of the sequence that this
-  // group begins with, or every row of a call so small that no group gets more than a few.
+  // Before that: rows that some group begins with whatever the plan says, those of the first roots, are asked into L2 while it runs, a
+  // sequence per group.  (All rows of a small call, of which every group gets a few at most, were too much: 74 chains of 7 drafts 33.7
+  // us per call, 37.0 with them; no row at all: 500 chains 105.6 instead of 104.3.)
   if (lane == 0 && tid >= NGRP * GT) {
-    const int G = gridDim.x * NGRP, me = ((tid - NGRP * GT) >> 5) * gridDim.x + blockIdx.x;
-    if (P.leaves) {
-      for (int c = me; c < P.B * R; c += G) ctx_prefetch_rows<UNC, !GREEDY, true>(P, c, rowbytes);
-    } else if (me < P.B) {
-      ctx_prefetch_rows<UNC, !GREEDY, true>(P, me * R, rowbytes);
-    }
+    const int me = ((tid - NGRP * GT) >> 5) * gridDim.x + blockIdx.x;
+    if (me < P.B) ctx_prefetch_rows<UNC, !GREEDY, true>(P, me * R, rowbytes);
   }
   grid_dependency_wait();
 
