@@ -374,7 +374,10 @@ __device__ __forceinline__ unsigned long long walk_exchange(Record* rec, unsigne
 // reads the words of 32 contexts at once, from the next one on, and follows those that lead on to the next: a chain's contexts do.
 // (29 chains of 443 drafts of 6664 fp32 logits 217 us per call, 1069 without it; 2 of 1024 drafts 73 and 722.  Paths of a few
 // contexts never get there.)
-constexpr int kWalkAlone = 6;
+// With the logit filter, where contexts take three times as long to decide, sequences of at most 64 contexts have all their words read at
+// once after three steps, and what was decided is followed without further round trips (1024 chains of 7 drafts 459 us per call, 467 to 473
+// without it; other variants lose by it: 2048 chains in greedy decoding 145.6 us without and 146.4 with it, 1000 trees 159.5 and 162.4).
+constexpr int kWalkAlone = 6, kWalkFilter = 3;
 __device__ __forceinline__ unsigned long long walk_look(const Record* rec) {
   unsigned long long w;
   asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(w) : "l"(&rec->word) : "memory");
@@ -593,15 +596,6 @@ __global__ void __launch_bounds__(SHAPE::THREADS, SHAPE::CTAS) lantern_context_k
         return true;
       }
       Record* recs = P.records + static_cast<size_t>(b) * R;
-      // Few sequences: most of a path has been decided by the time the walk comes along.  The words of all its contexts (two to a
-      // lane) travel together with the first exchange, and what was decided is followed without further round trips.
-      unsigned long long seen0 = 0, seen1 = 0;
-      bool looked = P.leaves && R <= 64;
-      auto look = [&]() {
-        if (lane < R) seen0 = walk_look(recs + lane);
-        if (lane + 32 < R) seen1 = walk_look(recs + lane + 32);
-      };
-      if (looked) look();
       // Algorithm 1 goes on from the accepted child only: every context behind another child is dead.  In
       // pre-order those are one contiguous range per child.
       const int cbase = p_cbase, span0 = p_span0, nchild = nc0 >> 16;
@@ -628,6 +622,7 @@ __global__ void __launch_bounds__(SHAPE::THREADS, SHAPE::CTAS) lantern_context_k
         int st = static_cast<int>(w >> 8) & 0xff, len = static_cast<int>(w >> 16) & 0xffff;
         const int len_before = len;
         int32_t* path = P.out_path ? P.out_path + static_cast<size_t>(b) * N : nullptr;
+        unsigned long long seen0 = 0, seen1 = 0;   // (TOPK) words of contexts `lane` and `lane` + 32
         for (int steps = 0;;) {
           st |= status;
           if (status & (LANTERN_ST_NONFINITE | LANTERN_ST_INTERNAL)) {
@@ -646,15 +641,17 @@ __global__ void __launch_bounds__(SHAPE::THREADS, SHAPE::CTAS) lantern_context_k
             ++len;
             at = accepted + 1;
             w = 0;
-            if (R <= 64) {
-              if (looked || steps > 2) {
-                if (!looked) look();
-                looked = true;
+            ++steps;
+            if (TOPK && R <= 64) {
+              if (steps > kWalkFilter) {
+                if (steps == kWalkFilter + 1) {
+                  if (lane < R) seen0 = walk_look(recs + lane);
+                  if (lane + 32 < R) seen1 = walk_look(recs + lane + 32);
+                }
                 const unsigned long long w0 = __shfl_sync(kFull, seen0, at & 31), w1 = __shfl_sync(kFull, seen1, at & 31);
                 w = at < 32 ? w0 : w1;
               }
-              ++steps;
-            } else if (++steps > kWalkAlone) {
+            } else if (steps > kWalkAlone) {
               // the contexts that were decided in favour of the node numbered as they are, from this one on, are followed at once
               for (int run = 32; run == 32;) {
                 const unsigned long long seen = at + lane < R ? walk_look(recs + at + lane) : 0;
