@@ -632,8 +632,17 @@ static void set_divisor(VerifyParams& P, float T) {
   P.T_inv_lo = pair(lo > 0.0f ? lo : 0x1p-126f);   // (a power of two leaves nothing; the product with -inf has to be -inf)
 }
 
-// Few contexts: the SMs have room for bonus draws ahead of time, and the call is short enough for the draw at its end to count.
-static bool leaves_pay(int B, int N, int sms) { return N > 0 && static_cast<long long>(B) * (N + 1) <= 4ll * sms; }
+// Does a call list its leaves, so that bonus draws are made ahead of the walk?  A draw ahead takes a group that would stand idle, and saves the walk
+// a dependent step at its end; where there is no such group it delays the contexts.  So calls of few contexts do, up to four per SM where the paths
+// are long enough to hide the draws, us per call without | with: 74 chains of 7 drafts 36.2 | 32.9, one tree of 60 20.2 | 17.6, five 28.0 | 25.5, nine
+// 29.9 | 28.2, but 16 of them (seven contexts per SM) 37.4 | 39.2.  Paths of one draft are not where a group has its SM for itself (25 chains
+// 15.2 | 17.1, 290 24.1 | 27.4), and rows of at most 8192 tokens, three groups to an SM, up to four drafts until every group has a context (one
+// chain of one draft 13.5 | 11.3, of 3 drafts 111 chains 17.6 | 16.0, 148 17.9 | 20.4; of one draft 200 15.6 | 15.4, 290 16.2 | 19.6).
+static bool leaves_pay(const VerifyParams& P, int sms) {
+  const long long contexts = static_cast<long long>(P.B) * P.R;
+  if (P.V > 8192) return P.N > 1 && contexts <= 4ll * sms;
+  return P.N > 0 && contexts <= (P.N > 4 ? 4ll : 3ll) * sms;
+}
 
 extern "C" lantern_status lantern_verify(const void* target_logits, const void* draft_logits, int dtype,
                                          float cfg_scale, int has_uncond, float T, const int32_t* draft_tokens,
@@ -732,7 +741,7 @@ static lantern_status verify_impl(const void* target_logits, const void* draft_l
   P.divergence = divergence;
   P.top_k = topk ? top_k : 0;
   P.dead = ws + L.dead;
-  P.leaves = leaves_pay(B, N, sms) ? reinterpret_cast<int32_t*>(ws + L.leaves) : nullptr;
+  P.leaves = leaves_pay(P, sms) ? reinterpret_cast<int32_t*>(ws + L.leaves) : nullptr;
   P.wait_tries = g_wait_tries;
   P.withhold_item = g_withhold_item;
 
