@@ -14,7 +14,7 @@
 
 namespace lantern {
 
-#define LANTERN_CONTEXT_KERNEL_REVISION 31   // bump on every change to the fused context kernel
+#define LANTERN_CONTEXT_KERNEL_REVISION 32   // bump on every change to the fused context kernel
 
 constexpr int MAX_N = 1024;
 
@@ -120,6 +120,7 @@ __device__ __forceinline__ int plan_word(int ranks, int leaves, int faults) { re
 struct PlanSummary {
   int slots, leaf_slots, faults;
 };
+template <bool LEAVES>   // they are listed
 __device__ __forceinline__ PlanSummary plan_summary(const VerifyParams& P, int lane) {
   int ranks = P.N > 0 ? 0 : 1, leaves = 0, bits = 0;
   const int blocks = (P.B + PLAN_SEQS - 1) / PLAN_SEQS;
@@ -130,12 +131,13 @@ __device__ __forceinline__ PlanSummary plan_summary(const VerifyParams& P, int l
     leaves = max(leaves, w >> 11 & 0x7ff);
     bits |= w >> 22;
   }
-  return {__reduce_max_sync(kFull, ranks) * P.B, P.leaves ? __reduce_max_sync(kFull, leaves) * P.B : 0, static_cast<int>(__reduce_or_sync(kFull, bits))};
+  return {__reduce_max_sync(kFull, ranks) * P.B, LEAVES ? __reduce_max_sync(kFull, leaves) * P.B : 0, static_cast<int>(__reduce_or_sync(kFull, bits))};
 }
 // The same without the fault bits: a chain has a context with a child for every draft, and one leaf.
+template <bool LEAVES>
 __device__ __forceinline__ PlanSummary plan_extent(const VerifyParams& P, int lane) {
-  if (!P.parents) return {(P.N > 0 ? P.N : 1) * P.B, P.leaves ? P.B : 0, 0};
-  return plan_summary(P, lane);
+  if (!P.parents) return {(P.N > 0 ? P.N : 1) * P.B, LEAVES ? P.B : 0, 0};
+  return plan_summary<LEAVES>(P, lane);
 }
 
 __device__ __forceinline__ float sum8(const float* v) {

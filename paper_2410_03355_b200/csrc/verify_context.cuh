@@ -391,7 +391,11 @@ __device__ __forceinline__ unsigned long long walk_look(const Record* rec) {
 // accepted iff sum_A q >= max_x q(x) (it is an arg max of q_{k,delta}(.|D = x~): the maximum over A's own members can never
 // exceed the sum), children are tried against the same q, and wherever the walk stops the token is arg max q.
 // TOPK = the logit filter is on (Appendix B.2): processed logits below the top_k-th largest of their row count as -inf.
-template <class SHAPE, int CH, bool BF16, bool UNC, bool TONE, bool JSD, bool TOPK, bool GREEDY>
+// FEW = a call of few contexts, whose leaves are listed (P.leaves): producers make bonus draws ahead of the walk.  At compile time, because
+// what they need for it costs the producers of large calls 1 to 5 per cent, also where it is stepped over (greedy decoding of 2048
+// chains of 7 drafts 146.4 us per call, 151.0 with one kernel for both; of 8192 tokens and 8 drafts 114.7 and 120.4; sampling, 8192 chains 952
+// and 973, 1600 trees of 8192 tokens 252 and 262).
+template <class SHAPE, int CH, bool BF16, bool UNC, bool TONE, bool JSD, bool TOPK, bool GREEDY, bool FEW>
 __global__ void __launch_bounds__(SHAPE::THREADS, SHAPE::CTAS) lantern_context_kernel(VerifyParams P) {
   constexpr int GT = SHAPE::GT, GW = GT / 32, NGRP = SHAPE::NGRP, AREAS = SHAPE::AREAS;
   constexpr int LOG_GT = GT == 512 ? 9 : 8;
@@ -473,7 +477,7 @@ __global__ void __launch_bounds__(SHAPE::THREADS, SHAPE::CTAS) lantern_context_k
     // round trip to the work list.
     int slots_seen = 0, live_seen = 0;
     // slots of the work list that are in use, and those of the list of leaves behind them
-    PlanSummary extent = {P.B * (N > 0 ? N : 1), P.leaves ? P.B * N : 0, 0};   // (at most, until the plan's summary has been read)
+    PlanSummary extent = {P.B * (N > 0 ? N : 1), FEW ? P.B * N : 0, 0};   // (at most, until the plan's summary has been read)
     auto batch_size = [&](int at) {
       const int share = (extent.slots + extent.leaf_slots - at) / (4 * G);
       const int live = share < 1 ? 1 : (share > 2 ? 2 : share);
@@ -492,7 +496,7 @@ __global__ void __launch_bounds__(SHAPE::THREADS, SHAPE::CTAS) lantern_context_k
         if (leaf < 0) {
           c.item = P.work[c.slot].item;
           c.mark = P.work[c.slot].mark;
-        } else if (leaf < extent.leaf_slots) {
+        } else if (FEW && leaf < extent.leaf_slots) {
           const int w = P.leaves[leaf], b = leaf % P.B;
           if (w >= 0) c.item = b * R + (w & 0xffff), c.mark = b * R + (w >> 16);
         }
@@ -501,7 +505,7 @@ __global__ void __launch_bounds__(SHAPE::THREADS, SHAPE::CTAS) lantern_context_k
     };
     // the rest, by the candidate's lane
     auto load_item = [&](const Cand& c, int4& lo, int4& hi) {
-      if (c.slot < extent.slots) {
+      if (!FEW || c.slot < extent.slots) {
         lo = *reinterpret_cast<const int4*>(P.work + c.slot);
         hi = *(reinterpret_cast<const int4*>(P.work + c.slot) + 1);
       } else {                 // nothing but a draw
@@ -522,7 +526,7 @@ __global__ void __launch_bounds__(SHAPE::THREADS, SHAPE::CTAS) lantern_context_k
     auto filter = [&](const Cand& c, bool first) -> unsigned {
       const bool has = c.item >= 0;
       const bool dead = has && !first && is_dead(c.mark);
-      n_skip += __popc(__ballot_sync(kFull, dead && c.slot < extent.slots));
+      n_skip += __popc(__ballot_sync(kFull, dead && (!FEW || c.slot < extent.slots)));
       const unsigned live = __ballot_sync(kFull, has && !dead);
       live_seen += __popc(live);
       return live;
@@ -534,10 +538,10 @@ __global__ void __launch_bounds__(SHAPE::THREADS, SHAPE::CTAS) lantern_context_k
     int4 lo = make_int4(-1, 0, 0, 0), hi = make_int4(0, 0, 0, 0);      // the description of this lane's candidate
     if (lane < b0 && cur.slot < extent.slots) load_item(cur, lo, hi);   // (the first batch at once, beside the summary)
     cur.item = lo.x, cur.mark = hi.w;
-    extent = plan_extent(P, lane);
+    extent = plan_extent<FEW>(P, lane);
     const int total = extent.slots + extent.leaf_slots;
     bool cur_end = me * b0 >= total, nxt_end = false, primed = false, described = true;   // (lo and hi: only of the first batch, and until used)
-    if (me * b0 + b0 > extent.slots) {   // (the leaves begin earlier than was assumed)
+    if (FEW && me * b0 + b0 > extent.slots) {   // (the leaves begin earlier than was assumed)
       cur = load_cand(me * b0, b0);
       if (cur.item >= 0) load_item(cur, lo, hi);
     }
@@ -688,7 +692,7 @@ __global__ void __launch_bounds__(SHAPE::THREADS, SHAPE::CTAS) lantern_context_k
     bool clean = true;
     // A context handed to a group that has siblings to try yet waits for all of them: in a small call of trees the next one is chosen
     // when the group's result is known (8 trees 38.0 -> 36.5 us per call; chains have no siblings, and lose by it).
-    const bool late = P.leaves && P.parents;
+    const bool late = FEW && P.parents;
     for (;;) {
       if (late && open && !take_result(i - 1)) {
         clean = false;
@@ -716,7 +720,7 @@ __global__ void __launch_bounds__(SHAPE::THREADS, SHAPE::CTAS) lantern_context_k
       } else {                 // (a work slot without children is a draw from the outset: a call without drafts)
         l = __ffs(mask) - 1;
         mask &= mask - 1;
-        leaf = __shfl_sync(kFull, cur.slot, l) >= extent.slots;
+        if (FEW) leaf = __shfl_sync(kFull, cur.slot, l) >= extent.slots;
         if (!described && lane == l) load_item(cur, lo, hi);   // in flight while the group is waited for
         described = false;
       }
@@ -793,7 +797,7 @@ __global__ void __launch_bounds__(SHAPE::THREADS, SHAPE::CTAS) lantern_context_k
       if (n_draw) atomicAdd(&P.counters->n_bonus, n_draw);
     }
     if (me == 0) {   // sequences that the plan found at fault
-      const int faults = plan_summary(P, lane).faults;
+      const int faults = plan_summary<FEW>(P, lane).faults;
       if (faults && lane == 0) atomicOr(&P.counters->status_or, faults);
     }
     return;

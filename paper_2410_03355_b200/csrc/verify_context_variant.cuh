@@ -5,10 +5,10 @@
 
 namespace lantern {
 
-template <class SHAPE, int CHC, bool BF16, bool UNC>
-static cudaError_t launch_shape(const VerifyParams& P, long long items, int sms, cudaStream_t st) {
+template <class SHAPE, int CHC, bool BF16, bool UNC, bool FEW>
+static cudaError_t launch_kernel(const VerifyParams& P, long long items, int sms, cudaStream_t st) {
   auto kc = lantern_context_kernel<SHAPE, CHC, BF16, UNC, LANTERN_VARIANT_TONE, LANTERN_VARIANT_JSD, LANTERN_VARIANT_TOPK,
-                                   LANTERN_VARIANT_GREEDY>;
+                                   LANTERN_VARIANT_GREEDY, FEW>;
   const size_t groups = SHAPE::NGRP * SHAPE::AREAS;
   const int ctas = sms * SHAPE::CTAS;
   const int grid = static_cast<int>(items < ctas ? items : ctas);   // a few contexts get an SM each
@@ -16,6 +16,11 @@ static cudaError_t launch_shape(const VerifyParams& P, long long items, int sms,
   const cudaError_t e = allow_shared_memory(kc, groups * ctx_area_bytes(CHC * SHAPE::GT * 8, BF16, UNC), ready);
   if (e != cudaSuccess) return e;
   return launch_dependent(kc, grid, SHAPE::THREADS, groups * ctx_area_bytes(P.V, BF16, UNC), st, P);
+}
+template <class SHAPE, int CHC, bool BF16, bool UNC>
+static cudaError_t launch_shape(const VerifyParams& P, long long items, int sms, cudaStream_t st) {
+  if (P.leaves) return launch_kernel<SHAPE, CHC, BF16, UNC, true>(P, items, sms, st);
+  return launch_kernel<SHAPE, CHC, BF16, UNC, false>(P, items, sms, st);
 }
 template <int CHC, bool BF16, bool UNC>
 static cudaError_t launch_one(const VerifyParams& P, long long items, int sms, cudaStream_t st) {
