@@ -22,8 +22,8 @@
 // read) and stay in the units of their slice; the shifts are tabulated, and because they are integers
 // a numerator comes to common units by an exact power of two.  One group barrier then publishes E,
 // the table and the per-warp maxima and sums.  Sums over many numerators average the ex2 unit's ~1e-7
-// rounding out; the two single probabilities that decide a position, q(x~) and p(x~), are formed by one
-// thread in double precision.
+// rounding out; the two single probabilities that decide a position, q(x~) and p(x~), are noted by a thread each
+// and formed by every thread in double precision.
 //
 // Deciding part, per child (Section 4.3 / Algorithm 2, second block): gather of the neighbour
 // row's numerators, double-precision scan against the strict bound (the per-warp totals tell every warp
@@ -154,6 +154,7 @@ struct alignas(16) GroupShared {
   // q(x~), p(x~) of the next child to test, not yet in common units, of context i in single[i & 1]: the first threads may note the next
   // context's before the last ones have read the current one's
   Exp2Split single[2][2];
+  double tested[2];             // (TOPK) the numerators of the tested token, common units
   double cut_sum;               // moved mass of A where the bound fell into a warp's slots
   double jsd_mass[2];           // the JSD bound as a mass, common units, by scan round (mod 2)
   double hist[32];              // drafter/target scale ratio of each earlier rejection round of this context
@@ -1161,10 +1162,40 @@ __global__ void __launch_bounds__(SHAPE::THREADS, SHAPE::CTAS) lantern_context_k
         int4 sib = make_int4(0, 0, 0, 0);
         if (ci + 1 < nchild) sib = *reinterpret_cast<const int4*>(kids + ci + 1);
         if (gt == 0) atomicAdd(&P.counters->n_tested, 1);   // work accounting (a fire-and-forget reduction)
+        // The tested token's two numerators in common units, in double precision from its raw logits, carried
+        // through every rejection round so far (E <- max(0, E - ratio_i * ep)); the sums they are compared
+        // with are sums of thousands of terms and do not suffer from cancellation.  A token that has lost its
+        // mass (it lay in an earlier A, or was itself rejected before) has none.  Every thread for itself behind the scan: by one warp, which
+        // the others then waited for, it took 0.5 us of a context's 5.8 (wide shape), and 0.9 for a second sibling.  With the logit filter
+        // the groups are bound by what they issue, and one warp does it ahead of the scan (4976 chains of 8192 tokens 1732 -> 1707 us,
+        // 1619 trees 584 -> 575; 1024 chains of 16384 tokens and small calls the same).
+        double e_xt = 0.0, p_xt = 0.0;
         // What the rejections so far have left of x~.  Read here, between the barrier that publishes the residual and the scan's: behind
         // the scan a warp that is ahead may have flagged it already.
         [[maybe_unused]] float bulk = 0.0f;
-        if (!GREEDY && ci > 0) bulk = mass(xt);
+        if (!GREEDY && ci > 0 && (!TOPK || gw == 0)) bulk = mass(xt);
+        [[maybe_unused]] auto numerators = [&]() {   // (by whole warps)
+          const Exp2Split q = S.single[iter & 1][0], p = S.single[iter & 1][1];
+          e_xt = q.y * exp2_int_d(q.n - static_cast<double>(Nq));
+          p_xt = p.y * exp2_int_d(p.n - static_cast<double>(Np));
+          if (ci > 0) {
+            if (ci <= 32) {
+              for (int i = 0; i < ci; ++i) e_xt = fmax(0.0, e_xt - S.hist[i] * p_xt);
+              if (bulk == 0.0f) e_xt = 0.0;
+            } else {
+              e_xt = static_cast<double>(bulk);
+            }
+            bool again = false;
+            for (int j = lane; j < ci; j += 32) again |= kids[j].token == xt;
+            if (__any_sync(kFull, again)) p_xt = 0.0;
+          }
+        };
+        if constexpr (!GREEDY && TOPK) {
+          if (gw == 0) {
+            numerators();
+            if (lane == 0) S.tested[0] = e_xt, S.tested[1] = p_xt;
+          }
+        }
 
         // ---- A_{k,delta}(x~): gather + prefix scan with the strict bound ----
         double thr = delta * Zq_c;   // the bound in the units of the unnormalised sums
@@ -1242,28 +1273,8 @@ __global__ void __launch_bounds__(SHAPE::THREADS, SHAPE::CTAS) lantern_context_k
             if (bad <= m) status |= LANTERN_ST_BAD_TABLE;
           }
         }
-        // The tested token's two numerators in common units, in double precision from its raw logits, carried
-        // through every rejection round so far (E <- max(0, E - ratio_i * ep)); the sums they are compared
-        // with are sums of thousands of terms and do not suffer from cancellation.  A token that has lost its
-        // mass (it lay in an earlier A, or was itself rejected before) has none.  Every thread for itself: by one thread, which
-        // the others then waited for, it took 0.5 us of a context's 5.8 (wide shape), and 0.9 for a second sibling.
-        double e_xt = 0.0, p_xt = 0.0;
-        if constexpr (!GREEDY) {
-          const Exp2Split q = S.single[iter & 1][0], p = S.single[iter & 1][1];
-          e_xt = q.y * exp2_int_d(q.n - static_cast<double>(Nq));
-          p_xt = p.y * exp2_int_d(p.n - static_cast<double>(Np));
-          if (ci > 0) {
-            if (ci <= 32) {
-              for (int i = 0; i < ci; ++i) e_xt = fmax(0.0, e_xt - S.hist[i] * p_xt);
-              if (bulk == 0.0f) e_xt = 0.0;
-            } else {
-              e_xt = static_cast<double>(bulk);
-            }
-            bool again = false;
-            for (int j = lane; j < ci; j += 32) again |= kids[j].token == xt;
-            if (__any_sync(kFull, again)) p_xt = 0.0;
-          }
-        }
+        if constexpr (!GREEDY && !TOPK) numerators();
+        if constexpr (!GREEDY && TOPK) e_xt = S.tested[0], p_xt = S.tested[1];
         // Section 4.3: accept iff r p(x~) < sum_A q, i.e. r p_xt / Zp_c < (e_xt + sm) / Zq_c, both sides times Zq_c Zp_c
         // (greedy decoding: x~ itself as every other numerator, so that the largest one compares equal to itself)
         const double qa_un = (GREEDY ? static_cast<double>(mass(xt)) : e_xt) + sm;
