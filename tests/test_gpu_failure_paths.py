@@ -10,7 +10,7 @@ import torch
 import lantern_inputs as li
 import oracle
 import paper_2410_03355_b200 as lt
-from parity import assert_parity, compare, run_gpu, to_device
+from parity import assert_parity, compare, run_gpu, tables, to_device
 
 pytestmark = pytest.mark.gpu
 
@@ -84,6 +84,37 @@ def test_a_wait_that_runs_out_in_a_large_call():
     for b in np.flatnonzero(flagged):
         assert g_tok[b] == -1 and 0 <= g_len[b] <= N
         assert np.array_equal(g_path[b, :g_len[b]], w_path[b, :g_len[b]]) and (g_path[b, g_len[b]:] == -1).all()
+
+
+@pytest.mark.parametrize("V", [512, 16384])
+def test_a_draw_made_ahead_that_runs_out(V):
+    """Few contexts, one per consumer group, every draft accepted: the copy of a leaf's row, which a group draws from ahead of the walk, is
+    never started.  Its group gives up and leaves the leaf undecided; the walk comes to it and ends there, with INTERNAL, no token and the
+    whole path.  The other sequences are what they are without it."""
+    B, N, bad = 4, 7, 2
+    inp = li.verify_inputs(B, N, V, dtype=li.BF16, has_uncond=True, cfg_scale=2.0, rho=0.9, sigma_draft=0.6, seed=3)
+    _, table = tables(li.codebook_gaussian(V, 8, seed=36), 8, inp.draft_tokens)
+    inp.draft_logits[:, :N] = inp.target_logits[0, :, :N]
+    inp.target_logits[1, :, :N] = inp.target_logits[0, :, :N]      # target and drafter are the same: accepted
+    d = to_device(inp)
+    want = _call(d, inp, table, 0.2)
+    assert (want.accept_len == N).all()
+    try:
+        lt.debug_wait_test(max_tries=3000, withhold_context=bad * (N + 1) + N)
+        ws = _poisoned_workspace(B, N, V, table.shape[1])
+        got = _call(d, inp, table, 0.2, ws)
+        bits = lt.last_status(ws)
+    finally:
+        lt.debug_wait_test(0, -1)
+    st = got.status.cpu().numpy()
+    assert st[bad] == lt.ST_INTERNAL and int(got.next_token[bad]) == -1 and int(got.accept_len[bad]) == N
+    others = np.arange(B) != bad
+    assert not st[others].any() and bits == lt.ST_INTERNAL
+    for f in ("accept_len", "next_token"):
+        assert torch.equal(getattr(got, f)[others], getattr(want, f)[others]), f
+    assert torch.equal(got.accept_path, want.accept_path)
+    again = _call(d, inp, table, 0.2)
+    assert torch.equal(again.next_token, want.next_token) and not again.status.any()
 
 
 def test_corrupt_table_entry_before_and_after_the_cut():

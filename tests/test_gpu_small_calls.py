@@ -1,4 +1,4 @@
-"""Calls of few contexts: bonus draws are made ahead of the walk, which follows what has been decided in one go; the plan has
+"""Calls of few contexts: bonus draws are made ahead of the walk, by kernels of their own; the plan has
 code of its own for chains and for trees of at most 64 drafts.  And the forms a call's arguments can take."""
 import dataclasses
 
@@ -23,12 +23,17 @@ def _inputs(B, N, tree, seed, V=512, **kw):
     return li.verify_inputs(B, N, V, dtype=li.BF16, has_uncond=True, cfg_scale=2.0, rho=0.9, sigma_draft=0.4, parents=par, seed=seed, **kw)
 
 
+def _many(N, many, V=512):
+    """One sequence; as many as have their bonus draws made ahead; one more."""
+    per_sm = 4 if N > 4 or V > 8192 else 3
+    return 1 if many == 0 else per_sm * _sms() // (N + 1) + many - 1
+
+
 @pytest.mark.parametrize("tree", [False, True])
 @pytest.mark.parametrize("N", [1, 2, 31, 32, 33, 63, 64, 70])
-@pytest.mark.parametrize("many", [0, 1, 2])   # one sequence; as many as have their bonus draws made ahead; one more
+@pytest.mark.parametrize("many", [0, 1, 2])
 def test_small_calls_against_oracle(N, tree, many):
-    B = 1 if many == 0 else 4 * _sms() // (N + 1) + many - 1
-    B = min(B, 40) if N < 31 and many == 1 else B
+    B = _many(N, many)
     inp = _inputs(B, N, tree, seed=7 * N + many)
     host, dev = tables(li.codebook_gaussian(512, 8, seed=18), 40, inp.draft_tokens)
     res = compare(inp, host, 0.4, run_gpu(inp, dev, 0.4))
@@ -36,12 +41,26 @@ def test_small_calls_against_oracle(N, tree, many):
     assert res["near"] <= near_ceiling(B)
 
 
+@pytest.mark.parametrize("N,tree,many", [(1, False, 1), (2, True, 1), (2, True, 2), (7, False, 1), (7, False, 2), (20, True, 1), (20, True, 2), (60, True, 0),
+                                         (60, True, 1), (64, True, 2)])
+def test_small_calls_of_long_rows_against_oracle(N, tree, many):
+    """The same where a group has sixteen warps and two staging areas; there are contexts enough for dynamic batches, that cross from the
+    contexts with children to those without."""
+    B = _many(N, many, 16384)
+    inp = _inputs(B, N, tree, seed=N, V=16384)
+    host, dev = tables(li.codebook_gaussian(16384, 8, seed=18), 300, inp.draft_tokens)
+    res = compare(inp, host, 0.4, run_gpu(inp, dev, 0.4))
+    assert_parity(res)
+    assert res["near"] <= near_ceiling(B)
+
+
+@pytest.mark.parametrize("V", [512, 16384])
 @pytest.mark.parametrize("N,tree", [(5, False), (20, True)])
-def test_draws_ahead_are_counted_once_and_repeat(N, tree):
+def test_draws_ahead_are_counted_once_and_repeat(N, tree, V):
     """Who makes a draw depends on timing; the outputs do not, and every sequence that ends on a leaf has one."""
     B = 12
-    inp = _inputs(B, N, tree, seed=N)
-    host, dev = tables(li.codebook_gaussian(512, 8, seed=18), 40, inp.draft_tokens)
+    inp = _inputs(B, N, tree, seed=N, V=V)
+    host, dev = tables(li.codebook_gaussian(V, 8, seed=18), 40, inp.draft_tokens)
     d = to_device(inp)
     ws = torch.empty(lt.verify_workspace_bytes(B, N, inp.V, 40), dtype=torch.uint8, device="cuda")
     want = None
