@@ -103,7 +103,7 @@ constexpr double kDegenerate = 1e-5;
 //   bits 0..1 state; walk waiting: bits 8..15 status so far, bits 16..31 drafts accepted so far;
 //   decided: bits 8..15 status, bits 16..31 accepted node + 1 (0 = none), bits 32..63 replacement token
 // A context without children starts as kWalkLeaf: the bonus draw is made by the walk when it gets there, or ahead of time by a
-// producer that has exchanged kWalkLeaf for kWalkPending first; its decided word carries kWalkDrawn.
+// producer that has put kWalkPending in the place of kWalkLeaf first (compare-and-swap); its decided word carries kWalkDrawn.
 enum : unsigned { kWalkPending = 0, kWalkWaiting = 1, kWalkDecided = 2, kWalkLeaf = 3, kWalkDrawn = 4 };
 __device__ __forceinline__ unsigned long long walk_word(unsigned state, unsigned status, unsigned count, int token = 0) {
   return state | (status << 8) | (static_cast<unsigned long long>(count) << 16) |

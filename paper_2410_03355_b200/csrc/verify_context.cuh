@@ -23,7 +23,7 @@
 // a numerator comes to common units by an exact power of two.  One group barrier then publishes E,
 // the table and the per-warp maxima and sums.  Sums over many numerators average the ex2 unit's ~1e-7
 // rounding out; the two single probabilities that decide a position, q(x~) and p(x~), are noted by a thread each
-// and formed by every thread in double precision.
+// and formed by every thread in double precision (with the logit filter by one warp).
 //
 // Deciding part, per child (Section 4.3 / Algorithm 2, second block): gather of the neighbour
 // row's numerators, double-precision scan against the strict bound (the per-warp totals tell every warp
@@ -46,7 +46,9 @@
 // as "walk waiting").  Whichever comes second goes on: along the accepted child, to the next word.  So a sequence
 // is walked by whoever completes the next piece of its path, nobody waits, and where the walk ends on
 // a context without children (or on one whose residual had no weight) the draw from that context's q
-// is the next thing the same group does.
+// is the next thing the same group does.  Two things save the walk time: a word that it has found decided by reading it, with others, is
+// followed without an exchange; and in calls of few contexts (FEW) a producer may claim a context without children ahead of the walk,
+// by compare-and-swap, so that its draw is a context like any other.
 #pragma once
 
 #include "verify_common.cuh"
@@ -460,7 +462,7 @@ __global__ void __launch_bounds__(SHAPE::THREADS, SHAPE::CTAS) lantern_context_k
   // One warp per consumer group hands out work, keeps that group's copies going and walks.  Its 32 lanes look
   // at up to 32 consecutive work slots at a time (a batch: the first one dealt statically, later ones
   // from a global counter, in sizes that shrink towards the end of the list so that the groups finish
-  // together), drop the empty and the dead ones, and lane 0 feeds the rest to the group one by one:
+  // together), drop the empty and the dead ones, and feed the rest to the group one by one, each by the lane that looked at it:
   // the context is chosen, and published, when the group has streamed the one before (so that it can go on to
   // the next drafter row without asking), and its target rows are copied as soon as a staging area is free.  The
   // next batch is loaded while the current one is being worked on, so that no round trip to the work list is
