@@ -14,7 +14,7 @@
 
 namespace lantern {
 
-#define LANTERN_CONTEXT_KERNEL_REVISION 33   // bump on every change to the fused context kernel
+#define LANTERN_CONTEXT_KERNEL_REVISION 34   // bump on every change to the fused context kernel
 
 constexpr int MAX_N = 1024;
 

@@ -326,26 +326,15 @@ __device__ __forceinline__ double warp_transposed_sum(const float (&v)[N], int l
 // q is +inf the row is reported, be it as +inf or as a NaN.)  For 2^-100 <= T <= 2^100, others are divided by.  Exact where remainder and
 // quotient are clear of the subnormal numbers, |l| >= 2^-100 and |l / T| >= 2^-125, or l = 0; below, the quotient can be off by a unit in
 // the last place.  Numerators do not see that: 2^(z log2 e - n) is 2^-n for any |z| < 2^-100.  The threshold of the logit filter does, which
-// has to be the very value of the tokens it is compared with (that of the tested one is a division's): LOOK looks for such logits, and divides
-// where there are any (1024 chains at T = 0.9 with the filter: 723 us by divisions, 587 without a look, 623 with it).
+// has to be the very value of the tokens it is compared with (that of the tested one is a division's): with the filter a thread looks for such
+// logits, in its part of the drafter row once, in the target row as it is processed, and divides where it has any (1024 chains at T = 0.9
+// with the filter: 723 us by divisions, 588 without a look, 603 with it, 622 with one at every use of the drafter row).
 static __device__ __noinline__ uint64_t divide_pair(uint64_t v, float T) {
   float lo, hi;
   unpack2(v, lo, hi);
   return pack2(__fdiv_rn(lo, T), __fdiv_rn(hi, T));
 }
-template <bool LOOK>
-__device__ __forceinline__ void divide_by_T(const VerifyParams& P, uint64_t (&z)[4]) {
-  bool fast = P.T_fast != 0;
-  if (LOOK) {
-    uint32_t least = 0xffffffffu;   // 2 bits(|l|) - 1: magnitudes in their order, zero as the largest
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      float lo, hi;
-      unpack2(z[i], lo, hi);
-      least = min(least, min(2u * __float_as_uint(lo) - 1u, 2u * __float_as_uint(hi) - 1u));
-    }
-    fast = fast && least >= P.T_least;
-  }
+__device__ __forceinline__ void divide_by_T(const VerifyParams& P, uint64_t (&z)[4], bool fast) {
   if (fast) {
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
@@ -358,6 +347,27 @@ __device__ __forceinline__ void divide_by_T(const VerifyParams& P, uint64_t (&z)
 #pragma unroll
     for (int i = 0; i < 4; ++i) z[i] = divide_pair(z[i], P.T);
   }
+}
+// the smallest of `least` and eight raw logits' magnitudes, each as 2 bits(|l|) - 1: zero is the largest.  (From the words as they lie there: with
+// the values widened first, which the sweeps widen again, the same call took 717 us.)
+template <bool BF16>
+__device__ __forceinline__ uint32_t least_magnitude(const Raw8<BF16>& d, uint32_t least) {
+  const uint32_t w[8] = {d.a.x, d.a.y, d.a.z, d.a.w, BF16 ? 0u : d.b.x, BF16 ? 0u : d.b.y, BF16 ? 0u : d.b.z, BF16 ? 0u : d.b.w};
+#pragma unroll
+  for (int i = 0; i < (BF16 ? 4 : 8); ++i)
+    least = BF16 ? min(least, min((w[i] << 17) - 1u, ((w[i] >> 16) << 17) - 1u)) : min(least, 2u * w[i] - 1u);
+  return least;
+}
+// are there four pairs of logits whose quotients divide_by_T forms without a division?
+__device__ __forceinline__ bool quotients_fast(const VerifyParams& P, const uint64_t (&z)[4]) {
+  uint32_t least = 0xffffffffu;
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    float lo, hi;
+    unpack2(z[i], lo, hi);
+    least = min(least, min(2u * __float_as_uint(lo) - 1u, 2u * __float_as_uint(hi) - 1u));
+  }
+  return least >= P.T_least;
 }
 
 // one bit per token of a thread
@@ -916,6 +926,7 @@ __global__ void __launch_bounds__(SHAPE::THREADS, SHAPE::CTAS) lantern_context_k
     auto sum_of = [&](int p) { return NP <= 2 ? tq_sum[NP <= 2 ? p : 0] : S.slice[1024 + p * GT + gt]; };
     float z_max = ninf;               // GREEDY: this thread's largest logit
     Raw8<BF16> raw[CH];           // the drafter row
+    bool fast_d = P.T_fast != 0;  // its quotients by the temperature are formed without a division
     auto load_drafter = [&](auto whole) {
 #pragma unroll
       for (int c = 0; c < CH; ++c) {
@@ -943,7 +954,7 @@ __global__ void __launch_bounds__(SHAPE::THREADS, SHAPE::CTAS) lantern_context_k
       for (int c = 0; c < CH; ++c) {
         uint64_t z2[4];
         raw8_pairs<BF16>(raw[c], z2);
-        if (!TONE) divide_by_T<TOPK>(P, z2);
+        if (!TONE) divide_by_T(P, z2, fast_d);
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
           float lo, hi;
@@ -989,7 +1000,7 @@ __global__ void __launch_bounds__(SHAPE::THREADS, SHAPE::CTAS) lantern_context_k
 #pragma unroll
               for (int i = 0; i < 4; ++i) c2[i] = fma2(s2, sub2(c2[i], u2[i]), u2[i]);   // l_u + s (l_c - l_u)
             }
-            if (!TONE && !TOPK) divide_by_T<false>(P, c2);
+            if (!TONE && !TOPK) divide_by_T(P, c2, P.T_fast != 0);
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
               uint64_t l2 = c2[i];
@@ -1041,22 +1052,26 @@ __global__ void __launch_bounds__(SHAPE::THREADS, SHAPE::CTAS) lantern_context_k
         if (full) load_drafter(std::true_type{});
         else load_drafter(std::false_type{});
       }
+      if constexpr (TOPK && !TONE) {
+        uint32_t least = ~0u;
+#pragma unroll
+        for (int c = 0; c < CH; ++c) least = least_magnitude<BF16>(raw[c], least);
+        fast_d = fast_d && least >= P.T_least;
+      }
       if constexpr (TOPK && !GREEDY) {   // the drafter row's threshold, from the registers that hold the row
-        auto own_value = [&](int c, float (&z)[8], auto look) {
+        auto own = [&](int c, float (&z)[8]) {
           uint64_t z2[4];
           raw8_pairs<BF16>(raw[c], z2);
-          if (!TONE) divide_by_T<decltype(look)::value>(P, z2);
+          if (!TONE) divide_by_T(P, z2, fast_d);
 #pragma unroll
           for (int i = 0; i < 4; ++i) unpack2(z2[i], z[2 * i], z[2 * i + 1]);
         };
-        auto sampled = [&](int c, float (&z)[8]) { own_value(c, z, std::false_type{}); };   // (it only decides where to look)
-        auto own = [&](int c, float (&z)[8]) { own_value(c, z, std::true_type{}); };
         auto again = [&](int c, float (&z)[8]) {
           row_logits<BF16, TONE>(P, P.draft, static_cast<size_t>(item) * V, c * GT + gt, z);
         };
         auto pairs = [&](int c, uint32_t (&w)[4]) { w[0] = raw[c].a.x, w[1] = raw[c].a.y, w[2] = raw[c].a.z, w[3] = raw[c].a.w; };
-        if constexpr (BF16 && TONE) tp = group_kth_largest<SHAPE, CH, CH, true>(P, sampled, pairs, own, again, V, S, grp, gt, search3);
-        else tp = group_kth_largest<SHAPE, CH, CH, false>(P, sampled, own, own, again, V, S, grp, gt, search3);
+        if constexpr (BF16 && TONE) tp = group_kth_largest<SHAPE, CH, CH, true>(P, own, pairs, own, again, V, S, grp, gt, search3);
+        else tp = group_kth_largest<SHAPE, CH, CH, false>(P, own, own, own, again, V, S, grp, gt, search3);
       }
       if (!GREEDY) reduce_drafter();
       if (!GREEDY && !TOPK && gt < 2) note_single();
@@ -1076,7 +1091,7 @@ __global__ void __launch_bounds__(SHAPE::THREADS, SHAPE::CTAS) lantern_context_k
 #pragma unroll
             for (int i = 0; i < 4; ++i) c2[i] = fma2(pack2(P.cfg_scale, P.cfg_scale), sub2(c2[i], u2[i]), u2[i]);
           }
-          if (!TONE) divide_by_T<decltype(look)::value>(P, c2);
+          if (!TONE) divide_by_T(P, c2, P.T_fast != 0 && (!decltype(look)::value || quotients_fast(P, c2)));
 #pragma unroll
           for (int i = 0; i < 4; ++i) unpack2(c2[i], z[2 * i], z[2 * i + 1]);
         };
@@ -1357,7 +1372,7 @@ __global__ void __launch_bounds__(SHAPE::THREADS, SHAPE::CTAS) lantern_context_k
               {
                 uint64_t z2[4];
                 raw8_pairs<BF16>(drafted, z2);
-                if (!TONE) divide_by_T<TOPK>(P, z2);
+                if (!TONE) divide_by_T(P, z2, fast_d);
 #pragma unroll
                 for (int i = 0; i < 4; ++i) {
                   unpack2(z2[i], z[2 * i], z[2 * i + 1]);
